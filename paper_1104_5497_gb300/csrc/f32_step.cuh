@@ -1,0 +1,216 @@
+// f32_step.cuh -- the building blocks of the FP32 group tracker (xy_track_group.cuh):
+// arithmetic in pairs (f32x2), compensated sums of pairs, and one path's step control.
+#pragma once
+
+#include "xy_track.cuh"
+
+// ------------------------------------------------------------- f32x2 pairs --
+__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ float2 f2dup(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 f2neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 f2add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 f2mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// a - b (the product with -1 is exact: one rounding, as a subtraction)
+__device__ __forceinline__ float2 f2sub(float2 a, float2 b) {
+    return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
+}
+__device__ __forceinline__ float2 f2i(float2 a) { return make_float2(-a.y, a.x); }   // i a
+__device__ __forceinline__ cx<float> f2c(float2 a) { return cx<float>{a.x, a.y}; }
+__device__ __forceinline__ float2 c2f(cx<float> a) { return make_float2(a.re, a.im); }
+
+// A pair of two-word numbers (EFT, nphc_internal.cuh): the same error-free transformations
+// on both halves.
+struct ext2 {
+    float2 hi, lo;
+};
+
+// acc += c v, nc = -c; as ext_acc
+__device__ __forceinline__ void acc2(ext2 &acc, float2 c, float2 nc, float2 v) {
+    const float2 np = f2mul(nc, v);        // -(the rounded product)
+    const float2 e = f2fma(c, v, np);      // its rounding error
+    const float2 s = f2sub(acc.hi, np);
+    const float2 bb = f2sub(s, acc.hi);
+    const float2 e2 = f2sub(f2sub(acc.hi, f2sub(s, bb)), f2add(np, bb));
+    acc.hi = s;
+    acc.lo = f2add(acc.lo, f2add(e, e2));
+}
+// acc += c (v.hi + v.lo); as ext_acc_ext
+__device__ __forceinline__ void acc2_ext(ext2 &acc, float2 c, float2 nc, const ext2 &v) {
+    acc2(acc, c, nc, v.hi);
+    acc.lo = f2fma(c, v.lo, acc.lo);
+}
+__device__ __forceinline__ void acc2_ext(ext2 &acc, float c, const ext2 &v) {
+    acc2_ext(acc, f2dup(c), f2dup(-c), v);
+}
+// (a.hi + a.lo) + (b.hi + b.lo)
+__device__ __forceinline__ ext2 ext2_add(const ext2 &a, const ext2 &b) {
+    const float2 s = f2add(a.hi, b.hi);
+    const float2 bb = f2sub(s, a.hi);
+    const float2 e = f2add(f2sub(a.hi, f2sub(s, bb)), f2sub(b.hi, bb));
+    return ext2{s, f2add(e, f2add(a.lo, b.lo))};
+}
+__device__ __forceinline__ ext2 ext2_scale(float c, const ext2 &a) {   // c a power of two
+    return ext2{f2mul(f2dup(c), a.hi), f2mul(f2dup(c), a.lo)};
+}
+__device__ __forceinline__ ext2 ext2_i(const ext2 &v) { return ext2{f2i(v.hi), f2i(v.lo)}; }
+// acc += a b for complex a, b: exact products
+__device__ __forceinline__ void acc2_cmul(ext2 &acc, float2 a, float2 b) {
+    acc2(acc, f2dup(a.x), f2dup(-a.x), b);
+    acc2(acc, f2dup(a.y), f2dup(-a.y), f2i(b));
+}
+
+// The rows (-H_f, -H_g) of one site at (p, q), compensated, from the compensated sums
+// U_p, U_q (xy_residual_comp in xy_solve.cuh, with the squares shared:
+// x^2 - 1 = B + h, y^2 - 1 = -B + h, B = (p^2 + q^2) / 4, h = G / 2 - 1 / 2, G = p q - 1).
+__device__ __forceinline__ void f32_residual_rows(float2 pk, float2 qk, const ext2 &up, const ext2 &uq,
+                                                  float s, float hs, float gr, float gi, float2 &rf,
+                                                  float2 &rg) {
+    const ext2 zero = {f2dup(0.0f), f2dup(0.0f)};
+    ext2 d = zero;   // D = q U_p - p U_q, f = i D / 2
+    acc2_ext(d, qk.x, up);
+    acc2_ext(d, qk.y, ext2_i(up));
+    acc2_ext(d, -pk.x, uq);
+    acc2_ext(d, -pk.y, ext2_i(uq));
+    ext2 G = {f2(-1.0f, 0.0f), f2dup(0.0f)}, B = zero;
+    acc2_cmul(G, pk, qk);
+    acc2_cmul(B, pk, pk);
+    acc2_cmul(B, qk, qk);
+    B = ext2_scale(0.25f, B);
+    const ext2 nB = {f2neg(B.hi), f2neg(B.lo)};
+    const ext2 half = {f2(-0.5f, 0.0f), f2dup(0.0f)};
+    const ext2 h = ext2_add(ext2_scale(0.5f, G), half);
+    const ext2 X = ext2_add(h, B), Y = ext2_add(h, nB);
+    ext2 hf = zero, hg = zero;   // H_f = gomt X + t f ;  H_g = gomt Y + t G
+    acc2_ext(hf, gr, X);
+    acc2_ext(hf, gi, ext2_i(X));
+    acc2_ext(hf, hs, ext2_i(d));
+    acc2_ext(hg, gr, Y);
+    acc2_ext(hg, gi, ext2_i(Y));
+    acc2_ext(hg, s, G);
+    rf = f2neg(f2add(hf.hi, hf.lo));
+    rg = f2neg(f2add(hg.hi, hg.lo));
+}
+
+// ------------------------------------------------------------ step control --
+// Time in units of 2^-53, the grid of the doubles in [1/2, 1): 1 - t is exact, and the step
+// logic costs no FP64 instruction (67 cycles of a scheduler each, measured, whatever the
+// number of lanes).
+typedef long long f32_time;
+#define F32_ONE (1ll << 53)
+__device__ __forceinline__ f32_time to_f32_time(double t) {   // clamped: beyond 256 no step differs
+    return __double2ll_rn(fmin(fmax(t, -256.0), 256.0) * 9007199254740992.0);
+}
+__device__ __forceinline__ float time_float(f32_time t) { return __ll2float_rn(t) * 1.1102230246251565e-16f; }
+__device__ __forceinline__ double time_double(f32_time t) { return __ll2double_rn(t) * 1.1102230246251565e-16; }
+
+struct F32Ctl {   // XYCtl in the trackers' own units
+    f32_time h0, hmax, hmin, tend, zone, near_end;
+    float rdiv, rband, eps, trust, kappa;
+    __device__ __forceinline__ explicit F32Ctl(const XYCtl &C)
+        : h0(to_f32_time(C.h0)), hmax(to_f32_time(C.hmax)), hmin(max(to_f32_time(C.hmin), (f32_time)1)),
+          tend(to_f32_time(C.t_end)), zone(to_f32_time(CRAWL_ZONE)), near_end(to_f32_time(NEAR_END)),
+          rdiv((float)C.rdiv), rband((float)(C.rdiv * (1.0 + RDIV_BAND))), eps((float)C.eps),
+          trust((float)C.trust), kappa((float)C.kappa) {}
+};
+
+// One path's step control: the rules of xy_track.cuh (track_body) for the FP32 pass.
+struct F32Step {
+    f32_time t, h, hacc, tck, hck, tmark;
+    float zlast;
+    int clean, since, run, rejects, attempts, steps, solves, newton;
+    bool have_ck, far;
+
+    __device__ __forceinline__ void start(f32_time t0, f32_time h0) {
+        t = t0;
+        h = hacc = h0;
+        tmark = F32_ONE - t0;
+        tck = hck = 0;
+        zlast = 0.0f;
+        clean = since = run = rejects = attempts = 0;
+        have_ck = far = false;
+    }
+    // a path heading out takes steps of at most KAPPA_FAR (1 - t)
+    __device__ __forceinline__ void cap() {
+        if (far) h = min(h, (f32_time)__umul64hi((unsigned long long)(F32_ONE - t),
+                                                 (unsigned long long)(KAPPA_FAR * 18446744073709551616.0)));
+    }
+    // length and end of the step
+    __device__ __forceinline__ void len(const F32Ctl &K, f32_time &hh, f32_time &t1) const {
+        const bool last = t + h >= K.tend;
+        t1 = last ? K.tend : t + h;
+        hh = last ? K.tend - t : h;
+    }
+    // The step to t1 is accepted at ||z||_inf = zi; returns the path's status.  save: the
+    // point becomes the hand-off checkpoint (the last clean point of the end zone: accepted,
+    // with the step before it accepted too).
+    __device__ __forceinline__ int accept(const F32Ctl &K, const XYCtl &C, f32_time t1, float zi, bool &save) {
+        int status = NPHC_PATH_RUNNING;
+        attempts++;
+        clean = rejects == 0 ? clean + 1 : 1;
+        t = t1;
+        const f32_time left = F32_ONE - t;
+        const bool zone = left < K.zone;
+        far = zone && zi > (float)FAR_NORM && zi > (float)FAR_GROWTH * zlast;
+        zlast = zi;
+        steps++;
+        rejects = 0;
+        hacc = h;
+        if (++run >= C.grow_after) {
+            run = 0;
+            h = min(2 * h, K.hmax);
+        }
+        if (zi > K.rdiv)   // marginal crossings close to t = 1 are FP64's to judge
+            status = (C.handoff && left < K.near_end && zi <= K.rband) ? NPHC_PATH_HANDOFF : NPHC_PATH_DIVERGED;
+        else if (t >= K.tend)
+            status = NPHC_PATH_REACHED;
+        save = C.handoff && (clean >= 2 || !have_ck) && status == NPHC_PATH_RUNNING && zone;
+        if (save) {
+            tck = t;
+            hck = hacc;
+            have_ck = true;
+        }
+        // crawl test near t = 1: 1 - t must at least halve every crawl_steps accepted steps
+        if (status == NPHC_PATH_RUNNING && C.crawl_steps > 0 && zone) {
+            if (++since >= C.crawl_steps) {
+                if (2 * left > tmark) status = C.handoff ? NPHC_PATH_HANDOFF : NPHC_PATH_MIN_STEP;
+                tmark = left;
+                since = 0;
+            }
+        } else {
+            tmark = left;
+            since = 0;
+        }
+        return status;
+    }
+    __device__ __forceinline__ int reject(const F32Ctl &K, const XYCtl &C) {
+        attempts++;
+        run = 0;
+        rejects++;
+        h >>= 1;
+        if (h < K.hmin) return C.handoff ? NPHC_PATH_HANDOFF : NPHC_PATH_MIN_STEP;
+        return C.handoff && rejects >= 10 ? NPHC_PATH_HANDOFF : NPHC_PATH_RUNNING;
+    }
+    // the step budget, after an attempt that left the path running
+    __device__ __forceinline__ int budget(const XYCtl &C, int status) const {
+        if (status != NPHC_PATH_RUNNING || attempts < C.max_steps) return status;
+        return C.handoff ? NPHC_PATH_HANDOFF : NPHC_PATH_STEP_BUDGET;
+    }
+    // what the endpoint arrays get besides the point (the checkpoint's, for a path handed off
+    // after one)
+    __device__ __forceinline__ bool from_checkpoint(int status) const {
+        return have_ck && (status == NPHC_PATH_HANDOFF || status == NPHC_PATH_HANDOFF_COND);
+    }
+    __device__ __forceinline__ void store(const EPView &ep, int64_t e, int status) const {
+        const bool handed = status == NPHC_PATH_HANDOFF || status == NPHC_PATH_HANDOFF_COND;
+        const bool ck = handed && have_ck;
+        ep.t[e] = time_double(ck ? tck : t);
+        ep.h[e] = time_double(ck ? hck : (handed ? hacc : h));
+        ep.status[e] = status;
+        ep.steps[e] = steps;
+        ep.solves[e] = solves;
+        ep.newton[e] = newton;
+    }
+};
+
+enum { F32_GO_ON, F32_ACCEPT, F32_REJECT, F32_ANCHORED };   // a step attempt's verdict

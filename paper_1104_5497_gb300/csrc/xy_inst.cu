@@ -3,6 +3,8 @@
 //   -DNPHC_INST_M=<M>  (free sites, N = M + 1)
 //   -DNPHC_INST_KIND=0 (FP32 tracker), 1 (FP64 tracker), 2 (FP64 refinement,
 //   certification, classification, adjoint) or 3 (Cauchy endgame)
+#include <algorithm>
+
 #include "xy_dispatch.cuh"
 
 #if NPHC_INST_KIND == 3
@@ -37,8 +39,120 @@ cudaError_t NPHC_CAT(launch_xy_cauchy_m, NPHC_INST_M)(const XYSys &sys, const EG
 }
 #endif
 
-#if NPHC_INST_KIND == 0 || NPHC_INST_KIND == 1
-#include "xy_track.cuh"
+#if NPHC_INST_KIND == 0
+#include "xy_track_group.cuh"
+
+// The FP32 pass has two kernels: one path per thread (xy_track.cuh) and four lanes per path
+// (xy_track_group.cuh).  One wave of the first takes its paths' latency (100 attempts of six
+// solves of one warp each) however few they are; four lanes shorten every solve, and sixteen
+// warps per SM hide each other's latency where seven cannot.  Measured (GB300, FP32 pass alone,
+// per-thread -> group, ms): 256 paths of N = 5 2.59 -> 1.02; 4,096 of N = 7 7.27 -> 2.40; 16,384 of
+// N = 8 11.3 -> 4.4; 65,536 of N = 9 25.4 -> 14.5; of N = 11, 12, 13: 262,144 154 -> 133, 262,144
+// 209 -> 148, 80,000 100 -> 55.6.  At M = 9 (N = 10) three of twelve row slots idle: 32,768 paths
+// 20.6 -> 18.9, 65,536 34.5 -> 33.9, but 262,144 109 -> 121.  So: the group kernel, unless over a
+// fifth of its slots idle and the per-thread kernel has more than two waves of paths.
+template <int M>
+static bool use_group(int64_t items, int64_t wave) {
+    return 5 * M >= 4 * GrpLayout<M>::ROWS || items <= 2 * wave;
+}
+
+static cudaError_t device_sms(int &sms) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return e;
+}
+
+// Shared memory limit and resident blocks per SM of a kernel (the limit is set once per process
+// and instantiation: attr).
+template <class K>
+static cudaError_t kernel_blocks(K k, int threads, size_t smem, bool &attr, int &per) {
+    if (!attr) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        attr = true;
+    }
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, threads, smem);
+    per = std::max(per, 1);
+    return e;
+}
+
+// Grid of a group launch over `items` paths: every SM filled (or with `warps` warps in all, if
+// given), but no more blocks than the paths need at one warp per scheduler first and eight
+// paths per warp then.
+static int group_grid(int sms, int per, int warps, int64_t items, int64_t state_threads) {
+    int64_t full = (int64_t)sms * per;
+    if (warps > 0) full = std::min<int64_t>(full, (warps + GRP_WARPS - 1) / GRP_WARPS);
+    const int64_t one = (int64_t)sms * GRP_WARPS;
+    const int64_t paths = std::min<int64_t>(std::max<int64_t>((items + one - 1) / one, 1), GRP_PATHS);
+    const int64_t need = std::max<int64_t>((items + paths * GRP_WARPS - 1) / (paths * GRP_WARPS), 1);
+    const int64_t cap = state_threads / (32 * GRP_WARPS);   // its checkpoints live in the scratch
+    return (int)std::min(std::min(full, need), cap);
+}
+
+cudaError_t NPHC_CAT(launch_xy_track_f32_m, NPHC_INST_M)(const XYSys &sys, const XYCtl &ctl,
+                                                         const EPView &ep, const WorkList &wl,
+                                                         int grid, cudaStream_t st) {
+    constexpr int M = NPHC_INST_M, BLK = NPHC_TRACK_BLOCK;
+    static bool attr_t = false, attr_g = false;
+    const size_t smem_t = xy_smem_per_thread<M, float>() * BLK, smem_g = grp_smem_per_block<M>(false);
+    auto kt = xy_track_kernel<M, float, BLK>;
+    auto kg = xy_track_group_kernel<M>;
+    int sms = 0, per_t = 0, per_g = 0;
+    cudaError_t e = device_sms(sms);
+    if (e == cudaSuccess) e = kernel_blocks(kt, BLK, smem_t, attr_t, per_t);
+    if (e == cudaSuccess) e = kernel_blocks(kg, 32 * GRP_WARPS, smem_g, attr_g, per_g);
+    if (e != cudaSuccess) return e;
+    if (use_group<M>(ep.count, (int64_t)sms * per_t * BLK)) {
+        const int gg = group_grid(sms, per_g, grid, ep.count, wl.state_threads);
+        if (gg <= 0) return cudaErrorInvalidValue;
+        kg<<<gg, 32 * GRP_WARPS, smem_g, st>>>(sys, ctl, ep, wl);
+    } else {
+        const int full = sms * per_t;   // persistent grid: every SM filled
+        if (grid <= 0 || grid > full) grid = full;
+        grid = std::min(grid, (int)(wl.state_threads / BLK));   // the scratch holds state for this many
+        if (grid <= 0) return cudaErrorInvalidValue;
+        kt<<<grid, BLK, smem_t, st>>>(sys, ctl, ep, wl);
+    }
+    nphc_launch_counter(1);
+    return cudaGetLastError();
+}
+
+// The FP32 pass of a batch group: one persistent grid over every path of the group's
+// instances (one queue), at most every SM filled.
+cudaError_t NPHC_CAT(launch_xy_track_f32_batch_m, NPHC_INST_M)(const BatchGroup &bg,
+                                                               const XYCtl &ctl,
+                                                               const WorkList &wl, int grid,
+                                                               cudaStream_t st) {
+    constexpr int M = NPHC_INST_M, BLK = NPHC_TRACK_BLOCK;
+    if (bg.total <= 0) return cudaSuccess;
+    static bool attr_t = false, attr_g = false;
+    const size_t smem_t = xy_smem_per_thread<M, float>() * BLK, smem_g = grp_smem_per_block<M>(true);
+    auto kt = xy_track_batch_kernel<M, float, BLK>;
+    auto kg = xy_track_group_batch_kernel<M>;
+    int sms = 0, per_t = 0, per_g = 0;
+    cudaError_t e = device_sms(sms);
+    if (e == cudaSuccess) e = kernel_blocks(kt, BLK, smem_t, attr_t, per_t);
+    if (e == cudaSuccess) e = kernel_blocks(kg, 32 * GRP_WARPS, smem_g, attr_g, per_g);
+    if (e != cudaSuccess) return e;
+    if (use_group<M>(bg.total, (int64_t)sms * per_t * BLK)) {
+        const int gg = group_grid(sms, per_g, grid, bg.total, wl.state_threads);
+        if (gg <= 0) return cudaErrorInvalidValue;
+        kg<<<gg, 32 * GRP_WARPS, smem_g, st>>>(bg.sys, bg.ep, bg.off, bg.n, ctl, wl);
+    } else {
+        const int full = sms * per_t;
+        if (grid <= 0 || grid > full) grid = full;
+        const int64_t need = (bg.total + BLK - 1) / BLK;   // no more threads than paths
+        if (grid > need) grid = (int)need;
+        grid = std::min(grid, (int)(wl.state_threads / BLK));
+        if (grid <= 0) return cudaErrorInvalidValue;
+        kt<<<grid, BLK, smem_t, st>>>(bg.sys, bg.ep, bg.off, bg.n, ctl, wl);
+    }
+    nphc_launch_counter(1);
+    return cudaGetLastError();
+}
+#endif
+
 #if NPHC_INST_KIND == 1
 #include "xy_track_warp.cuh"
 
@@ -74,23 +188,12 @@ cudaError_t NPHC_CAT(launch_xy_track_f64w_m, NPHC_INST_M)(const XYSys &sys, cons
     nphc_launch_counter(1);
     return cudaGetLastError();
 }
-#endif
-
-#if NPHC_INST_KIND == 0
-using RT = float;
-constexpr int BLK = NPHC_TRACK_BLOCK;
-#define NPHC_FN NPHC_CAT(launch_xy_track_f32_m, NPHC_INST_M)
-#else
-using RT = double;
-constexpr int BLK = NPHC_TRACK_BLOCK;
-#define NPHC_FN NPHC_CAT(launch_xy_track_f64_m, NPHC_INST_M)
-#endif
-
-cudaError_t NPHC_FN(const XYSys &sys, const XYCtl &ctl, const EPView &ep, const WorkList &wl,
-                    int grid, cudaStream_t st) {
-    constexpr int M = NPHC_INST_M;
-    const size_t smem = xy_smem_per_thread<M, RT>() * BLK;
-    auto k = xy_track_kernel<M, RT, BLK>;
+cudaError_t NPHC_CAT(launch_xy_track_f64_m, NPHC_INST_M)(const XYSys &sys, const XYCtl &ctl,
+                                                         const EPView &ep, const WorkList &wl,
+                                                         int grid, cudaStream_t st) {
+    constexpr int M = NPHC_INST_M, BLK = NPHC_TRACK_BLOCK;
+    const size_t smem = xy_smem_per_thread<M, double>() * BLK;
+    auto k = xy_track_kernel<M, double, BLK>;
     static bool attr_set = false;   // once per process for this instantiation
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -111,43 +214,9 @@ cudaError_t NPHC_FN(const XYSys &sys, const XYCtl &ctl, const EPView &ep, const 
     nphc_launch_counter(1);
     return cudaGetLastError();
 }
-
-#if NPHC_INST_KIND == 0
-// The FP32 pass of a batch group: one persistent grid over every path of the group's
-// instances (one queue), at most every SM filled.
-cudaError_t NPHC_CAT(launch_xy_track_f32_batch_m, NPHC_INST_M)(const BatchGroup &bg,
-                                                               const XYCtl &ctl,
-                                                               const WorkList &wl, int grid,
-                                                               cudaStream_t st) {
-    constexpr int M = NPHC_INST_M;
-    if (bg.total <= 0) return cudaSuccess;
-    const size_t smem = xy_smem_per_thread<M, RT>() * BLK;
-    auto k = xy_track_batch_kernel<M, RT, BLK>;
-    static bool attr_set = false;   // once per process for this instantiation
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
-    int dev = 0, sms = 0, per = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, BLK, smem);
-    if (e != cudaSuccess) return e;
-    const int full = sms * (per > 0 ? per : 1);
-    if (grid <= 0 || grid > full) grid = full;
-    const int64_t need = (bg.total + BLK - 1) / BLK;   // no more threads than paths
-    if (grid > need) grid = (int)need;
-    const int cap = (int)(wl.state_threads / BLK);
-    if (grid > cap) grid = cap;
-    if (grid <= 0) return cudaErrorInvalidValue;
-    k<<<grid, BLK, smem, st>>>(bg.sys, bg.ep, bg.off, bg.n, ctl, wl);
-    nphc_launch_counter(1);
-    return cudaGetLastError();
-}
 #endif
 
-#elif NPHC_INST_KIND == 2
+#if NPHC_INST_KIND == 2
 #include "xy_endgame.cuh"
 
 cudaError_t NPHC_CAT(launch_xy_refine_certify_m, NPHC_INST_M)(const XYSys &sys, double tol_sol,
