@@ -191,7 +191,7 @@ struct QuadProblem {
     }
 };
 
-// Endgame policy (see EGXY): P, DP dense from the terms, z in G's X.
+// Refinement policy (see refine_body): P, DP dense from the terms, z in G's X.
 template <int NV>
 struct EGQuad {
     using Sys = QSys;
@@ -249,7 +249,7 @@ struct EGQuad {
                 if (T.b >= 0) G.setS(i, T.b, cadd(G.S(i, T.b), cmul(c, wa)));
             }
         }
-        // ||DP||_F, kept in the unused second half of R for jac_fro
+        // ||DP||_F, kept in the spare entry of R for jac_fro
         double f = 0.0;
 #pragma unroll 1
         for (int c = 0; c < NV; c++)
@@ -292,7 +292,7 @@ template <int NV>
 __global__ void __launch_bounds__(EG_BLOCK)
     quad_refine_certify_kernel(const __grid_constant__ QSys S, double tol_sol, double refine_eps,
                                int refine_iters, const EPView ep, const WorkList wl) {
-    refine_body<EGQuad<NV>>(S, tol_sol, refine_eps, refine_iters, ep, wl, 0);
+    refine_body<EGQuad<NV>>(S, tol_sol, refine_eps, refine_iters, ep, wl);
 }
 
 template <int NV>

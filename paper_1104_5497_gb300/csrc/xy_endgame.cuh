@@ -24,17 +24,17 @@
 //   [[0, D^-1], [S^-1, -S^-1 C D^-1]],
 // so a solve costs one M x M system, and, W being unitary,
 //   ||DP^-1||_F^2 = sum_j iv_j^2 + ||S^-1||_F^2 + ||S^-1 C D^-1||_F^2
-// needs only 2M triangular solves after one Householder QR of S (stored: R above the
-// diagonal with a real diagonal, the reflectors below, conj(tau) aside).
+// needs only 2M triangular solves after one factorisation of S.  The XY ring's kernel is
+// xy_refine_group.cuh (four lanes per endpoint); this file holds the classification and the
+// adjoint, and the rules of refinement and certification as a generic body, one endpoint per
+// thread with a Householder QR of DP, for quadratic systems (quad.cuh).
 //
 // The refinement certifies the iterate whose Newton correction met the tolerance, from
 // the factorisation of that iteration, and outputs its Newton iterate.
 //
-// Storage: one endpoint per thread, interleaved across the 32 threads of a block
-// (element i of a thread's array at [i * 32 + lane]) so that the rolled loops index it
-// at run time without local memory: the per-site arrays, point and vectors in shared
-// memory, the M x M factor in shared memory too or, when a solve provides a scratch
-// buffer, in global memory (L2-resident), which leaves room for more warps per SM.
+// Storage of the generic body: interleaved across the 32 threads of a block in shared memory
+// (element i of a thread's array at [i * 32 + lane]), so that the rolled loops index it at run
+// time without local memory.
 #pragma once
 
 #include "nphc_internal.cuh"
@@ -55,109 +55,30 @@ struct EGVec {
     __device__ __forceinline__ void set(int i, cx<double> v) const { p[i * EG_BLOCK] = v; }
 };
 
-// Per-thread working set of the endgame (complex doubles, in this order).  The M x M
-// matrix S comes last: in shared memory with the rest, or (refinement launches given a
-// scratch buffer) in global memory, interleaved across the launch's threads, so that the
-// shared part alone sets the occupancy.
+// Per-thread working set of the refinement (complex doubles, in this order).
 template <int M>
 struct EGLayout {
     static constexpr int TQ = 0;                // conj(tau) of the reflectors
-    static constexpr int AH = TQ + M;           // frame a^
-    static constexpr int BH = AH + M;           // frame b^
-    static constexpr int IV = BH + M;           // iv (real part)
-    static constexpr int AD = IV + M;           // d f_j / d c_j
-    static constexpr int BD = AD + M;           // d f_j / d s_j
-    static constexpr int X = BD + M;            // c_1..c_M
-    static constexpr int Y = X + M;             // s_1..s_M
-    static constexpr int R = Y + M;             // right-hand side / residual, 2M
-    static constexpr int D = R + 2 * M;         // solution, 2M
-    static constexpr int S = D + 2 * M;         // M x M, column-major: entry (i, c) at c M + i
+    static constexpr int X = TQ + M;            // z
+    static constexpr int R = X + M;             // right-hand side / residual (and one scalar)
+    static constexpr int D = R + M + 1;         // solution
+    static constexpr int S = D + M;             // M x M, column-major: entry (i, c) at c M + i
     static constexpr int TOTAL = S + M * M;
 };
 
-// Shared memory per thread, with S or without it (S in a global scratch buffer).
 template <int M>
-constexpr size_t eg_smem_per_thread(bool with_s = true) {
-    return sizeof(cx<double>) * (size_t)(with_s ? EGLayout<M>::TOTAL : EGLayout<M>::S);
+constexpr size_t eg_smem_per_thread() {
+    return sizeof(cx<double>) * (size_t)EGLayout<M>::TOTAL;
 }
 
 template <int M>
 struct EG {
     cx<double> *base;   // this thread's first entry in shared memory (stride EG_BLOCK)
-    cx<double> *sp;     // this thread's entry (0, 0) of S, in shared or global memory
-    int64_t ss;         // S's stride between entries
+    cx<double> *sp;     // this thread's entry (0, 0) of S
     __device__ __forceinline__ EGVec v(int off) const { return EGVec{base + off * EG_BLOCK}; }
-    __device__ __forceinline__ cx<double> S(int i, int c) const { return sp[(c * M + i) * ss]; }
-    __device__ __forceinline__ void setS(int i, int c, cx<double> a) const { sp[(c * M + i) * ss] = a; }
+    __device__ __forceinline__ cx<double> S(int i, int c) const { return sp[(c * M + i) * EG_BLOCK]; }
+    __device__ __forceinline__ void setS(int i, int c, cx<double> a) const { sp[(c * M + i) * EG_BLOCK] = a; }
 };
-
-// P(z) with exact products and double-double sums, rounded once: at ||z|| >> 1 the
-// terms of P are ~||z||^2 and a plain double sum is dominated by rounding, which would
-// limit the refinement and inflate beta (hence alpha) of large-norm solutions.
-struct dd {
-    double hi, lo;
-};
-
-__device__ __forceinline__ dd dd_two_prod(double a, double b) {
-    const double p = __dmul_rn(a, b);
-    return dd{p, __fma_rn(a, b, -p)};
-}
-
-__device__ __forceinline__ dd dd_add(dd a, dd b) {
-    const double s = __dadd_rn(a.hi, b.hi);
-    const double bb = __dsub_rn(s, a.hi);
-    const double e = __dadd_rn(__dsub_rn(a.hi, __dsub_rn(s, bb)), __dsub_rn(b.hi, bb));
-    const double lo = __dadd_rn(e, __dadd_rn(a.lo, b.lo));
-    const double hi = __dadd_rn(s, lo);
-    return dd{hi, __dsub_rn(lo, __dsub_rn(hi, s))};
-}
-
-// a * b with a double-double, b double
-__device__ __forceinline__ dd dd_mul_d(dd a, double b) {
-    const dd p = dd_two_prod(a.hi, b);
-    const double lo = __fma_rn(a.lo, b, p.lo);
-    const double hi = __dadd_rn(p.hi, lo);
-    return dd{hi, __dsub_rn(lo, __dsub_rn(hi, p.hi))};
-}
-
-__device__ __forceinline__ double dd_val(dd a) { return __dadd_rn(a.hi, a.lo); }
-
-// -P(z) into R, with exact products and double-double sums; returns ||P||_inf.
-template <int M>
-__device__ double eg_minus_p(const EG<M> &G, const double *__restrict__ J) {
-    const EGVec X = G.v(EGLayout<M>::X), Y = G.v(EGLayout<M>::Y), R = G.v(EGLayout<M>::R);
-    double res = 0.0;
-#pragma unroll 1
-    for (int k = 0; k < M; k++) {
-        const double *Jk = J + k * NPHC_JSTRIDE;
-        dd ur = {Jk[M], 0.0}, ui = {0.0, 0.0}, wr = {0.0, 0.0}, wi = {0.0, 0.0};
-#pragma unroll 1
-        for (int l = 0; l < M; l++) {   // J_kk = 0 adds exact zeros
-            const cx<double> xl = X.get(l), yl = Y.get(l);
-            ur = dd_add(ur, dd_two_prod(Jk[l], xl.re));
-            ui = dd_add(ui, dd_two_prod(Jk[l], xl.im));
-            wr = dd_add(wr, dd_two_prod(Jk[l], yl.re));
-            wi = dd_add(wi, dd_two_prod(Jk[l], yl.im));
-        }
-        const cx<double> xk = X.get(k), yk = Y.get(k);
-        // f = y u - x w
-        const dd fr = dd_add(dd_add(dd_mul_d(ur, yk.re), dd_mul_d(ui, -yk.im)),
-                             dd_add(dd_mul_d(wr, -xk.re), dd_mul_d(wi, xk.im)));
-        const dd fi = dd_add(dd_add(dd_mul_d(ui, yk.re), dd_mul_d(ur, yk.im)),
-                             dd_add(dd_mul_d(wi, -xk.re), dd_mul_d(wr, -xk.im)));
-        // g = c^2 + s^2 - 1
-        dd gr = dd_add(dd_add(dd_two_prod(xk.re, xk.re), dd_two_prod(-xk.im, xk.im)),
-                       dd_add(dd_two_prod(yk.re, yk.re), dd_two_prod(-yk.im, yk.im)));
-        gr = dd_add(gr, dd{-1.0, 0.0});
-        const dd gi = dd_add(dd_two_prod(2.0 * xk.re, xk.im), dd_two_prod(2.0 * yk.re, yk.im));
-        const cx<double> f = cx<double>{dd_val(fr), dd_val(fi)};
-        const cx<double> g = cx<double>{dd_val(gr), dd_val(gi)};
-        res = fmax(res, fmax(sqrt(cabs2(f)), sqrt(cabs2(g))));
-        R.set(k, cx<double>{-f.re, -f.im});
-        R.set(M + k, cx<double>{-g.re, -g.im});
-    }
-    return res;
-}
 
 // Householder QR of the M x M matrix G.S in place: R above the diagonal with a real
 // diagonal (stored as (beta, 0)), the reflectors (1, v) below it, conj(tau) in TQ.
@@ -195,49 +116,6 @@ __device__ bool eg_qr(const EG<M> &G) {
     return ok;
 }
 
-// Frames, diagonal Jacobian entries and the Householder QR of S at the point (X, Y).
-// Returns false when S is singular.
-template <int M>
-__device__ bool eg_factor(const EG<M> &G, const double *__restrict__ J) {
-    using L = EGLayout<M>;
-    const EGVec X = G.v(L::X), Y = G.v(L::Y), AH = G.v(L::AH), BH = G.v(L::BH), IV = G.v(L::IV),
-                AD = G.v(L::AD), BD = G.v(L::BD);
-#pragma unroll 1
-    for (int j = 0; j < M; j++) {
-        const double *Jj = J + j * NPHC_JSTRIDE;
-        cx<double> u = cx<double>{Jj[M], 0.0}, w = cx<double>{0.0, 0.0};
-#pragma unroll 1
-        for (int l = 0; l < M; l++) {
-            const cx<double> xl = X.get(l), yl = Y.get(l);
-            u.re += Jj[l] * xl.re;
-            u.im += Jj[l] * xl.im;
-            w.re += Jj[l] * yl.re;
-            w.im += Jj[l] * yl.im;
-        }
-        AD.set(j, cx<double>{-w.re, -w.im});
-        BD.set(j, u);
-        const cx<double> a = cscale(2.0, X.get(j)), b = cscale(2.0, Y.get(j));
-        const double iv = rsqrt(cabs2(a) + cabs2(b));
-        IV.set(j, cx<double>{iv, 0.0});
-        AH.set(j, cscale(iv, a));
-        BH.set(j, cscale(iv, b));
-    }
-#pragma unroll 1
-    for (int j = 0; j < M; j++) {
-        const cx<double> ah = AH.get(j), bh = BH.get(j);
-#pragma unroll 1
-        for (int k = 0; k < M; k++) {
-            cx<double> e;
-            if (k == j)
-                e = csub(cmul(AD.get(j), bh), cmul(BD.get(j), ah));
-            else
-                e = cscale(J[k * NPHC_JSTRIDE + j], cadd(cmul(Y.get(k), bh), cmul(X.get(k), ah)));
-            G.setS(k, j, e);
-        }
-    }
-    return eg_qr<M>(G);
-}
-
 // b <- R^-1 Q^H b (b: M entries of a per-thread array); returns ||b||^2 afterwards.
 template <int M>
 __device__ double eg_schur_solve(const EG<M> &G, const EGVec &b) {
@@ -265,68 +143,6 @@ __device__ double eg_schur_solve(const EG<M> &G, const EGVec &b) {
     return n2;
 }
 
-// C_kj (the q_j-coefficient of gradient row k in the frame).
-template <int M>
-__device__ __forceinline__ cx<double> eg_C(const EG<M> &G, const double *__restrict__ J, int k,
-                                           int j) {
-    using L = EGLayout<M>;
-    const cx<double> ah = G.v(L::AH).get(j), bh = G.v(L::BH).get(j);
-    if (k == j)
-        return cadd(cmulc(ah, G.v(L::AD).get(j)), cmulc(bh, G.v(L::BD).get(j)));
-    const double Jkj = J[k * NPHC_JSTRIDE + j];
-    return cscale(Jkj, csub(cmulc(ah, G.v(L::Y).get(k)), cmulc(bh, G.v(L::X).get(k))));
-}
-
-// D <- DP^-1 R (after eg_factor); returns ||D||^2.
-template <int M>
-__device__ double eg_solve(const EG<M> &G, const double *__restrict__ J) {
-    using L = EGLayout<M>;
-    const EGVec R = G.v(L::R), Dv = G.v(L::D), IV = G.v(L::IV), AH = G.v(L::AH), BH = G.v(L::BH);
-    // q_j = iv_j r_gj into D[M + j]; Schur right-hand side r_fk - sum_j C_kj q_j into D[k]
-#pragma unroll 1
-    for (int j = 0; j < M; j++) Dv.set(M + j, cscale(IV.get(j).re, R.get(M + j)));
-#pragma unroll 1
-    for (int k = 0; k < M; k++) {
-        cx<double> acc = R.get(k);
-#pragma unroll 1
-        for (int j = 0; j < M; j++) acc = csub(acc, cmul(eg_C<M>(G, J, k, j), Dv.get(M + j)));
-        Dv.set(k, acc);
-    }
-    eg_schur_solve<M>(G, Dv);
-    double n2 = 0.0;
-#pragma unroll 1
-    for (int j = 0; j < M; j++) {
-        const cx<double> ah = AH.get(j), bh = BH.get(j), q = Dv.get(M + j), sj = Dv.get(j);
-        const cx<double> dx = cadd(cmulc(ah, q), cmul(bh, sj));
-        const cx<double> dy = csub(cmulc(bh, q), cmul(ah, sj));
-        Dv.set(j, dx);
-        Dv.set(M + j, dy);
-        n2 += cabs2(dx) + cabs2(dy);
-    }
-    return n2;
-}
-
-// ||DP^-1||_F after eg_factor (block formula above); uses D as scratch.
-template <int M>
-__device__ double eg_inv_fro(const EG<M> &G, const double *__restrict__ J) {
-    using L = EGLayout<M>;
-    const EGVec Dv = G.v(L::D), IV = G.v(L::IV);
-    double s = 0.0;
-#pragma unroll 1
-    for (int j = 0; j < M; j++) s += IV.get(j).re * IV.get(j).re;
-    // columns of S^-1 and of S^-1 C D^-1
-#pragma unroll 1
-    for (int col = 0; col < 2 * M; col++) {
-        const int j = col < M ? col : col - M;
-#pragma unroll 1
-        for (int k = 0; k < M; k++)
-            Dv.set(k, col < M ? cx<double>{k == j ? 1.0 : 0.0, 0.0}
-                              : cscale(IV.get(j).re, eg_C<M>(G, J, k, j)));
-        s += eg_schur_solve<M>(G, Dv);
-    }
-    return sqrt(s);
-}
-
 // shortcut = 1: entries handed off by the FP32 pass close to t = 1 are refined at t = 1
 // directly (Newton on P from the hand-off point: for a path to a nonsingular solution xi,
 // z(t) = xi + (1 - t) z'(1) + ..., so the point is already in xi's Newton basin).  The
@@ -334,50 +150,10 @@ __device__ double eg_inv_fro(const EG<M> &G, const double *__restrict__ J) {
 // certifies becomes NPHC_PATH_REACHED, any other entry is left untouched.
 #define SHORTCUT_TRUST 1e-2
 
-// The system an endgame kernel works on, as a policy for refine_body: the unknowns
-// (NZ, stored in G's X then Y), -P into R, the factorisation of DP, the Newton step
-// D = DP^-1 R, ||DP^-1||_F and ||D^2 P / 2||.  EGXY: the XY ring (frames + Schur QR).
-template <int M>
-struct EGXY {
-    using Sys = XYSys;
-    static constexpr int DIM = M;        // EG<DIM> storage
-    static constexpr int NZ = 2 * M;
-    static __device__ __forceinline__ cx<double> zget(const EG<M> &G, int k) {
-        return k < M ? G.v(EGLayout<M>::X).get(k) : G.v(EGLayout<M>::Y).get(k - M);
-    }
-    static __device__ __forceinline__ void zset(const EG<M> &G, int k, cx<double> v) {
-        if (k < M) G.v(EGLayout<M>::X).set(k, v);
-        else G.v(EGLayout<M>::Y).set(k - M, v);
-    }
-    static __device__ __forceinline__ double minus_p(const EG<M> &G, const Sys &S) {
-        return eg_minus_p<M>(G, S.Jd);
-    }
-    static __device__ __forceinline__ bool factor(const EG<M> &G, const Sys &S) {
-        return eg_factor<M>(G, S.Jd);
-    }
-    static __device__ __forceinline__ double solve(const EG<M> &G, const Sys &S) {
-        return eg_solve<M>(G, S.Jd);
-    }
-    static __device__ __forceinline__ double inv_fro(const EG<M> &G, const Sys &S) {
-        return eg_inv_fro<M>(G, S.Jd);
-    }
-    // ||DP||_F after factor: gradient row k has J_kj y_k, -J_kj x_k (free j != k), -w_k,
-    // u_k; constraint row k has 2 x_k, 2 y_k
-    static __device__ __forceinline__ double jac_fro(const EG<M> &G, const Sys &S) {
-        using L = EGLayout<M>;
-        double f = 0.0;
-#pragma unroll 1
-        for (int k = 0; k < M; k++) {
-            const double xy = cabs2(G.v(L::X).get(k)) + cabs2(G.v(L::Y).get(k));
-            double jj = 0.0;
-#pragma unroll 1
-            for (int j = 0; j < M; j++) jj += S.Jd[k * NPHC_JSTRIDE + j] * S.Jd[k * NPHC_JSTRIDE + j];
-            f += jj * xy + cabs2(G.v(L::AD).get(k)) + cabs2(G.v(L::BD).get(k)) + 4.0 * xy;
-        }
-        return sqrt(f);
-    }
-    static __device__ __forceinline__ double d2norm(const Sys &S) { return S.d2norm; }
-};
+// The system a refinement kernel works on is a policy Q for refine_body (EGQuad in quad.cuh):
+// the unknowns (NZ of them, stored in G's X), -P into R, the factorisation of DP, the Newton
+// step D = DP^-1 R, ||DP||_F, ||DP^-1||_F and ||D^2 P / 2||.  The XY ring has a kernel of its own
+// (xy_refine_group.cuh) that follows the same rules.
 
 // beta = ||DP^-1 P||, ||DP^-1||_F and ||P||_inf at the point in G.  False if singular:
 // at a point of a positive-dimensional solution set P vanishes to double-double precision
@@ -415,26 +191,23 @@ __device__ bool eg_beta_invnorm_p(const EG<Q::DIM> &G, const typename Q::Sys &S,
 template <class Q>
 __device__ bool eg_refine_certify_one(const EG<Q::DIM> &G, const typename Q::Sys &S,
                                       double tol_sol, double refine_eps, int refine_iters,
-                                      const EPView &ep, int64_t e, int shortcut) {
+                                      const EPView &ep, int64_t e) {
     constexpr int NZ = Q::NZ;
     const EGVec Dv = G.v(EGLayout<Q::DIM>::D);
     const int64_t cnt = ep.count;
     const double alpha0 = NPHC_ALPHA_CERT;
     const int st = ep.status[e];
-    const bool sc = shortcut && (st == NPHC_PATH_HANDOFF || st == NPHC_PATH_HANDOFF_COND);
-    if (!sc) {
-        ep.alpha[e] = INFINITY;
-        ep.beta[e] = INFINITY;
-        ep.gamma[e] = INFINITY;
-        ep.resid[e] = INFINITY;
-        if (st == NPHC_PATH_DIVERGED) {
-            ep.cls[e] = NPHC_END_NONE;
-            return false;
-        }
-        if (st != NPHC_PATH_REACHED) {
-            ep.cls[e] = NPHC_END_FAILED;
-            return false;
-        }
+    ep.alpha[e] = INFINITY;
+    ep.beta[e] = INFINITY;
+    ep.gamma[e] = INFINITY;
+    ep.resid[e] = INFINITY;
+    if (st == NPHC_PATH_DIVERGED) {
+        ep.cls[e] = NPHC_END_NONE;
+        return false;
+    }
+    if (st != NPHC_PATH_REACHED) {
+        ep.cls[e] = NPHC_END_FAILED;
+        return false;
     }
 #pragma unroll 1
     for (int k = 0; k < NZ; k++) Q::zset(G, k, cx<double>{ep.z_re[k * cnt + e], ep.z_im[k * cnt + e]});
@@ -455,7 +228,6 @@ __device__ bool eg_refine_certify_one(const EG<Q::DIM> &G, const typename Q::Sys
         double z2 = 0.0;
 #pragma unroll 1
         for (int k = 0; k < NZ; k++) z2 += cabs2(Q::zget(G, k));
-        if (sc && it == 0 && !(dn <= SHORTCUT_TRUST * (1.0 + sqrt(z2)))) return false;   // not in a basin
         if (!isfinite(dn) || !isfinite(z2)) {
             finite = false;
             break;
@@ -509,16 +281,10 @@ __device__ bool eg_refine_certify_one(const EG<Q::DIM> &G, const typename Q::Sys
     } else {
         beta = INFINITY;
     }
-    if (sc && !(real_test || cls == NPHC_END_NONREAL || cls == NPHC_END_UNDECIDED))
-        return false;   // left for FP64 tracking
     ep.alpha[e] = alpha;
     ep.beta[e] = beta;
     ep.gamma[e] = gam;
     ep.resid[e] = finite ? res : INFINITY;
-    if (sc) {
-        ep.status[e] = NPHC_PATH_REACHED;
-        ep.t[e] = 1.0;
-    }
 #pragma unroll 1
     for (int k = 0; k < NZ; k++) {
         const cx<double> zk = Q::zget(G, k);
@@ -551,26 +317,18 @@ __device__ void eg_real_test(const EG<Q::DIM> &G, const typename Q::Sys &S, cons
         ep.cls[e] = sqrt(im2) > 2.0 * ep.beta[e] ? NPHC_END_NONREAL : NPHC_END_UNDECIDED;
 }
 
-// One warp per block.  Entries are taken 32 at a time; the few that need the real test
-// (about one in thirty at N = 10) go to a per-warp queue that is drained 32 at a time,
-// so that the test runs on full warps instead of costing most warps a pass with one
-// active lane.  With wl.state set (a scratch buffer of at least gridDim.x x EG_BLOCK
-// threads' matrices), S lives there: the launch then needs shared memory for the rest
-// only, and fits more warps per SM (GB300's FP64 pipes are per SM sub-partition: at M = 9
-// four warps use all four where the 3 KB per thread of the whole set allowed two).
+// One warp per block.  Entries are taken 32 at a time; the few that need the real test go to
+// a per-warp queue that is drained 32 at a time, so that the test runs on full warps.
 template <class Q>
 __device__ __forceinline__ void refine_body(const typename Q::Sys &S, double tol_sol,
                                             double refine_eps, int refine_iters, const EPView &ep,
-                                            const WorkList &wl, int shortcut) {
+                                            const WorkList &wl) {
     using L = EGLayout<Q::DIM>;
     extern __shared__ __align__(16) unsigned char egraw[];
     __shared__ int64_t rq[2 * EG_BLOCK];
     const int lane = threadIdx.x;
     cx<double> *const sb = reinterpret_cast<cx<double> *>(egraw) + lane;
-    const EG<Q::DIM> G = wl.state
-        ? EG<Q::DIM>{sb, reinterpret_cast<cx<double> *>(wl.state) + (int64_t)blockIdx.x * EG_BLOCK + lane,
-                     (int64_t)gridDim.x * EG_BLOCK}
-        : EG<Q::DIM>{sb, sb + L::S * EG_BLOCK, EG_BLOCK};
+    const EG<Q::DIM> G{sb, sb + L::S * EG_BLOCK};
     const int64_t total = worklist_size(wl, ep.count);
     int qn = 0;   // queued real tests (the same in every lane)
     for (int64_t base = (int64_t)blockIdx.x * EG_BLOCK; base < total;
@@ -580,7 +338,7 @@ __device__ __forceinline__ void refine_body(const typename Q::Sys &S, double tol
         bool rt = false;
         if (i < total) e = worklist_entry(wl, i, ep.count);   // -1: rejected (debug)
         if (e >= 0)
-            rt = eg_refine_certify_one<Q>(G, S, tol_sol, refine_eps, refine_iters, ep, e, shortcut);
+            rt = eg_refine_certify_one<Q>(G, S, tol_sol, refine_eps, refine_iters, ep, e);
         const unsigned m = __ballot_sync(0xffffffffu, rt);
         if (rt) rq[qn + __popc(m & ((1u << lane) - 1u))] = e;
         qn += __popc(m);
@@ -592,13 +350,6 @@ __device__ __forceinline__ void refine_body(const typename Q::Sys &S, double tol
         }
     }
     if (lane < qn) eg_real_test<Q>(G, S, ep, rq[lane]);
-}
-
-template <int M>
-__global__ void __launch_bounds__(EG_BLOCK)
-    xy_refine_certify_kernel(const __grid_constant__ XYSys S, double tol_sol, double refine_eps,
-                             int refine_iters, const EPView ep, const WorkList wl, int shortcut) {
-    refine_body<EGXY<M>>(S, tol_sol, refine_eps, refine_iters, ep, wl, shortcut);
 }
 
 template <int M>

@@ -217,7 +217,7 @@ cudaError_t NPHC_CAT(launch_xy_track_f64_m, NPHC_INST_M)(const XYSys &sys, const
 #endif
 
 #if NPHC_INST_KIND == 2
-#include "xy_endgame.cuh"
+#include "xy_refine_group.cuh"
 
 cudaError_t NPHC_CAT(launch_xy_refine_certify_m, NPHC_INST_M)(const XYSys &sys, double tol_sol,
                                                              double refine_eps, int refine_iters,
@@ -226,32 +226,24 @@ cudaError_t NPHC_CAT(launch_xy_refine_certify_m, NPHC_INST_M)(const XYSys &sys, 
                                                              cudaStream_t st) {
     if (cap <= 0) return cudaSuccess;
     constexpr int M = NPHC_INST_M;
-    // with a scratch buffer (wl.state, wl.state_threads threads) S lives there and the
-    // shared memory holds the rest only
-    const bool gs = wl.state != nullptr && wl.state_threads >= EG_BLOCK;
-    const size_t smem = eg_smem_per_thread<M>(!gs) * EG_BLOCK;
-    auto k = xy_refine_certify_kernel<M>;
-    static bool attr_set = false;   // once per process for this instantiation (the larger size)
+    const size_t smem = rg_smem_per_block<M>();
+    auto k = xy_refine_group_kernel<M>;
+    static bool attr_set = false;   // once per process for this instantiation
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)(eg_smem_per_thread<M>() * EG_BLOCK));
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
     int dev = 0, sms = 0, per = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, EG_BLOCK, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 32, smem);
     if (e != cudaSuccess) return e;
-    // grid-stride over the entries: at most every SM filled, at most one entry per thread,
-    // and no more threads than the scratch buffer holds
-    const int64_t need = (cap + EG_BLOCK - 1) / EG_BLOCK;
-    int64_t full = (int64_t)sms * (per > 0 ? per : 1);
-    if (gs && full > wl.state_threads / EG_BLOCK) full = wl.state_threads / EG_BLOCK;
-    const int grid = (int)(need < full ? need : full);
-    WorkList w = wl;
-    if (!gs) w.state = nullptr;
-    k<<<grid, EG_BLOCK, smem, st>>>(sys, tol_sol, refine_eps, refine_iters, ep, w, shortcut);
+    // one or two warps on each of an SM's four schedulers (the FP64 pipes are per scheduler,
+    // and the entries are dealt out evenly), at most one entry per warp
+    const int64_t full = (int64_t)sms * (per >= 8 ? 8 : per >= 4 ? 4 : per > 0 ? per : 1);
+    const int grid = (int)(cap < full ? cap : full);
+    k<<<grid, 32, smem, st>>>(sys, tol_sol, refine_eps, refine_iters, ep, wl, shortcut);
     nphc_launch_counter(1);
     return cudaGetLastError();
 }
