@@ -106,7 +106,7 @@ struct nphc_system {
     XYSys xs;                // coupling tables; gamma is filled per call
     bool quad = false;       // generic quadratic system (nphc_system_create_quadratic)
     QSys qs;                 // its device term list; gamma is filled per call
-    void *qdev = nullptr;    // device allocation holding qs.row and qs.terms
+    void *qdev = nullptr;    // device allocation holding qs' arrays
 };
 
 struct nphc_result {
@@ -338,6 +338,27 @@ nphc_status nphc_system_create_quadratic(int n, int nterms, const int32_t *eq, c
     double d2 = 0.0;
     for (int i = 0; i < n; i++)
         for (double v : m2[i]) d2 += v * v;
+    // the Jacobian's entries: per (variable, equation) cell the list of c w(other)
+    std::vector<std::vector<QTerm>> cell((size_t)n * n);
+    for (int i = 0; i < n; i++)
+        for (int t = row[i]; t < row[i + 1]; t++) {
+            QTerm q = terms[t];
+            const int32_t a = q.a, b = q.b;
+            if (a >= 0) {
+                q.a = b;
+                cell[(size_t)a * n + i].push_back(q);
+            }
+            if (b >= 0) {
+                q.a = a;
+                cell[(size_t)b * n + i].push_back(q);
+            }
+        }
+    std::vector<int32_t> jrow(1, 0);
+    std::vector<QTerm> jac;
+    for (const std::vector<QTerm> &c : cell) {
+        jac.insert(jac.end(), c.begin(), c.end());
+        jrow.push_back((int32_t)jac.size());
+    }
     nphc_system *S = new (std::nothrow) nphc_system;
     if (!S) return fail(NPHC_ENOMEM, "host allocation");
     S->N = 0;
@@ -347,7 +368,9 @@ nphc_status nphc_system_create_quadratic(int n, int nterms, const int32_t *eq, c
     std::memset(&S->xs, 0, sizeof(S->xs));
     S->quad = true;
     const size_t rbytes = align256(sizeof(int32_t) * (n + 1));
-    const size_t bytes = rbytes + sizeof(QTerm) * nterms;
+    const size_t tbytes = align256(sizeof(QTerm) * nterms);
+    const size_t jbytes = align256(sizeof(int32_t) * jrow.size());
+    const size_t bytes = rbytes + tbytes + jbytes + sizeof(QTerm) * std::max<size_t>(jac.size(), 1);
     if (cudaMalloc(&S->qdev, bytes) != cudaSuccess) {
         cudaGetLastError();
         delete S;
@@ -357,6 +380,10 @@ nphc_status nphc_system_create_quadratic(int n, int nterms, const int32_t *eq, c
     cudaError_t e = cudaMemcpy(d, row.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(d + rbytes, terms.data(), sizeof(QTerm) * nterms, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(d + rbytes + tbytes, jrow.data(), sizeof(int32_t) * jrow.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && !jac.empty())
+        e = cudaMemcpy(d + rbytes + tbytes + jbytes, jac.data(), sizeof(QTerm) * jac.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         nphc_system_destroy(S);
         return fail(NPHC_ECUDA, std::string("term list upload: ") + cudaGetErrorString(e));
@@ -364,6 +391,8 @@ nphc_status nphc_system_create_quadratic(int n, int nterms, const int32_t *eq, c
     S->qs.n = n;
     S->qs.row = reinterpret_cast<const int32_t *>(d);
     S->qs.terms = reinterpret_cast<const QTerm *>(d + rbytes);
+    S->qs.jrow = reinterpret_cast<const int32_t *>(d + rbytes + tbytes);
+    S->qs.jac = reinterpret_cast<const QTerm *>(d + rbytes + tbytes + jbytes);
     S->qs.gre = 1.0;
     S->qs.gim = 0.0;
     S->qs.d2norm = std::sqrt(d2);
@@ -488,7 +517,7 @@ nphc_status track_impl(const nphc_system *S, const nphc_options *o, nphc_precisi
     }
     const EPView v = view(ep);
     if (S->quad)
-        NPHC_CK(launch_quad_track(S->n, quad_with_gamma(S, o), ctl, v, wl, 0, st));
+        NPHC_CK(launch_quad_track(S->n, quad_with_gamma(S, o), ctl, v, wl, st));
     else if (!f32 && list != nullptr && o->threads_per_path != 1)   // one path per warp
         NPHC_CK(launch_xy_track_f64_warp_bps(S->M, xs, ctl, v, wl, o->list_blocks_per_sm, st));
     else if (!f32 && list != nullptr)   // FP64 lists, one path per thread, full warps

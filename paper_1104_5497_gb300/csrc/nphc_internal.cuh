@@ -217,6 +217,10 @@ struct QSys {
     int n;
     const int32_t *row;    // [n + 1] term offsets per equation (device)
     const QTerm *terms;    // [row[n]] (device)
+    // dP_i/dz_v = sum of c w(a) over the entries jrow[v n + i] .. jrow[v n + i + 1] - 1 of jac (a
+    // term c w(a) w(b) gives v = a one with w(b) and v = b one with w(a); the b of an entry is unused)
+    const int32_t *jrow;   // [n n + 1] (device)
+    const QTerm *jac;      // [jrow[n n]] (device)
     double gre, gim;       // gamma
     double d2norm;         // ||D^2 P / 2|| bound
     double kappa_sing;     // singular above kappa_sing max(1, ||z||_inf^2)
@@ -255,7 +259,7 @@ cudaError_t launch_xy_classify(int M, const XYSys &sys, const EPView &ep, double
                                cudaStream_t st, const int32_t *list = nullptr,
                                const int32_t *list_count = nullptr);
 cudaError_t launch_quad_track(int n, const QSys &sys, const XYCtl &ctl, const EPView &ep,
-                              const WorkList &wl, int grid, cudaStream_t st);
+                              const WorkList &wl, cudaStream_t st);
 cudaError_t launch_quad_refine_certify(int n, const QSys &sys, double tol_sol, double refine_eps,
                                        int refine_iters, const EPView &ep, int64_t cap,
                                        const WorkList &wl, cudaStream_t st);

@@ -24,20 +24,19 @@ cudaError_t persistent_grid(K k, int block, size_t smem, int &grid) {
 
 }  // namespace
 
+constexpr int QUAD_WARPS = 4;   // warps per block of the one-path-per-warp kernels
+
 cudaError_t NPHC_CAT(launch_quad_track_n, NPHC_QUAD_NV)(const QSys &sys, const XYCtl &ctl,
                                                         const EPView &ep, const WorkList &wl,
-                                                        int grid, cudaStream_t st) {
-    using P = QuadProblem<NPHC_QUAD_NV>;
-    const size_t smem = track_smem_per_thread<P>() * P::BLOCK;
-    auto k = quad_track_kernel<NPHC_QUAD_NV>;
+                                                        cudaStream_t st) {
+    if (ep.count <= 0) return cudaSuccess;
+    const size_t smem = sizeof(cx<double>) * QuadLayout<NPHC_QUAD_NV>::TOTAL * QUAD_WARPS;
+    auto k = quad_track_warp_kernel<NPHC_QUAD_NV, QUAD_WARPS>;
     int full = 0;
-    cudaError_t e = persistent_grid(k, P::BLOCK, smem, full);
+    cudaError_t e = persistent_grid(k, 32 * QUAD_WARPS, smem, full);
     if (e != cudaSuccess) return e;
-    if (grid <= 0 || grid > full) grid = full;
-    const int cap = (int)(wl.state_threads / P::BLOCK);   // the scratch holds state for this many
-    if (grid > cap) grid = cap;
-    if (grid <= 0) return cudaErrorInvalidValue;
-    k<<<grid, P::BLOCK, smem, st>>>(sys, ctl, ep, wl);
+    const int64_t need = (ep.count + QUAD_WARPS - 1) / QUAD_WARPS;   // a list is at most ep.count long
+    k<<<(int)(need < full ? need : full), 32 * QUAD_WARPS, smem, st>>>(sys, ctl, ep, wl);
     nphc_launch_counter(1);
     return cudaGetLastError();
 }
@@ -49,16 +48,14 @@ cudaError_t NPHC_CAT(launch_quad_refine_certify_n, NPHC_QUAD_NV)(const QSys &sys
                                                                  const WorkList &wl,
                                                                  cudaStream_t st) {
     if (cap <= 0) return cudaSuccess;
-    const size_t smem = eg_smem_per_thread<NPHC_QUAD_NV>() * EG_BLOCK;
-    auto k = quad_refine_certify_kernel<NPHC_QUAD_NV>;
+    const size_t smem = sizeof(cx<double>) * QuadRefineLayout<NPHC_QUAD_NV>::TOTAL * QUAD_WARPS;
+    auto k = quad_refine_warp_kernel<NPHC_QUAD_NV, QUAD_WARPS>;
     int full = 0;
-    cudaError_t e = persistent_grid(k, EG_BLOCK, smem, full);
+    cudaError_t e = persistent_grid(k, 32 * QUAD_WARPS, smem, full);
     if (e != cudaSuccess) return e;
-    const int64_t need = (cap + EG_BLOCK - 1) / EG_BLOCK;
-    const int grid = (int)(need < full ? need : full);
-    WorkList w = wl;
-    w.state = nullptr;   // S in shared memory (the launch is sized for it)
-    k<<<grid, EG_BLOCK, smem, st>>>(sys, tol_sol, refine_eps, refine_iters, ep, w);
+    const int64_t need = (cap + QUAD_WARPS - 1) / QUAD_WARPS;
+    k<<<(int)(need < full ? need : full), 32 * QUAD_WARPS, smem, st>>>(sys, tol_sol, refine_eps, refine_iters,
+                                                                       ep, wl);
     nphc_launch_counter(1);
     return cudaGetLastError();
 }

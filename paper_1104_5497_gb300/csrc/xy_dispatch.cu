@@ -66,8 +66,8 @@ int xy_track_f32_block(int M) { (void)M; return NPHC_TRACK_BLOCK; }
 int xy_track_f64_block(int M) { (void)M; return NPHC_TRACK_BLOCK; }
 
 cudaError_t launch_quad_track(int n, const QSys &sys, const XYCtl &ctl, const EPView &ep,
-                              const WorkList &wl, int grid, cudaStream_t st) {
-#define C(NN) case NN: return launch_quad_track_n##NN(sys, ctl, ep, wl, grid, st);
+                              const WorkList &wl, cudaStream_t st) {
+#define C(NN) case NN: return launch_quad_track_n##NN(sys, ctl, ep, wl, st);
     switch (n) { NPHC_FOR_EACH_QN(C) default: return cudaErrorInvalidValue; }
 #undef C
 }

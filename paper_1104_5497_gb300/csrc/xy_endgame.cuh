@@ -2,7 +2,8 @@
 //   refinement: Newton's method on P to full double precision (section "Numerical
 //     Polynomial Homotopy Continuation Method" refines every endpoint to machine
 //     precision before certifying it), with P evaluated by exact products and
-//     double-double sums (eg_minus_p);
+//     compensated sums (at ||z|| >> 1 the terms of P are ~||z||^2, and a plain sum's
+//     rounding would limit the refinement and inflate beta);
 //   the solution tolerance Delta_sol on ||P(z)||_inf;
 //   alpha-theory certification (the alphaCertified step of the same section):
 //     beta = ||DP^-1 P||_2, gamma <= ||DP^-1||_F ||D^2 P / 2|| (P is quadratic, so
@@ -25,21 +26,14 @@
 // so a solve costs one M x M system, and, W being unitary,
 //   ||DP^-1||_F^2 = sum_j iv_j^2 + ||S^-1||_F^2 + ||S^-1 C D^-1||_F^2
 // needs only 2M triangular solves after one factorisation of S.  The XY ring's kernel is
-// xy_refine_group.cuh (four lanes per endpoint); this file holds the classification and the
-// adjoint, and the rules of refinement and certification as a generic body, one endpoint per
-// thread with a Householder QR of DP, for quadratic systems (quad.cuh).
+// xy_refine_group.cuh (four lanes per endpoint), a quadratic system's quad_warp.cuh (one
+// endpoint per warp); this file holds what they share, the classification and the adjoint.
 //
 // The refinement certifies the iterate whose Newton correction met the tolerance, from
 // the factorisation of that iteration, and outputs its Newton iterate.
-//
-// Storage of the generic body: interleaved across the 32 threads of a block in shared memory
-// (element i of a thread's array at [i * 32 + lane]), so that the rolled loops index it at run
-// time without local memory.
 #pragma once
 
 #include "nphc_internal.cuh"
-
-#define EG_BLOCK 32
 
 // The certification threshold: half of Smale's (13 - 3 sqrt 17) / 4.  alphaCertified
 // decides in exact arithmetic; an FP64 test keeps a factor of two so that rounding cannot
@@ -47,310 +41,12 @@
 // point of the positive-dimensional family reached alpha = 0.115 < 0.158).
 #define NPHC_ALPHA_CERT (0.5 * (13.0 - 3.0 * sqrt(17.0)) / 4.0)
 
-
-// One thread's array of complex doubles in shared memory.
-struct EGVec {
-    cx<double> *p;
-    __device__ __forceinline__ cx<double> get(int i) const { return p[i * EG_BLOCK]; }
-    __device__ __forceinline__ void set(int i, cx<double> v) const { p[i * EG_BLOCK] = v; }
-};
-
-// Per-thread working set of the refinement (complex doubles, in this order).
-template <int M>
-struct EGLayout {
-    static constexpr int TQ = 0;                // conj(tau) of the reflectors
-    static constexpr int X = TQ + M;            // z
-    static constexpr int R = X + M;             // right-hand side / residual (and one scalar)
-    static constexpr int D = R + M + 1;         // solution
-    static constexpr int S = D + M;             // M x M, column-major: entry (i, c) at c M + i
-    static constexpr int TOTAL = S + M * M;
-};
-
-template <int M>
-constexpr size_t eg_smem_per_thread() {
-    return sizeof(cx<double>) * (size_t)EGLayout<M>::TOTAL;
-}
-
-template <int M>
-struct EG {
-    cx<double> *base;   // this thread's first entry in shared memory (stride EG_BLOCK)
-    cx<double> *sp;     // this thread's entry (0, 0) of S
-    __device__ __forceinline__ EGVec v(int off) const { return EGVec{base + off * EG_BLOCK}; }
-    __device__ __forceinline__ cx<double> S(int i, int c) const { return sp[(c * M + i) * EG_BLOCK]; }
-    __device__ __forceinline__ void setS(int i, int c, cx<double> a) const { sp[(c * M + i) * EG_BLOCK] = a; }
-};
-
-// Householder QR of the M x M matrix G.S in place: R above the diagonal with a real
-// diagonal (stored as (beta, 0)), the reflectors (1, v) below it, conj(tau) in TQ.
-// Returns false when the matrix is singular.
-template <int M>
-__device__ bool eg_qr(const EG<M> &G) {
-    const EGVec TQ = G.v(EGLayout<M>::TQ);
-    bool ok = true;
-#pragma unroll 1
-    for (int k = 0; k < M; k++) {
-        const cx<double> al = G.S(k, k);
-        double xn2 = 0.0;
-#pragma unroll 1
-        for (int i = k + 1; i < M; i++) xn2 += cabs2(G.S(i, k));
-        const double an = sqrt(cabs2(al) + xn2);
-        ok = ok && an > 0.0;
-        const double beta = al.re >= 0.0 ? -an : an;
-        const cx<double> tauc = cx<double>{(beta - al.re) / beta, al.im / beta};
-        const cx<double> sc = crecip(cx<double>{al.re - beta, al.im});
-#pragma unroll 1
-        for (int i = k + 1; i < M; i++) G.setS(i, k, cmul(G.S(i, k), sc));
-        G.setS(k, k, cx<double>{beta, 0.0});
-        TQ.set(k, tauc);
-#pragma unroll 1
-        for (int c = k + 1; c < M; c++) {
-            cx<double> wv = G.S(k, c);
-#pragma unroll 1
-            for (int i = k + 1; i < M; i++) wv = cadd(wv, cmulc(G.S(i, k), G.S(i, c)));
-            wv = cmul(tauc, wv);
-            G.setS(k, c, csub(G.S(k, c), wv));
-#pragma unroll 1
-            for (int i = k + 1; i < M; i++) G.setS(i, c, csub(G.S(i, c), cmul(G.S(i, k), wv)));
-        }
-    }
-    return ok;
-}
-
-// b <- R^-1 Q^H b (b: M entries of a per-thread array); returns ||b||^2 afterwards.
-template <int M>
-__device__ double eg_schur_solve(const EG<M> &G, const EGVec &b) {
-    const EGVec TQ = G.v(EGLayout<M>::TQ);
-#pragma unroll 1
-    for (int k = 0; k < M; k++) {
-        cx<double> wv = b.get(k);
-#pragma unroll 1
-        for (int i = k + 1; i < M; i++) wv = cadd(wv, cmulc(G.S(i, k), b.get(i)));
-        wv = cmul(TQ.get(k), wv);
-        b.set(k, csub(b.get(k), wv));
-#pragma unroll 1
-        for (int i = k + 1; i < M; i++) b.set(i, csub(b.get(i), cmul(G.S(i, k), wv)));
-    }
-    double n2 = 0.0;
-#pragma unroll 1
-    for (int k = M - 1; k >= 0; k--) {
-        cx<double> acc = b.get(k);
-#pragma unroll 1
-        for (int c = k + 1; c < M; c++) acc = csub(acc, cmul(G.S(k, c), b.get(c)));
-        acc = cscale(1.0 / G.S(k, k).re, acc);
-        b.set(k, acc);
-        n2 += cabs2(acc);
-    }
-    return n2;
-}
-
 // shortcut = 1: entries handed off by the FP32 pass close to t = 1 are refined at t = 1
 // directly (Newton on P from the hand-off point: for a path to a nonsingular solution xi,
 // z(t) = xi + (1 - t) z'(1) + ..., so the point is already in xi's Newton basin).  The
 // first Newton correction must stay below SHORTCUT_TRUST (1 + ||z||); an entry that
 // certifies becomes NPHC_PATH_REACHED, any other entry is left untouched.
 #define SHORTCUT_TRUST 1e-2
-
-// The system a refinement kernel works on is a policy Q for refine_body (EGQuad in quad.cuh):
-// the unknowns (NZ of them, stored in G's X), -P into R, the factorisation of DP, the Newton
-// step D = DP^-1 R, ||DP||_F, ||DP^-1||_F and ||D^2 P / 2||.  The XY ring has a kernel of its own
-// (xy_refine_group.cuh) that follows the same rules.
-
-// beta = ||DP^-1 P||, ||DP^-1||_F and ||P||_inf at the point in G.  False if singular:
-// at a point of a positive-dimensional solution set P vanishes to double-double precision
-// (beta is tiny) while rounding leaves the computed DP^-1 merely huge, and the soft alpha
-// test alone can pass there, so a Frobenius condition number ||DP||_F ||DP^-1||_F above
-// kappa_sing max(1, ||z||_inf^2) counts as singular.  The bound grows with ||z||_inf^2 like
-// the solution tolerance: the equations are quadratic, the Jacobian's entries grow like
-// ||z|| and an isolated solution near the solution set at infinity has a smallest singular
-// value shrinking like 1 / ||z|| (a solution of norm 1e6 has a condition number ~1e12).
-// The same from a factorisation already made at the point in G: fro = ||DP||_F, dn =
-// ||DP^-1 P|| from its solve (inv_fro takes D as scratch).
-template <class Q>
-__device__ bool eg_certify_factored(const EG<Q::DIM> &G, const typename Q::Sys &S, double fro,
-                                    double dn, double &beta, double &invF) {
-    beta = dn;
-    invF = Q::inv_fro(G, S);
-    double zi = 0.0;
-#pragma unroll 1
-    for (int k = 0; k < Q::NZ; k++) zi = fmax(zi, sqrt(cabs2(Q::zget(G, k))));
-    return isfinite(beta) && isfinite(invF) && fro * invF <= S.kappa_sing * fmax(1.0, zi * zi);
-}
-
-template <class Q>
-__device__ bool eg_beta_invnorm_p(const EG<Q::DIM> &G, const typename Q::Sys &S, double &beta,
-                                  double &invF, double &res) {
-    res = Q::minus_p(G, S);
-    if (!Q::factor(G, S)) return false;
-    const double fro = Q::jac_fro(G, S);
-    const double dn = sqrt(Q::solve(G, S));
-    return eg_certify_factored<Q>(G, S, fro, dn, beta, invF);
-}
-
-// Refinement and certification of entry e.  Returns true when e still needs the
-// alpha-test at Re z (its refined z is already written out; the caller runs the test).
-template <class Q>
-__device__ bool eg_refine_certify_one(const EG<Q::DIM> &G, const typename Q::Sys &S,
-                                      double tol_sol, double refine_eps, int refine_iters,
-                                      const EPView &ep, int64_t e) {
-    constexpr int NZ = Q::NZ;
-    const EGVec Dv = G.v(EGLayout<Q::DIM>::D);
-    const int64_t cnt = ep.count;
-    const double alpha0 = NPHC_ALPHA_CERT;
-    const int st = ep.status[e];
-    ep.alpha[e] = INFINITY;
-    ep.beta[e] = INFINITY;
-    ep.gamma[e] = INFINITY;
-    ep.resid[e] = INFINITY;
-    if (st == NPHC_PATH_DIVERGED) {
-        ep.cls[e] = NPHC_END_NONE;
-        return false;
-    }
-    if (st != NPHC_PATH_REACHED) {
-        ep.cls[e] = NPHC_END_FAILED;
-        return false;
-    }
-#pragma unroll 1
-    for (int k = 0; k < NZ; k++) Q::zset(G, k, cx<double>{ep.z_re[k * cnt + e], ep.z_im[k * cnt + e]});
-    int cls = NPHC_END_SINGULAR;
-    bool finite = true;
-    double beta = INFINITY, invF = INFINITY, res = INFINITY;
-    bool certified = false, cert_ok = false;
-    // Newton refinement on P.  The iteration whose correction meets refine_eps certifies its
-    // own point z_k from the factorisation it has just made (beta = ||dz_k||, exactly what a
-    // separate certification at z_k computes), and the output is z_k's Newton iterate
-    // z_k + dz_k, closer still to the same zero: one evaluation, factorisation and solve
-    // less than certifying the output point afresh
-#pragma unroll 1
-    for (int it = 0; it < refine_iters; it++) {
-        const double rk = Q::minus_p(G, S);
-        if (!Q::factor(G, S)) break;
-        const double dn = sqrt(Q::solve(G, S));
-        double z2 = 0.0;
-#pragma unroll 1
-        for (int k = 0; k < NZ; k++) z2 += cabs2(Q::zget(G, k));
-        if (!isfinite(dn) || !isfinite(z2)) {
-            finite = false;
-            break;
-        }
-        const bool last = dn <= refine_eps * (1.0 + sqrt(z2));
-        const EGVec Step = last ? G.v(EGLayout<Q::DIM>::R) : Dv;
-        if (last) {
-#pragma unroll 1
-            for (int k = 0; k < NZ; k++) Step.set(k, Dv.get(k));   // inv_fro takes D as scratch
-            const double fro = Q::jac_fro(G, S);
-            cert_ok = eg_certify_factored<Q>(G, S, fro, dn, beta, invF);
-            res = rk;
-            certified = true;
-        }
-        double zn = 0.0;
-#pragma unroll 1
-        for (int k = 0; k < NZ; k++) {
-            const cx<double> zk = cadd(Q::zget(G, k), Step.get(k));
-            Q::zset(G, k, zk);
-            zn += cabs2(zk);
-        }
-        if (!isfinite(zn)) {
-            finite = false;
-            break;
-        }
-        if (last) break;
-    }
-    if (finite && !certified) cert_ok = eg_beta_invnorm_p<Q>(G, S, beta, invF, res);
-    double alpha = INFINITY, gam = INFINITY;
-    bool real_test = false;
-    if (finite && cert_ok) {
-        gam = invF * Q::d2norm(S);
-        alpha = beta * gam;
-        // Delta_sol relative to the size of the (quadratic) terms: max(1, ||z||_inf^2)
-        double zi = 0.0, im2 = 0.0;
-#pragma unroll 1
-        for (int k = 0; k < NZ; k++) {
-            const cx<double> zk = Q::zget(G, k);
-            zi = fmax(zi, sqrt(cabs2(zk)));
-            im2 += zk.im * zk.im;
-        }
-        if (res <= tol_sol * fmax(1.0, zi * zi) && alpha < alpha0) {
-            // z and Re z share their associated zero when alpha < 0.03 and
-            // ||Im z|| < 1 / (20 gamma): then the real test at Re z decides (queued)
-            const double im = sqrt(im2);
-            if (alpha < 0.03 && im < 1.0 / (20.0 * gam))
-                real_test = true;
-            else
-                cls = im > 2.0 * beta ? NPHC_END_NONREAL : NPHC_END_UNDECIDED;
-        }
-    } else {
-        beta = INFINITY;
-    }
-    ep.alpha[e] = alpha;
-    ep.beta[e] = beta;
-    ep.gamma[e] = gam;
-    ep.resid[e] = finite ? res : INFINITY;
-#pragma unroll 1
-    for (int k = 0; k < NZ; k++) {
-        const cx<double> zk = Q::zget(G, k);
-        ep.z_re[k * cnt + e] = zk.re;
-        ep.z_im[k * cnt + e] = zk.im;
-    }
-    if (!real_test) ep.cls[e] = cls;
-    return real_test;
-}
-
-// The alpha-test at Re z of a certified entry e that shares its zero with Re z: real
-// when it passes there; otherwise non-real when ||Im z|| > 2 beta (z and conj z then
-// have distinct zeros), else undecided.
-template <class Q>
-__device__ void eg_real_test(const EG<Q::DIM> &G, const typename Q::Sys &S, const EPView &ep,
-                             int64_t e) {
-    const int64_t cnt = ep.count;
-    const double alpha0 = NPHC_ALPHA_CERT;
-    double im2 = 0.0;
-#pragma unroll 1
-    for (int k = 0; k < Q::NZ; k++) {
-        const double yi = ep.z_im[k * cnt + e];
-        im2 += yi * yi;
-        Q::zset(G, k, cx<double>{ep.z_re[k * cnt + e], 0.0});
-    }
-    double br, ir, rr;
-    if (eg_beta_invnorm_p<Q>(G, S, br, ir, rr) && br * ir * Q::d2norm(S) < alpha0)
-        ep.cls[e] = NPHC_END_REAL;
-    else
-        ep.cls[e] = sqrt(im2) > 2.0 * ep.beta[e] ? NPHC_END_NONREAL : NPHC_END_UNDECIDED;
-}
-
-// One warp per block.  Entries are taken 32 at a time; the few that need the real test go to
-// a per-warp queue that is drained 32 at a time, so that the test runs on full warps.
-template <class Q>
-__device__ __forceinline__ void refine_body(const typename Q::Sys &S, double tol_sol,
-                                            double refine_eps, int refine_iters, const EPView &ep,
-                                            const WorkList &wl) {
-    using L = EGLayout<Q::DIM>;
-    extern __shared__ __align__(16) unsigned char egraw[];
-    __shared__ int64_t rq[2 * EG_BLOCK];
-    const int lane = threadIdx.x;
-    cx<double> *const sb = reinterpret_cast<cx<double> *>(egraw) + lane;
-    const EG<Q::DIM> G{sb, sb + L::S * EG_BLOCK};
-    const int64_t total = worklist_size(wl, ep.count);
-    int qn = 0;   // queued real tests (the same in every lane)
-    for (int64_t base = (int64_t)blockIdx.x * EG_BLOCK; base < total;
-         base += (int64_t)gridDim.x * EG_BLOCK) {
-        const int64_t i = base + lane;
-        int64_t e = -1;
-        bool rt = false;
-        if (i < total) e = worklist_entry(wl, i, ep.count);   // -1: rejected (debug)
-        if (e >= 0)
-            rt = eg_refine_certify_one<Q>(G, S, tol_sol, refine_eps, refine_iters, ep, e);
-        const unsigned m = __ballot_sync(0xffffffffu, rt);
-        if (rt) rq[qn + __popc(m & ((1u << lane) - 1u))] = e;
-        qn += __popc(m);
-        __syncwarp();
-        if (qn >= EG_BLOCK) {
-            eg_real_test<Q>(G, S, ep, rq[qn - EG_BLOCK + lane]);
-            qn -= EG_BLOCK;
-            __syncwarp();
-        }
-    }
-    if (lane < qn) eg_real_test<Q>(G, S, ep, rq[lane]);
-}
 
 template <int M>
 __global__ void __launch_bounds__(128)

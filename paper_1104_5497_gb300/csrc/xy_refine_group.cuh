@@ -287,7 +287,7 @@ __device__ void rg_norms(const RGPath<M> &G, unsigned long long perm, double &in
     zi2 = rg_max(G.m, zi);
 }
 
-// The rules of eg_refine_certify_one and eg_real_test (xy_endgame.cuh).
+// Refinement, certification and the real test of every selected entry that reached t = 1.
 template <int M>
 __global__ void __launch_bounds__(32)
     xy_refine_group_kernel(const __grid_constant__ XYSys S, double tol_sol, double refine_eps,

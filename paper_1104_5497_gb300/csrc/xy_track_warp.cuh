@@ -233,6 +233,82 @@ __device__ void warp_residual(const WarpPath<M> &P, const double *__restrict__ J
     __syncwarp();
 }
 
+// Solves the M x M system [A | b0 | b1] (column-major, M rows; b1 only when two_rhs) by LU with
+// partial pivoting over the warp; cur: entry lane % 16 of the solution for right-hand side
+// lane / 16.  False when the matrix is singular.
+template <int M>
+__device__ __forceinline__ bool warp_lu_solve(cx<double> *A, int lane, bool two_rhs, cx<double> &cur) {
+    static_assert(M <= 16, "one row per lane of each half-warp");
+    auto at = [&](int i, int c) -> cx<double> & { return A[c * M + i]; };
+    const int hrow = lane & 15, r = lane >> 4;
+    // ---- LU with partial pivoting of [S | b0 | b1]; the pivot's reciprocal replaces it
+    const int ncol = two_rhs ? M + 2 : M + 1;
+    bool ok = true;
+#pragma unroll 1
+    for (int k = 0; k < M; k++) {
+        // the row of the largest |re| + |im| at or below k (ties: the lowest row); the
+        // bit patterns of non-negative doubles order as the values do
+        unsigned long long key = 0ull;
+        int idx = lane;
+        if (lane >= k && lane < M) {
+            const cx<double> a = at(lane, k);
+            key = (unsigned long long)__double_as_longlong(fabs(a.re) + fabs(a.im));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long ko = __shfl_xor_sync(0xffffffffu, key, o);
+            const int io = __shfl_xor_sync(0xffffffffu, idx, o);
+            if (ko > key || (ko == key && io < idx)) {
+                key = ko;
+                idx = io;
+            }
+        }
+        int p = idx;
+        if (key == 0ull) {   // the column is zero from row k down: S is singular
+            ok = false;
+            p = k;
+        }
+        if (p != k) {   // uniform
+            if (lane >= k && lane < ncol) {
+                const cx<double> a = at(k, lane);
+                at(k, lane) = at(p, lane);
+                at(p, lane) = a;
+            }
+            __syncwarp();
+        }
+        const cx<double> a = at(k, k);
+        const double rd = 1.0 / fma(a.re, a.re, a.im * a.im);
+        const cx<double> ip = cx<double>{a.re * rd, -a.im * rd};
+        if (lane > k && lane < M) at(lane, k) = cmul(at(lane, k), ip);
+        __syncwarp();
+        const int nr = M - 1 - k, nc = ncol - 1 - k;
+#pragma unroll 1
+        for (int e = lane; e < nr * nc; e += 32) {
+            const int c = k + 1 + e / nr, i = k + 1 + (e - (e / nr) * nr);
+            at(i, c) = cfnms(at(i, c), at(i, k), at(k, c));
+        }
+        if (lane == 31) at(k, k) = ip;   // nothing reads the pivot in this step's update
+        __syncwarp();
+    }
+
+    // ---- back substitution U x = b in registers: right-hand side r, row hrow
+    const bool act = r == 0 || two_rhs;
+    cur = cx<double>{0.0, 0.0};
+    if (act && hrow < M) cur = at(hrow, M + r);
+#pragma unroll 1
+    for (int k = M - 1; k >= 0; k--) {
+        const int src = (lane & 16) | k;
+        const cx<double> bk = cx<double>{__shfl_sync(0xffffffffu, cur.re, src),
+                                         __shfl_sync(0xffffffffu, cur.im, src)};
+        if (hrow <= k) {
+            const cx<double> xk = cmul(bk, at(k, k));   // the pivot's reciprocal
+            cur = hrow == k ? xk : cfnms(cur, at(hrow, k), xk);
+        }
+    }
+
+    return ok;
+}
+
 // H_z(ZC, t) d = r, the per-thread xy_solve's Schur reduction shared out over the warp;
 // ZC and d in (x, y) (LC == false) or in the light-cone coordinates (p, q).
 //   two_rhs false: r = -H_t, d into W1.
@@ -345,70 +421,9 @@ __device__ bool warp_solve(const WarpPath<M> &P, const double *__restrict__ J, d
     }
     __syncwarp();
 
-    // ---- LU with partial pivoting of [S | b0 | b1]; the pivot's reciprocal replaces it
-    const int ncol = two_rhs ? M + 2 : M + 1;
-    bool ok = true;
-#pragma unroll 1
-    for (int k = 0; k < M; k++) {
-        // the row of the largest |re| + |im| at or below k (ties: the lowest row); the
-        // bit patterns of non-negative doubles order as the values do
-        unsigned long long key = 0ull;
-        int idx = lane;
-        if (lane >= k && lane < M) {
-            const cx<double> a = P.A(lane, k);
-            key = (unsigned long long)__double_as_longlong(fabs(a.re) + fabs(a.im));
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long ko = __shfl_xor_sync(0xffffffffu, key, o);
-            const int io = __shfl_xor_sync(0xffffffffu, idx, o);
-            if (ko > key || (ko == key && io < idx)) {
-                key = ko;
-                idx = io;
-            }
-        }
-        int p = idx;
-        if (key == 0ull) {   // the column is zero from row k down: S is singular
-            ok = false;
-            p = k;
-        }
-        if (p != k) {   // uniform
-            if (lane >= k && lane < ncol) {
-                const cx<double> a = P.A(k, lane);
-                P.A(k, lane) = P.A(p, lane);
-                P.A(p, lane) = a;
-            }
-            __syncwarp();
-        }
-        const cx<double> a = P.A(k, k);
-        const double rd = 1.0 / fma(a.re, a.re, a.im * a.im);
-        const cx<double> ip = cx<double>{a.re * rd, -a.im * rd};
-        if (lane > k && lane < M) P.A(lane, k) = cmul(P.A(lane, k), ip);
-        __syncwarp();
-        const int nr = M - 1 - k, nc = ncol - 1 - k;
-#pragma unroll 1
-        for (int e = lane; e < nr * nc; e += 32) {
-            const int c = k + 1 + e / nr, i = k + 1 + (e - (e / nr) * nr);
-            P.A(i, c) = cfnms(P.A(i, c), P.A(i, k), P.A(k, c));
-        }
-        if (lane == 31) P.A(k, k) = ip;   // nothing reads the pivot in this step's update
-        __syncwarp();
-    }
-
-    // ---- back substitution U x = b in registers: right-hand side r, row hrow
+    cx<double> cur;   // the solution: right-hand side r, row hrow
+    const bool ok = warp_lu_solve<M>(P.s + L::A, lane, two_rhs, cur);
     const bool act = r == 0 || two_rhs;
-    cx<double> cur = cx<double>{0.0, 0.0};
-    if (act && hrow < M) cur = P.A(hrow, M + r);
-#pragma unroll 1
-    for (int k = M - 1; k >= 0; k--) {
-        const int src = (lane & 16) | k;
-        const cx<double> bk = cx<double>{__shfl_sync(0xffffffffu, cur.re, src),
-                                         __shfl_sync(0xffffffffu, cur.im, src)};
-        if (hrow <= k) {
-            const cx<double> xk = cmul(bk, P.A(k, k));   // the pivot's reciprocal
-            cur = hrow == k ? xk : cfnms(cur, P.A(hrow, k), xk);
-        }
-    }
 
     // ---- back to (dx, dy) or (dp, dq) = (sp dwp, sq dwq): site j of right-hand side r on
     // lane 16 r + j, (dwp, dwq) = conj(a^, b^) q_j + (b^, -a^) s_j
@@ -434,24 +449,100 @@ __device__ bool warp_solve(const WarpPath<M> &P, const double *__restrict__ J, d
     return ok && isfinite(chk);
 }
 
-// One path per warp; the control flow of track_body in FP64, uniform over the warp.  The
-// path's state is in light-cone coordinates (p_k, q_k) = (x_k + i y_k, x_k - i y_k), like
-// the per-thread trackers' (xy_track.cuh): near infinity one of them is far below x_k and
-// y_k, and in (x, y) FP64 would lose it to cancellation.  Norms are those of (x, y):
-// ||(x, y)||_2 = sqrt(1/2) ||(p, q)||_2 and ||(x, y)||_inf = max_k max(|p + q|, |p - q|) / 2.
-template <int M, int WARPS>
-__global__ void __launch_bounds__(32 * WARPS)
-    xy_track_warp64_kernel(const __grid_constant__ XYSys S, const __grid_constant__ XYCtl C,
-                           const EPView ep, const WorkList wl) {
+// The problem a warp tracker runs on, as a policy for warp_track_body: the unknowns (NV), the
+// shared layout with the step vectors Z0, K1, AC, ZC, W1, the start point with its dz/dt, the
+// residual -H at ZC into W1, the linear solve, and the state's relation to the endpoint
+// arrays' z (load, store, NORM2: the factor from the state's squared 2-norm to z's, and this
+// lane's share of ||z||_inf at ZC).  WarpXY: the XY ring, its state in light-cone coordinates
+// (p_k, q_k) = (x_k + i y_k, x_k - i y_k), like the per-thread trackers' (xy_track.cuh): near
+// infinity one of them is far below x_k and y_k, and in (x, y) FP64 would lose it to
+// cancellation.  ||(x, y)||_2 = sqrt(1/2) ||(p, q)||_2, ||(x, y)||_inf = max_k max(|p + q|, |p - q|) / 2.
+template <int M>
+struct WarpXY {
+    using Sys = XYSys;
     using L = WarpLayout<M>;
-    constexpr int NV = 2 * M;
+    using Path = WarpPath<M>;
+    static constexpr int NV = 2 * M;
+    static constexpr double NORM2 = 0.5;
+    static __device__ __forceinline__ void load(const Path &P, const EPView &ep, int64_t e) {
+        const int64_t cnt = ep.count;
+        const int lane = P.lane;
+        if (lane < M) {   // (x, y) to (p, q)
+            const int k = lane;
+            const double xr = ep.z_re[k * cnt + e], xi = ep.z_im[k * cnt + e];
+            const double yr = ep.z_re[(M + k) * cnt + e], yi = ep.z_im[(M + k) * cnt + e];
+            P.at(L::Z0, k) = cx<double>{xr - yi, xi + yr};
+            P.at(L::Z0, M + k) = cx<double>{xr + yi, xi - yr};
+        }
+    }
+    static __device__ __forceinline__ void start(const Path &P, const Sys &S, int64_t p) {
+        const int lane = P.lane, i = lane;
+        const double *J = S.Jd;
+        const cx<double> gam = cx<double>{S.gre, S.gim};
+        if (i < NV) P.at(L::Z0, i) = cx<double>{((p >> i) & 1) ? -1.0 : 1.0, 0.0};
+        __syncwarp();
+        if (lane < M) {   // dz/dt at t = 0: -P_i(z) / (2 gamma z_i)
+            const int k = lane;
+            const cx<double> xk = P.at(L::Z0, k), yk = P.at(L::Z0, M + k);
+            const double *Jk = J + k * NPHC_JSTRIDE;
+            cx<double> u = cx<double>{Jk[M], 0.0}, w = cx<double>{0.0, 0.0};
+#pragma unroll 1
+            for (int l = 0; l < M; l++) {
+                u.re += Jk[l] * P.at(L::Z0, l).re;
+                w.re += Jk[l] * P.at(L::Z0, M + l).re;
+            }
+            cx<double> rf, rg;
+            minus_ht_rows<double>(xk, yk, u, w, gam, rf, rg);
+            const cx<double> ig = crecip(gam);
+            const cx<double> dx = cscale(0.5 * xk.re, cmul(ig, rf));
+            const cx<double> dy = cscale(0.5 * yk.re, cmul(ig, rg));
+            P.at(L::K1, k) = cadd(dx, cmul_i(dy));       // dp = dx + i dy
+            P.at(L::K1, M + k) = csub(dx, cmul_i(dy));   // dq = dx - i dy
+        }
+        __syncwarp();
+        if (lane < M) {   // p = x + i y, q = x - i y (x, y real at the start)
+            const int k = lane;
+            const double xk = P.at(L::Z0, k).re, yk = P.at(L::Z0, M + k).re;
+            P.at(L::Z0, k) = cx<double>{xk, yk};
+            P.at(L::Z0, M + k) = cx<double>{xk, -yk};
+        }
+    }
+    static __device__ __forceinline__ void residual(const Path &P, const Sys &S, double s, double omt) {
+        warp_residual<M, true>(P, S.Jd, s, omt, cx<double>{S.gre, S.gim});
+    }
+    static __device__ __forceinline__ bool solve(const Path &P, const Sys &S, double s, double omt,
+                                                 bool two_rhs, int out2) {
+        return warp_solve<M, true>(P, S.Jd, s, omt, cx<double>{S.gre, S.gim}, two_rhs, out2);
+    }
+    static __device__ __forceinline__ double norminf(const Path &P) {
+        if (P.lane >= M) return 0.0;
+        const cx<double> pk = P.at(L::ZC, P.lane), qk = P.at(L::ZC, M + P.lane);
+        return 0.5 * sqrt(fmax(cabs2(cadd(pk, qk)), cabs2(csub(pk, qk))));
+    }
+    static __device__ __forceinline__ void store(const Path &P, const EPView &ep, int64_t e) {
+        const int64_t cnt = ep.count;
+        const int lane = P.lane;
+        if (lane < M) {   // x = (p + q) / 2, y = -i (p - q) / 2
+            const int k = lane;
+            const cx<double> pk = P.at(L::Z0, k), qk = P.at(L::Z0, M + k);
+            ep.z_re[k * cnt + e] = 0.5 * (pk.re + qk.re);
+            ep.z_im[k * cnt + e] = 0.5 * (pk.im + qk.im);
+            ep.z_re[(M + k) * cnt + e] = 0.5 * (pk.im - qk.im);
+            ep.z_im[(M + k) * cnt + e] = -0.5 * (pk.re - qk.re);
+        }
+    }
+};
+
+// One path per warp; the control flow of track_body in FP64, uniform over the warp.
+template <class Q>
+__device__ __forceinline__ void warp_track_body(const typename Q::Sys &S, const XYCtl &C,
+                                                const EPView &ep, const WorkList &wl) {
+    using L = typename Q::L;
+    constexpr int NV = Q::NV;
     extern __shared__ __align__(16) unsigned char wraw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const WarpPath<M> P{reinterpret_cast<cx<double> *>(wraw) + (size_t)wid * L::TOTAL, lane};
-    const double *J = S.Jd;
-    const cx<double> gam = cx<double>{S.gre, S.gim};
+    const typename Q::Path P{reinterpret_cast<cx<double> *>(wraw) + (size_t)wid * L::TOTAL, lane};
     const int64_t total = worklist_size(wl, ep.count);
-    const int64_t cnt = ep.count;
     const int i = lane;   // vector component of this lane (i < NV)
     for (;;) {
         unsigned long long q = 0;
@@ -464,13 +555,7 @@ __global__ void __launch_bounds__(32 * WARPS)
         double t, h, hacc;
         bool need_k1;
         if (C.resume) {
-            if (lane < M) {   // (x, y) to (p, q)
-                const int k = lane;
-                const double xr = ep.z_re[k * cnt + e], xi = ep.z_im[k * cnt + e];
-                const double yr = ep.z_re[(M + k) * cnt + e], yi = ep.z_im[(M + k) * cnt + e];
-                P.at(L::Z0, k) = cx<double>{xr - yi, xi + yr};
-                P.at(L::Z0, M + k) = cx<double>{xr + yi, xi - yr};
-            }
+            Q::load(P, ep, e);
             t = ep.t[e];
             h = fmin(fmax(ep.h[e], 0.125 * (1.0 - t)), C.hmax);
             h = fmax(h, C.hmin * 4.0);
@@ -479,34 +564,7 @@ __global__ void __launch_bounds__(32 * WARPS)
             newton = ep.newton[e];
             need_k1 = true;
         } else {
-            const int64_t p = ep.path[e];
-            if (i < NV) P.at(L::Z0, i) = cx<double>{((p >> i) & 1) ? -1.0 : 1.0, 0.0};
-            __syncwarp();
-            if (lane < M) {   // dz/dt at t = 0: -P_i(z) / (2 gamma z_i)
-                const int k = lane;
-                const cx<double> xk = P.at(L::Z0, k), yk = P.at(L::Z0, M + k);
-                const double *Jk = J + k * NPHC_JSTRIDE;
-                cx<double> u = cx<double>{Jk[M], 0.0}, w = cx<double>{0.0, 0.0};
-#pragma unroll 1
-                for (int l = 0; l < M; l++) {
-                    u.re += Jk[l] * P.at(L::Z0, l).re;
-                    w.re += Jk[l] * P.at(L::Z0, M + l).re;
-                }
-                cx<double> rf, rg;
-                minus_ht_rows<double>(xk, yk, u, w, gam, rf, rg);
-                const cx<double> ig = crecip(gam);
-                const cx<double> dx = cscale(0.5 * xk.re, cmul(ig, rf));
-                const cx<double> dy = cscale(0.5 * yk.re, cmul(ig, rg));
-                P.at(L::K1, k) = cadd(dx, cmul_i(dy));       // dp = dx + i dy
-                P.at(L::K1, M + k) = csub(dx, cmul_i(dy));   // dq = dx - i dy
-            }
-            __syncwarp();
-            if (lane < M) {   // p = x + i y, q = x - i y (x, y real at the start)
-                const int k = lane;
-                const double xk = P.at(L::Z0, k).re, yk = P.at(L::Z0, M + k).re;
-                P.at(L::Z0, k) = cx<double>{xk, yk};
-                P.at(L::Z0, M + k) = cx<double>{xk, -yk};
-            }
+            Q::start(P, S, ep.path[e]);
             t = 0.0;
             h = C.h0;
             steps = C.accumulate ? ep.steps[e] : 0;
@@ -543,8 +601,8 @@ __global__ void __launch_bounds__(32 * WARPS)
                     }
                     __syncwarp();
                 }
-                if (corr) warp_residual<M, true>(P, J, te, 1.0 - te, gam);
-                const bool oks = warp_solve<M, true>(P, J, te, 1.0 - te, gam, corr, L::AC);
+                if (corr) Q::residual(P, S, te, 1.0 - te);
+                const bool oks = Q::solve(P, S, te, 1.0 - te, corr, L::AC);
                 solves++;
                 if (ph == 0) {   // pull the resumed point onto the FP64 path; dz/dt there
                     if (i < NV) {
@@ -571,12 +629,12 @@ __global__ void __launch_bounds__(32 * WARPS)
                             P.at(L::ZC, i) = zp;
                             zz = cabs2(zp);
                         }
-                        zpn = sqrt(0.5 * warp_sum(zz));
+                        zpn = sqrt(Q::NORM2 * warp_sum(zz));
                     }
                     __syncwarp();
                 } else {
                     newton++;
-                    const double dn = sqrt(0.5 * warp_sum(i < NV ? cabs2(P.at(L::W1, i)) : 0.0));
+                    const double dn = sqrt(Q::NORM2 * warp_sum(i < NV ? cabs2(P.at(L::W1, i)) : 0.0));
                     if (!oks || !isfinite(dn)) {
                         bad = true;
                     } else if (ph == 4 && dn > C.trust * (1.0 + zpn)) {
@@ -588,7 +646,7 @@ __global__ void __launch_bounds__(32 * WARPS)
                             P.at(L::ZC, i) = zn;
                             zz = cabs2(zn);
                         }
-                        zz = 0.5 * warp_sum(zz);
+                        zz = Q::NORM2 * warp_sum(zz);
                         if (dn <= C.eps * (1.0 + sqrt(zz))) conv = true;
                     }
                     __syncwarp();
@@ -597,16 +655,11 @@ __global__ void __launch_bounds__(32 * WARPS)
             if (status != NPHC_PATH_RUNNING) break;
             attempts++;
             if (conv) {
-                double zi = 0.0;   // ||(x, y)||_inf
                 if (i < NV) {
                     P.at(L::Z0, i) = P.at(L::ZC, i);
                     P.at(L::K1, i) = P.at(L::AC, i);
                 }
-                if (lane < M) {
-                    const cx<double> pk = P.at(L::ZC, lane), qk = P.at(L::ZC, M + lane);
-                    zi = 0.5 * sqrt(fmax(cabs2(cadd(pk, qk)), cabs2(csub(pk, qk))));
-                }
-                zi = warp_max(zi);
+                const double zi = warp_max(Q::norminf(P));   // of the endpoint arrays' z
                 __syncwarp();
                 t = t1;
                 far = 1.0 - t < CRAWL_ZONE && zi > FAR_NORM && zi > FAR_GROWTH * zlast;
@@ -628,14 +681,7 @@ __global__ void __launch_bounds__(32 * WARPS)
             }
             if (status == NPHC_PATH_RUNNING && attempts >= C.max_steps) status = NPHC_PATH_STEP_BUDGET;
         }
-        if (lane < M) {   // x = (p + q) / 2, y = -i (p - q) / 2
-            const int k = lane;
-            const cx<double> pk = P.at(L::Z0, k), qk = P.at(L::Z0, M + k);
-            ep.z_re[k * cnt + e] = 0.5 * (pk.re + qk.re);
-            ep.z_im[k * cnt + e] = 0.5 * (pk.im + qk.im);
-            ep.z_re[(M + k) * cnt + e] = 0.5 * (pk.im - qk.im);
-            ep.z_im[(M + k) * cnt + e] = -0.5 * (pk.re - qk.re);
-        }
+        Q::store(P, ep, e);
         if (lane == 0) {
             ep.t[e] = t;
             ep.h[e] = h;
@@ -646,4 +692,11 @@ __global__ void __launch_bounds__(32 * WARPS)
         }
         __syncwarp();
     }
+}
+
+template <int M, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS)
+    xy_track_warp64_kernel(const __grid_constant__ XYSys S, const __grid_constant__ XYCtl C,
+                           const EPView ep, const WorkList wl) {
+    warp_track_body<WarpXY<M>>(S, C, ep, wl);
 }
