@@ -659,9 +659,17 @@ nphc_status nphc_classify(const nphc_system *S, const nphc_endpoints *ep, double
     if ((s = check_ep(S, ep, true)) != NPHC_OK) return s;
     if (!theta || !index || !energy) return fail(NPHC_EINVAL, "output arrays missing");
     if (S->quad) return fail(NPHC_EINVAL, "classification needs an XY system");
-    XYSys xs = S->xs;
-    NPHC_CK(launch_xy_classify(S->M, xs, view(ep), theta, index, energy, min_abs_eig, log_abs_det,
-                               (cudaStream_t)stream));
+    if (ep->count == 0) return NPHC_OK;
+    const XYSys xs = S->xs;
+    cudaStream_t st = (cudaStream_t)stream;
+    // defaults for every entry, then the real ones
+    const size_t row = sizeof(double) * ep->count;
+    NPHC_CK(cudaMemsetAsync(theta, 0, row * S->M, st));
+    NPHC_CK(cudaMemsetAsync(energy, 0, row, st));
+    if (min_abs_eig) NPHC_CK(cudaMemsetAsync(min_abs_eig, 0, row, st));
+    if (log_abs_det) NPHC_CK(cudaMemsetAsync(log_abs_det, 0, row, st));
+    NPHC_CK(cudaMemsetAsync(index, 0xff, sizeof(int32_t) * ep->count, st));
+    NPHC_CK(launch_xy_classify(S->M, xs, view(ep), theta, index, energy, min_abs_eig, log_abs_det, st));
     return NPHC_OK;
 }
 

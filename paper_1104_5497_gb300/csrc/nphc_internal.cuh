@@ -251,8 +251,8 @@ cudaError_t launch_xy_track_f64_warp(int M, const XYSys &sys, const XYCtl &ctl, 
 cudaError_t launch_xy_refine_certify(int M, const XYSys &sys, double tol_sol, double refine_eps,
                                      int refine_iters, const EPView &ep, int64_t cap,
                                      const WorkList &wl, int shortcut, cudaStream_t st);
-// Classification of every entry, or (list, device list_count) of listed real entries only,
-// 32 to a warp (the other entries' outputs are then left as they are).
+// Classification of the real entries, all of them or (list, device list_count) the listed
+// ones; the other entries' outputs are left as they are.
 cudaError_t launch_xy_classify(int M, const XYSys &sys, const EPView &ep, double *theta,
                                int32_t *index, double *energy, double *min_eig,
                                double *log_abs_det,

@@ -253,8 +253,23 @@ cudaError_t NPHC_CAT(launch_xy_adjoint_m, NPHC_INST_M)(const XYSys &sys, int64_t
                                                       const double *g_theta, double *dJ,
                                                       cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
-    const int grid = (int)((count + 127) / 128);
-    xy_adjoint_kernel<NPHC_INST_M><<<grid, 128, 0, st>>>(sys, count, theta, g_energy, g_theta, dJ);
+    constexpr int M = NPHC_INST_M;
+    const size_t smem = adj_smem_per_block<M>();
+    auto k = xy_adjoint_kernel<M>;
+    static bool attr_set = false;   // once per process for this instantiation
+    if (!attr_set) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    // a warp per scheduler (the FP64 pipe is busy with one), fewer when a warp per point is fewer
+    const int64_t need = (count + ADJ_WARPS - 1) / ADJ_WARPS;
+    const int grid = (int)(need < sms ? need : sms);
+    k<<<grid, 32 * ADJ_WARPS, smem, st>>>(sys, count, theta, g_energy, g_theta, dJ);
     nphc_launch_counter(1);
     return cudaGetLastError();
 }
@@ -266,10 +281,23 @@ cudaError_t NPHC_CAT(launch_xy_classify_m, NPHC_INST_M)(const XYSys &sys, const 
                                                        const int32_t *list_count,
                                                        cudaStream_t st) {
     if (ep.count <= 0) return cudaSuccess;
-    // a list is at most ep.count long (its length is on the device)
-    const int grid = (int)((ep.count + 127) / 128);
-    xy_classify_kernel<NPHC_INST_M><<<grid, 128, 0, st>>>(sys, ep, theta, index, energy, min_eig,
-                                                                   log_abs_det, list, list_count);
+    constexpr int M = NPHC_INST_M;
+    const size_t smem = cls_smem_per_block<M>();
+    auto k = xy_classify_kernel<M>;
+    static bool attr_set = false;   // once per process for this instantiation
+    if (!attr_set) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    // a warp per scheduler, at most one point per warp (a list is at most ep.count long)
+    const int64_t full = (int64_t)sms * 4;
+    const int grid = (int)(ep.count < full ? ep.count : full);
+    k<<<grid, 32, smem, st>>>(sys, ep, theta, index, energy, min_eig, log_abs_det, list, list_count);
     nphc_launch_counter(1);
     return cudaGetLastError();
 }

@@ -80,6 +80,14 @@ struct RGPath {
     __device__ __forceinline__ void sync() const { __syncwarp(m); }
 };
 
+// Warps (one-warp blocks) of a launch with up to two per scheduler that share `total` items,
+// `slots` side by side in each: half of them while that is enough, so that no scheduler runs
+// two FP64 chains where one would do.
+__device__ __forceinline__ int fill_warps(int64_t total, int slots) {
+    const int half = ((int)gridDim.x + 1) / 2;
+    return total <= (int64_t)half * slots ? half : (int)gridDim.x;
+}
+
 // P, the factorisation of DP and the Newton correction D = -DP^-1 P (into QA, QB) at Z.  res = ||P||_inf,
 // dn2 = ||D||_2^2, z2 = ||z||_2^2; perm: the row of S behind each row of the factor, four bits
 // each.  False when the Schur matrix is singular.
@@ -312,8 +320,10 @@ __global__ void __launch_bounds__(32)
     const int64_t cnt = ep.count, total = worklist_size(wl, cnt);
 
     // entries one per warp before more per warp: i = endpoint slot * warps + warp
-    int64_t next = (int64_t)pth * gridDim.x + blockIdx.x;
-    const int64_t stride = (int64_t)RG_PATHS * gridDim.x;
+    const int warps = fill_warps(total, RG_PATHS);
+    if ((int)blockIdx.x >= warps) return;
+    int64_t next = (int64_t)pth * warps + blockIdx.x;
+    const int64_t stride = (int64_t)RG_PATHS * warps;
     enum { IDLE, EVALUATE, CERTIFY, DONE };
     enum { NEWTON, LAST, FINAL, REAL };   // what the evaluation is for: a Newton step, the one
                                           // whose correction met the tolerance, a certificate
