@@ -212,5 +212,3 @@ struct F32Step {
         ep.newton[e] = newton;
     }
 };
-
-enum { F32_GO_ON, F32_ACCEPT, F32_REJECT, F32_ANCHORED };   // a step attempt's verdict

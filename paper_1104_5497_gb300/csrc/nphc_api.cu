@@ -490,6 +490,13 @@ EPView view(const nphc_endpoints *e) {
     return v;
 }
 
+// FP64 tracking: paths per scheduler from which four lanes per path (xy_track_group64.cuh) beat
+// a warp per path (xy_track_warp.cuh).  Whole passes, measured (warp / group, ms): 2,500 paths of
+// N = 8 52 / 70, 4,096 79 / 73, 16,384 281 / 122; of N = 10 4,096 102 / 129, 8,192 185 / 136.  Lists
+// (hand-offs, re-tracks) hold paths of very different lengths, and a group's chain is three
+// times a warp's: the 9,493 hand-offs of an N = 10 ring take 20 ms by warps and 29 by groups.
+constexpr int64_t kFewPerScheduler = 7, kFewListedPerScheduler = 32;
+
 nphc_status track_impl(const nphc_system *S, const nphc_options *o, nphc_precision prec,
                        const nphc_endpoints *ep, const int32_t *list, const int32_t *list_count,
                        bool resume, bool accumulate, void *ws, int queue_slot, cudaStream_t st,
@@ -508,24 +515,26 @@ nphc_status track_impl(const nphc_system *S, const nphc_options *o, nphc_precisi
     wl.state = static_cast<char *>(ws) + ws_layout(S->n, 0).state;
     wl.state_threads = NPHC_TRACK_MAX_THREADS;
     NPHC_CK(cudaMemsetAsync(wl.queue, 0, sizeof(unsigned long long), st));
-    int grid = 0;
-    if (f32 && o->blocks_per_sm > 0) {
-        int dev = 0, sms = 0;
-        NPHC_CK(cudaGetDevice(&dev));
-        NPHC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        grid = sms * o->blocks_per_sm;
-    }
+    int dev = 0, sms = 0;
+    NPHC_CK(cudaGetDevice(&dev));
+    NPHC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const EPView v = view(ep);
-    if (S->quad)
+    if (S->quad) {
         NPHC_CK(launch_quad_track(S->n, quad_with_gamma(S, o), ctl, v, wl, st));
-    else if (!f32 && list != nullptr && o->threads_per_path != 1)   // one path per warp
-        NPHC_CK(launch_xy_track_f64_warp_bps(S->M, xs, ctl, v, wl, o->list_blocks_per_sm, st));
-    else if (!f32 && list != nullptr)   // FP64 lists, one path per thread, full warps
+    } else if (f32) {
+        NPHC_CK(launch_xy_track_f32(S->M, xs, ctl, v, wl, 0, sms * o->blocks_per_sm, st));
+    } else if (list != nullptr && o->threads_per_path == 1) {   // one path per thread, full warps
         NPHC_CK(launch_xy_track_f64(S->M, xs, ctl, v, wl, 0, 0, st));
-    else if (f32)
-        NPHC_CK(launch_xy_track_f32(S->M, xs, ctl, v, wl, 0, grid, st));
-    else
-        NPHC_CK(launch_xy_track_f64(S->M, xs, ctl, v, wl, 0, 0, st));
+    } else if (list != nullptr && o->threads_per_path == 32) {
+        NPHC_CK(launch_xy_track_f64_warp(S->M, xs, ctl, v, wl, o->list_blocks_per_sm, INT64_MAX, st));
+    } else {
+        // One path per warp for few paths, four lanes per path for many; the length of a list
+        // is on the device, so both kernels get it and one of them returns at once.
+        const int64_t few = (list != nullptr ? kFewListedPerScheduler : kFewPerScheduler) * 4 * sms;
+        if (list != nullptr || ep->count < few)
+            NPHC_CK(launch_xy_track_f64_warp(S->M, xs, ctl, v, wl, o->list_blocks_per_sm, few, st));
+        NPHC_CK(launch_xy_track_f64_group(S->M, xs, ctl, v, wl, few, st));
+    }
     return NPHC_OK;
 }
 

@@ -245,9 +245,6 @@ cudaError_t launch_xy_track_f64(int M, const XYSys &sys, const XYCtl &ctl, const
 // The FP32 pass over every path of a batch group (ring size M), one persistent launch.
 cudaError_t launch_xy_track_f32_batch(int M, const BatchGroup &bg, const XYCtl &ctl,
                                       const WorkList &wl, int grid, cudaStream_t st);
-// FP64 tracking with one path per warp (xy_track_warp.cuh), for short lists.
-cudaError_t launch_xy_track_f64_warp(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
-                                     const WorkList &wl, cudaStream_t st);
 cudaError_t launch_xy_refine_certify(int M, const XYSys &sys, double tol_sol, double refine_eps,
                                      int refine_iters, const EPView &ep, int64_t cap,
                                      const WorkList &wl, int shortcut, cudaStream_t st);

@@ -19,7 +19,9 @@
     cudaError_t launch_xy_track_f64_m##MM(const XYSys &, const XYCtl &, const EPView &,     \
                                           const WorkList &, int, cudaStream_t);              \
     cudaError_t launch_xy_track_f64w_m##MM(const XYSys &, const XYCtl &, const EPView &,    \
-                                           const WorkList &, int, cudaStream_t);            \
+                                           const WorkList &, int, int64_t, cudaStream_t);   \
+    cudaError_t launch_xy_track_f64g_m##MM(const XYSys &, const XYCtl &, const EPView &,    \
+                                           const WorkList &, int64_t, cudaStream_t);        \
     cudaError_t launch_xy_refine_certify_m##MM(const XYSys &, double, double, int,          \
                                                const EPView &, int64_t, const WorkList &,   \
                                                int, cudaStream_t);                          \
@@ -45,8 +47,10 @@ NPHC_FOR_EACH_M(NPHC_DECL)
 NPHC_FOR_EACH_QN(NPHC_QDECL)
 #undef NPHC_QDECL
 
-// The FP64 list tracker with a chosen number of blocks per SM (0: automatic); the
-// launcher of nphc_internal.cuh is this one with 0.
-cudaError_t launch_xy_track_f64_warp_bps(int M, const XYSys &sys, const XYCtl &ctl,
-                                         const EPView &ep, const WorkList &wl, int blocks_per_sm,
-                                         cudaStream_t st);
+// FP64 tracking with one path per warp (blocks_per_sm blocks of four, 0: two) of launches and
+// lists shorter than max_paths, and with four lanes per path of those of min_paths or more.
+cudaError_t launch_xy_track_f64_warp(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
+                                     const WorkList &wl, int blocks_per_sm, int64_t max_paths,
+                                     cudaStream_t st);
+cudaError_t launch_xy_track_f64_group(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
+                                      const WorkList &wl, int64_t min_paths, cudaStream_t st);

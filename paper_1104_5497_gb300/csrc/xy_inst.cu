@@ -154,13 +154,14 @@ cudaError_t NPHC_CAT(launch_xy_track_f32_batch_m, NPHC_INST_M)(const BatchGroup 
 #endif
 
 #if NPHC_INST_KIND == 1
-#include "xy_track_warp.cuh"
+#include "xy_track_group64.cuh"
 
 // one path per warp (short FP64 lists), 4 warps per block, blocks_per_sm blocks per SM
 // (0: two)
 cudaError_t NPHC_CAT(launch_xy_track_f64w_m, NPHC_INST_M)(const XYSys &sys, const XYCtl &ctl,
                                                           const EPView &ep, const WorkList &wl,
-                                                          int blocks_per_sm, cudaStream_t st) {
+                                                          int blocks_per_sm, int64_t max_paths,
+                                                          cudaStream_t st) {
     constexpr int M = NPHC_INST_M, WARPS = 4;
     if (ep.count <= 0) return cudaSuccess;
     const size_t smem = warp_track_smem_per_warp<M>() * WARPS;
@@ -182,9 +183,37 @@ cudaError_t NPHC_CAT(launch_xy_track_f64w_m, NPHC_INST_M)(const XYSys &sys, cons
     // the mean and the others idled half the launch)
     const int want = blocks_per_sm > 0 ? blocks_per_sm : 2;
     const int64_t full = (int64_t)sms * (per < want ? (per > 0 ? per : 1) : want);
-    const int64_t need = (ep.count + WARPS - 1) / WARPS;   // the list is at most ep.count long
+    // at most max_paths run here, and the list is at most ep.count long
+    const int64_t most = ep.count < max_paths ? ep.count : max_paths;
+    const int64_t need = (most + WARPS - 1) / WARPS;
     const int grid = (int)(need < full ? need : full);
-    k<<<grid, 32 * WARPS, smem, st>>>(sys, ctl, ep, wl);
+    k<<<grid, 32 * WARPS, smem, st>>>(sys, ctl, ep, wl, max_paths);
+    nphc_launch_counter(1);
+    return cudaGetLastError();
+}
+
+// four lanes per path, for min_paths paths or more
+cudaError_t NPHC_CAT(launch_xy_track_f64g_m, NPHC_INST_M)(const XYSys &sys, const XYCtl &ctl,
+                                                          const EPView &ep, const WorkList &wl,
+                                                          int64_t min_paths, cudaStream_t st) {
+    constexpr int M = NPHC_INST_M;
+    if (ep.count <= 0 || ep.count < min_paths) return cudaSuccess;
+    const size_t smem = g64_smem_per_block<M>();
+    auto k = xy_track_group64_kernel<M>;
+    static bool attr_set = false;   // once per process for this instantiation
+    if (!attr_set) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
+    int dev = 0, sms = 0, per = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 32, smem);
+    if (e != cudaSuccess) return e;
+    // one or two warps on each scheduler (paths are pulled from a queue)
+    const int64_t grid = (int64_t)sms * (per >= 8 ? 8 : per >= 4 ? 4 : per > 0 ? per : 1);
+    k<<<(int)std::min(grid, ep.count), 32, smem, st>>>(sys, ctl, ep, wl, min_paths);
     nphc_launch_counter(1);
     return cudaGetLastError();
 }

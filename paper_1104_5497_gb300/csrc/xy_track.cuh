@@ -70,6 +70,9 @@ struct JSel<double> {
 #define FAR_NORM 10.0
 #define FAR_GROWTH 1.01
 #define KAPPA_FAR 0.38
+// What a group tracker knows of a step attempt after a solve (ANCHORED: a resumed point has been
+// pulled onto this precision's path).
+enum { STEP_GO_ON, STEP_ACCEPT, STEP_REJECT, STEP_ANCHORED };
 #define NEAR_END 1e-5     // FP32 radius crossings with 1 - t below this ...
 #define RDIV_BAND 1e-3    // ... and ||z||_inf within rdiv (1 + RDIV_BAND) go to FP64
 

@@ -581,7 +581,7 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
         const bool corr = nc > 0 && 2 * nc >= np;
         const bool w = act && wants_c == corr;
         const f32_time te = ph == 0 ? P.t : ph < 3 ? P.t + hh / 2 : t1;
-        int verdict = F32_GO_ON, status = NPHC_PATH_RUNNING;
+        int verdict = STEP_GO_ON, status = NPHC_PATH_RUNNING;
         float zi = 0.0f;
         GrpStep<SL> dt, dr;
         float kest;
@@ -617,7 +617,7 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
             if (w) {
                 zpn = sqrtf(0.5f * zz);   // ||(x, y)||_2 of the predicted point
                 ph++;
-                if (ph == 4 && bad) verdict = F32_REJECT;
+                if (ph == 4 && bad) verdict = STEP_REJECT;
             }
         } else {
             // ---- corrector iteration (phase 0: a resumed point pulled onto this precision's
@@ -652,20 +652,20 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
                 P.newton++;
                 kstep = fmaxf(kstep, kest);
                 if (ph == 0) {
-                    verdict = F32_ANCHORED;
+                    verdict = STEP_ANCHORED;
                     if (!oks) status = C.handoff ? NPHC_PATH_HANDOFF : NPHC_PATH_NONFINITE;
                 } else if (move && dn <= K.eps * (1.0f + sqrtf(0.5f * zz))) {
                     // a converged step whose systems' condition estimate exceeds kappa (0: no
                     // test) is not taken: FP64 continues the path from its last accepted
                     // point (or the end zone's clean checkpoint)
-                    verdict = F32_ACCEPT;
+                    verdict = STEP_ACCEPT;
                     if (K.kappa > 0.0f && !(kstep <= K.kappa)) status = NPHC_PATH_HANDOFF_COND;
                 } else if (fail || ph + 1 >= 4 + C.max_newton) {
-                    verdict = F32_REJECT;
+                    verdict = STEP_REJECT;
                 } else {
                     ph++;
                 }
-                if ((verdict == F32_ACCEPT || verdict == F32_ANCHORED) && status == NPHC_PATH_RUNNING) {
+                if ((verdict == STEP_ACCEPT || verdict == STEP_ANCHORED) && status == NPHC_PATH_RUNNING) {
 #pragma unroll
                     for (int q = 0; q < SL; q++)
                         if (own(q)) {
@@ -677,17 +677,17 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
             }
         }
         // ---- the step attempt is over
-        if (verdict != F32_GO_ON) {
+        if (verdict != STEP_GO_ON) {
             bool save = false;
-            if (verdict == F32_ACCEPT && status == NPHC_PATH_RUNNING) status = P.accept(K, C, t1, zi, save);
-            else if (verdict == F32_REJECT) status = P.reject(K, C);
+            if (verdict == STEP_ACCEPT && status == NPHC_PATH_RUNNING) status = P.accept(K, C, t1, zi, save);
+            else if (verdict == STEP_REJECT) status = P.reject(K, C);
             status = P.budget(C, status);
             if (save) {
 #pragma unroll
                 for (int q = 0; q < SL; q++)
                     if (own(q)) ck[(g + 4 * q) * slots] = at(L::PQ, g + 4 * q);
             }
-            if (verdict != F32_ANCHORED) kstep = 0.0f;
+            if (verdict != STEP_ANCHORED) kstep = 0.0f;
             start = status == NPHC_PATH_RUNNING;
             if (!start) {
                 const EPView &ep = src.eps(inst);

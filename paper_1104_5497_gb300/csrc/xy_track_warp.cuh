@@ -534,15 +534,18 @@ struct WarpXY {
 };
 
 // One path per warp; the control flow of track_body in FP64, uniform over the warp.
+// A list of max_paths entries or more is left to the group kernel (xy_track_group64.cuh).
 template <class Q>
 __device__ __forceinline__ void warp_track_body(const typename Q::Sys &S, const XYCtl &C,
-                                                const EPView &ep, const WorkList &wl) {
+                                                const EPView &ep, const WorkList &wl,
+                                                int64_t max_paths = INT64_MAX) {
     using L = typename Q::L;
     constexpr int NV = Q::NV;
     extern __shared__ __align__(16) unsigned char wraw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const typename Q::Path P{reinterpret_cast<cx<double> *>(wraw) + (size_t)wid * L::TOTAL, lane};
     const int64_t total = worklist_size(wl, ep.count);
+    if (total >= max_paths) return;
     const int i = lane;   // vector component of this lane (i < NV)
     for (;;) {
         unsigned long long q = 0;
@@ -697,6 +700,6 @@ __device__ __forceinline__ void warp_track_body(const typename Q::Sys &S, const 
 template <int M, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS)
     xy_track_warp64_kernel(const __grid_constant__ XYSys S, const __grid_constant__ XYCtl C,
-                           const EPView ep, const WorkList wl) {
-    warp_track_body<WarpXY<M>>(S, C, ep, wl);
+                           const EPView ep, const WorkList wl, int64_t max_paths) {
+    warp_track_body<WarpXY<M>>(S, C, ep, wl, max_paths);
 }
