@@ -478,5 +478,8 @@ __global__ void __launch_bounds__(32)
                 }
             }
         }
+        // an entry's unknowns are loaded by other lanes than those that have just written out the
+        // slot's last one
+        __syncwarp();
     }
 }
