@@ -1,23 +1,54 @@
-// f32_step.cuh -- the building blocks of the FP32 group tracker (xy_track_group.cuh):
-// arithmetic in pairs (f32x2), compensated sums of pairs, and one path's step control.
+// f32_step.cuh -- what the FP32 trackers (xy_track_group.cuh, xy_track_lane.cuh) share: arithmetic
+// in pairs (f32x2), compensated sums of pairs, the terms of one site, one path's step control.
 #pragma once
 
 #include "xy_track.cuh"
 
 // ------------------------------------------------------------- f32x2 pairs --
+// A pair is a complex number (re, im) or two neighbours.  The paired instructions take their
+// operands negated, swapped or one half twice at no cost (static instruction counts), so
+// f2dup, f2neg and f2i below are free as operands, and a complex product is two instructions.
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ float2 f2dup(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 f2neg(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 f2add(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 f2mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-// a - b (the product with -1 is exact: one rounding, as a subtraction)
-__device__ __forceinline__ float2 f2sub(float2 a, float2 b) {
-    return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
-}
+__device__ __forceinline__ float2 f2sub(float2 a, float2 b) { return __fadd2_rn(a, f2neg(b)); }
 __device__ __forceinline__ float2 f2i(float2 a) { return make_float2(-a.y, a.x); }   // i a
-__device__ __forceinline__ cx<float> f2c(float2 a) { return cx<float>{a.x, a.y}; }
-__device__ __forceinline__ float2 c2f(cx<float> a) { return make_float2(a.re, a.im); }
+__device__ __forceinline__ float2 f2scale(float s, float2 a) { return f2mul(f2dup(s), a); }
+__device__ __forceinline__ float f2abs2(float2 a) { return fmaf(a.x, a.x, a.y * a.y); }
+// complex a b, conj(a) b, c + a b, c - a b
+__device__ __forceinline__ float2 f2cmul(float2 a, float2 b) { return f2fma(f2dup(a.y), f2i(b), f2mul(f2dup(a.x), b)); }
+__device__ __forceinline__ float2 f2cmulc(float2 a, float2 b) {
+    return f2fma(f2dup(-a.y), f2i(b), f2mul(f2dup(a.x), b));
+}
+__device__ __forceinline__ float2 f2cfma(float2 a, float2 b, float2 c) {
+    return f2fma(f2dup(a.y), f2i(b), f2fma(f2dup(a.x), b, c));
+}
+__device__ __forceinline__ float2 f2cfms(float2 a, float2 b, float2 c) {
+    return f2fma(f2dup(-a.y), f2i(b), f2fma(f2dup(-a.x), b, c));
+}
+
+// Square root and reciprocal square root for the light-cone scales and frames (any scale solves
+// the same system, and the frame's error of two ulp is the row's own rounding), and a pivot's
+// reciprocal with one Newton step: one to three instructions where the IEEE forms take
+// thirteen to fifteen.
+__device__ __forceinline__ float f32_sqrt(float x) {
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float f32_rsqrt(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float f32_recip(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return fmaf(fmaf(-x, r, 1.0f), r, r);
+}
 
 // A pair of two-word numbers (EFT, nphc_internal.cuh): the same error-free transformations
 // on both halves.
@@ -25,23 +56,20 @@ struct ext2 {
     float2 hi, lo;
 };
 
-// acc += c v, nc = -c; as ext_acc
-__device__ __forceinline__ void acc2(ext2 &acc, float2 c, float2 nc, float2 v) {
-    const float2 np = f2mul(nc, v);        // -(the rounded product)
-    const float2 e = f2fma(c, v, np);      // its rounding error
-    const float2 s = f2sub(acc.hi, np);
+// acc += c v; as ext_acc
+__device__ __forceinline__ void acc2(ext2 &acc, float2 c, float2 v) {
+    const float2 p = f2mul(c, v);
+    const float2 e = f2fma(c, v, f2neg(p));   // the product's rounding error
+    const float2 s = f2add(acc.hi, p);
     const float2 bb = f2sub(s, acc.hi);
-    const float2 e2 = f2sub(f2sub(acc.hi, f2sub(s, bb)), f2add(np, bb));
+    const float2 e2 = f2add(f2sub(acc.hi, f2sub(s, bb)), f2sub(p, bb));
     acc.hi = s;
     acc.lo = f2add(acc.lo, f2add(e, e2));
 }
 // acc += c (v.hi + v.lo); as ext_acc_ext
-__device__ __forceinline__ void acc2_ext(ext2 &acc, float2 c, float2 nc, const ext2 &v) {
-    acc2(acc, c, nc, v.hi);
-    acc.lo = f2fma(c, v.lo, acc.lo);
-}
 __device__ __forceinline__ void acc2_ext(ext2 &acc, float c, const ext2 &v) {
-    acc2_ext(acc, f2dup(c), f2dup(-c), v);
+    acc2(acc, f2dup(c), v.hi);
+    acc.lo = f2fma(f2dup(c), v.lo, acc.lo);
 }
 // (a.hi + a.lo) + (b.hi + b.lo)
 __device__ __forceinline__ ext2 ext2_add(const ext2 &a, const ext2 &b) {
@@ -56,8 +84,8 @@ __device__ __forceinline__ ext2 ext2_scale(float c, const ext2 &a) {   // c a po
 __device__ __forceinline__ ext2 ext2_i(const ext2 &v) { return ext2{f2i(v.hi), f2i(v.lo)}; }
 // acc += a b for complex a, b: exact products
 __device__ __forceinline__ void acc2_cmul(ext2 &acc, float2 a, float2 b) {
-    acc2(acc, f2dup(a.x), f2dup(-a.x), b);
-    acc2(acc, f2dup(a.y), f2dup(-a.y), f2i(b));
+    acc2(acc, f2dup(a.x), b);
+    acc2(acc, f2dup(a.y), f2i(b));
 }
 
 // The rows (-H_f, -H_g) of one site at (p, q), compensated, from the compensated sums
@@ -90,6 +118,45 @@ __device__ __forceinline__ void f32_residual_rows(float2 pk, float2 qk, const ex
     acc2_ext(hg, s, G);
     rf = f2neg(f2add(hf.hi, hf.lo));
     rg = f2neg(f2add(hg.hi, hg.lo));
+}
+
+// The terms of site j at (p, q) = (p_j, q_j) with U_p, U_q (xy_solve.cuh): the scaled light-cone
+// frame (g_frame_lc) sb = sp b^, sa = sq a^, the Schur matrix's diagonal entry sjj, and for a
+// right-hand side (rf, rg) X, Y (xy_solve.cuh) and the site's own share d = rf - A px - B py.
+struct F32Site {
+    float2 ah, bh, sb, sa, sjj, Ajj, Bjj;
+    float iv, sp, sq;
+    __device__ __forceinline__ void rhs(float2 rf, float2 rg, float2 &x, float2 &y, float2 &d) const {
+        const float2 c = f2scale(iv, rg);
+        const float2 px = f2cmulc(ah, c), py = f2cmulc(bh, c);
+        x = f2scale(sp, px);
+        y = f2scale(sq, py);
+        d = f2cfms(Bjj, py, f2cfms(Ajj, px, rf));
+    }
+};
+
+// Also -H_t's rows (lc_minus_ht_rows) into htf, htg.  hs = t / 2, hgomt = gamma (1 - t) / 2.
+__device__ __forceinline__ F32Site f32_site(float2 p, float2 q, float2 Up, float2 Uq, float s, float hs,
+                                            float2 hgomt, float2 gam, float2 &htf, float2 &htg) {
+    F32Site v;
+    const float2 one = f2(1.0f, 0.0f), a = f2add(p, q), d = f2sub(p, q);
+    const float2 D = f2cfms(p, Uq, f2cmul(q, Up));   // f = i D / 2
+    htf = f2cfma(gam, f2fma(f2dup(0.25f), f2cmul(a, a), f2neg(one)), f2scale(-0.5f, f2i(D)));
+    htg = f2cfma(gam, f2fma(f2dup(-0.25f), f2cmul(d, d), f2neg(one)), f2cfms(p, q, one));
+    v.sp = fmaxf(1.0f, f32_sqrt(f2abs2(p)));
+    v.sq = fmaxf(1.0f, f32_sqrt(f2abs2(q)));
+    const float2 hd = f2cmul(hgomt, d);
+    const float2 ra = f2scale(v.sp, f2fma(f2dup(s), q, f2neg(hd))), rb = f2scale(v.sq, f2fma(f2dup(s), p, hd));
+    v.iv = f32_rsqrt(f2abs2(ra) + f2abs2(rb));
+    v.ah = f2scale(v.iv, ra);
+    v.bh = f2scale(v.iv, rb);
+    v.sb = f2scale(v.sp, v.bh);
+    v.sa = f2scale(v.sq, v.ah);
+    const float2 g = f2cmul(hgomt, a);
+    v.Ajj = f2scale(v.sp, f2fma(f2dup(-hs), f2i(Uq), g));
+    v.Bjj = f2scale(v.sq, f2fma(f2dup(hs), f2i(Up), g));
+    v.sjj = f2cfms(v.Bjj, v.ah, f2cmul(v.Ajj, v.bh));
+    return v;
 }
 
 // ------------------------------------------------------------ step control --

@@ -8,8 +8,8 @@
 
 #include "nphc.h"
 
-#define NPHC_MAXN NPHC_MAX_N          // couplings are stored in NPHC_MAXN x NPHC_MAXN tables
-#define NPHC_JSTRIDE NPHC_MAXN
+#define NPHC_MAXN NPHC_MAX_N          // couplings are stored in NPHC_MAXN rows of
+#define NPHC_JSTRIDE 16               // NPHC_JSTRIDE numbers (128-bit loads of four)
 
 // ------------------------------------------------------------------ complex --
 template <class R>
@@ -119,8 +119,9 @@ __device__ __forceinline__ R ext_val(ext<R> a) { return EFT<R>::add(a.hi, a.lo);
 // unrolled kernels read them as constant-bank operands.
 struct XYSys {
     int N;                                  // ring size; M = N - 1 free sites
-    float Jf[NPHC_MAXN * NPHC_MAXN];        // J in FP32 (row k, column j at k * NPHC_JSTRIDE + j)
-    double Jd[NPHC_MAXN * NPHC_MAXN];       // J in FP64
+    alignas(16) float Jf[NPHC_MAXN * NPHC_JSTRIDE];   // J in FP32 (row k, column j at
+                                                      // k * NPHC_JSTRIDE + j; zeros beyond)
+    double Jd[NPHC_MAXN * NPHC_JSTRIDE];    // J in FP64
     double gre, gim;                        // gamma
     double d2norm;                          // ||D^2 P / 2|| bound (alpha-theory gamma)
     double kappa_sing;                      // singular above kappa_sing max(1, ||z||_inf^2)

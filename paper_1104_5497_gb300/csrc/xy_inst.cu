@@ -41,19 +41,26 @@ cudaError_t NPHC_CAT(launch_xy_cauchy_m, NPHC_INST_M)(const XYSys &sys, const EG
 
 #if NPHC_INST_KIND == 0
 #include "xy_track_group.cuh"
+#include "xy_track_lane.cuh"
 
-// The FP32 pass has two kernels: one path per thread (xy_track.cuh) and four lanes per path
-// (xy_track_group.cuh).  One wave of the first takes its paths' latency (100 attempts of six
-// solves of one warp each) however few they are; four lanes shorten every solve, and sixteen
-// warps per SM hide each other's latency where seven cannot.  Measured (GB300, FP32 pass alone,
-// per-thread -> group, ms): 256 paths of N = 5 2.59 -> 1.02; 4,096 of N = 7 7.27 -> 2.40; 16,384 of
-// N = 8 11.3 -> 4.4; 65,536 of N = 9 25.4 -> 14.5; of N = 11, 12, 13: 262,144 154 -> 133, 262,144
-// 209 -> 148, 80,000 100 -> 55.6.  At M = 9 (N = 10) three of twelve row slots idle: 32,768 paths
-// 20.6 -> 18.9, 65,536 34.5 -> 33.9, but 262,144 109 -> 121.  So: the group kernel, unless over a
-// fifth of its slots idle and the per-thread kernel has more than two waves of paths.
+// The FP32 pass has two kernels: one path per thread (xy_track_lane.cuh) and four lanes per path
+// (xy_track_group.cuh).  The first takes fewer instructions per path but one wave of it (19,000 to
+// 90,000 paths) takes its paths' latency however few they are; four lanes shorten every solve
+// and sixteen warps per SM hide each other's latency where four to ten cannot, at the price of
+// the rows that pad M to a multiple of four.  Measured (GB300, FP32 pass alone, group / lane, ms):
+//   no padding    N = 13 80,000 paths (4.1 waves of lanes) 58.1 / 65.6, 262,144 (13.5) 183.7 / 185.6;
+//                 N = 9 65,536 (1.5) 13.8 / 16.8, batches of 262,144 (6) 74 / 74, 524,288 (12) 225 / 188
+//   one row       N = 12 32,768 (1.3) 24.3 / 27.8, 65,536 (2.7) 43.0 / 41.1, 262,144 (11) 154 / 133;
+//                 N = 8 batches of 65,536 (1.2) 19.5 / 20.1, 262,144 (4.9) 86 / 80
+//   two rows      N = 11 32,768 (1.1) 18.7 / 20.6, 49,152 (1.7) 25.7 / 26.4, 65,536 (2.2) 33.2 / 30.0,
+//                 262,144 (9) 118 / 93
+//   three rows    N = 10 16,384 (0.5) 9.0 / 13.5, 24,576 (0.7) 14.0 / 13.6, 32,768 (1.0) 16.4 / 13.8,
+//                 262,144 (7.7) 106 / 73
+// So lanes from that many quarter waves on, by the number of padding rows:
 template <int M>
 static bool use_group(int64_t items, int64_t wave) {
-    return 5 * M >= 4 * GrpLayout<M>::ROWS || items <= 2 * wave;
+    constexpr int quarters[4] = {32, 11, 8, 3};
+    return 4 * items < quarters[GrpLayout<M>::ROWS - M] * wave;
 }
 
 static cudaError_t device_sms(int &sms) {
@@ -95,8 +102,8 @@ cudaError_t NPHC_CAT(launch_xy_track_f32_m, NPHC_INST_M)(const XYSys &sys, const
                                                          int grid, cudaStream_t st) {
     constexpr int M = NPHC_INST_M, BLK = NPHC_TRACK_BLOCK;
     static bool attr_t = false, attr_g = false;
-    const size_t smem_t = xy_smem_per_thread<M, float>() * BLK, smem_g = grp_smem_per_block<M>(false);
-    auto kt = xy_track_kernel<M, float, BLK>;
+    const size_t smem_t = lane_smem_per_block<M>(false), smem_g = grp_smem_per_block<M>(false);
+    auto kt = xy_track_lane_kernel<M>;
     auto kg = xy_track_group_kernel<M>;
     int sms = 0, per_t = 0, per_g = 0;
     cudaError_t e = device_sms(sms);
@@ -127,8 +134,8 @@ cudaError_t NPHC_CAT(launch_xy_track_f32_batch_m, NPHC_INST_M)(const BatchGroup 
     constexpr int M = NPHC_INST_M, BLK = NPHC_TRACK_BLOCK;
     if (bg.total <= 0) return cudaSuccess;
     static bool attr_t = false, attr_g = false;
-    const size_t smem_t = xy_smem_per_thread<M, float>() * BLK, smem_g = grp_smem_per_block<M>(true);
-    auto kt = xy_track_batch_kernel<M, float, BLK>;
+    const size_t smem_t = lane_smem_per_block<M>(true), smem_g = grp_smem_per_block<M>(true);
+    auto kt = xy_track_lane_batch_kernel<M>;
     auto kg = xy_track_group_batch_kernel<M>;
     int sms = 0, per_t = 0, per_g = 0;
     cudaError_t e = device_sms(sms);

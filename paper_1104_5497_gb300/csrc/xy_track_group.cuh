@@ -64,36 +64,20 @@ struct GrpLayout {
     static constexpr int BLOCKS = M <= 10 ? 4 : 3;   // resident blocks per SM aimed at
 };
 
-// single: one table per block, (J, J, -J, -J) per entry; batch: one per path, a float per entry
+// the coupling table: one per block, or (batch) one per path
 template <int M>
 constexpr size_t grp_smem_per_block(bool batch) {
     using L = GrpLayout<M>;
-    return sizeof(float4) * (size_t)(GRP_WARPS * GRP_PATHS * L::TOTAL + (batch ? 0 : L::JB)) +
-           (batch ? sizeof(float) * (size_t)GRP_WARPS * GRP_PATHS * L::JB : 0);
+    return sizeof(float4) * (size_t)(GRP_WARPS * GRP_PATHS * L::TOTAL) +
+           sizeof(float) * (size_t)L::JB * (batch ? GRP_WARPS * GRP_PATHS : 1);
 }
 
 template <int M, bool BATCH>
 struct GrpJ {
-    const void *base;   // this lane's row g of the table
-    __device__ __forceinline__ void get(int s, int l, float2 &c, float2 &nc) const {
-        if (BATCH) {
-            const float v = static_cast<const float *>(base)[(4 * s * (M + 1) + l) * GRP_PATHS];
-            c = f2dup(v);
-            nc = f2dup(-v);
-        } else {
-            const float4 v = static_cast<const float4 *>(base)[4 * s * (M + 1) + l];
-            c = f2(v.x, v.y);
-            nc = f2(v.z, v.w);
-        }
-    }
-    __device__ __forceinline__ float2 dup(int s, int l) const {
-        if (BATCH) return f2dup(static_cast<const float *>(base)[(4 * s * (M + 1) + l) * GRP_PATHS]);
-        return *reinterpret_cast<const float2 *>(static_cast<const float4 *>(base) + 4 * s * (M + 1) + l);
-    }
-    __device__ __forceinline__ float val(int s, int l) const {
-        if (BATCH) return static_cast<const float *>(base)[(4 * s * (M + 1) + l) * GRP_PATHS];
-        return static_cast<const float4 *>(base)[4 * s * (M + 1) + l].x;
-    }
+    const float *base;   // this lane's row g of the table
+    static constexpr int STEP = BATCH ? GRP_PATHS : 1;
+    __device__ __forceinline__ float val(int s, int l) const { return base[(4 * s * (M + 1) + l) * STEP]; }
+    __device__ __forceinline__ float2 dup(int s, int l) const { return f2dup(val(s, l)); }
 };
 
 __device__ __forceinline__ float grp_sum(float v) {   // over a path's four lanes
@@ -122,7 +106,7 @@ __device__ __forceinline__ bool grp_solve(float4 *__restrict__ sm, const GrpJ<M,
                                           GrpStep<GrpLayout<M>::SL> &dr, float &kest) {
     using L = GrpLayout<M>;
     constexpr int SL = L::SL, NP = L::NP, NPT = L::NPT;
-    const cx<float> gomt = cscale(omt, gam);
+    const float2 gm = f2(gam.re, gam.im), hgomt = f2scale(0.5f * omt, gm);
     const float hs = 0.5f * s;
     auto at = [&](int off, int i) -> float4 & { return sm[(off + i) * GRP_PATHS]; };
     auto own = [&](int q) { return q < SL - 1 || M % 4 == 0 || g + 4 * q < M; };   // site g + 4 q exists
@@ -141,10 +125,9 @@ __device__ __forceinline__ bool grp_solve(float4 *__restrict__ sm, const GrpJ<M,
 #pragma unroll 1
             for (int l = 0; l < M; l++) {
                 const float4 v = at(L::PQ, l);
-                float2 c, nc;
-                J.get(q, l, c, nc);
-                acc2(up, c, nc, f2(v.x, v.y));
-                acc2(uq, c, nc, f2(v.z, v.w));
+                const float2 c = J.dup(q, l);
+                acc2(up, c, f2(v.x, v.y));
+                acc2(uq, c, f2(v.z, v.w));
             }
             f32_residual_rows(f2(z.x, z.y), f2(z.z, z.w), up, uq, s, hs, __fmul_rn(omt, gam.re),
                               __fmul_rn(omt, gam.im), rf, rg);
@@ -157,40 +140,26 @@ __device__ __forceinline__ bool grp_solve(float4 *__restrict__ sm, const GrpJ<M,
                 uq.hi = f2fma(c, f2(v.z, v.w), uq.hi);
             }
         }
-        const cx<float> pj = {z.x, z.y}, qj = {z.z, z.w};
-        const cx<float> Up = f2c(up.hi), Uq = f2c(uq.hi);
-        cx<float> htf, htg;
-        lc_minus_ht_rows<float>(pj, qj, Up, Uq, gam, htf, htg);
-        cx<float> ah, bh;
-        float iv, sp, sq;
-        g_frame_lc<float>(pj, qj, s, gomt, ah, bh, iv, sp, sq);
-        const cx<float> gpq = cmul(gomt, cadd(pj, qj));
-        const cx<float> Ajj = cscale(0.5f * sp, csub(gpq, cmul_i(cscale(s, Uq))));
-        const cx<float> Bjj = cscale(0.5f * sq, cadd(gpq, cmul_i(cscale(s, Up))));
-        const cx<float> sb = cscale(sp, bh), sa = cscale(sq, ah);
-        const cx<float> qT = cscale(iv, htg);
-        const cx<float> pxT = cmulc(ah, qT), pyT = cmulc(bh, qT);
-        const cx<float> sjj = csub(cmul(Ajj, bh), cmul(Bjj, ah));
-        const cx<float> bT = csub(htf, cadd(cmul(Ajj, pxT), cmul(Bjj, pyT)));
+        float2 htf, htg, x, y, d;
+        const F32Site v = f32_site(f2(z.x, z.y), f2(z.z, z.w), up.hi, uq.hi, s, hs, hgomt, gm, htf, htg);
+        v.rhs(htf, htg, x, y, d);
         if (own(q)) {
-            at(L::XY, j) = make_float4(sp * pxT.re, sp * pxT.im, sq * pyT.re, sq * pyT.im);
-            at(L::FR, j) = make_float4(sb.re, sb.im, sa.re, sa.im);
-            at(L::W0, j) = make_float4(sjj.re, sjj.im, bT.re, bT.im);
+            at(L::XY, j) = make_float4(x.x, x.y, y.x, y.y);
+            at(L::FR, j) = make_float4(v.sb.x, v.sb.y, v.sa.x, v.sa.y);
+            at(L::W0, j) = make_float4(v.sjj.x, v.sjj.y, d.x, d.y);
             // column pair j / 2: (re, re', im, im') of cb = i t/2 sp b^ and ca = i t/2 sq a^
             float *cb = reinterpret_cast<float *>(&at(L::U, j >> 1)) + (j & 1);
             float *ca = reinterpret_cast<float *>(&at(L::U, L::NPM + (j >> 1))) + (j & 1);
-            cb[0] = -hs * sb.im;
-            cb[2] = hs * sb.re;
-            ca[0] = -hs * sa.im;
-            ca[2] = hs * sa.re;
+            cb[0] = -hs * v.sb.y;
+            cb[2] = hs * v.sb.x;
+            ca[0] = -hs * v.sa.y;
+            ca[2] = hs * v.sa.x;
         }
         if (corr) {
-            const cx<float> qR = cscale(iv, f2c(rg));
-            const cx<float> pxR = cmulc(ah, qR), pyR = cmulc(bh, qR);
-            const cx<float> bR = csub(f2c(rf), cadd(cmul(Ajj, pxR), cmul(Bjj, pyR)));
+            v.rhs(rf, rg, x, y, d);
             if (own(q)) {
-                if (w) at(L::AC, j) = make_float4(sp * pxR.re, sp * pxR.im, sq * pyR.re, sq * pyR.im);
-                at(L::W1, j) = make_float4(bR.re, bR.im, 0.0f, 0.0f);
+                if (w) at(L::AC, j) = make_float4(x.x, x.y, y.x, y.y);
+                at(L::W1, j) = make_float4(d.x, d.y, 0.0f, 0.0f);
             }
         }
     }
@@ -263,14 +232,13 @@ __device__ __forceinline__ bool grp_solve(float4 *__restrict__ sm, const GrpJ<M,
 #pragma unroll
         for (int q = 0; q < SL; q++) {
             const float4 z = at(L::PQ, site(q));
-            const cx<float> pk = {z.x, z.y}, qk = {z.z, z.w};
-            const cx<float> vT = csub(cmul(qk, f2c(sx[q])), cmul(pk, f2c(sy[q])));
-            const cx<float> vR = csub(cmul(qk, f2c(rx[q])), cmul(pk, f2c(ry[q])));
+            const float2 ip = f2scale(hs, f2i(f2(z.x, z.y))), iq = f2scale(-hs, f2i(f2(z.z, z.w)));
             const float4 dg = at(L::W0, site(q)), dr1 = at(L::W1, site(q));
             const float mine = own(q) ? 1.0f : 0.0f;   // rows that do not exist are zero
-            const float tr = mine * (dg.z + hs * vT.im), ti = mine * (dg.w - hs * vT.re);
-            const float rr = corr ? mine * (dr1.x + hs * vR.im) : 0.0f;
-            const float ri = corr ? mine * (dr1.y - hs * vR.re) : 0.0f;
+            const float2 t = f2scale(mine, f2cfma(ip, sy[q], f2cfma(iq, sx[q], f2(dg.z, dg.w))));
+            float2 r = f2dup(0.0f);
+            if (corr) r = f2scale(mine, f2cfma(ip, ry[q], f2cfma(iq, rx[q], f2(dr1.x, dr1.y))));
+            const float tr = t.x, ti = t.y, rr = r.x, ri = r.y;
             if (M % 2) {
                 re[q][M / 2].y = tr;
                 im[q][M / 2].y = ti;
@@ -285,24 +253,25 @@ __device__ __forceinline__ bool grp_solve(float4 *__restrict__ sm, const GrpJ<M,
     __syncwarp();
 
     // ---- LU with partial pivoting; U's rows go to shared memory
-    unsigned done = 0;   // bit q: own row g + 4 q is a pivot row already (or does not exist)
-    if (!own(SL - 1)) done = 1u << (SL - 1);
+    unsigned live[SL];   // all but the low four bits while own row g + 4 q waits to be a pivot row, else 0
+#pragma unroll
+    for (int q = 0; q < SL; q++) live[q] = own(q) ? ~15u : 0u;
     bool ok = true;
     float umax = 0.0f, umin = INFINITY;   // of |U_kk|^2
-    cx<float> ip[M];
+    float2 ip[M];
 #pragma unroll
     for (int k = 0; k < M; k++) {
         const int kp = k / 2;
-        cx<float> a[SL];
-        unsigned key = 0;
+        float2 a[SL];
+        unsigned key = 0;   // rows done or absent count as zeros
 #pragma unroll
         for (int q = 0; q < SL; q++) {
-            a[q] = k % 2 ? cx<float>{re[q][kp].y, im[q][kp].y} : cx<float>{re[q][kp].x, im[q][kp].x};
-            const unsigned v = (__float_as_uint(cabs2(a[q])) & ~15u) | (unsigned)(15 - 4 * q - g);
-            if (!((done >> q) & 1u)) key = max(key, v);
+            a[q] = k % 2 ? f2(re[q][kp].y, im[q][kp].y) : f2(re[q][kp].x, im[q][kp].x);
+            key = max(key, (__float_as_uint(f2abs2(a[q])) & live[q]) | (unsigned)(15 - 4 * q - g));
         }
         key = max(key, __shfl_xor_sync(0xffffffffu, key, 8));
         key = max(key, __shfl_xor_sync(0xffffffffu, key, 16));
+        ok = ok && key > 15u;
         const int prow = 15 - (int)(key & 15u);
         const int uo = L::U + L::uoff(k) - kp;
 #pragma unroll
@@ -310,26 +279,24 @@ __device__ __forceinline__ bool grp_solve(float4 *__restrict__ sm, const GrpJ<M,
             if (g + 4 * q == prow) {
 #pragma unroll
                 for (int c = kp; c < NP; c++) at(uo, c) = make_float4(re[q][c].x, re[q][c].y, im[q][c].x, im[q][c].y);
-                done |= 1u << q;
+                live[q] = 0;
             }
         }
         __syncwarp();
         const float4 u0 = at(uo, kp);
-        const cx<float> piv = k % 2 ? cx<float>{u0.y, u0.w} : cx<float>{u0.x, u0.z};
-        const float best = cabs2(piv);
-        ok = ok && best > 0.0f;
+        const float2 piv = k % 2 ? f2(u0.y, u0.w) : f2(u0.x, u0.z);
+        const float best = f2abs2(piv);
         umax = fmaxf(umax, best);
         umin = fminf(umin, best);
-        const float rb = recip_r(best);
-        ip[k] = cx<float>{piv.re * rb, -piv.im * rb};
+        ip[k] = f2scale(f32_recip(best), f2(piv.x, -piv.y));
         if (k < M - 1) {
             float2 lr[SL], li[SL], nli[SL];   // -Re, Im, -Im of the multipliers
 #pragma unroll
             for (int q = 0; q < SL; q++) {
-                const cx<float> l = cmul(a[q], ip[k]);
-                lr[q] = f2dup(-l.re);
-                li[q] = f2dup(l.im);
-                nli[q] = f2dup(-l.im);
+                const float2 l = f2cmul(a[q], ip[k]);
+                lr[q] = f2dup(-l.x);
+                li[q] = f2dup(l.y);
+                nli[q] = f2dup(-l.y);
             }
             auto update = [&](int c) {
                 const float4 u = c == kp ? u0 : at(uo, c);
@@ -365,18 +332,18 @@ __device__ __forceinline__ bool grp_solve(float4 *__restrict__ sm, const GrpJ<M,
             si = f2fma(ui, xr[c], f2fma(ur, xi[c], si));
         }
         const float4 ut = at(uo, M / 2);
-        cx<float> b = M % 2 ? cx<float>{ut.y, ut.w} : cx<float>{ut.x, ut.z};
+        float2 b = M % 2 ? f2(ut.y, ut.w) : f2(ut.x, ut.z);
         if (mine_r) {
             const float4 ub = at(uo, NP - 1);
-            b = M % 2 ? cx<float>{ub.x, ub.z} : cx<float>{ub.y, ub.w};
+            b = M % 2 ? f2(ub.x, ub.z) : f2(ub.y, ub.w);
         }
-        const cx<float> x = cmul(cx<float>{b.re - (sr.x + sr.y), b.im - (si.x + si.y)}, ip[k]);
+        const float2 x = f2cmul(f2(b.x - (sr.x + sr.y), b.y - (si.x + si.y)), ip[k]);
         if (k % 2) {
-            xr[k / 2].y = x.re;
-            xi[k / 2].y = x.im;
+            xr[k / 2].y = x.x;
+            xi[k / 2].y = x.y;
         } else {
-            xr[k / 2].x = x.re;
-            xi[k / 2].x = x.im;
+            xr[k / 2].x = x.x;
+            xi[k / 2].x = x.y;
         }
     }
     __syncwarp();
@@ -395,20 +362,16 @@ __device__ __forceinline__ bool grp_solve(float4 *__restrict__ sm, const GrpJ<M,
     for (int q = 0; q < SL; q++) {
         const int j = site(q);
         const float4 x = at(L::U, j), f = at(L::FR, j), v = at(L::XY, j);
-        const cx<float> sb = {f.x, f.y}, sa = {f.z, f.w}, sT = {x.x, x.y};
-        const cx<float> p0 = cadd(cx<float>{v.x, v.y}, cmul(sb, sT));
-        const cx<float> q0 = csub(cx<float>{v.z, v.w}, cmul(sa, sT));
-        chk += cabs2(p0) + cabs2(q0);
-        dt.p[q] = c2f(p0);
-        dt.q[q] = c2f(q0);
+        const float2 sb = f2(f.x, f.y), sa = f2(f.z, f.w), sT = f2(x.x, x.y);
+        dt.p[q] = f2cfma(sb, sT, f2(v.x, v.y));
+        dt.q[q] = f2cfms(sa, sT, f2(v.z, v.w));
+        chk += f2abs2(dt.p[q]) + f2abs2(dt.q[q]);
         if (corr) {
             const float4 r = at(L::AC, j);
-            const cx<float> sR = {x.z, x.w};
-            const cx<float> p1 = cadd(cx<float>{r.x, r.y}, cmul(sb, sR));
-            const cx<float> q1 = csub(cx<float>{r.z, r.w}, cmul(sa, sR));
-            chk += cabs2(p1) + cabs2(q1);
-            dr.p[q] = c2f(p1);
-            dr.q[q] = c2f(q1);
+            const float2 sR = f2(x.z, x.w);
+            dr.p[q] = f2cfma(sb, sR, f2(r.x, r.y));
+            dr.q[q] = f2cfms(sa, sR, f2(r.z, r.w));
+            chk += f2abs2(dr.p[q]) + f2abs2(dr.q[q]);
         }
     }
     chk = grp_sum(chk);
@@ -423,19 +386,17 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int g = lane >> 3, pth = lane & 7;
     float4 *const sm = grp_raw + wid * (GRP_PATHS * L::TOTAL) + pth;
-    float4 *const jtab = grp_raw + GRP_WARPS * (GRP_PATHS * L::TOTAL);
+    float *const jtab = reinterpret_cast<float *>(grp_raw + GRP_WARPS * (GRP_PATHS * L::TOTAL));
     auto at = [&](int off, int i) -> float4 & { return sm[(off + i) * GRP_PATHS]; };
     auto own = [&](int q) { return q < SL - 1 || M % 4 == 0 || g + 4 * q < M; };
     auto site = [&](int q) { return own(q) ? g + 4 * q : M - 1; };
-    float *const jpath = reinterpret_cast<float *>(jtab) + wid * (GRP_PATHS * L::JB) + pth;   // batch
-    const GrpJ<M, BATCH> J{BATCH ? static_cast<const void *>(jpath + g * (M + 1) * GRP_PATHS)
-                                 : static_cast<const void *>(jtab + g * (M + 1))};
+    float *const jpath = jtab + wid * (GRP_PATHS * L::JB) + pth;   // batch
+    const GrpJ<M, BATCH> J{BATCH ? jpath + g * (M + 1) * GRP_PATHS : jtab + g * (M + 1)};
     if (!BATCH) {
         const float *Jf = src.sys(0).Jf;
         for (int i = threadIdx.x; i < L::JB; i += blockDim.x) {
             const int r = i / (M + 1), l = i - r * (M + 1);
-            const float v = r < M ? Jf[r * NPHC_JSTRIDE + l] : 0.0f;
-            jtab[i] = make_float4(v, v, -v, -v);
+            jtab[i] = r < M ? Jf[r * NPHC_JSTRIDE + l] : 0.0f;
         }
         __syncthreads();
     }
@@ -594,7 +555,7 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
             float zz = 0.0f;
             if (w) {
                 const float hr = time_float(hh);
-                const float2 c = f2dup(ph == 1 ? 0.5f * hr : ph == 2 ? hr : hr / 6.0f);
+                const float2 c = f2dup(ph == 1 ? 0.5f * hr : ph == 2 ? hr : hr * (1.0f / 6.0f));
                 bad = bad || !oks;
                 P.solves++;
                 kstep = fmaxf(kstep, kest);
