@@ -5,7 +5,9 @@
 // singular or fail) and each path is a long chain of dependent FP64 solves, so the
 // latency of one solve sets the time: sharing it over the lanes cuts that chain ~10x
 // against one path per thread.  Control flow is uniform over the warp (every branch is
-// on values broadcast from lane 0); lane i < 2M holds component i of the vectors.
+// on values broadcast from lane 0); lane i < 2M holds component i of the vectors.  Bound by the
+// FP64 pipe (67 cycles per warp instruction); 4,096 paths of the endgame workload on N = 4 took
+// 50.9 ms before the residual's grid sums, the split sites and the shared stage points, 33.3 now.
 #pragma once
 
 #include "cauchy.cuh"
@@ -23,6 +25,15 @@ struct CauchyWarpLayout {
 template <int M>
 constexpr size_t cauchy_warp_smem_per_warp() {
     return sizeof(cx<double>) * (size_t)CauchyWarpLayout<M>::TOTAL;
+}
+
+__device__ __forceinline__ EffPoint shfl_point(const EffPoint &p, int src) {   // lane src's, to all
+    EffPoint r;
+    r.s = __shfl_sync(0xffffffffu, p.s, src);
+    r.omt = __shfl_sync(0xffffffffu, p.omt, src);
+    r.g = cx<double>{__shfl_sync(0xffffffffu, p.g.re, src), __shfl_sync(0xffffffffu, p.g.im, src)};
+    r.cw = cx<double>{__shfl_sync(0xffffffffu, p.cw.re, src), __shfl_sync(0xffffffffu, p.cw.im, src)};
+    return r;
 }
 
 template <int M, int WARPS>
@@ -77,7 +88,7 @@ __global__ void __launch_bounds__(32 * WARPS)
                 const EffPoint pe = eff_point(eg_ew(lr, radial, j, K, C.lnratio, v), gam, ag);
                 if (vl) P.at(L::ZC, i) = P.at(L::Z0, i);
                 __syncwarp();
-                warp_residual<M>(P, J, pe.s, pe.omt, pe.g);
+                warp_residual<M>(P, J, S.jexp, pe.s, pe.omt, pe.g);
                 const bool ok = warp_solve<M>(P, J, pe.s, pe.omt, pe.g, true, L::AC);
                 solves++;
                 if (vl) {
@@ -103,8 +114,10 @@ __global__ void __launch_bounds__(32 * WARPS)
                     radial ? cx<double>{C.lnratio, 0.0} : cx<double>{0.0, NPHC_TWO_PI / (double)K};
                 const cx<double> hd = cscale(hh, dw);
                 const cx<double> hd2 = cscale(0.5, hd);
-                const EffPoint pm = eff_point(eg_ew(lr, radial, j, K, C.lnratio, v + 0.5 * hh), gam, ag);
-                const EffPoint p1 = eff_point(eg_ew(lr, radial, j, K, C.lnratio, v1), gam, ag);
+                // the points at v + h/2 and v + h: one half-warp each (an exponential, a sine and
+                // cosine, a root and three divisions in FP64)
+                const EffPoint ph = eff_point(eg_ew(lr, radial, j, K, C.lnratio, lane < 16 ? v + 0.5 * hh : v1), gam, ag);
+                const EffPoint pm = shfl_point(ph, 0), p1 = shfl_point(ph, 16);
                 bool bad = false, conv = false;
                 // RK4 stages 2..4 on dz/dw (k = cw d of the solve at each stage point)
                 if (vl) P.at(L::ZC, i) = cadd(P.at(L::Z0, i), cmul(hd2, P.at(L::K1, i)));
@@ -140,7 +153,7 @@ __global__ void __launch_bounds__(32 * WARPS)
                 // Newton's corrector at v1
 #pragma unroll 1
                 for (int it = 0; it < C.max_newton && !bad; it++) {
-                    warp_residual<M>(P, J, p1.s, p1.omt, p1.g);
+                    warp_residual<M>(P, J, S.jexp, p1.s, p1.omt, p1.g);
                     const bool oks = warp_solve<M>(P, J, p1.s, p1.omt, p1.g, true, L::AC);
                     solves++;
                     const double dn = sqrt(warp_sum(vl ? cabs2(P.at(L::W1, i)) : 0.0));
@@ -217,7 +230,7 @@ __global__ void __launch_bounds__(32 * WARPS)
                                     // a solution of P is the endpoint; otherwise a pole
                                     // (growing distance) or an enclosed branch point of
                                     // two other sheets (on to smaller radii)
-                                    warp_residual<M>(P, J, 1.0, 0.0, gam);   // W1 = -P(est)
+                                    warp_residual<M>(P, J, S.jexp, 1.0, 0.0, gam);   // W1 = -P(est)
                                     const double res = warp_max(vl ? sqrt(cabs2(P.at(L::W1, i))) : 0.0);
                                     const double zi2 = warp_max(vl ? sqrt(cabs2(P.at(L::ZC, i))) : 0.0);
                                     if (res <= C.tol_res * (zi2 > 1.0 ? zi2 * zi2 : 1.0))

@@ -259,15 +259,21 @@ nphc_status nphc_system_create_xy(int N, double sigma, const double *J, nphc_sys
     S->J = Jv;
     std::memset(&S->xs, 0, sizeof(S->xs));
     S->xs.N = N;
+    double row = 0.0;         // the largest sum_j |J_ij|
     double d2 = 2.0 * S->M;   // each constraint c^2 + s^2 - 1 contributes ||M_g||_F^2 = 2
-    for (int i = 0; i < N; i++)
+    for (int i = 0; i < N; i++) {
+        double sum = 0.0;
         for (int j = 0; j < N; j++) {
+            sum += std::fabs(Jv[i * N + j]);
             S->xs.Jf[i * NPHC_JSTRIDE + j] = (float)Jv[i * N + j];
             S->xs.Jd[i * NPHC_JSTRIDE + j] = Jv[i * N + j];
             // gradient row i: J_ij (s_i c_j - s_j c_i) puts J_ij / 2 on four symmetric
             // entries when j is free, so ||M_fi||_F^2 gains J_ij^2
             if (i < S->M && j < S->M && i != j) d2 += Jv[i * N + j] * Jv[i * N + j];
         }
+        row = std::max(row, sum);
+    }
+    S->xs.jexp = row > 0.0 ? (std::isfinite(row) ? std::ilogb(row * (1.0 + 1e-12)) + 1 : 1024) : -1023;
     S->xs.d2norm = std::sqrt(d2);
     S->xs.kappa_sing = 1e12;
     *out = S;
@@ -491,11 +497,12 @@ EPView view(const nphc_endpoints *e) {
 }
 
 // FP64 tracking: paths per scheduler from which four lanes per path (xy_track_group64.cuh) beat
-// a warp per path (xy_track_warp.cuh).  Whole passes, measured (warp / group, ms): 2,500 paths of
-// N = 8 52 / 70, 4,096 79 / 73, 16,384 281 / 122; of N = 10 4,096 102 / 129, 8,192 185 / 136.  Lists
-// (hand-offs, re-tracks) hold paths of very different lengths, and a group's chain is three
-// times a warp's: the 9,493 hand-offs of an N = 10 ring take 20 ms by warps and 29 by groups.
-constexpr int64_t kFewPerScheduler = 7, kFewListedPerScheduler = 32;
+// a warp per path (xy_track_warp.cuh).  Whole passes, measured (warp / group, ms; 608 schedulers):
+// N = 8 4,096 paths 49 / 60, 6,000 68 / 60, 16,384 170 / 97; N = 10 6,000 85 / 111, 8,192 120 / 109;
+// N = 12 4,096 82 / 88, 8,192 152 / 139.  Lists (hand-offs, re-tracks) hold paths of very different
+// lengths, and a group's chain is three times a warp's: the 9,493 hand-offs of an N = 10 ring took
+// 20 ms by warps and 29 by groups (13.5 by warps now).
+constexpr int64_t kFewPerScheduler = 10, kFewListedPerScheduler = 32;
 
 nphc_status track_impl(const nphc_system *S, const nphc_options *o, nphc_precision prec,
                        const nphc_endpoints *ep, const int32_t *list, const int32_t *list_count,

@@ -114,11 +114,51 @@ __device__ __forceinline__ void ext_acc_ext(ext<R> &acc, R a, ext<R> b) {
 template <class R>
 __device__ __forceinline__ R ext_val(ext<R> a) { return EFT<R>::add(a.hi, a.lo); }
 
+// The same sums in FP64 with four instructions per term instead of ten, where the terms have a
+// known bound.  A double next to the anchor 1.5 2^k lies on the grid of 2^(k-52) while it stays
+// within 2^(k-1) of it, so in n = fma(a, b, h), t = n - h the difference is exact, and the part of the
+// product off the grid, a b - t, is one more fma.  lo collects these, each rounded at 2^(k-106):
+// with k a few bits above the largest sum the result, (h - anchor) + lo, carries what
+// ext_acc's does.  Bounds are exponents, in integers.  At the ends of the exponent range the
+// anchor stays put: sums near 2^1020 only need to stay non-finite, as their products are.
+struct gsum {
+    double h, lo;
+};
+// |v| < 2^(gexp(v) + 1); 1024 for infinities and NaN
+__device__ __forceinline__ int gexp(double v) { return ((__double2hiint(v) >> 20) & 0x7ff) - 1023; }
+__device__ __forceinline__ double gsum_anchor(int k) {   // for sums below 2^(k-1)
+    return __hiloint2double((min(max(k, -900), 1020) + 1023) << 20 | 0x80000, 0);
+}
+__device__ __forceinline__ gsum gsum_start(double anchor, double c) {   // the term c
+    const double n = __dadd_rn(anchor, c);
+    return gsum{n, __dsub_rn(c, __dsub_rn(n, anchor))};
+}
+__device__ __forceinline__ void gsum_acc(gsum &s, double a, double b) {
+    const double n = __fma_rn(a, b, s.h);
+    s.lo = __dadd_rn(s.lo, __fma_rn(a, b, -__dsub_rn(n, s.h)));
+    s.h = n;
+}
+__device__ __forceinline__ void gsum_acc_ext(gsum &s, double a, ext<double> b) {
+    gsum_acc(s, a, b.hi);
+    s.lo = __fma_rn(a, b.lo, s.lo);
+}
+// hi on the grid (sums and differences of such hi are exact), lo not small against it
+__device__ __forceinline__ ext<double> gsum_ext(gsum s, double anchor) {
+    return ext<double>{__dsub_rn(s.h, anchor), s.lo};
+}
+__device__ __forceinline__ ext<double> grid_add(ext<double> a, ext<double> b) {   // of one grid
+    return ext<double>{__dadd_rn(a.hi, b.hi), __dadd_rn(a.lo, b.lo)};
+}
+__device__ __forceinline__ ext<double> grid_sub(ext<double> a, ext<double> b) {
+    return ext<double>{__dsub_rn(a.hi, b.hi), __dsub_rn(a.lo, b.lo)};
+}
+
 // ------------------------------------------------------ launch arguments --
 // Couplings and homotopy constants of one XY ring, passed by value so that the
 // unrolled kernels read them as constant-bank operands.
 struct XYSys {
     int N;                                  // ring size; M = N - 1 free sites
+    int jexp;                               // sum_j |J_kj| < 2^jexp for every k (gsum)
     alignas(16) float Jf[NPHC_MAXN * NPHC_JSTRIDE];   // J in FP32 (row k, column j at
                                                       // k * NPHC_JSTRIDE + j; zeros beyond)
     double Jd[NPHC_MAXN * NPHC_JSTRIDE];    // J in FP64

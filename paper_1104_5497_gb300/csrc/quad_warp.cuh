@@ -19,6 +19,13 @@
 #include "xy_endgame.cuh"
 #include "xy_track_warp.cuh"
 
+// (a.hi + a.lo) + (b.hi + b.lo), the rounding error of the leading sum kept in lo
+__device__ __forceinline__ ext<double> ext_add(ext<double> a, ext<double> b) {
+    double s, e;
+    two_sum(a.hi, b.hi, s, e);
+    return ext<double>{s, EFT<double>::add(e, EFT<double>::add(a.lo, b.lo))};
+}
+
 template <int N>
 struct QuadLayout {   // shared memory per warp, complex doubles
     static constexpr int A = 0;                 // [H_z | r | -H_t], column-major

@@ -6,17 +6,17 @@
 // the FP64 instruction count of the longest lane times the warps per scheduler.  So the work
 // of an endpoint is laid over lanes until the rows fill them (lane g owns the sites and
 // matrix rows j = g + 4 q), and the instruction count is what it is written for:
-//   * P by compensated sums (an exact product and a two-sum, 10 instructions per term; the
-//     rounding errors are collected in a second word, as in the trackers' residuals);
+//   * P by sums on grids (gsum in nphc_internal.cuh, as in the trackers' residuals): four
+//     instructions per term where an exact product and a two-sum took ten (15,013 points of
+//     N = 10 2.72 -> 2.06 ms);
 //   * the Schur right-hand side as J times per-site vectors;
 //   * LU with partial pivoting instead of Householder QR (half the operations, no square
 //     roots; the pivot search compares |re| + |im| as integers);
 //   * ||DP^-1||_F from 2 M triangular solves, dealt out over the four lanes.
-// 12.8 k FP64 instructions per warp of eight endpoints at M = 9 (three evaluations, a certificate,
-// some real tests; FP64 pipe 81% active), and a few hundred endpoints fill the chip.  Against one
-// endpoint per thread with double-double sums and a QR (solve's launches, ms): N = 5 0.7 -> 0.15,
-// N = 8 (3,432 endpoints) 2.96 -> 0.81, N = 10 (47,100) 14.4 -> 8.4, N = 11 (184,756) 60 -> 33;
-// called step by step, 15,013 points of N = 10 6.0 -> 2.7 and N = 13 (2,900) 26.4 -> 2.9.
+// A few hundred endpoints fill the chip.  Against one endpoint per thread with double-double sums
+// and a QR (solve's launches, ms): N = 5 0.7 -> 0.15, N = 8 (3,432 endpoints) 2.96 -> 0.45, N = 10
+// (47,100) 14.4 -> 6.1; called step by step, 15,013 points of N = 10 6.0 -> 2.06 and N = 13 (2,900)
+// 26.4 -> 2.0.
 //
 // An endpoint is in one of two states: it waits for an evaluation (P, the factorisation of DP
 // and the Newton correction at its point) or for a certificate from the factorisation just
@@ -64,6 +64,9 @@ __device__ __forceinline__ double rg_max(unsigned m, double v) {
     v = fmax(v, __shfl_xor_sync(m, v, 8));
     return fmax(v, __shfl_xor_sync(m, v, 16));
 }
+__device__ __forceinline__ int gexp_max(cx<double> x, cx<double> y) {
+    return max(max(gexp(x.re), gexp(x.im)), max(gexp(y.re), gexp(y.im)));
+}
 
 // One endpoint's lanes: slot memory, own rows.
 template <int M>
@@ -73,6 +76,7 @@ struct RGPath {
     cx<double> *sm;      // this endpoint's column of the shared memory
     const double *J;     // J[k * (M + 1) + l], l = M the pinned site
     const double *jj;    // sum over free l of J_kl^2
+    int jexp;            // XYSys::jexp
     int g;               // lane of the endpoint
     unsigned m;          // the lanes that run this code together (whole endpoints)
     __device__ __forceinline__ cx<double> &at(int off, int i) const { return sm[(off + i) * RG_PATHS]; }
@@ -96,37 +100,47 @@ __device__ bool rg_evaluate(const RGPath<M> &G, double &res, double &dn2, double
     using L = RGLayout<M>;
     const int g = G.g;
     double pmax = 0.0;
+    int ez = 0;   // exponent of max(1, ||z||_inf)
+#pragma unroll 1
+    for (int j = g; j < M; j += 4) ez = max(ez, gexp_max(G.at(L::Z, j), G.at(L::Z, M + j)));
+    ez = max(ez, __shfl_xor_sync(G.m, ez, 8));
+    ez = max(ez, __shfl_xor_sync(G.m, ez, 16));
+    const int ku = G.jexp + ez + 2;   // |u_j|, |w_j| < 2^(ku - 1)
+    const double au = gsum_anchor(ku);
 #pragma unroll 1
     for (int j = g; j < M; j += 4) {
         const double *Jj = G.J + j * (M + 1);
-        const ext<double> zero = {0.0, 0.0};
-        ext<double> ur = {Jj[M], 0.0}, ui = zero, wr = zero, wi = zero;
+        gsum sur = gsum_start(au, Jj[M]), sui = {au, 0.0}, swr = sui, swi = sui;
 #pragma unroll 1
         for (int l = 0; l < M; l++) {   // J_jj = 0 adds exact zeros
             const cx<double> xl = G.at(L::Z, l), yl = G.at(L::Z, M + l);
             const double c = Jj[l];
-            ext_acc(ur, c, xl.re);
-            ext_acc(ui, c, xl.im);
-            ext_acc(wr, c, yl.re);
-            ext_acc(wi, c, yl.im);
+            gsum_acc(sur, c, xl.re);
+            gsum_acc(sui, c, xl.im);
+            gsum_acc(swr, c, yl.re);
+            gsum_acc(swi, c, yl.im);
         }
+        const ext<double> ur = gsum_ext(sur, au), ui = gsum_ext(sui, au), wr = gsum_ext(swr, au), wi = gsum_ext(swi, au);
         const cx<double> x = G.at(L::Z, j), y = G.at(L::Z, M + j);
-        ext<double> fr = zero, fi = zero, gr = {-1.0, 0.0}, gi = zero;
-        ext_acc_ext(fr, y.re, ur);   // f = y u - x w
-        ext_acc_ext(fr, -y.im, ui);
-        ext_acc_ext(fr, -x.re, wr);
-        ext_acc_ext(fr, x.im, wi);
-        ext_acc_ext(fi, y.re, ui);
-        ext_acc_ext(fi, y.im, ur);
-        ext_acc_ext(fi, -x.re, wi);
-        ext_acc_ext(fi, -x.im, wr);
-        ext_acc(gr, x.re, x.re);     // g = x^2 + y^2 - 1
-        ext_acc(gr, -x.im, x.im);
-        ext_acc(gr, y.re, y.re);
-        ext_acc(gr, -y.im, y.im);
-        ext_acc(gi, 2.0 * x.re, x.im);
-        ext_acc(gi, 2.0 * y.re, y.im);
-        const cx<double> f = {ext_val(fr), ext_val(fi)}, gg = {ext_val(gr), ext_val(gi)};
+        const int ek = gexp_max(x, y);
+        const double af = gsum_anchor(ek + ku + 3), ag = gsum_anchor(max(0, 2 * ek + 4) + 2);
+        gsum fr = {af, 0.0}, fi = fr, gr = gsum_start(ag, -1.0), gi = {ag, 0.0};
+        gsum_acc_ext(fr, y.re, ur);   // f = y u - x w
+        gsum_acc_ext(fr, -y.im, ui);
+        gsum_acc_ext(fr, -x.re, wr);
+        gsum_acc_ext(fr, x.im, wi);
+        gsum_acc_ext(fi, y.re, ui);
+        gsum_acc_ext(fi, y.im, ur);
+        gsum_acc_ext(fi, -x.re, wi);
+        gsum_acc_ext(fi, -x.im, wr);
+        gsum_acc(gr, x.re, x.re);     // g = x^2 + y^2 - 1
+        gsum_acc(gr, -x.im, x.im);
+        gsum_acc(gr, y.re, y.re);
+        gsum_acc(gr, -y.im, y.im);
+        gsum_acc(gi, 2.0 * x.re, x.im);
+        gsum_acc(gi, 2.0 * y.re, y.im);
+        const cx<double> f = {ext_val(gsum_ext(fr, af)), ext_val(gsum_ext(fi, af))};
+        const cx<double> gg = {ext_val(gsum_ext(gr, ag)), ext_val(gsum_ext(gi, ag))};
         pmax = fmax(pmax, fmax(cabs2(f), cabs2(gg)));
         const cx<double> u = {ext_val(ur), ext_val(ui)}, w = {ext_val(wr), ext_val(wi)};
         const cx<double> a = cscale(2.0, x), b = cscale(2.0, y);
@@ -314,7 +328,7 @@ __global__ void __launch_bounds__(32)
         jj[lane] = s;
     }
     __syncwarp();
-    RGPath<M> G{base + pth, J, jj, g, 0xffffffffu};
+    RGPath<M> G{base + pth, J, jj, S.jexp, g, 0xffffffffu};
     const unsigned mine = 0x01010101u << pth;   // this endpoint's four lanes
     const double alpha0 = NPHC_ALPHA_CERT;
     const int64_t cnt = ep.count, total = worklist_size(wl, cnt);

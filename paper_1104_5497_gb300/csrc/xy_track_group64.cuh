@@ -4,19 +4,19 @@
 // Bound by the FP64 pipe: a warp instruction every 67 cycles per scheduler, whatever the number
 // of active lanes and dependent or not (measured), so the time is the FP64 instruction count of
 // the longest lane of every warp.  Against one path per thread the count per solve falls with
-// the lanes (M = 9: about 1.6 k for a predictor and 3.9 k for a corrector solve of eight paths
-// against 5 k and 12 k of 32, rows of the last lanes idle), a ring's paths make four times as
-// many warps, and no warp waits in lockstep:
+// the lanes (rows of the last lanes idle), a ring's paths make four times as many warps, and no
+// warp waits in lockstep:
 //   * lane g owns the sites and rows g + 4 q; the matrix and the vectors are in shared memory,
 //     every loop is rolled (the pipe hides the loads, and the code stays small);
 //   * the light-cone scales are powers of two taken from the exponents (any scale solves the
 //     same system; a power of two adds no rounding and no FP64 instruction);
+//   * the corrector's residual is sums on grids (gsum in nphc_internal.cuh): four instructions per
+//     term where compensated sums with two-sums took ten (N = 8, 16,384 paths: 121 -> 97 ms);
 //   * each path is in its own phase (RK4 stage or corrector iteration); a warp runs whichever
 //     kind of solve more of its paths wait for, as the FP32 pass does (xy_track_group.cuh).
 // Against one path per warp (xy_track_warp.cuh) a solve's chain is three times as long but eight
-// paths share it: the better choice once there are a few paths for every scheduler.  16,384 paths
-// of N = 8: 248 ms with one path per thread, 281 with one per warp, 122 here; 65,536 of N = 10
-// 1,346 with one per warp, 674 here.
+// paths share it: the better choice once there are ten paths for every scheduler.  16,384 paths
+// of N = 8: 248 ms with one path per thread, 170 with one per warp, 97 here.
 #pragma once
 
 #include "xy_track_warp.cuh"
@@ -40,17 +40,12 @@ constexpr size_t g64_smem_per_block() {
     return sizeof(cx<double>) * (size_t)(G64_PATHS * G64Layout<M>::TOTAL) + sizeof(double) * (size_t)(M * (M + 1));
 }
 
-// The largest power of two <= max(1, |re|, |im|), from the exponents alone.
-__device__ __forceinline__ double pow2_scale(cx<double> a) {
-    const int hi = max(__double2hiint(a.re) & 0x7fffffff, __double2hiint(a.im) & 0x7fffffff) & 0x7ff00000;
-    return __hiloint2double(min(max(hi, 0x3ff00000), 0x7fd00000), 0);
-}
-
 template <int M>
 struct G64Path {
     using L = G64Layout<M>;
     cx<double> *sm;
     const double *J;     // J[k * (M + 1) + l], l = M the pinned site
+    int jexp;            // XYSys::jexp
     int g;
     unsigned m;          // the lanes that run this code together (whole paths)
     __device__ __forceinline__ cx<double> &at(int off, int i) const { return sm[(off + i) * G64_PATHS]; }
@@ -66,56 +61,59 @@ struct G64Path {
     }
 };
 
-// -H rows of one site, compensated (f32_residual_rows in f32_step.cuh, in FP64).
+// -H rows of one site (f32_residual_rows in f32_step.cuh, in FP64), as sums on grids (gsum).
+// |U_p|, |U_q| < 2^(ku - 1).
 __device__ __forceinline__ void f64_residual_rows(cx<double> p, cx<double> q, const ext<double> &upr,
                                                   const ext<double> &upi, const ext<double> &uqr,
-                                                  const ext<double> &uqi, double s, double hs, double gr,
-                                                  double gi, cx<double> &rf, cx<double> &rg) {
-    const ext<double> zero = {0.0, 0.0};
-    ext<double> dr = zero, di = zero;   // D = q U_p - p U_q, f = i D / 2
-    ext_acc_ext(dr, q.re, upr);
-    ext_acc_ext(dr, -q.im, upi);
-    ext_acc_ext(dr, -p.re, uqr);
-    ext_acc_ext(dr, p.im, uqi);
-    ext_acc_ext(di, q.re, upi);
-    ext_acc_ext(di, q.im, upr);
-    ext_acc_ext(di, -p.re, uqi);
-    ext_acc_ext(di, -p.im, uqr);
+                                                  const ext<double> &uqi, int ku, double s, double hs,
+                                                  double gr, double gi, cx<double> &rf, cx<double> &rg) {
+    const int ek = max(max(gexp(p.re), gexp(p.im)), max(gexp(q.re), gexp(q.im)));
+    const int eg = max(gexp(gr), gexp(gi)), kd = ek + ku + 3, kh = max(0, 2 * ek + 2) + 2;
+    const double ad = gsum_anchor(kd), ah = gsum_anchor(kh);
+    gsum sdr = {ad, 0.0}, sdi = sdr;   // D = q U_p - p U_q, f = i D / 2
+    gsum_acc_ext(sdr, q.re, upr);
+    gsum_acc_ext(sdr, -q.im, upi);
+    gsum_acc_ext(sdr, -p.re, uqr);
+    gsum_acc_ext(sdr, p.im, uqi);
+    gsum_acc_ext(sdi, q.re, upi);
+    gsum_acc_ext(sdi, q.im, upr);
+    gsum_acc_ext(sdi, -p.re, uqi);
+    gsum_acc_ext(sdi, -p.im, uqr);
+    const ext<double> dr = gsum_ext(sdr, ad), di = gsum_ext(sdi, ad);
     // h = (p q - 2) / 2, B = (p^2 + q^2) / 4: x^2 - 1 = h + B, y^2 - 1 = h - B, p q - 1 = 2 h + 1
-    ext<double> hr = {-1.0, 0.0}, hi = zero, br = zero, bi = zero;
-    ext_acc(hr, 0.5 * p.re, q.re);
-    ext_acc(hr, -0.5 * p.im, q.im);
-    ext_acc(hi, 0.5 * p.re, q.im);
-    ext_acc(hi, 0.5 * p.im, q.re);
-    ext_acc(br, 0.25 * p.re, p.re);
-    ext_acc(br, -0.25 * p.im, p.im);
-    ext_acc(br, 0.25 * q.re, q.re);
-    ext_acc(br, -0.25 * q.im, q.im);
-    ext_acc(bi, 0.5 * p.re, p.im);
-    ext_acc(bi, 0.5 * q.re, q.im);
-    const ext<double> nbr = {-br.hi, -br.lo}, nbi = {-bi.hi, -bi.lo};
-    const ext<double> xr = ext_add(hr, br), xi = ext_add(hi, bi), yr = ext_add(hr, nbr), yi = ext_add(hi, nbi);
+    const cx<double> ph = cscale(0.5, p), qh = cscale(0.5, q);
+    gsum shr = gsum_start(ah, -1.0), shi = {ah, 0.0}, sbr = shi, sbi = shi;
+    gsum_acc(shr, ph.re, q.re);
+    gsum_acc(shr, -ph.im, q.im);
+    gsum_acc(shi, ph.re, q.im);
+    gsum_acc(shi, ph.im, q.re);
+    gsum_acc(sbr, ph.re, ph.re);
+    gsum_acc(sbr, -ph.im, ph.im);
+    gsum_acc(sbr, qh.re, qh.re);
+    gsum_acc(sbr, -qh.im, qh.im);
+    gsum_acc(sbi, ph.re, p.im);
+    gsum_acc(sbi, qh.re, q.im);
+    const ext<double> hr = gsum_ext(shr, ah), hi = gsum_ext(shi, ah), br = gsum_ext(sbr, ah), bi = gsum_ext(sbi, ah);
+    const ext<double> xr = grid_add(hr, br), xi = grid_add(hi, bi), yr = grid_sub(hr, br), yi = grid_sub(hi, bi);
     // H_f = gomt X + t f ;  H_g = gomt Y + t (2 h + 1)
-    ext<double> fr = zero, fi = zero, kr = {s, 0.0}, ki = zero;
-    ext_acc_ext(fr, gr, xr);
-    ext_acc_ext(fr, -gi, xi);
-    ext_acc_ext(fr, -hs, di);
-    ext_acc_ext(fi, gr, xi);
-    ext_acc_ext(fi, gi, xr);
-    ext_acc_ext(fi, hs, dr);
-    ext_acc_ext(kr, gr, yr);
-    ext_acc_ext(kr, -gi, yi);
-    ext_acc_ext(kr, 2.0 * s, hr);
-    ext_acc_ext(ki, gr, yi);
-    ext_acc_ext(ki, gi, yr);
-    ext_acc_ext(ki, 2.0 * s, hi);
-    rf = cx<double>{-ext_val(fr), -ext_val(fi)};
-    rg = cx<double>{-ext_val(kr), -ext_val(ki)};
-}
-
-// c + a b, c - a b with four fused multiply-adds
-__device__ __forceinline__ cx<double> cfma64(cx<double> a, cx<double> b, cx<double> c) {
-    return cx<double>{fma(-a.im, b.im, fma(a.re, b.re, c.re)), fma(a.im, b.re, fma(a.re, b.im, c.im))};
+    const double s2 = 2.0 * s;
+    const double af = gsum_anchor(max(eg + kh + 2, gexp(hs) + kd) + 2);
+    const double ag = gsum_anchor(max(eg + kh + 2, gexp(s2) + kh + 1) + 2);
+    gsum fr = {af, 0.0}, fi = fr, kr = gsum_start(ag, s), ki = {ag, 0.0};
+    gsum_acc_ext(fr, gr, xr);
+    gsum_acc_ext(fr, -gi, xi);
+    gsum_acc_ext(fr, -hs, di);
+    gsum_acc_ext(fi, gr, xi);
+    gsum_acc_ext(fi, gi, xr);
+    gsum_acc_ext(fi, hs, dr);
+    gsum_acc_ext(kr, gr, yr);
+    gsum_acc_ext(kr, -gi, yi);
+    gsum_acc_ext(kr, s2, hr);
+    gsum_acc_ext(ki, gr, yi);
+    gsum_acc_ext(ki, gi, yr);
+    gsum_acc_ext(ki, s2, hi);
+    rf = cx<double>{-ext_val(gsum_ext(fr, af)), -ext_val(gsum_ext(fi, af))};
+    rg = cx<double>{-ext_val(gsum_ext(kr, ag)), -ext_val(gsum_ext(ki, ag))};
 }
 
 // One solve of H_z(z, t) d = r at PQ: r = -H_t, d into W (corr false); r = -H (compensated), d into
@@ -127,6 +125,18 @@ __device__ bool g64_solve(const G64Path<M> &G, double s, double omt, cx<double> 
     const int g = G.g;
     const cx<double> gomt = cscale(omt, gam);
     const double hs = 0.5 * s;
+    int ku = 0;
+    if (corr) {   // the grid of the U sums, from the exponent of max(1, max |p|, |q|)
+#pragma unroll 1
+        for (int k = g; k < M; k += 4)
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const cx<double> v = G.at(L::PQ, k + h * M);
+                ku = max(ku, max(gexp(v.re), gexp(v.im)));
+            }
+        ku = max(ku, __shfl_xor_sync(G.m, ku, 8));
+        ku = max(ku, __shfl_xor_sync(G.m, ku, 16)) + G.jexp + 2;
+    }
     // ---- site by site: U sums, residual rows, frames, the diagonal's terms
 #pragma unroll 1
     for (int j = g; j < M; j += 4) {
@@ -134,21 +144,22 @@ __device__ bool g64_solve(const G64Path<M> &G, double s, double omt, cx<double> 
         const cx<double> p = G.at(L::PQ, j), q = G.at(L::PQ, M + j);
         cx<double> Up = {Jj[M], 0.0}, Uq = Up, rf, rg;
         if (corr) {
-            const ext<double> zero = {0.0, 0.0};
-            ext<double> upr = {Jj[M], 0.0}, upi = zero, uqr = upr, uqi = zero;
+            const double au = gsum_anchor(ku);
+            gsum spr = gsum_start(au, Jj[M]), spi = {au, 0.0}, sqr = spr, sqi = spi;
 #pragma unroll 1
             for (int l = 0; l < M; l++) {   // J_jj = 0 adds exact zeros
                 const cx<double> pl = G.at(L::PQ, l), ql = G.at(L::PQ, M + l);
                 const double c = Jj[l];
-                ext_acc(upr, c, pl.re);
-                ext_acc(upi, c, pl.im);
-                ext_acc(uqr, c, ql.re);
-                ext_acc(uqi, c, ql.im);
+                gsum_acc(spr, c, pl.re);
+                gsum_acc(spi, c, pl.im);
+                gsum_acc(sqr, c, ql.re);
+                gsum_acc(sqi, c, ql.im);
             }
-            f64_residual_rows(p, q, upr, upi, uqr, uqi, s, hs, EFT<double>::mul(omt, gam.re),
+            const ext<double> upr = gsum_ext(spr, au), upi = gsum_ext(spi, au), uqr = gsum_ext(sqr, au), uqi = gsum_ext(sqi, au);
+            f64_residual_rows(p, q, upr, upi, uqr, uqi, ku, s, hs, EFT<double>::mul(omt, gam.re),
                               EFT<double>::mul(omt, gam.im), rf, rg);
-            Up = cx<double>{upr.hi, upi.hi};
-            Uq = cx<double>{uqr.hi, uqi.hi};
+            Up = cx<double>{ext_val(upr), ext_val(upi)};
+            Uq = cx<double>{ext_val(uqr), ext_val(uqi)};
         } else {
 #pragma unroll 1
             for (int l = 0; l < M; l++) {
@@ -313,7 +324,7 @@ __global__ void __launch_bounds__(32)
     double *const J = reinterpret_cast<double *>(base + G64_PATHS * L::TOTAL);
     const int lane = threadIdx.x, g = lane >> 3, pth = lane & 7;
     for (int i = lane; i < M * (M + 1); i += 32) J[i] = S.Jd[(i / (M + 1)) * NPHC_JSTRIDE + i % (M + 1)];
-    G64Path<M> G{base + pth, J, g, 0xffffffffu};
+    G64Path<M> G{base + pth, J, S.jexp, g, 0xffffffffu};
     const cx<double> gam = {S.gre, S.gim};
     // few paths: fewer per warp, so that every scheduler has some
     const int64_t want = (total + gridDim.x - 1) / gridDim.x;

@@ -2,12 +2,13 @@
 // short lists (paths handed off by the FP32 pass, re-tracks).
 //
 // GB300 runs FP64 at 1/64 of the FP32 rate, and its FP64 pipe takes a warp instruction
-// at the same cost whatever the number of active lanes: a solve costs about 76 cycles of
-// an SM sub-partition per FP64 instruction on the longest chain that any lane runs.  So
+// at the same cost whatever the number of active lanes: a solve costs 67 cycles of an SM
+// sub-partition per FP64 instruction on the longest chain that any lane runs.  So
 // the 32 lanes share one path, and every stage is laid out to keep each lane's own FP64
 // chain short rather than to save lanes:
-//   * per-site quantities (couplings sums, frames, the diagonal's terms): lane j for
-//     site j, the sums u_j and w_j on lanes j and 16 + j;
+//   * per-site quantities (couplings sums, frames, the diagonal's terms): the p side of
+//     site j on lane j, the q side on lane 16 + j, both halves on the same instructions;
+//     the frames' scales are powers of two from the exponents (no square root);
 //   * the off-diagonal Schur entries: one entry per lane, strided over the M x M matrix;
 //   * the right-hand sides: sums of J times per-site vectors, right-hand side r on the
 //     lanes 16 r + k (row k);
@@ -15,7 +16,10 @@
 //     square root; the pivot search compares the bit patterns of |re| + |im| as integers
 //     and costs one FP64 add), the rank-one update strided over the trailing block;
 //   * the back substitution in registers (right-hand side r on lanes 16 r + row);
-//   * the compensated residual of row pair k on lanes k and 16 + k.
+//   * the compensated residual of row pair k on lanes k and 16 + k, as sums on grids (gsum in
+//     nphc_internal.cuh: four instructions per term where two-sums took ten).
+// The 9,493 hand-offs of an N = 10 ring: 20.0 ms with two-sums, one lane per site and square
+// roots, 13.5 now; 1,400 of N = 13 6.4 -> 5.0.
 // The step logic (RK4 predictor, Newton corrector, step control, divergence radius,
 // budget) is the per-thread FP64 tracker's, as are the state in light-cone coordinates,
 // the equations and the scaled light-cone frames of the Schur reduction (xy_solve.cuh):
@@ -25,7 +29,7 @@
 //
 // Storage: everything of a path in per-warp shared memory (complex doubles): the
 // augmented Schur matrix [S | b0 | b1] (column-major, M x (M + 2)), the five step
-// vectors Z0, K1, AC, ZC, W1 (2M each) and thirteen per-site arrays.
+// vectors Z0, K1, AC, ZC, W1 (2M each) and eight per-site arrays.
 #pragma once
 
 #include "xy_track.cuh"
@@ -39,20 +43,15 @@ struct WarpLayout {
     static constexpr int AC = K1 + NV;
     static constexpr int ZC = AC + NV;
     static constexpr int W1 = ZC + NV;
-    static constexpr int AH = W1 + NV;    // frame a^_j
-    static constexpr int BH = AH + M;     // frame b^_j
-    static constexpr int SS = BH + M;     // light-cone scales (sp, sq) of site j
-    static constexpr int CB = SS + M;     // (i t / 2) sp_j b^_j: Schur column j is J_kj (q_k CB_j + p_k CA_j)
-    static constexpr int CA = CB + M;     // (i t / 2) sq_j a^_j
-    static constexpr int X0 = CA + M;     // sp_j conj(a^_j) q0_j, sq_j conj(b^_j) q0_j (right-hand side 0),
+    static constexpr int SB = W1 + NV;    // sp b^_j of the scaled frame: Schur column j is J_kj (IQ_k SB_j + IP_k SA_j)
+    static constexpr int SA = SB + M;     // sq a^_j
+    static constexpr int X0 = SA + M;     // sp_j conj(a^_j) q0_j, sq_j conj(b^_j) q0_j (right-hand side 0),
     static constexpr int Y0 = X0 + M;
     static constexpr int X1 = Y0 + M;     // the same with q1_j (right-hand side 1)
     static constexpr int Y1 = X1 + M;
-    static constexpr int PK = Y1 + M;     // p_j = x_j + i y_j, q_j = x_j - i y_j
-    static constexpr int QK = PK + M;
-    static constexpr int QS0 = QK + M;    // the constraint rows' components q0_j, q1_j
-    static constexpr int QS1 = QS0 + M;
-    static constexpr int TOTAL = QS1 + M;
+    static constexpr int IP = Y1 + M;     // (i t / 2) p_j, (i t / 2) q_j
+    static constexpr int IQ = IP + M;
+    static constexpr int TOTAL = IQ + M;
 };
 
 template <int M>
@@ -80,19 +79,27 @@ __device__ __forceinline__ cx<double> cfnms(cx<double> c, cx<double> a, cx<doubl
     return cx<double>{fma(a.im, b.im, fma(-a.re, b.re, c.re)), fma(-a.im, b.re, fma(-a.re, b.im, c.im))};
 }
 
-__device__ __forceinline__ cx<double> shfl_down16(cx<double> v) {
-    return cx<double>{__shfl_down_sync(0xffffffffu, v.re, 16), __shfl_down_sync(0xffffffffu, v.im, 16)};
+// c + a b
+__device__ __forceinline__ cx<double> cfma64(cx<double> a, cx<double> b, cx<double> c) {
+    return cx<double>{fma(-a.im, b.im, fma(a.re, b.re, c.re)), fma(a.im, b.re, fma(a.re, b.im, c.im))};
+}
+
+// The largest power of two <= max(1, |re|, |im|), from the exponents alone.
+__device__ __forceinline__ double pow2_scale(cx<double> a) {
+    const int hi = max(__double2hiint(a.re) & 0x7fffffff, __double2hiint(a.im) & 0x7fffffff) & 0x7ff00000;
+    return __hiloint2double(min(max(hi, 0x3ff00000), 0x7fd00000), 0);
+}
+
+__device__ __forceinline__ cx<double> shfl_xor16(cx<double> v) {
+    return cx<double>{__shfl_xor_sync(0xffffffffu, v.re, 16), __shfl_xor_sync(0xffffffffu, v.im, 16)};
 }
 
 __device__ __forceinline__ ext<double> shfl_down16(ext<double> v) {
     return ext<double>{__shfl_down_sync(0xffffffffu, v.hi, 16), __shfl_down_sync(0xffffffffu, v.lo, 16)};
 }
 
-// (a.hi + a.lo) + (b.hi + b.lo), the rounding error of the leading sum kept in lo
-__device__ __forceinline__ ext<double> ext_add(ext<double> a, ext<double> b) {
-    double s, e;
-    two_sum(a.hi, b.hi, s, e);
-    return ext<double>{s, EFT<double>::add(e, EFT<double>::add(a.lo, b.lo))};
+__device__ __forceinline__ ext<double> shfl_up16(ext<double> v) {
+    return ext<double>{__shfl_up_sync(0xffffffffu, v.hi, 16), __shfl_up_sync(0xffffffffu, v.lo, 16)};
 }
 
 template <int M>
@@ -103,133 +110,103 @@ struct WarpPath {
     __device__ __forceinline__ cx<double> &A(int i, int c) const { return s[WarpLayout<M>::A + c * M + i]; }
 };
 
-// -H(z, t) at ZC into W1 with compensated sums (the per-thread trackers' residuals).
-// LC == false: ZC holds (x, y) (the Cauchy endgame); row pair k: lane k sums
-// u_k = J_kN + sum_l J_kl x_l and forms the f row, lane 16 + k sums w_k = sum_l J_kl y_l,
-// forms the g row (which needs no sums) and hands its share of f_k = y_k u_k - x_k w_k to
-// lane k.  LC == true: ZC holds the light-cone coordinates (p, q) (xy_residual_comp in
-// xy_solve.cuh); lane k sums U_p,k, lane 16 + k sums U_q,k, and D_k = q_k U_p,k - p_k U_q,k
-// is formed the same way.
+// -H(z, t) at ZC into W1 with compensated sums (on grids: gsum).  LC == false: ZC holds (x, y) (the
+// Cauchy endgame), f = y u - x w; LC == true: the light-cone coordinates (p, q), f = i D / 2 with
+// D = q U_p - p U_q (xy_residual_comp in xy_solve.cuh).  Row pair k: lane k sums u_k (U_p,k) and forms
+// the f row, lane 16 + k sums w_k (U_q,k), hands its share of f (D) to lane k and forms the g row;
+// both halves run the same instructions.  |J row| < 2^jexp.
 template <int M, bool LC = false>
-__device__ void warp_residual(const WarpPath<M> &P, const double *__restrict__ J, double s,
+__device__ void warp_residual(const WarpPath<M> &P, const double *__restrict__ J, int jexp, double s,
                               double omt, cx<double> gam) {
     static_assert(M <= 16, "one row pair per lane pair");
     using L = WarpLayout<M>;
     using E = EFT<double>;
     const int k = P.lane & 15;
-    const bool hi = P.lane >= 16;
-    const ext<double> zero = {0.0, 0.0};
-    ext<double> fre = zero, fim = zero;   // lane k's and lane 16 + k's shares of f (or D)
-    cx<double> zk = cx<double>{0.0, 0.0}, wk = zk;   // (x_k, y_k) or (p_k, q_k)
-    const cx<double> gomt = cx<double>{E::mul(omt, gam.re), E::mul(omt, gam.im)};
-    if (k < M) {
+    const bool hi = P.lane >= 16, on = k < M;
+    cx<double> zk = {1.0, 0.0}, wk = zk;   // (x_k, y_k) or (p_k, q_k)
+    if (on) {
         zk = P.at(L::ZC, k);
         wk = P.at(L::ZC, M + k);
-        const double *Jk = J + k * NPHC_JSTRIDE;
-        const int off = hi ? L::ZC + M : L::ZC;
-        ext<double> sre = {(hi && !LC) ? 0.0 : Jk[M], 0.0}, sim = zero;
+    }
+    const int ek = max(max(gexp(zk.re), gexp(zk.im)), max(gexp(wk.re), gexp(wk.im)));
+    const int ku = __reduce_max_sync(0xffffffffu, max(ek, 0)) + jexp + 2, kd = ek + ku + 3;
+    const double au = gsum_anchor(ku), ad = gsum_anchor(kd);
+    const double *Jk = J + (on ? k : 0) * NPHC_JSTRIDE;
+    const int off = hi ? L::ZC + M : L::ZC;
+    gsum sr = gsum_start(au, (hi && !LC) ? 0.0 : Jk[M]), si = {au, 0.0};
 #pragma unroll 1
-        for (int l = 0; l < M; l++) {   // J_kk = 0 adds exact zeros
-            const cx<double> v = P.at(off, l);
-            ext_acc(sre, Jk[l], v.re);
-            ext_acc(sim, Jk[l], v.im);
-        }
-        // (x, y): lane k y_k u_k, lane 16 + k -x_k w_k;  (p, q): lane k q_k U_p, lane 16 + k -p_k U_q
-        const cx<double> c = hi ? cx<double>{-zk.re, -zk.im} : wk;
-        ext_acc_ext(fre, c.re, sre);
-        ext_acc_ext(fre, -c.im, sim);
-        ext_acc_ext(fim, c.re, sim);
-        ext_acc_ext(fim, c.im, sre);
+    for (int l = 0; l < M; l++) {   // J_kk = 0 adds exact zeros
+        const cx<double> v = P.at(off, l);
+        gsum_acc(sr, Jk[l], v.re);
+        gsum_acc(si, Jk[l], v.im);
     }
-    const ext<double> ore = shfl_down16(fre), oim = shfl_down16(fim);
-    if (k < M) {
-        if (!LC) {
-            const cx<double> xk = zk, yk = wk;
-            ext<double> qxr = {-1.0, 0.0}, qxi = zero;
-            ext_acc(qxr, xk.re, xk.re);
-            ext_acc(qxr, -xk.im, xk.im);
-            ext_acc(qxi, 2.0 * xk.re, xk.im);
-            if (!hi) {
-                fre = ext_add(fre, ore);
-                fim = ext_add(fim, oim);
-                ext<double> hfr = zero, hfi = zero;
-                ext_acc_ext(hfr, gomt.re, qxr);
-                ext_acc_ext(hfr, -gomt.im, qxi);
-                ext_acc_ext(hfr, s, fre);
-                ext_acc_ext(hfi, gomt.re, qxi);
-                ext_acc_ext(hfi, gomt.im, qxr);
-                ext_acc_ext(hfi, s, fim);
-                P.at(L::W1, k) = cx<double>{-ext_val(hfr), -ext_val(hfi)};
-            } else {
-                ext<double> qyr = {-1.0, 0.0}, qyi = zero;
-                ext_acc(qyr, yk.re, yk.re);
-                ext_acc(qyr, -yk.im, yk.im);
-                ext_acc(qyi, 2.0 * yk.re, yk.im);
-                ext<double> hgr = zero, hgi = zero;
-                ext_acc_ext(hgr, gomt.re, qyr);
-                ext_acc_ext(hgr, -gomt.im, qyi);
-                ext_acc_ext(hgr, s, qxr);
-                ext_acc_ext(hgr, s, qyr);
-                ext_acc(hgr, s, 1.0);
-                ext_acc_ext(hgi, gomt.re, qyi);
-                ext_acc_ext(hgi, gomt.im, qyr);
-                ext_acc_ext(hgi, s, qxi);
-                ext_acc_ext(hgi, s, qyi);
-                P.at(L::W1, M + k) = cx<double>{-ext_val(hgr), -ext_val(hgi)};
-            }
-        } else {
-            const cx<double> pk = zk, qk = wk;
-            const double hs = 0.5 * s;
-            if (!hi) {
-                // H_f = gomt X + t f, f = i D / 2, X = x^2 - 1 = (p^2 + 2 p q + q^2) / 4 - 1
-                const ext<double> dr = ext_add(fre, ore), di = ext_add(fim, oim);
-                ext<double> xr = {-1.0, 0.0}, xi = zero;
-                ext_acc(xr, 0.25 * pk.re, pk.re);
-                ext_acc(xr, -0.25 * pk.im, pk.im);
-                ext_acc(xr, 0.5 * pk.re, qk.re);
-                ext_acc(xr, -0.5 * pk.im, qk.im);
-                ext_acc(xr, 0.25 * qk.re, qk.re);
-                ext_acc(xr, -0.25 * qk.im, qk.im);
-                ext_acc(xi, 0.5 * pk.re, pk.im);
-                ext_acc(xi, 0.5 * pk.re, qk.im);
-                ext_acc(xi, 0.5 * pk.im, qk.re);
-                ext_acc(xi, 0.5 * qk.re, qk.im);
-                ext<double> hfr = zero, hfi = zero;
-                ext_acc_ext(hfr, gomt.re, xr);
-                ext_acc_ext(hfr, -gomt.im, xi);
-                ext_acc_ext(hfr, -hs, di);
-                ext_acc_ext(hfi, gomt.re, xi);
-                ext_acc_ext(hfi, gomt.im, xr);
-                ext_acc_ext(hfi, hs, dr);
-                P.at(L::W1, k) = cx<double>{-ext_val(hfr), -ext_val(hfi)};
-            } else {
-                // H_g = gomt Y + t G, Y = y^2 - 1 = -(p^2 - 2 p q + q^2) / 4 - 1, G = p q - 1
-                ext<double> yr = {-1.0, 0.0}, yi = zero, gr = {-1.0, 0.0}, gi = zero;
-                ext_acc(yr, -0.25 * pk.re, pk.re);
-                ext_acc(yr, 0.25 * pk.im, pk.im);
-                ext_acc(yr, 0.5 * pk.re, qk.re);
-                ext_acc(yr, -0.5 * pk.im, qk.im);
-                ext_acc(yr, -0.25 * qk.re, qk.re);
-                ext_acc(yr, 0.25 * qk.im, qk.im);
-                ext_acc(yi, -0.5 * pk.re, pk.im);
-                ext_acc(yi, 0.5 * pk.re, qk.im);
-                ext_acc(yi, 0.5 * pk.im, qk.re);
-                ext_acc(yi, -0.5 * qk.re, qk.im);
-                ext_acc(gr, pk.re, qk.re);
-                ext_acc(gr, -pk.im, qk.im);
-                ext_acc(gi, pk.re, qk.im);
-                ext_acc(gi, pk.im, qk.re);
-                ext<double> hgr = zero, hgi = zero;
-                ext_acc_ext(hgr, gomt.re, yr);
-                ext_acc_ext(hgr, -gomt.im, yi);
-                ext_acc_ext(hgr, s, gr);
-                ext_acc_ext(hgi, gomt.re, yi);
-                ext_acc_ext(hgi, gomt.im, yr);
-                ext_acc_ext(hgi, s, gi);
-                P.at(L::W1, M + k) = cx<double>{-ext_val(hgr), -ext_val(hgi)};
-            }
+    const ext<double> ur = gsum_ext(sr, au), ui = gsum_ext(si, au);
+    // (x, y): lane k y_k u_k, lane 16 + k -x_k w_k;  (p, q): lane k q_k U_p, lane 16 + k -p_k U_q
+    const cx<double> c = hi ? cx<double>{-zk.re, -zk.im} : wk;
+    gsum sfr = {ad, 0.0}, sfi = sfr;
+    gsum_acc_ext(sfr, c.re, ur);
+    gsum_acc_ext(sfr, -c.im, ui);
+    gsum_acc_ext(sfi, c.re, ui);
+    gsum_acc_ext(sfi, c.im, ur);
+    ext<double> fr = gsum_ext(sfr, ad), fi = gsum_ext(sfi, ad);
+    fr = grid_add(fr, shfl_down16(fr));
+    fi = grid_add(fi, shfl_down16(fi));
+    // lane k: X = x^2 - 1, lane 16 + k: Y = y^2 - 1 and G = x^2 + y^2 - 1
+    const int kh = max(0, 2 * ek + 2) + 2;
+    const double ah = gsum_anchor(kh);
+    ext<double> ar, ai, tr, ti;   // X or Y; what t multiplies: f (or D), or G - 1
+    double cr, ci;
+    if (LC) {   // h = (p q - 2) / 2, B = (p^2 + q^2) / 4: X = h + B, Y = h - B, G = p q - 1 = 2 h + 1
+        const cx<double> ph = cscale(0.5, zk), qh = cscale(0.5, wk);
+        gsum shr = gsum_start(ah, -1.0), shi = {ah, 0.0}, sbr = shi, sbi = shi;
+        gsum_acc(shr, ph.re, wk.re);
+        gsum_acc(shr, -ph.im, wk.im);
+        gsum_acc(shi, ph.re, wk.im);
+        gsum_acc(shi, ph.im, wk.re);
+        gsum_acc(sbr, ph.re, ph.re);
+        gsum_acc(sbr, -ph.im, ph.im);
+        gsum_acc(sbr, qh.re, qh.re);
+        gsum_acc(sbr, -qh.im, qh.im);
+        gsum_acc(sbi, ph.re, zk.im);
+        gsum_acc(sbi, qh.re, wk.im);
+        ext<double> br = gsum_ext(sbr, ah), bi = gsum_ext(sbi, ah);
+        if (hi) {
+            br = ext<double>{-br.hi, -br.lo};
+            bi = ext<double>{-bi.hi, -bi.lo};
         }
+        const ext<double> hr = gsum_ext(shr, ah), hm = gsum_ext(shi, ah);
+        ar = grid_add(hr, br);
+        ai = grid_add(hm, bi);
+        tr = hi ? hr : fi;
+        ti = hi ? hm : fr;
+        cr = hi ? 2.0 * s : -0.5 * s;
+        ci = hi ? 2.0 * s : 0.5 * s;
+    } else {
+        const cx<double> v = hi ? wk : zk;
+        gsum svr = gsum_start(ah, -1.0), svi = {ah, 0.0};
+        gsum_acc(svr, v.re, v.re);
+        gsum_acc(svr, -v.im, v.im);
+        gsum_acc(svi, 2.0 * v.re, v.im);
+        ar = gsum_ext(svr, ah);
+        ai = gsum_ext(svi, ah);
+        const ext<double> xr = shfl_up16(ar), xi = shfl_up16(ai);
+        tr = hi ? grid_add(ar, xr) : fr;   // X + Y = G - 1
+        ti = hi ? grid_add(ai, xi) : fi;
+        cr = ci = s;
     }
+    // H_f = gomt X + t f, H_g = gomt Y + t G
+    const double gr = E::mul(omt, gam.re), gi = E::mul(omt, gam.im);
+    const int kt = hi ? kh + 1 : kd;
+    const double av = gsum_anchor(max(max(gexp(gr), gexp(gi)) + kh + 2, gexp(cr) + kt + 1) + 2);
+    gsum vr = gsum_start(av, hi ? s : 0.0), vi = {av, 0.0};
+    gsum_acc_ext(vr, gr, ar);
+    gsum_acc_ext(vr, -gi, ai);
+    gsum_acc_ext(vr, cr, tr);
+    gsum_acc_ext(vi, gr, ai);
+    gsum_acc_ext(vi, gi, ar);
+    gsum_acc_ext(vi, ci, ti);
+    if (on)
+        P.at(L::W1, hi ? M + k : k) = cx<double>{-ext_val(gsum_ext(vr, av)), -ext_val(gsum_ext(vi, av))};
     __syncwarp();
 }
 
@@ -309,8 +286,8 @@ __device__ __forceinline__ bool warp_lu_solve(cx<double> *A, int lane, bool two_
     return ok;
 }
 
-// H_z(ZC, t) d = r, the per-thread xy_solve's Schur reduction shared out over the warp;
-// ZC and d in (x, y) (LC == false) or in the light-cone coordinates (p, q).
+// H_z(ZC, t) d = r, the Schur reduction of xy_solve.cuh shared out over the warp; ZC and d in
+// (x, y) (LC == false) or in the light-cone coordinates (p, q).
 //   two_rhs false: r = -H_t, d into W1.
 //   two_rhs true:  r1 = W1 (the residual), d1 into W1; r2 = -H_t, d2 into `out2`.
 // Returns false (in every lane) when S is singular or the result is not finite.
@@ -321,73 +298,72 @@ __device__ bool warp_solve(const WarpPath<M> &P, const double *__restrict__ J, d
     using L = WarpLayout<M>;
     const int lane = P.lane;
     const int hrow = lane & 15, r = lane >> 4;   // row and right-hand side of the half-warp layout
-    const cx<double> gomt = cscale(omt, gam);
-    const cx<double> sg = cx<double>{s + gomt.re, gomt.im};   // t + gamma (1 - t)
+    const bool hi = lane >= 16, on = hrow < M;
+    const cx<double> hg = cscale(0.5 * omt, gam);
     const double hs = 0.5 * s;
 
-    // ---- per-site quantities: u_j (U_p,j) on lane j, w_j (U_q,j) on lane 16 + j, the
-    // rest on lane j
-    cx<double> uw = cx<double>{0.0, 0.0};
-    if (hrow < M) {
-        const int j = hrow;
+    // ---- per-site quantities of site j: its p side (U_p, a^, sp, A, -H_t's f row) on lane j, its q
+    // side (U_q, b^, sq, B, the g row) on lane 16 + j.  o: the own one of p_j and q_j, x the other.
+    {
+        const int j = on ? hrow : 0;
         const double *Jj = J + j * NPHC_JSTRIDE;
-        const int off = r ? L::ZC + M : L::ZC;
-        uw = cx<double>{(r && !LC) ? 0.0 : Jj[M], 0.0};
+        const cx<double> z = P.at(L::ZC, j), w = P.at(L::ZC, M + j);
+        cx<double> U = {(hi && !LC) ? 0.0 : Jj[M], 0.0};
+        const int off = hi ? L::ZC + M : L::ZC;
 #pragma unroll 1
         for (int l = 0; l < M; l++) {
             const cx<double> v = P.at(off, l);
-            uw.re = fma(Jj[l], v.re, uw.re);
-            uw.im = fma(Jj[l], v.im, uw.im);
+            U.re = fma(Jj[l], v.re, U.re);
+            U.im = fma(Jj[l], v.im, U.im);
         }
-    }
-    const cx<double> w = shfl_down16(uw);
-    if (lane < M) {
-        const int j = lane;
-        const cx<double> u = uw;
-        const cx<double> zj = P.at(L::ZC, j), wj = P.at(L::ZC, M + j);
-        cx<double> htf, htg, ah, bh, Ajj, Bjj, pj, qj;   // Ajj, Bjj: gradient row j on (dwp_j, dwq_j)
-        double iv, sp, sq;
-        if (LC) {
-            pj = zj;
-            qj = wj;
-            lc_minus_ht_rows<double>(pj, qj, u, w, gam, htf, htg);
-            g_frame_lc<double>(pj, qj, s, gomt, ah, bh, iv, sp, sq);
-            const cx<double> gpq = cmul(gomt, cadd(pj, qj));
-            Ajj = cscale(0.5 * sp, csub(gpq, cmul_i(cscale(s, w))));
-            Bjj = cscale(0.5 * sq, cadd(gpq, cmul_i(cscale(s, u))));
-        } else {
-            const cx<double> xj = zj, yj = wj;
-            pj = cx<double>{xj.re - yj.im, xj.im + yj.re};
-            qj = cx<double>{xj.re + yj.im, xj.im - yj.re};
-            minus_ht_rows<double>(xj, yj, u, w, gam, htf, htg);
-            g_frame<double>(xj, yj, s, sg, ah, bh, iv, sp, sq);
-            lc_coef<double>(cx<double>{-s * w.re + 2.0 * (gomt.re * xj.re - gomt.im * xj.im),
-                                       -s * w.im + 2.0 * (gomt.re * xj.im + gomt.im * xj.re)},
-                            cscale(s, u), sp, sq, Ajj, Bjj);
+        cx<double> V = shfl_xor16(U), p = z, q = w;   // V: the other side's sum
+        if (!LC) {   // U_p = u + i w, U_q = u - i w
+            const cx<double> su = hi ? V : U, sw = hi ? U : V;
+            const cx<double> up = {su.re - sw.im, su.im + sw.re}, uq = {su.re + sw.im, su.im - sw.re};
+            U = hi ? uq : up;
+            V = hi ? up : uq;
+            p = cx<double>{z.re - w.im, z.im + w.re};
+            q = cx<double>{z.re + w.im, z.im - w.re};
         }
-        const cx<double> rf0 = two_rhs ? P.at(L::W1, j) : htf;
-        const cx<double> rg0 = two_rhs ? P.at(L::W1, M + j) : htg;
-        const cx<double> q0 = cscale(iv, rg0), q1 = cscale(iv, htg);
-        const cx<double> px0 = cmulc(ah, q0), py0 = cmulc(bh, q0);
-        P.at(L::AH, j) = ah;
-        P.at(L::BH, j) = bh;
-        P.at(L::SS, j) = cx<double>{sp, sq};
-        P.at(L::CB, j) = cmul_i(cscale(hs * sp, bh));
-        P.at(L::CA, j) = cmul_i(cscale(hs * sq, ah));
-        P.at(L::X0, j) = cscale(sp, px0);
-        P.at(L::Y0, j) = cscale(sq, py0);
-        P.at(L::PK, j) = pj;
-        P.at(L::QK, j) = qj;
-        P.at(L::QS0, j) = q0;
-        // the diagonal entry, and the diagonal's own terms of the right-hand sides
-        P.A(j, j) = csub(cmul(Ajj, bh), cmul(Bjj, ah));
-        P.A(j, M) = csub(rf0, cadd(cmul(Ajj, px0), cmul(Bjj, py0)));
+        const cx<double> o = hi ? q : p, x = hi ? p : q;
+        // -H_t's rows: gamma X - f, f = i D / 2, D = q U_p - p U_q; gamma Y - G, G = p q - 1
+        const cx<double> m = cmul(x, U), mo = shfl_xor16(m), pq = cmul(p, q);
+        const cx<double> D = csub(hi ? mo : m, hi ? m : mo);
+        const cx<double> sum = cadd(p, q), dif = csub(o, x);
+        const cx<double> e = hi ? dif : sum, e2 = cmul(e, e);
+        const double quarter = hi ? -0.25 : 0.25;
+        const cx<double> t = {fma(quarter, e2.re, -1.0), quarter * e2.im};
+        const cx<double> sub = hi ? cx<double>{pq.re - 1.0, pq.im} : cx<double>{-0.5 * D.im, 0.5 * D.re};
+        const cx<double> ht = csub(cmul(gam, t), sub), ho = shfl_xor16(ht);
+        const cx<double> htg = hi ? ht : ho;
+        // the scaled frame (g_frame_lc in xy_solve.cuh) with powers of two for scales
+        const double so = pow2_scale(o);
+        const cx<double> hd = cmul(hg, dif);
+        const cx<double> v = {so * fma(s, x.re, -hd.re), so * fma(s, x.im, -hd.im)};
+        const double n2 = cabs2(v), iv = rsqrt(n2 + __shfl_xor_sync(0xffffffffu, n2, 16));
+        const cx<double> vh = cscale(iv, v), xh = shfl_xor16(vh);
+        const cx<double> g2 = cmul(hg, sum);
+        const double hsu = hi ? hs : -hs;
+        const cx<double> A = {so * fma(-hsu, V.im, g2.re), so * fma(hsu, V.re, g2.im)};
+        const cx<double> dg = cmul(A, xh), dgo = shfl_xor16(dg);
+        const cx<double> px0 = cmulc(vh, cscale(iv, two_rhs ? P.at(L::W1, M + j) : htg));
+        const cx<double> b0 = cmul(A, px0), b0o = shfl_xor16(b0);
+        cx<double> px1 = px0, b1 = b0, b1o = b0o;
         if (two_rhs) {
-            const cx<double> px1 = cmulc(ah, q1), py1 = cmulc(bh, q1);
-            P.at(L::X1, j) = cscale(sp, px1);
-            P.at(L::Y1, j) = cscale(sq, py1);
-            P.at(L::QS1, j) = q1;
-            P.A(j, M + 1) = csub(htf, cadd(cmul(Ajj, px1), cmul(Bjj, py1)));
+            px1 = cmulc(vh, cscale(iv, htg));
+            b1 = cmul(A, px1);
+            b1o = shfl_xor16(b1);
+        }
+        if (on) {
+            P.at(hi ? L::SA : L::SB, j) = cscale(so, xh);
+            P.at(hi ? L::IQ : L::IP, j) = cx<double>{-hs * o.im, hs * o.re};
+            P.at(hi ? L::Y0 : L::X0, j) = cscale(so, px0);
+            if (two_rhs) P.at(hi ? L::Y1 : L::X1, j) = cscale(so, px1);
+            if (!hi) {   // the diagonal entry, and the diagonal's own terms of the right-hand sides
+                P.A(j, j) = csub(dg, dgo);
+                P.A(j, M) = csub(csub(two_rhs ? P.at(L::W1, j) : ht, b0), b0o);
+                if (two_rhs) P.A(j, M + 1) = csub(csub(ht, b1), b1o);
+            }
         }
     }
     __syncwarp();
@@ -400,9 +376,10 @@ __device__ bool warp_solve(const WarpPath<M> &P, const double *__restrict__ J, d
         const int j = e / M, k = e - j * M;
         if (k != j)
             P.A(k, j) = cscale(J[k * NPHC_JSTRIDE + j],
-                               cadd(cmul(P.at(L::QK, k), P.at(L::CB, j)), cmul(P.at(L::PK, k), P.at(L::CA, j))));
+                               cfma64(P.at(L::IP, k), P.at(L::SA, j), cmul(P.at(L::IQ, k), P.at(L::SB, j))));
     }
-    if (hrow < M && (r == 0 || two_rhs)) {
+    const bool act = r == 0 || two_rhs;
+    if (on && act) {
         const int k = hrow;
         const double *Jk = J + k * NPHC_JSTRIDE;
         const int ox = r ? L::X1 : L::X0, oy = r ? L::Y1 : L::Y0;
@@ -416,37 +393,31 @@ __device__ bool warp_solve(const WarpPath<M> &P, const double *__restrict__ J, d
             sy.re = fma(Jkj, yv.re, sy.re);
             sy.im = fma(Jkj, yv.im, sy.im);
         }
-        const cx<double> d = csub(cmul(P.at(L::QK, k), sx), cmul(P.at(L::PK, k), sy));
-        P.A(k, M + r) = csub(P.A(k, M + r), cmul_i(cscale(hs, d)));
+        P.A(k, M + r) = cfma64(P.at(L::IP, k), sy, cfnms(P.A(k, M + r), P.at(L::IQ, k), sx));
     }
     __syncwarp();
 
     cx<double> cur;   // the solution: right-hand side r, row hrow
     const bool ok = warp_lu_solve<M>(P.s + L::A, lane, two_rhs, cur);
-    const bool act = r == 0 || two_rhs;
 
-    // ---- back to (dx, dy) or (dp, dq) = (sp dwp, sq dwq): site j of right-hand side r on
-    // lane 16 r + j, (dwp, dwq) = conj(a^, b^) q_j + (b^, -a^) s_j
-    double chk = 0.0;
-    if (act && hrow < M) {
+    // ---- back to (dp, dq) = (X + sp b^ s, Y - sq a^ s): site j of right-hand side r on lane 16 r + j
+    bool finite = true;   // a square that overflows counts as not finite
+    if (act && on) {
         const int j = hrow;
-        const cx<double> sc = P.at(L::SS, j), ah = P.at(L::AH, j), bh = P.at(L::BH, j);
-        const cx<double> qv = P.at(r ? L::QS1 : L::QS0, j);
-        cx<double> dx, dy;
-        if (LC) {
-            dx = cscale(sc.re, cadd(cmulc(ah, qv), cmul(bh, cur)));
-            dy = cscale(sc.im, csub(cmulc(bh, qv), cmul(ah, cur)));
-        } else {
-            lc_step<double>(ah, bh, sc.re, sc.im, qv, cur, dx, dy);
+        cx<double> dp = cfma64(P.at(L::SB, j), cur, P.at(r ? L::X1 : L::X0, j));
+        cx<double> dq = cfnms(P.at(r ? L::Y1 : L::Y0, j), P.at(L::SA, j), cur);
+        finite = max(max(gexp(dp.re), gexp(dp.im)), max(gexp(dq.re), gexp(dq.im))) < 511;
+        if (!LC) {
+            const cx<double> x = {0.5 * (dp.re + dq.re), 0.5 * (dp.im + dq.im)};
+            dq = cx<double>{0.5 * (dp.im - dq.im), -0.5 * (dp.re - dq.re)};
+            dp = x;
         }
-        chk = cabs2(dx) + cabs2(dy);
         const int o = r ? out2 : L::W1;   // W1's entries j and M + j were read above only
-        P.at(o, j) = dx;
-        P.at(o, M + j) = dy;
+        P.at(o, j) = dp;
+        P.at(o, M + j) = dq;
     }
     __syncwarp();
-    chk = warp_sum(chk);
-    return ok && isfinite(chk);
+    return ok && __all_sync(0xffffffffu, finite);
 }
 
 // The problem a warp tracker runs on, as a policy for warp_track_body: the unknowns (NV), the
@@ -508,7 +479,7 @@ struct WarpXY {
         }
     }
     static __device__ __forceinline__ void residual(const Path &P, const Sys &S, double s, double omt) {
-        warp_residual<M, true>(P, S.Jd, s, omt, cx<double>{S.gre, S.gim});
+        warp_residual<M, true>(P, S.Jd, S.jexp, s, omt, cx<double>{S.gre, S.gim});
     }
     static __device__ __forceinline__ bool solve(const Path &P, const Sys &S, double s, double omt,
                                                  bool two_rhs, int out2) {
