@@ -680,11 +680,13 @@ nphc_status nphc_classify(const nphc_system *S, const nphc_endpoints *ep, double
     cudaStream_t st = (cudaStream_t)stream;
     // defaults for every entry, then the real ones
     const size_t row = sizeof(double) * ep->count;
-    NPHC_CK(cudaMemsetAsync(theta, 0, row * S->M, st));
-    NPHC_CK(cudaMemsetAsync(energy, 0, row, st));
-    if (min_abs_eig) NPHC_CK(cudaMemsetAsync(min_abs_eig, 0, row, st));
-    if (log_abs_det) NPHC_CK(cudaMemsetAsync(log_abs_det, 0, row, st));
-    NPHC_CK(cudaMemsetAsync(index, 0xff, sizeof(int32_t) * ep->count, st));
+    FillSet f;
+    f.add(theta, row * S->M, 0);
+    f.add(energy, row, 0);
+    if (min_abs_eig) f.add(min_abs_eig, row, 0);
+    if (log_abs_det) f.add(log_abs_det, row, 0);
+    f.add(index, sizeof(int32_t) * ep->count, 0xffffffffu);
+    NPHC_CK(launch_fill(f, st));
     NPHC_CK(launch_xy_classify(S->M, xs, view(ep), theta, index, energy, min_abs_eig, log_abs_det, st));
     return NPHC_OK;
 }
@@ -845,10 +847,12 @@ nphc_status solve_into_impl(const nphc_system *S, const nphc_options *o, nphc_re
     const DedupScratch dsc = dedup_scratch(R->ws, L);
     R->solved = false;
     const int64_t launches0 = nphc_launch_counter(0);
-    NPHC_CK(cudaMemsetAsync(R->flags, 0, sizeof(int32_t) * R->P, st));
-    NPHC_CK(cudaMemsetAsync(R->lcount, 0, sizeof(int32_t) * 8, st));
-    NPHC_CK(cudaMemsetAsync(R->cycle, 0, sizeof(int32_t) * R->P, st));
-    NPHC_CK(cudaMemsetAsync(R->egst, 0, sizeof(int32_t) * R->P, st));
+    FillSet init;
+    init.add(R->flags, sizeof(int32_t) * R->P, 0);
+    init.add(R->lcount, sizeof(int32_t) * 8, 0);
+    init.add(R->cycle, sizeof(int32_t) * R->P, 0);
+    init.add(R->egst, sizeof(int32_t) * R->P, 0);
+    NPHC_CK(launch_fill(init, st));
     const bool mixed = o->precision == NPHC_PREC_MIXED;
     // the Cauchy endgame on the paths that end singular or failed; the result keeps its
     // tracking statuses (the endgame's own go to a scratch array)
@@ -958,11 +962,13 @@ nphc_status solve_into_impl(const nphc_system *S, const nphc_options *o, nphc_re
         const Range r("classify");
         // defaults for every entry (theta, energy, |lambda|_min, log|det H| 0; index -1), then
         // the real stationary points, compacted so that they fill whole warps
-        NPHC_CK(cudaMemsetAsync(R->theta, 0, sizeof(double) * R->M * R->P, st));
-        NPHC_CK(cudaMemsetAsync(R->energy, 0, sizeof(double) * R->P, st));
-        NPHC_CK(cudaMemsetAsync(R->mineig, 0, sizeof(double) * R->P, st));
-        NPHC_CK(cudaMemsetAsync(R->logdet, 0, sizeof(double) * R->P, st));
-        NPHC_CK(cudaMemsetAsync(R->index, 0xff, sizeof(int32_t) * R->P, st));
+        FillSet f;
+        f.add(R->theta, sizeof(double) * R->M * R->P, 0);
+        f.add(R->energy, sizeof(double) * R->P, 0);
+        f.add(R->mineig, sizeof(double) * R->P, 0);
+        f.add(R->logdet, sizeof(double) * R->P, 0);
+        f.add(R->index, sizeof(int32_t) * R->P, 0xffffffffu);
+        NPHC_CK(launch_fill(f, st));
         NPHC_CK(launch_real_list(v, R->real_list, R->lcount + 4, st));
         NPHC_CK(launch_xy_classify(S->M, xs, v, R->theta, R->index, R->energy, R->mineig, R->logdet, st,
                                    R->real_list, R->lcount + 4));
@@ -1221,8 +1227,8 @@ nphc_status nphc_dedup_noalloc(const nphc_system *S, const nphc_options *o,
     off += align256(sizeof(int32_t) * ep->count);
     w.table_size = tsize;
     if (tsize > kNoallocTable || off > kNoallocBytes) return fail(NPHC_EINVAL, "scratch layout overflow");
-    // launch_dedup clears the cell keys, list heads, flags and *dup_count itself with
-    // cudaMemsetAsync on `stream`; the list links are written before they are read.
+    // launch_dedup clears the cell keys, list heads, flags and *dup_count itself on
+    // `stream`; the list links are written before they are read.
     NPHC_CK(launch_dedup(view(ep), S->n, kDedupDelta, w, dup_list, dup_count, (cudaStream_t)stream));
     return NPHC_OK;
 }

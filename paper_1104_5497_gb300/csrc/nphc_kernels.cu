@@ -105,21 +105,34 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
     return z ^ (z >> 31);
 }
 
-__device__ __forceinline__ double dd_pitch(double delta0, int level) {
+// Per level: 1 / pitch, and the largest beta that looks the level up (4 beta <= DD_BAND pitch).
+struct DDGrid {
+    double inv[DD_LEVELS], beta[DD_LEVELS];
+};
+static DDGrid dd_grid(double delta0) {
+    DDGrid g;
     double d = delta0;
-    for (int l = 0; l < level; l++) d *= 100.0;
-    return d;
+    for (int L = 0; L < DD_LEVELS; L++, d *= 100.0) {
+        g.inv[L] = 1.0 / d;
+        g.beta[L] = 0.25 * (DD_BAND * d);
+    }
+    return g;
 }
 
 // The projections' weights, fixed pseudo-random numbers in [-1, 1) (splitmix64 of (i, r),
-// r = 2k: Re z_k, 2k + 1: Im z_k), and the prefix sums of their squares that normalise a
+// r = 2k: Re z_k, 2k + 1: Im z_k), and the factors that normalise a
 // projection over the first 2n real coordinates; built at compile time.  A point has at
 // most DD_MAXR real coordinates (24 unknowns: the N = 13 ring).
 #define DD_MAXR 48
 struct DDTable {
     double w[4][DD_MAXR];
-    double n2[4][DD_MAXR + 1];
+    double rn[4][DD_MAXR + 1];   // 1 / sqrt(sum of the first r squares)
 };
+constexpr double dd_rsqrt(double a) {   // Newton; a in (1e-3, DD_MAXR]
+    double y = a < 0.1 ? 3.0 : 0.14;
+    for (int i = 0; i < 60; i++) y *= 1.5 - 0.5 * a * y * y;
+    return y;
+}
 constexpr uint64_t dd_splitmix(uint64_t z) {
     z += 0x9E3779B97F4A7C15ull;
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
@@ -129,12 +142,13 @@ constexpr uint64_t dd_splitmix(uint64_t z) {
 constexpr DDTable dd_make_table() {
     DDTable t{};
     for (int i = 0; i < 4; i++) {
-        t.n2[i][0] = 0.0;
+        double n2 = 0.0;
         for (int r = 0; r < DD_MAXR; r++) {
             const uint64_t h = dd_splitmix(0x5851F42D4C957F2Dull ^ ((uint64_t)i << 32) ^ (uint64_t)r);
             const double w = (double)(int64_t)h * (1.0 / 9223372036854775808.0);
             t.w[i][r] = w;
-            t.n2[i][r + 1] = t.n2[i][r] + w * w;
+            n2 += w * w;
+            t.rn[i][r + 1] = dd_rsqrt(n2);
         }
     }
     return t;
@@ -153,7 +167,7 @@ __device__ __forceinline__ void dd_project(const EPView &ep, int n, int64_t e, d
             dot[i] = fma(dd_tab.w[i][2 * k], re, fma(dd_tab.w[i][2 * k + 1], im, dot[i]));
     }
 #pragma unroll
-    for (int i = 0; i < 4; i++) u[i] = dot[i] / sqrt(dd_tab.n2[i][2 * n]);
+    for (int i = 0; i < 4; i++) u[i] = dot[i] * dd_tab.rn[i][2 * n];
 }
 
 __device__ __forceinline__ uint64_t dd_cell_key(int level, const long long (&q)[4]) {
@@ -165,30 +179,46 @@ __device__ __forceinline__ uint64_t dd_cell_key(int level, const long long (&q)[
 // alpha-theory: the same solution when alpha < 0.03 and ||za - zb|| < 1 / (20 gamma) for
 // either point; a pair that is not provably distinct (||za - zb|| > 2 (beta_a + beta_b))
 // counts as the same solution too.
+// Most candidates of a coarse cell are far apart, and a chain of them is walked by one thread:
+// the sum stops once it exceeds every distance that could count (with a margin of 1e-5 on its
+// square for the FP32 bounds), usually after two of the n components.
 __device__ __forceinline__ bool same_solution(const EPView &ep, int n, int64_t a, int64_t b) {
     const int64_t cnt = ep.count;
+    const double ba = ep.beta[a], bb = ep.beta[b], ga = ep.gamma[a], gb = ep.gamma[b];
+    const bool ca = ba * ga < 0.03, cb = bb * gb < 0.03;
+    const double sep = 2.0 * (ba + bb);
+    const float ra = ca ? 1.0f / (20.0f * (float)ga) : 0.0f, rb = cb ? 1.0f / (20.0f * (float)gb) : 0.0f;
+    const float r = fmaxf(fmaxf(ra, rb), (float)sep);
+    const double far = (double)r * (double)r * (1.0 + 1e-5) + 1e-300;
     double d2 = 0.0;
-    for (int i = 0; i < n; i++) {
-        const double dr = ep.z_re[i * cnt + a] - ep.z_re[i * cnt + b];
-        const double di = ep.z_im[i * cnt + a] - ep.z_im[i * cnt + b];
-        d2 += dr * dr + di * di;
+    for (int i = 0; i < n; i += 2) {
+#pragma unroll
+        for (int k = i; k < i + 2; k++)
+            if (k < n) {
+                const double dr = ep.z_re[k * cnt + a] - ep.z_re[k * cnt + b];
+                const double di = ep.z_im[k * cnt + a] - ep.z_im[k * cnt + b];
+                d2 += dr * dr + di * di;
+            }
+        if (d2 > far) return false;
     }
     const double d = sqrt(d2);
-    const bool sa = ep.beta[a] * ep.gamma[a] < 0.03 && d * 20.0 * ep.gamma[a] < 1.0;
-    const bool sb = ep.beta[b] * ep.gamma[b] < 0.03 && d * 20.0 * ep.gamma[b] < 1.0;
-    const bool distinct = d > 2.0 * (ep.beta[a] + ep.beta[b]);
+    const bool sa = ca && d * 20.0 * ga < 1.0;
+    const bool sb = cb && d * 20.0 * gb < 1.0;
+    const bool distinct = d > sep;
     return sa || sb || !distinct;
 }
 
 // finest level at which e's copies with smaller beta are within the band; DD_LEVELS if none
-__device__ __forceinline__ int dd_level(double beta, double delta0) {
+__device__ __forceinline__ int dd_level(double beta, const DDGrid &grid) {
     for (int L = 0; L < DD_LEVELS; L++)
-        if (4.0 * beta <= DD_BAND * dd_pitch(delta0, L)) return L;
+        if (beta <= grid.beta[L]) return L;
     return DD_LEVELS;
 }
 
 // phase 1: list every certified endpoint under its cell at every level
-__global__ void dedup_insert_kernel(const EPView ep, int n, double delta0, DedupScratch w) {
+__global__ void dedup_insert_kernel(const EPView ep, int n, const __grid_constant__ DDGrid grid, DedupScratch w,
+                                    const int32_t *mcount) {
+    if (mcount && *mcount == 0) return;   // nothing to match: nobody reads the tables
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= ep.count) return;
     for (int L = 0; L < DD_LEVELS; L++) w.next[L * ep.count + e] = -1;
@@ -197,9 +227,8 @@ __global__ void dedup_insert_kernel(const EPView ep, int n, double delta0, Dedup
     double u[4];
     dd_project(ep, n, e, u);
     for (int L = 0; L < DD_LEVELS; L++) {
-        const double inv = 1.0 / dd_pitch(delta0, L);
         long long q[4];
-        for (int i = 0; i < 4; i++) q[i] = (long long)floor(u[i] * inv);
+        for (int i = 0; i < 4; i++) q[i] = __double2ll_rd(u[i] * grid.inv[L]);
         const unsigned long long key = dd_cell_key(L, q);
         unsigned long long *keys = w.keys + L * w.table_size;
         int32_t *head = w.head + L * w.table_size;
@@ -248,24 +277,24 @@ __device__ __forceinline__ int64_t dd_entry(const EPView &ep, const int32_t *mli
     return i < ep.count ? i : -1;
 }
 
-__global__ void dedup_match_kernel(const EPView ep, int n, double delta0, DedupScratch w,
+__global__ void dedup_match_kernel(const EPView ep, int n, const __grid_constant__ DDGrid grid, DedupScratch w,
                                    int32_t *list, int32_t *count, const int32_t *mlist,
                                    const int32_t *mcount) {
     const int64_t e = dd_entry(ep, mlist, mcount);
     if (e < 0 || !is_certified(ep.cls[e])) return;
-    const int L = dd_level(ep.beta[e], delta0);
+    const int L = dd_level(ep.beta[e], grid);
     if (L >= DD_LEVELS) return;   // phase 3
     double v[4];
     long long q0[4];
     int dir[4];
     dd_project(ep, n, e, v);
-    const double inv = 1.0 / dd_pitch(delta0, L);
-    for (int i = 0; i < 4; i++) v[i] *= inv;
+    for (int i = 0; i < 4; i++) v[i] *= grid.inv[L];
     for (int i = 0; i < 4; i++) {
-        q0[i] = (long long)floor(v[i]);
+        q0[i] = __double2ll_rd(v[i]);
         const double f = v[i] - (double)q0[i];
         dir[i] = f < DD_BAND ? -1 : (f > 1.0 - DD_BAND ? 1 : 0);
     }
+    const int64_t pe = ep.path[e];
     const uint64_t mask = (uint64_t)w.table_size - 1;
     const unsigned long long *keys = w.keys + L * w.table_size;
     const int32_t *head = w.head + L * w.table_size;
@@ -293,17 +322,25 @@ __global__ void dedup_match_kernel(const EPView ep, int n, double delta0, DedupS
         }
         for (int64_t guard = 0; o >= 0 && guard < ep.count; guard++) {
             if (!NPHC_VALID(o < ep.count, 3)) break;
-            if (o != e && same_solution(ep, n, e, o)) dd_pair(ep, w, list, count, e, o);
-            o = next[o];
+            const int32_t nx = next[o];
+            if (o != e) {
+                // a pair whose entries are both listed and whose higher path is marked has nothing
+                // to add (marks are only ever set); a solution reached by hundreds of paths
+                // would be compared pair by pair
+                const int64_t hi = ep.path[o] < pe ? e : o;
+                const bool known = __ldcg(&w.inlist[e]) && __ldcg(&w.inlist[o]) && __ldcg(&ep.cls[hi]) == NPHC_END_DUPLICATE;
+                if (!known && same_solution(ep, n, e, o)) dd_pair(ep, w, list, count, e, o);
+            }
+            o = nx;
         }
     }
 }
 
-__global__ void dedup_unhashed_kernel(const EPView ep, int n, double delta0, DedupScratch w,
+__global__ void dedup_unhashed_kernel(const EPView ep, int n, const __grid_constant__ DDGrid grid, DedupScratch w,
                                       int32_t *list, int32_t *count, const int32_t *mlist,
                                       const int32_t *mcount) {
     const int64_t e = dd_entry(ep, mlist, mcount);
-    if (e < 0 || !is_certified(ep.cls[e]) || dd_level(ep.beta[e], delta0) < DD_LEVELS) return;
+    if (e < 0 || !is_certified(ep.cls[e]) || dd_level(ep.beta[e], grid) < DD_LEVELS) return;
     for (int64_t j = 0; j < ep.count; j++) {
         if (j == e) continue;
         const int cj = ep.cls[j];
@@ -319,38 +356,37 @@ __global__ void counts_kernel(const EPView ep, const int32_t *flags, const int32
     for (int i = threadIdx.x; i < NPHC_NCOUNTS; i += blockDim.x) loc[i] = 0;
     __syncthreads();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < ep.count) {
-        atomicAdd(&loc[NPHC_COUNT_PATHS], 1ull);
-        const int st = ep.status[e];
-        if (st == NPHC_PATH_REACHED) atomicAdd(&loc[NPHC_COUNT_REACHED], 1ull);
-        else if (st == NPHC_PATH_DIVERGED) atomicAdd(&loc[NPHC_COUNT_DIVERGED], 1ull);
-        else atomicAdd(&loc[NPHC_COUNT_FAILED], 1ull);
-        const int c = ep.cls[e];
-        if (c == NPHC_END_REAL) atomicAdd(&loc[NPHC_COUNT_REAL], 1ull);
-        else if (c == NPHC_END_NONREAL) atomicAdd(&loc[NPHC_COUNT_NONREAL], 1ull);
-        else if (c == NPHC_END_UNDECIDED) atomicAdd(&loc[NPHC_COUNT_UNDECIDED], 1ull);
-        else if (c == NPHC_END_SINGULAR) atomicAdd(&loc[NPHC_COUNT_SINGULAR], 1ull);
-        else if (c == NPHC_END_DUPLICATE) atomicAdd(&loc[NPHC_COUNT_DUPLICATE], 1ull);
-        if (flags) {
-            if (flags[e] & FLAG_FP64_CONTINUED) atomicAdd(&loc[NPHC_COUNT_HANDOFF], 1ull);
-            if (flags[e] & FLAG_COND) atomicAdd(&loc[NPHC_COUNT_HANDOFF_COND], 1ull);
-            if (flags[e] & (FLAG_RETRACKED | FLAG_RETRACKED_DUP)) atomicAdd(&loc[NPHC_COUNT_RETRACKED], 1ull);
-        }
-        atomicAdd(&loc[NPHC_COUNT_SOLVES], (unsigned long long)ep.solves[e]);
-        if (c == NPHC_END_REAL && index) {
-            const int ix = index[e];
-            if (ix >= 0 && ix < NPHC_MAX_N) atomicAdd(&loc[NPHC_COUNT_INDEX0 + ix], 1ull);
-        }
-        if (egst && egst[e] != NPHC_EG_NONE) {
-            const int g = egst[e];
-            atomicAdd(&loc[NPHC_COUNT_EG_RUN], 1ull);
-            if (g == NPHC_EG_CONVERGED) {
-                atomicAdd(&loc[NPHC_COUNT_EG_CONVERGED], 1ull);
-                if (cycle[e] >= 2) atomicAdd(&loc[NPHC_COUNT_EG_MULTIPLE], 1ull);
-            } else if (g == NPHC_EG_AT_INFINITY || g == NPHC_EG_DIVERGED) {
-                atomicAdd(&loc[NPHC_COUNT_EG_AT_INFINITY], 1ull);
-            }
-        }
+    const bool on = e < ep.count;
+    // one shared atomic per warp and counter (per thread they queue up: 15 us)
+    auto tally = [&](int k, bool yes) {
+        const unsigned m = __ballot_sync(0xffffffffu, on && yes);
+        if (m && (threadIdx.x & 31) == 0) atomicAdd(&loc[k], (unsigned long long)__popc(m));
+    };
+    const int st = on ? ep.status[e] : 0, c = on ? ep.cls[e] : 0, fl = on && flags ? flags[e] : 0;
+    const int g = on && egst ? egst[e] : NPHC_EG_NONE;
+    tally(NPHC_COUNT_PATHS, true);
+    tally(NPHC_COUNT_REACHED, st == NPHC_PATH_REACHED);
+    tally(NPHC_COUNT_DIVERGED, st == NPHC_PATH_DIVERGED);
+    tally(NPHC_COUNT_FAILED, st != NPHC_PATH_REACHED && st != NPHC_PATH_DIVERGED);
+    tally(NPHC_COUNT_REAL, c == NPHC_END_REAL);
+    tally(NPHC_COUNT_NONREAL, c == NPHC_END_NONREAL);
+    tally(NPHC_COUNT_UNDECIDED, c == NPHC_END_UNDECIDED);
+    tally(NPHC_COUNT_SINGULAR, c == NPHC_END_SINGULAR);
+    tally(NPHC_COUNT_DUPLICATE, c == NPHC_END_DUPLICATE);
+    tally(NPHC_COUNT_HANDOFF, fl & FLAG_FP64_CONTINUED);
+    tally(NPHC_COUNT_HANDOFF_COND, fl & FLAG_COND);
+    tally(NPHC_COUNT_RETRACKED, fl & (FLAG_RETRACKED | FLAG_RETRACKED_DUP));
+    tally(NPHC_COUNT_EG_RUN, g != NPHC_EG_NONE);
+    tally(NPHC_COUNT_EG_CONVERGED, g == NPHC_EG_CONVERGED);
+    tally(NPHC_COUNT_EG_MULTIPLE, g == NPHC_EG_CONVERGED && cycle[e] >= 2);
+    tally(NPHC_COUNT_EG_AT_INFINITY, g == NPHC_EG_AT_INFINITY || g == NPHC_EG_DIVERGED);
+    // the sum of the solves in two halves, so that 32 of them cannot overflow
+    const unsigned sv = on ? (unsigned)ep.solves[e] : 0u;
+    const unsigned lo = __reduce_add_sync(0xffffffffu, sv & 0xffffu), hi = __reduce_add_sync(0xffffffffu, sv >> 16);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&loc[NPHC_COUNT_SOLVES], ((unsigned long long)hi << 16) + lo);
+    if (c == NPHC_END_REAL && index) {
+        const int ix = index[e];
+        if (ix >= 0 && ix < NPHC_MAX_N) atomicAdd(&loc[NPHC_COUNT_INDEX0 + ix], 1ull);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < NPHC_NCOUNTS; i += blockDim.x)
@@ -393,6 +429,33 @@ __global__ void gather_sps_kernel(const EPView ep, int M, const int32_t *list, c
 // ------------------------------------------------------------- launchers --
 static inline int blocks_for(int64_t n, int b) { return (int)((n + b - 1) / b); }
 
+// Several arrays set in one launch (a memset each costs 3 us of the stream, 29 of them a tenth of
+// a solve of N = 5).
+__global__ void fill_kernel(const __grid_constant__ FillSet f) {
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    const bool skip = f.gate && *f.gate == 0;
+    for (int s = 0; s < f.n; s++) {
+        if (skip && s >= f.n_always) return;
+        const uint32_t v = f.value[s];
+        if (((reinterpret_cast<uintptr_t>(f.ptr[s]) | (uintptr_t)f.bytes[s]) & 15) == 0) {
+            for (int64_t i = i0; i < f.bytes[s] / 16; i += step)
+                static_cast<uint4 *>(f.ptr[s])[i] = make_uint4(v, v, v, v);
+        } else {
+            for (int64_t i = i0; i < f.bytes[s] / 4; i += step) static_cast<uint32_t *>(f.ptr[s])[i] = v;
+        }
+    }
+}
+
+cudaError_t launch_fill(const FillSet &f, cudaStream_t st) {
+    int64_t most = 0;
+    for (int s = 0; s < f.n; s++) most = f.bytes[s] > most ? f.bytes[s] : most;
+    if (most == 0) return cudaSuccess;
+    const int64_t blocks = (most / 16 + 255) / 256;
+    fill_kernel<<<(int)(blocks < 1 ? 1 : blocks > 2048 ? 2048 : blocks), 256, 0, st>>>(f);
+    nphc_launch_counter(1);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_compact(const EPView &ep, int pred, int32_t *flags, int32_t *list,
                            int32_t *count, cudaStream_t st) {
     if (ep.count == 0) return cudaSuccess;
@@ -414,18 +477,24 @@ cudaError_t launch_dedup(const EPView &ep, int n, double delta, DedupScratch w, 
                          const int32_t *mcount) {
     cudaError_t err;
     // *count is an output of every call, an empty set included
-    if (count && (err = cudaMemsetAsync(count, 0, sizeof(int32_t), st))) return err;
-    if (ep.count == 0) return cudaSuccess;
+    if (ep.count == 0) return count ? cudaMemsetAsync(count, 0, sizeof(int32_t), st) : cudaSuccess;
     const size_t slots = (size_t)DD_LEVELS * w.table_size;
-    if ((err = cudaMemsetAsync(w.keys, 0, sizeof(unsigned long long) * slots, st))) return err;
-    if ((err = cudaMemsetAsync(w.head, 0xff, sizeof(int32_t) * slots, st))) return err;
-    if ((err = cudaMemsetAsync(w.inlist, 0, sizeof(int32_t) * ep.count, st))) return err;
-    const int g = blocks_for(ep.count, 256);
-    dedup_insert_kernel<<<g, 256, 0, st>>>(ep, n, delta, w);
+    FillSet f;
+    f.gate = mcount;
+    if (count) f.always(count, sizeof(int32_t), 0);
+    f.add(w.keys, sizeof(unsigned long long) * slots, 0);
+    f.add(w.head, sizeof(int32_t) * slots, 0xffffffffu);
+    f.add(w.inlist, sizeof(int32_t) * ep.count, 0);
+    if ((err = launch_fill(f, st))) return err;
+    // blocks of two warps: a thread's FP64 (one projection) takes 67 cycles an instruction per
+    // scheduler, and 15,000 endpoints in blocks of 256 leave 90 SMs idle
+    const DDGrid grid = dd_grid(delta);
+    const int g = blocks_for(ep.count, 64);
+    dedup_insert_kernel<<<g, 64, 0, st>>>(ep, n, grid, w, mcount);
     nphc_launch_counter(1);
-    dedup_match_kernel<<<g, 256, 0, st>>>(ep, n, delta, w, list, count, mlist, mcount);
+    dedup_match_kernel<<<g, 64, 0, st>>>(ep, n, grid, w, list, count, mlist, mcount);
     nphc_launch_counter(1);
-    dedup_unhashed_kernel<<<g, 256, 0, st>>>(ep, n, delta, w, list, count, mlist, mcount);
+    dedup_unhashed_kernel<<<g, 64, 0, st>>>(ep, n, grid, w, list, count, mlist, mcount);
     nphc_launch_counter(1);
     return cudaGetLastError();
 }

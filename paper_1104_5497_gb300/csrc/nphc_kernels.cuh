@@ -25,6 +25,26 @@ struct DedupScratch {
     int32_t *inlist;
 };
 
+// Arrays to set to a repeated 32-bit value in one launch (bytes: multiples of 4).  With a gate (a
+// device counter) of 0 only those of `always` are set; they come first.
+struct FillSet {
+    void *ptr[6];
+    int64_t bytes[6];
+    uint32_t value[6];
+    int n = 0, n_always = 0;
+    const int32_t *gate = nullptr;
+    void add(void *p, size_t b, uint32_t v) {
+        ptr[n] = p;
+        bytes[n] = (int64_t)b;
+        value[n++] = v;
+    }
+    void always(void *p, size_t b, uint32_t v) {
+        add(p, b, v);
+        n_always = n;
+    }
+};
+cudaError_t launch_fill(const FillSet &f, cudaStream_t st);
+
 // The debug build's first failed index check (0 if none), cleared; -1 in a release build.
 cudaError_t nphc_debug_read(int *code);
 
@@ -34,7 +54,8 @@ cudaError_t launch_flag_list(const int32_t *list, const int32_t *count, int64_t 
                              int32_t *flags, int32_t bit, cudaStream_t st);
 // Marks duplicates among the certified entries of ep.  mlist / mcount (device, may be
 // NULL): only the pairs with an entry of mlist are examined (every other pair was
-// settled by an earlier dedup and its entries left unchanged since).
+// settled by an earlier dedup and its entries left unchanged since); with an empty mlist the
+// launches return at once.
 cudaError_t launch_dedup(const EPView &ep, int n, double delta, DedupScratch w, int32_t *list,
                          int32_t *count, cudaStream_t st, const int32_t *mlist = nullptr,
                          const int32_t *mcount = nullptr);
