@@ -93,6 +93,12 @@ DedupScratch dedup_scratch(void *ws, const WsLayout &L) {
     return w;
 }
 
+// k with s < 2^k for a rounded sum s >= 0 of non-negative numbers
+int sum_exponent(double s) {
+    if (!(s > 0.0)) return -1023;
+    return std::isfinite(s) ? std::ilogb(s * (1.0 + 1e-12)) + 1 : 1024;
+}
+
 unsigned long long *ws_queue(void *ws, int slot) {
     return reinterpret_cast<unsigned long long *>(static_cast<char *>(ws)) + slot;
 }
@@ -273,7 +279,7 @@ nphc_status nphc_system_create_xy(int N, double sigma, const double *J, nphc_sys
         }
         row = std::max(row, sum);
     }
-    S->xs.jexp = row > 0.0 ? (std::isfinite(row) ? std::ilogb(row * (1.0 + 1e-12)) + 1 : 1024) : -1023;
+    S->xs.jexp = sum_exponent(row);
     S->xs.d2norm = std::sqrt(d2);
     S->xs.kappa_sing = 1e12;
     *out = S;
@@ -341,9 +347,13 @@ nphc_status nphc_system_create_quadratic(int n, int nterms, const int32_t *eq, c
             }
         }
     }
-    double d2 = 0.0;
-    for (int i = 0; i < n; i++)
+    double d2 = 0.0, most = 0.0;
+    for (int i = 0; i < n; i++) {
         for (double v : m2[i]) d2 += v * v;
+        double sum = 0.0;
+        for (int t = row[i]; t < row[i + 1]; t++) sum += std::fabs(terms[t].cre) + std::fabs(terms[t].cim);
+        most = std::max(most, sum);
+    }
     // the Jacobian's entries: per (variable, equation) cell the list of c w(other)
     std::vector<std::vector<QTerm>> cell((size_t)n * n);
     for (int i = 0; i < n; i++)
@@ -395,6 +405,7 @@ nphc_status nphc_system_create_quadratic(int n, int nterms, const int32_t *eq, c
         return fail(NPHC_ECUDA, std::string("term list upload: ") + cudaGetErrorString(e));
     }
     S->qs.n = n;
+    S->qs.cexp = sum_exponent(most);
     S->qs.row = reinterpret_cast<const int32_t *>(d);
     S->qs.terms = reinterpret_cast<const QTerm *>(d + rbytes);
     S->qs.jrow = reinterpret_cast<const int32_t *>(d + rbytes + tbytes);

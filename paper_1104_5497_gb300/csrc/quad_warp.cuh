@@ -7,7 +7,7 @@
 // whatever the number of lanes; a dense residual and QR of n = 10 take 40 k).  So the lanes
 // share a path:
 //   * sums over an equation's terms: 32 / n lanes per equation, each a share of the terms,
-//     their (compensated) sums combined by shuffles;
+//     their (compensated: gsum in nphc_internal.cuh) sums combined by shuffles;
 //   * the Jacobian: one (variable, equation) cell per lane at a time, from the list of the
 //     terms that contribute to it;
 //   * the linear solve: warp_lu_solve (xy_track_warp.cuh).
@@ -18,13 +18,6 @@
 
 #include "xy_endgame.cuh"
 #include "xy_track_warp.cuh"
-
-// (a.hi + a.lo) + (b.hi + b.lo), the rounding error of the leading sum kept in lo
-__device__ __forceinline__ ext<double> ext_add(ext<double> a, ext<double> b) {
-    double s, e;
-    two_sum(a.hi, b.hi, s, e);
-    return ext<double>{s, EFT<double>::add(e, EFT<double>::add(a.lo, b.lo))};
-}
 
 template <int N>
 struct QuadLayout {   // shared memory per warp, complex doubles
@@ -63,7 +56,7 @@ struct QuadSum {
 #pragma unroll 1
             for (int t = S.row[i] + lane % LE; t < S.row[i + 1]; t += LE) {
                 const QTerm T = S.terms[t];
-                p = cadd(p, cmul(cx<double>{T.cre, T.cim}, cmul(quad_w(z, T.a), quad_w(z, T.b))));
+                p = cfma64(cx<double>{T.cre, T.cim}, cmul(quad_w(z, T.a), quad_w(z, T.b)), p);
             }
         }
 #pragma unroll
@@ -73,34 +66,41 @@ struct QuadSum {
         }
         return p;
     }
+    // With exact products and compensated sums, on grids (gsum); |P's parts| < 2^(kp - 1).
     static __device__ __forceinline__ void compensated(const QSys &S, const cx<double> *z, int lane,
-                                                       ext<double> &pr, ext<double> &pi) {
-        const ext<double> zero = {0.0, 0.0};
-        pr = pi = zero;
+                                                       ext<double> &pr, ext<double> &pi, int &kp) {
+        const cx<double> zl = z[lane < N ? lane : 0];
+        const int ez = __reduce_max_sync(0xffffffffu, max(max(gexp(zl.re), gexp(zl.im)), 0));
+        kp = S.cexp + 2 * ez + 4;
+        const double am = gsum_anchor(2 * ez + 4), ap = gsum_anchor(kp);
+        gsum sr = {ap, 0.0}, si = sr;
         const int i = lane / LE;
         if (i < N) {
 #pragma unroll 1
             for (int t = S.row[i] + lane % LE; t < S.row[i + 1]; t += LE) {
                 const QTerm T = S.terms[t];
                 const cx<double> wa = quad_w(z, T.a), wb = quad_w(z, T.b);
-                ext<double> mr = zero, mi = zero;   // wa wb
-                ext_acc(mr, wa.re, wb.re);
-                ext_acc(mr, -wa.im, wb.im);
-                ext_acc(mi, wa.re, wb.im);
-                ext_acc(mi, wa.im, wb.re);
-                ext_acc_ext(pr, T.cre, mr);
-                ext_acc_ext(pr, -T.cim, mi);
-                ext_acc_ext(pi, T.cre, mi);
-                ext_acc_ext(pi, T.cim, mr);
+                gsum smr = {am, 0.0}, smi = smr;   // wa wb
+                gsum_acc(smr, wa.re, wb.re);
+                gsum_acc(smr, -wa.im, wb.im);
+                gsum_acc(smi, wa.re, wb.im);
+                gsum_acc(smi, wa.im, wb.re);
+                const ext<double> mr = gsum_ext(smr, am), mi = gsum_ext(smi, am);
+                gsum_acc_ext(sr, T.cre, mr);
+                gsum_acc_ext(sr, -T.cim, mi);
+                gsum_acc_ext(si, T.cre, mi);
+                gsum_acc_ext(si, T.cim, mr);
             }
         }
+        pr = gsum_ext(sr, ap);
+        pi = gsum_ext(si, ap);
 #pragma unroll
         for (int o = 1; o < LE; o <<= 1) {
             const ext<double> qr = {__shfl_down_sync(0xffffffffu, pr.hi, o), __shfl_down_sync(0xffffffffu, pr.lo, o)};
             const ext<double> qi = {__shfl_down_sync(0xffffffffu, pi.hi, o), __shfl_down_sync(0xffffffffu, pi.lo, o)};
             if (lane % LE % (2 * o) == 0 && lane % LE + o < LE) {
-                pr = ext_add(pr, qr);
-                pi = ext_add(pi, qi);
+                pr = grid_add(pr, qr);
+                pi = grid_add(pi, qi);
             }
         }
     }
@@ -113,7 +113,7 @@ __device__ __forceinline__ cx<double> quad_jac(const QSys &S, const cx<double> *
 #pragma unroll 1
     for (int t = S.jrow[cell]; t < S.jrow[cell + 1]; t++) {
         const QTerm T = S.jac[t];
-        d = cadd(d, cmul(cx<double>{T.cre, T.cim}, quad_w(z, T.a)));
+        d = cfma64(cx<double>{T.cre, T.cim}, quad_w(z, T.a), d);
     }
     return d;
 }
@@ -154,23 +154,27 @@ struct WarpQuad {
         using E = EFT<double>;
         const int lane = P.lane, i = QuadSum<N>::eq(lane);
         ext<double> pr, pi;
-        QuadSum<N>::compensated(S, P.s + L::ZC, lane, pr, pi);
+        int kp;
+        QuadSum<N>::compensated(S, P.s + L::ZC, lane, pr, pi, kp);
         if (QuadSum<N>::first(lane)) {
             const double g1r = E::mul(omt, S.gre), g1i = E::mul(omt, S.gim);
-            const ext<double> zero = {0.0, 0.0};
             const cx<double> zi = P.at(L::ZC, i);
-            ext<double> qr = {-1.0, 0.0}, qi = zero;   // z_i^2 - 1
-            ext_acc(qr, zi.re, zi.re);
-            ext_acc(qr, -zi.im, zi.im);
-            ext_acc(qi, 2.0 * zi.re, zi.im);
-            ext<double> hr = zero, hi = zero;
-            ext_acc_ext(hr, g1r, qr);
-            ext_acc_ext(hr, -g1i, qi);
-            ext_acc_ext(hr, s, pr);
-            ext_acc_ext(hi, g1r, qi);
-            ext_acc_ext(hi, g1i, qr);
-            ext_acc_ext(hi, s, pi);
-            P.at(L::W1, i) = cx<double>{-ext_val(hr), -ext_val(hi)};
+            const int kq = max(0, 2 * max(gexp(zi.re), gexp(zi.im)) + 2) + 2;
+            const double aq = gsum_anchor(kq);
+            gsum sqr = gsum_start(aq, -1.0), sqi = {aq, 0.0};   // z_i^2 - 1
+            gsum_acc(sqr, zi.re, zi.re);
+            gsum_acc(sqr, -zi.im, zi.im);
+            gsum_acc(sqi, 2.0 * zi.re, zi.im);
+            const ext<double> qr = gsum_ext(sqr, aq), qi = gsum_ext(sqi, aq);
+            const double ah = gsum_anchor(max(max(gexp(g1r), gexp(g1i)) + kq + 1, gexp(s) + kp) + 2);
+            gsum hr = {ah, 0.0}, hi = hr;
+            gsum_acc_ext(hr, g1r, qr);
+            gsum_acc_ext(hr, -g1i, qi);
+            gsum_acc_ext(hr, s, pr);
+            gsum_acc_ext(hi, g1r, qi);
+            gsum_acc_ext(hi, g1i, qr);
+            gsum_acc_ext(hi, s, pi);
+            P.at(L::W1, i) = cx<double>{-ext_val(gsum_ext(hr, ah)), -ext_val(gsum_ext(hi, ah))};
             P.at(L::PV, i) = cx<double>{ext_val(pr), ext_val(pi)};
         }
         __syncwarp();
@@ -234,7 +238,8 @@ __device__ QuadEval quad_evaluate(const QuadPath &W, const QSys &S) {
     const cx<double> *z = W.s + L::Z;
     QuadEval v;
     ext<double> pr, pi;
-    QuadSum<N>::compensated(S, z, lane, pr, pi);
+    int kp;
+    QuadSum<N>::compensated(S, z, lane, pr, pi, kp);
     double pm = 0.0;
     if (QuadSum<N>::first(lane)) {
         const cx<double> p = {ext_val(pr), ext_val(pi)};
