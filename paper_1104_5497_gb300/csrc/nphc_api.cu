@@ -1097,15 +1097,21 @@ nphc_status nphc_result_copy_endpoints(const nphc_result *R, int64_t cap, double
     if (k == 0) return NPHC_OK;
     const int n = R->n;
     if (z_re || z_im) {
-        std::vector<double> buf(R->P);
+        // blocks of entries through a buffer that stays in the cache (and in touched pages: a copy to
+        // untouched pageable memory takes 2 ms per 1.8 MB), each transposed by reading n streams and
+        // writing one; a copy and a strided scatter per component took 1.0 ms for N = 8
+        const int64_t block = std::min<int64_t>(k, std::max<int64_t>(256, 65536 / n));
+        std::vector<double> buf((size_t)n * block);
         for (int part = 0; part < 2; part++) {
             double *dst = part ? z_im : z_re;
             if (!dst) continue;
             const double *src = part ? R->ep.z_im : R->ep.z_re;
-            for (int i = 0; i < n; i++) {
-                NPHC_CK(cudaMemcpy(buf.data(), src + (size_t)i * R->P, sizeof(double) * k,
-                                   cudaMemcpyDeviceToHost));
-                for (int64_t e = 0; e < k; e++) dst[e * n + i] = buf[e];
+            for (int64_t e0 = 0; e0 < k; e0 += block) {
+                const int64_t m = std::min(block, k - e0);
+                NPHC_CK(cudaMemcpy2D(buf.data(), sizeof(double) * m, src + e0, sizeof(double) * R->P,
+                                     sizeof(double) * m, n, cudaMemcpyDeviceToHost));
+                for (int64_t e = 0; e < m; e++)
+                    for (int i = 0; i < n; i++) dst[(e0 + e) * n + i] = buf[(size_t)i * m + e];
             }
         }
     }

@@ -314,11 +314,13 @@ class Result:
         s = self.system
         n = ctypes.c_int64()
         P = s.npaths
-        zr, zi = np.zeros((P, s.n)), np.zeros((P, s.n))
-        st, cl = np.zeros(P, np.int32), np.zeros(P, np.int32)
+        zr, zi = np.empty((P, s.n)), np.empty((P, s.n))
+        st, cl = np.empty(P, np.int32), np.empty(P, np.int32)
         _check("nphc_result_copy_endpoints", lib().nphc_result_copy_endpoints(
             self.handle, P, _pd(zr), _pd(zi), _pi32(st), _pi32(cl), ctypes.byref(n)))
-        return dict(z=zr + 1j * zi, status=st, cls=cl)
+        z = np.empty((P, s.n), np.complex128)
+        z.real, z.imag = zr, zi
+        return dict(z=z, status=st, cls=cl)
 
     def device_endpoints(self) -> nphc_endpoints:
         ep = nphc_endpoints()
