@@ -229,7 +229,7 @@ cudaError_t NPHC_CAT(launch_xy_track_f64_m, NPHC_INST_M)(const XYSys &sys, const
                                                          int grid, cudaStream_t st) {
     constexpr int M = NPHC_INST_M, BLK = NPHC_TRACK_BLOCK;
     const size_t smem = xy_smem_per_thread<M, double>() * BLK;
-    auto k = xy_track_kernel<M, double, BLK>;
+    auto k = xy_track_kernel<M, BLK>;
     static bool attr_set = false;   // once per process for this instantiation
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

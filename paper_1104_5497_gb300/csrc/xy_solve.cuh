@@ -84,8 +84,6 @@ struct SMat {
 template <int M, class R>
 constexpr size_t xy_smem_per_thread() { return sizeof(cx<R>) * (size_t)(M * (M + 2) + 2 * M); }
 
-__device__ __forceinline__ void compiler_fence() { asm volatile("" ::: "memory"); }
-
 // -H_t rows of site k (H_t = P - gamma Q) at the point (xk, yk) with u_k, w_k given.
 template <class R>
 __device__ __forceinline__ void minus_ht_rows(cx<R> xk, cx<R> yk, cx<R> u, cx<R> w, cx<R> gam,
@@ -94,13 +92,6 @@ __device__ __forceinline__ void minus_ht_rows(cx<R> xk, cx<R> yk, cx<R> u, cx<R>
     const cx<R> x2 = cmul(xk, xk), y2 = cmul(yk, yk);
     rf = csub(cmul(gam, cx<R>{x2.re - R(1), x2.im}), f);
     rg = csub(cmul(gam, cx<R>{y2.re - R(1), y2.im}), cx<R>{x2.re + y2.re - R(1), x2.im + y2.im});
-}
-
-// -H_t constraint row only (needs no couplings).
-template <class R>
-__device__ __forceinline__ cx<R> minus_ht_g(cx<R> xk, cx<R> yk, cx<R> gam) {
-    const cx<R> x2 = cmul(xk, xk), y2 = cmul(yk, yk);
-    return csub(cmul(gam, cx<R>{y2.re - R(1), y2.im}), cx<R>{x2.re + y2.re - R(1), x2.im + y2.im});
 }
 
 // u_k = J_{k,N} + sum_l J_kl x_l and w_k = sum_l J_kl y_l (J_kk = 0, so the sum may run over
@@ -121,46 +112,6 @@ __device__ __forceinline__ void xy_uw(const R *__restrict__ J, const cx<R> (&x)[
     }
 }
 
-// Coefficients (al, be) of a row on (dx_j, dy_j) as coefficients on the scaled light-cone
-// step (dwp_j, dwq_j): (sp (al - i be) / 2, sq (al + i be) / 2).
-template <class R>
-__device__ __forceinline__ void lc_coef(cx<R> al, cx<R> be, R sp, R sq, cx<R> &alp, cx<R> &bep) {
-    alp = cscale(R(0.5) * sp, cx<R>{al.re + be.im, al.im - be.re});
-    bep = cscale(R(0.5) * sq, cx<R>{al.re - be.im, al.im + be.re});
-}
-
-// Scales of site j's light-cone coordinates: max(1, |x + i y|) and max(1, |x - i y|).
-template <class R>
-__device__ __forceinline__ void lc_scales(cx<R> xj, cx<R> yj, R &sp, R &sq) {
-    const cx<R> p = cx<R>{xj.re - yj.im, xj.im + yj.re}, q = cx<R>{xj.re + yj.im, xj.im - yj.re};
-    sp = fmax(R(1), sqrt_r(cabs2(p)));
-    sq = fmax(R(1), sqrt_r(cabs2(q)));
-}
-
-// Frame of constraint row j in site j's scaled light-cone coordinates: (a^, b^), the
-// inverse of the row's norm |(a'_j, b'_j)| and the scales sp, sq.
-template <class R>
-__device__ __forceinline__ void g_frame(cx<R> xj, cx<R> yj, R s, cx<R> sg, cx<R> &ah, cx<R> &bh,
-                                        R &iv, R &sp, R &sq) {
-    lc_scales<R>(xj, yj, sp, sq);
-    cx<R> a, bb;
-    lc_coef<R>(cscale(R(2) * s, xj), cscale(R(2), cmul(sg, yj)), sp, sq, a, bb);
-    iv = rsqrt_r(cabs2(a) + cabs2(bb));
-    ah = cscale(iv, a);
-    bh = cscale(iv, bb);
-}
-
-// (dx_j, dy_j) from the light-cone step (dwp, dwq) = conj(a^, b^) q + (b^, -a^) s.
-template <class R>
-__device__ __forceinline__ void lc_step(cx<R> ah, cx<R> bh, R sp, R sq, cx<R> q, cx<R> s,
-                                        cx<R> &dx, cx<R> &dy) {
-    const cx<R> wp = cscale(sp, cadd(cmulc(ah, q), cmul(bh, s)));
-    const cx<R> wq = cscale(sq, csub(cmulc(bh, q), cmul(ah, s)));
-    dx = cscale(R(0.5), cadd(wp, wq));
-    const cx<R> d = csub(wp, wq);
-    dy = cx<R>{R(0.5) * d.im, R(-0.5) * d.re};   // -i (wp - wq) / 2
-}
-
 // i c
 template <class R>
 __device__ __forceinline__ cx<R> cmul_i(cx<R> c) { return cx<R>{-c.im, c.re}; }
@@ -169,14 +120,10 @@ __device__ __forceinline__ cx<R> cmul_i(cx<R> c) { return cx<R>{-c.im, c.re}; }
 // [S | b0 | b1] (b1 only when two_rhs) by Householder QR: Q^H [S | b] = [R | Q^H b] with a
 // real diagonal (stored as (beta, 0) on the diagonal of S), then back substitution in
 // place: the solutions end in columns M and M + 1.  Returns false when S is singular.
-// kest (may be NULL) receives max_k |R_kk| / min_k |R_kk|, a lower bound on the condition
-// number of S that costs two comparisons per column.
 template <int M, class R, int BLOCK>
-__device__ __forceinline__ bool aug_qr_solve(const SMat<M, R, BLOCK> &A, bool two_rhs,
-                                             R *kest = nullptr) {
+__device__ __forceinline__ bool aug_qr_solve(const SMat<M, R, BLOCK> &A, bool two_rhs) {
     const int ncol = two_rhs ? M + 2 : M + 1;
     bool ok = true;
-    R rmax = R(0), rmin = R(0);
 #pragma unroll 1
     for (int k = 0; k < M; k++) {
         const int n = M - k;   // active rows k .. M-1, relative index i = 0 .. n-1
@@ -199,8 +146,6 @@ __device__ __forceinline__ bool aug_qr_solve(const SMat<M, R, BLOCK> &A, bool tw
         }
         const R an = sqrt_r(cabs2(al) + (xa + xb));
         ok = ok && (an > R(0));
-        rmax = fmax(rmax, an);
-        rmin = k == 0 ? an : fmin(rmin, an);
         const R beta = al.re >= R(0) ? -an : an;
         const R ib = recip_r(beta);
         const cx<R> tauc = cx<R>{(beta - al.re) * ib, al.im * ib};   // conj(tau)
@@ -264,7 +209,6 @@ __device__ __forceinline__ bool aug_qr_solve(const SMat<M, R, BLOCK> &A, bool tw
         }
     }
 
-    if (kest) *kest = rmin > R(0) ? rmax / rmin : R(INFINITY);
     return ok;
 }
 
@@ -275,14 +219,10 @@ __device__ __forceinline__ bool aug_qr_solve(const SMat<M, R, BLOCK> &A, bool tw
 // conflict-free in the interleaved layout) and the rows below take a rank-one update,
 // a load, four FMAs and a store per complex entry, against Householder's extra dot
 // product per entry.  The pivot's reciprocal replaces U_kk for the back substitution.
-// kest (may be NULL) receives max_k |U_kk| / min_k |U_kk|, the usual cheap estimate of the
-// condition number from a pivoted factorisation.
 template <int M, class R, int BLOCK>
-__device__ __forceinline__ bool aug_lu_solve(const SMat<M, R, BLOCK> &A, bool two_rhs,
-                                             R *kest = nullptr) {
+__device__ __forceinline__ bool aug_lu_solve(const SMat<M, R, BLOCK> &A, bool two_rhs) {
     const int ncol = two_rhs ? M + 2 : M + 1;
     bool ok = true;
-    R umax = R(0), umin = R(0);
 #pragma unroll 1
     for (int k = 0; k < M; k++) {
         const int n = M - k;   // active rows k .. M-1, relative index i = 0 .. n-1
@@ -304,9 +244,6 @@ __device__ __forceinline__ bool aug_lu_solve(const SMat<M, R, BLOCK> &A, bool tw
             }
         }
         ok = ok && (best > R(0));
-        const R um = sqrt_r(best);
-        umax = fmax(umax, um);
-        umin = k == 0 ? um : fmin(umin, um);
         const cx<R> ip = crecip(piv);
         // multipliers of rows 1 .. n-1 after the swap (row p holds the old row k)
 #pragma unroll
@@ -358,7 +295,6 @@ __device__ __forceinline__ bool aug_lu_solve(const SMat<M, R, BLOCK> &A, bool tw
         }
     }
 
-    if (kest) *kest = umin > R(0) ? umax / umin : R(INFINITY);
     return ok;
 }
 
@@ -436,8 +372,7 @@ template <int M, class R, int BLOCK, class Out2>
 __device__ __forceinline__ bool xy_solve(const R *__restrict__ J, const SMat<M, R, BLOCK> &A,
                                          const SVec<R, BLOCK> &pt, R s, R omt, cx<R> gam,
                                          bool two_rhs, const SVec<R, BLOCK> &res,
-                                         const SVec<R, BLOCK> &out1, const Out2 &out2, bool wr,
-                                         R *kest = nullptr) {
+                                         const SVec<R, BLOCK> &out1, const Out2 &out2, bool wr) {
     const cx<R> gomt = cscale(omt, gam);
 
     cx<R> p[M], q[M];
@@ -506,7 +441,7 @@ __device__ __forceinline__ bool xy_solve(const R *__restrict__ J, const SMat<M, 
             A.set(k, M + 1, csub(A.get(k, M + 1), cmul_i(cscale(hs, csub(cmul(q[k], sx1[k]), cmul(p[k], sy1[k]))))));
     }
 
-    bool ok = aug_lu_solve<M, R, BLOCK>(A, two_rhs, kest);
+    bool ok = aug_lu_solve<M, R, BLOCK>(A, two_rhs);
 
     // ---- back to (dp, dq) = (sp dwp, sq dwq),
     // (dwp, dwq) = conj(a^, b^) q_j + (b^, -a^) s_j

@@ -3,22 +3,26 @@
 // Q_i = z_i^2 - 1, start points z_i = +-1, tracked from t = 0 to t = 1 with a
 // predictor and Newton's corrector).
 //
-// Layout: one path per thread; a persistent grid pulls paths from a device work
-// counter (warp-aggregated atomics) until the list is drained.  The warp runs its 32
-// paths in lockstep through the same phases of a step -- three RK4 stage solves, then
-// up to max_newton corrector solves -- in a loop with a single call site of the solve,
-// so the heavy solve is never divergent and its unrolled code is instantiated once
-// (instruction-cache resident); lanes whose path has finished take the next one at
-// the step boundary.  The M x M Schur matrix, the evaluation point and the solve
-// output of each path live in shared memory (xy_solve.cuh); the accepted point, its
-// derivative and the RK4 sum live in a global scratch (coalesced, L2-resident).
+// This file: the method, what every tracker shares, and the FP64 tracker with one path per
+// thread, which lists take when asked to (options.threads_per_path = 1).  The others: one path
+// per thread or four lanes per path in FP32 (xy_track_lane.cuh, xy_track_group.cuh), four lanes
+// or a warp per path in FP64 (xy_track_group64.cuh, xy_track_warp.cuh).
+//
+// Layout here: a persistent grid pulls paths from a device work counter (warp-aggregated
+// atomics) until the list is drained.  The warp runs its 32 paths in lockstep through the same
+// phases of a step -- three RK4 stage solves, then up to max_newton corrector solves -- in a
+// loop with a single call site of the solve, so the heavy solve is never divergent and its
+// unrolled code is instantiated once (instruction-cache resident); lanes whose path has
+// finished take the next one at the step boundary.  The M x M Schur matrix, the evaluation
+// point and the solve output of each path live in shared memory (xy_solve.cuh); the accepted
+// point, its derivative and the RK4 sum live in a global scratch (coalesced, L2-resident).
 //
 // Predictor: classical RK4 on dz/dt = -H_z^-1 H_t.  The derivative at the start of a
 // step is taken from the previous step's last corrector solve (second right-hand
 // side, same factorisation), and at t = 0 it is known in closed form
 // (H_z = 2 gamma diag(z), H_t = P(z)), so each step costs 3 stage solves.
 // Corrector: Newton at t + h, its residual evaluated with compensated sums
-// (xy_residual_comp: float-float in FP32, double-double in FP64).  A step is accepted when ||dz|| <= eps (1 + ||z||)
+// (float-float in FP32, double-double in FP64).  A step is accepted when ||dz|| <= eps (1 + ||z||)
 // within max_newton iterations, and rejected when the first correction exceeds
 // trust (1 + ||z||).  Step size doubles after grow_after consecutive accepts and halves
 // on a reject; the final step lands exactly on t = t_end (1, or 1 - r0 before the Cauchy
@@ -43,17 +47,6 @@
 #pragma once
 
 #include "xy_solve.cuh"
-
-template <class R>
-struct JSel;
-template <>
-struct JSel<float> {
-    static __device__ __forceinline__ const float *get(const XYSys &S) { return S.Jf; }
-};
-template <>
-struct JSel<double> {
-    static __device__ __forceinline__ const double *get(const XYSys &S) { return S.Jd; }
-};
 
 #define CRAWL_ZONE 1e-3   // the crawl test applies once 1 - t < CRAWL_ZONE
 // A path in the end zone whose ||z||_inf exceeds FAR_NORM and grew by more than FAR_GROWTH
@@ -84,14 +77,6 @@ __device__ __forceinline__ R vnorm2(const V &v) {
     return sqrt_r(s);
 }
 
-template <int NV, class R, class V>
-__device__ __forceinline__ R vnorminf(const V &v) {
-    R s = R(0);
-#pragma unroll 1
-    for (int i = 0; i < NV; i++) s = fmax(s, sqrt_r(cabs2(v.get(i))));
-    return s;
-}
-
 // The problem a tracker runs on, as a policy for track_body: the unknowns (NV), the
 // per-thread shared matrix (MD x (MD + 2)), the start point with its dz/dt, the
 // corrector residual -H, the linear solve, and the tracker state's relation to the
@@ -99,9 +84,9 @@ __device__ __forceinline__ R vnorminf(const V &v) {
 // z's inf-norm).  XYProblem: the XY ring (structured Schur solve, M = N - 1 free sites,
 // NV = 2M), its state in light-cone coordinates p_k = x_k + i y_k, q_k = x_k - i y_k
 // (xy_solve.cuh): a unitary map times sqrt(2), so 2-norms are the state's over sqrt(2).
-template <int M, class RT, int BLK>
+template <int M, int BLK>
 struct XYProblem {
-    using R = RT;
+    using R = double;
     using Sys = XYSys;
     static constexpr int BLOCK = BLK;
     static constexpr int NV = 2 * M;
@@ -150,7 +135,7 @@ struct XYProblem {
     // H_t = P(z), so dz_i/dt = -P_i(z) / (2 gamma z_i); both in light-cone coordinates
     static __device__ __forceinline__ void start(const Sys &S, int64_t p, const GVec<R> &Z0,
                                                  const GVec<R> &K1) {
-        const R *J = JSel<R>::get(S);
+        const R *J = S.Jd;
         const cx<R> gam = cx<R>{(R)S.gre, (R)S.gim};
         cx<R> x[M], y[M];
 #pragma unroll
@@ -177,7 +162,7 @@ struct XYProblem {
 
     static __device__ __forceinline__ void residual(const Sys &S, const SVec<R, BLOCK> &pt, R s,
                                                     R omt, const SVec<R, BLOCK> &out, bool wr) {
-        residual_g(S, pt, s, omt, cx<R>{(R)S.gre, (R)S.gim}, out, wr);
+        xy_residual_comp<M, R, BLOCK>(S.Jd, pt, s, omt, cx<R>{S.gre, S.gim}, out, wr);
     }
 
     template <class Out2>
@@ -185,28 +170,9 @@ struct XYProblem {
                                                  const SVec<R, BLOCK> &pt, R s, R omt,
                                                  bool two_rhs, const SVec<R, BLOCK> &res,
                                                  const SVec<R, BLOCK> &out1, const Out2 &out2,
-                                                 bool wr, R *kest = nullptr) {
-        return solve_g(S, A, pt, s, omt, cx<R>{(R)S.gre, (R)S.gim}, two_rhs, res, out1, out2, wr,
-                       kest);
-    }
-
-    // the same with an explicit gamma (per thread: the Cauchy endgame's equivalent real-t
-    // homotopy at a complex t)
-    static __device__ __forceinline__ void residual_g(const Sys &S, const SVec<R, BLOCK> &pt, R s,
-                                                      R omt, cx<R> gam,
-                                                      const SVec<R, BLOCK> &out, bool wr) {
-        xy_residual_comp<M, R, BLOCK>(JSel<R>::get(S), pt, s, omt, gam, out, wr);
-    }
-
-    template <class Out2>
-    static __device__ __forceinline__ bool solve_g(const Sys &S, const SMat<M, R, BLOCK> &A,
-                                                   const SVec<R, BLOCK> &pt, R s, R omt,
-                                                   cx<R> gam, bool two_rhs,
-                                                   const SVec<R, BLOCK> &res,
-                                                   const SVec<R, BLOCK> &out1, const Out2 &out2,
-                                                   bool wr, R *kest = nullptr) {
-        return xy_solve<M, R, BLOCK>(JSel<R>::get(S), A, pt, s, omt, gam, two_rhs, res, out1, out2,
-                                     wr, kest);
+                                                 bool wr) {
+        return xy_solve<M, R, BLOCK>(S.Jd, A, pt, s, omt, cx<R>{S.gre, S.gim}, two_rhs, res, out1,
+                                     out2, wr);
     }
 };
 
@@ -260,8 +226,9 @@ struct BatchSrc {
     __device__ __forceinline__ const EPView &eps(int g) const { return ep[g]; }
 };
 
-template <class P, class Src>
-__device__ __forceinline__ void track_body(const Src &src, const XYCtl &C, const WorkList &wl) {
+template <class P>
+__device__ __forceinline__ void track_body(const typename P::Sys &S, const XYCtl &C, const EPView &ep,
+                                           const WorkList &wl) {
     using R = typename P::R;
     constexpr int BLOCK = P::BLOCK, NV = P::NV, MD = P::MD;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -277,8 +244,7 @@ __device__ __forceinline__ void track_body(const Src &src, const XYCtl &C, const
     const GVec<R> Z0{st + (0 * NV) * nth + gtid, nth};       // accepted point
     const GVec<R> K1{st + (1 * NV) * nth + gtid, nth};       // dz/dt at Z0
     const GVec<R> AC{st + (2 * NV) * nth + gtid, nth};       // RK4 sum; next K1 in correction
-    const GVec<R> CK{st + (3 * NV) * nth + gtid, nth};       // FP32 pass: hand-off checkpoint
-    const int64_t total = src.total();
+    const int64_t total = worklist_size(wl, ep.count);
 
     // short lists: at most `lanes` paths per warp, so that the list spreads over every SM
     // instead of filling the first warps 32 at a time (FP64 continuation of a few
@@ -290,14 +256,8 @@ __device__ __forceinline__ void track_body(const Src &src, const XYCtl &C, const
         lanes = per < 1 ? 1 : (per > 32 ? 32 : (int)per);
     }
     int64_t e = (lane >= lanes) ? -2 : -1;   // entry index; -1 idle, -2 drained
-    int g = 0;                                // instance of the entry (batches)
-    double t = 0.0, h = 0.0, hacc = 0.0;
-    double tck = 0.0, hck = 0.0;   // checkpoint: the last clean accepted point with 1 - t < CRAWL_ZONE
-    bool have_ck = false;
-    int clean = 0;                 // accepted steps in a row without a reject between them
-    double tmark = 0.0;   // 1 - t recorded every CRAWL_STEPS accepted steps near t = 1
-    int since = 0;
-    int status = 0, run = 0, rejects = 0, attempts = 0, steps = 0, solves = 0, newton = 0;
+    double t = 0.0, h = 0.0;
+    int status = 0, run = 0, attempts = 0, steps = 0, solves = 0, newton = 0;
     bool need_k1 = false;
     bool far = false;      // heading out: steps capped at KAPPA_FAR (1 - t)
     double zlast = 0.0;    // ||z||_inf at the last accepted point
@@ -313,17 +273,13 @@ __device__ __forceinline__ void track_body(const Src &src, const XYCtl &C, const
             base = __shfl_sync(0xffffffffu, base, leader);
             if (idle) {
                 const int64_t i = (int64_t)base + __popc(need & ((1u << lane) - 1u));
-                if (i < total) src.take(i, g, e);   // -1 (skipped) if the debug build rejects it
+                if (i < total) e = worklist_entry(wl, i, ep.count);   // -1 (skipped) if the debug build rejects it
                 if (i >= total) {
                     e = -2;
                 } else if (e >= 0) {
-                    const EPView &ep = src.eps(g);
                     status = NPHC_PATH_RUNNING;
                     run = 0;
-                    rejects = 0;
                     attempts = 0;
-                    have_ck = false;
-                    clean = 0;
                     if (C.resume) {
                         P::load(ep, e, Z0);
                         t = ep.t[e];
@@ -336,7 +292,7 @@ __device__ __forceinline__ void track_body(const Src &src, const XYCtl &C, const
                         newton = ep.newton[e];
                         need_k1 = true;
                     } else {
-                        P::start(src.sys(g), ep.path[e], Z0, K1);
+                        P::start(S, ep.path[e], Z0, K1);
                         t = 0.0;
                         h = C.h0;
                         steps = C.accumulate ? ep.steps[e] : 0;
@@ -344,9 +300,6 @@ __device__ __forceinline__ void track_body(const Src &src, const XYCtl &C, const
                         newton = C.accumulate ? ep.newton[e] : 0;
                         need_k1 = false;
                     }
-                    hacc = h;
-                    tmark = 1.0 - t;
-                    since = 0;
                     far = false;
                     zlast = 0.0;
                 }
@@ -369,7 +322,6 @@ __device__ __forceinline__ void track_body(const Src &src, const XYCtl &C, const
         bool go = act && !need_k1;
         bool conv = false, bad = false;
         R zpn = R(0);
-        R kstep = R(0);   // the largest condition estimate of this attempt's solves
         const int ph0 = __any_sync(0xffffffffu, act && need_k1) ? 0 : 1;
         const int nph = 4 + C.max_newton;
 #pragma unroll 1
@@ -403,12 +355,10 @@ __device__ __forceinline__ void track_body(const Src &src, const XYCtl &C, const
                 }
             }
             const R tr = (R)te, omt = (R)(1.0 - te);
-            if (corr) P::residual(src.sys(g), ZC, tr, omt, W1, w);
-            R kest = R(0);
-            const bool oks = P::solve(src.sys(g), A, ZC, tr, omt, corr, W1, W1, AC, w, &kest);
+            if (corr) P::residual(S, ZC, tr, omt, W1, w);
+            const bool oks = P::solve(S, A, ZC, tr, omt, corr, W1, W1, AC, w);
             if (!w) continue;
             solves++;
-            kstep = fmax(kstep, kest);
             if (ph == 0) {
                 // z0 += Newton correction at t; dz/dt from the second right-hand side
 #pragma unroll 6
@@ -418,7 +368,7 @@ __device__ __forceinline__ void track_body(const Src &src, const XYCtl &C, const
                 }
                 newton++;
                 need_k1 = false;
-                if (!oks) status = C.handoff ? NPHC_PATH_HANDOFF : NPHC_PATH_NONFINITE;
+                if (!oks) status = NPHC_PATH_NONFINITE;
             } else if (!corr) {
                 bad = bad || !oks;
                 if (ph == 1) {
@@ -459,19 +409,6 @@ __device__ __forceinline__ void track_body(const Src &src, const XYCtl &C, const
         }
         go = go && status == NPHC_PATH_RUNNING;
 
-        // ---- FP32 pass: a converged step whose Schur systems' condition estimate exceeds
-        // kappa (kappa = 0 outside the FP32 pass) is not taken; FP64 continues the path from
-        // its last accepted point (or the end zone's clean checkpoint), where the estimate
-        // was below kappa: the FP32 solve's relative error grows like the condition number
-        // times 6e-8, and a step across an ill-conditioned stretch (two paths passing
-        // close) can land on the neighbouring path.  A step that did not converge lands
-        // nowhere: it is rejected and halved as usual, whatever its estimate (a poor
-        // prediction far off the path can see a large one)
-        if (go && conv && C.kappa > 0.0 && !((double)kstep <= C.kappa)) {
-            status = NPHC_PATH_HANDOFF_COND;
-            go = false;
-        }
-
         // ---- accept or reject
         if (go) {
             attempts++;
@@ -482,79 +419,27 @@ __device__ __forceinline__ void track_body(const Src &src, const XYCtl &C, const
                     K1.set(k, AC.get(k));
                 }
                 const R zi = P::norminf(ZC);
-                clean = rejects == 0 ? clean + 1 : 1;
                 t = t1;
                 far = 1.0 - t < CRAWL_ZONE && (double)zi > FAR_NORM && (double)zi > FAR_GROWTH * zlast;
                 zlast = (double)zi;
                 steps++;
-                rejects = 0;
-                hacc = h;
                 if (++run >= C.grow_after) {
                     run = 0;
                     h = fmin(2.0 * h, C.hmax);
                 }
-                if ((double)zi > C.rdiv)
-                    // An FP32 point is accurate to ~eps relative, so a crossing by more
-                    // than RDIV_BAND is one in FP64 too; FP32 leaves only the marginal
-                    // crossings close to t = 1 to FP64
-                    status = (C.handoff && 1.0 - t < NEAR_END &&
-                              (double)zi <= C.rdiv * (1.0 + RDIV_BAND))
-                                 ? NPHC_PATH_HANDOFF
-                                 : NPHC_PATH_DIVERGED;
-                else if (t >= C.t_end)
-                    status = NPHC_PATH_REACHED;
-                // FP32 pass: in the end zone keep the last clean point (accepted, with the
-                // step before it accepted too); a path that the pass later hands off
-                // resumes in FP64 from there, not from the point where FP32 precision ran
-                // out, which can sit off the path.  A converged FP32 point in light-cone
-                // coordinates is on its path to the corrector's tolerance; in (x, y) the
-                // small light-cone coordinate of a far point was lost to cancellation, so
-                // such points could look converged while off the path, and the checkpoint
-                // then had to stay at the end zone's entry.
-                if (C.handoff && (clean >= 2 || !have_ck) && status == NPHC_PATH_RUNNING &&
-                    1.0 - t < CRAWL_ZONE) {
-#pragma unroll 6
-                    for (int k = 0; k < NV; k++) CK.set(k, Z0.get(k));
-                    tck = t;
-                    hck = hacc;
-                    have_ck = true;
-                }
-                // crawl test near t = 1: 1 - t must at least halve every CRAWL_STEPS
-                // accepted steps (paths to nonsingular endpoints finish in a few steps;
-                // a crawl means a singular endpoint, infinity, or precision exhausted)
-                if (status == NPHC_PATH_RUNNING && C.crawl_steps > 0 && 1.0 - t < CRAWL_ZONE) {
-                    if (++since >= C.crawl_steps) {
-                        if (1.0 - t > 0.5 * tmark)
-                            status = C.handoff ? NPHC_PATH_HANDOFF : NPHC_PATH_MIN_STEP;
-                        tmark = 1.0 - t;
-                        since = 0;
-                    }
-                } else {
-                    tmark = 1.0 - t;
-                    since = 0;
-                }
+                if ((double)zi > C.rdiv) status = NPHC_PATH_DIVERGED;
+                else if (t >= C.t_end) status = NPHC_PATH_REACHED;
             } else {
                 run = 0;
-                rejects++;
                 h *= 0.5;
-                if (h < C.hmin)
-                    status = C.handoff ? NPHC_PATH_HANDOFF : NPHC_PATH_MIN_STEP;
-                else if (C.handoff && rejects >= 10)
-                    status = NPHC_PATH_HANDOFF;
+                if (h < C.hmin) status = NPHC_PATH_MIN_STEP;
             }
-            if (status == NPHC_PATH_RUNNING && attempts >= C.max_steps)
-                status = C.handoff ? NPHC_PATH_HANDOFF : NPHC_PATH_STEP_BUDGET;
+            if (status == NPHC_PATH_RUNNING && attempts >= C.max_steps) status = NPHC_PATH_STEP_BUDGET;
         }
         if (act && status != NPHC_PATH_RUNNING) {
-            const EPView &ep = src.eps(g);
-            const bool handed = status == NPHC_PATH_HANDOFF || status == NPHC_PATH_HANDOFF_COND;
-            const bool from_ck = handed && have_ck;
-            if (from_ck)
-                P::store(ep, e, CK);
-            else
-                P::store(ep, e, Z0);
-            ep.t[e] = from_ck ? tck : t;
-            ep.h[e] = from_ck ? hck : (handed ? hacc : h);
+            P::store(ep, e, Z0);
+            ep.t[e] = t;
+            ep.h[e] = h;
             ep.status[e] = status;
             ep.steps[e] = steps;
             ep.solves[e] = solves;
@@ -564,19 +449,9 @@ __device__ __forceinline__ void track_body(const Src &src, const XYCtl &C, const
     }
 }
 
-template <int M, class R, int BLOCK>
+template <int M, int BLOCK>
 __global__ void __launch_bounds__(BLOCK)
     xy_track_kernel(const __grid_constant__ XYSys S, const __grid_constant__ XYCtl C,
                     const EPView ep, const WorkList wl) {
-    track_body<XYProblem<M, R, BLOCK>>(SingleSrc<XYSys>{S, ep, wl}, C, wl);
-}
-
-// The FP32 pass of a batch: every path of every instance of one ring size in one
-// persistent launch, pulled from one queue (BatchSrc).
-template <int M, class R, int BLOCK>
-__global__ void __launch_bounds__(BLOCK)
-    xy_track_batch_kernel(const XYSys *__restrict__ sys, const EPView *__restrict__ eps,
-                          const int64_t *__restrict__ off, int n,
-                          const __grid_constant__ XYCtl C, const WorkList wl) {
-    track_body<XYProblem<M, R, BLOCK>>(BatchSrc<XYSys>{sys, eps, off, n}, C, wl);
+    track_body<XYProblem<M, BLOCK>>(S, C, ep, wl);
 }
