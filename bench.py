@@ -123,8 +123,8 @@ class ClockSampler:
 
 
 def solve_flops(M: int, corrector: bool) -> tuple[float, float]:
-    """FP32 flops of one structured solve of the per-thread tracker as implemented
-    (xy_solve.cuh, light-cone coordinates), as (method, overhead).  method: the Schur
+    """FP32 flops of one structured solve of the XY ring's trackers (xy_solve.cuh, light-cone
+    coordinates), as (method, overhead).  method: the Schur
     build (couplings sums, -H_t rows, frames, M x M entries and right-hand sides), the
     LU factorisation with partial pivoting, back substitution and recovery; a corrector
     solve adds the second
@@ -153,7 +153,7 @@ def solve_flops(M: int, corrector: bool) -> tuple[float, float]:
 def kernel_source_sha() -> str:
     h = hashlib.sha256()
     d = os.path.join(ROOT, "paper_1104_5497_gb300", "csrc")
-    for f in ("xy_solve.cuh", "xy_track.cuh", "nphc_internal.cuh"):
+    for f in ("xy_track_lane.cuh", "f32_step.cuh", "nphc_internal.cuh"):
         h.update(open(os.path.join(d, f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -506,7 +506,7 @@ def run_mine(args):
                         "untuned_value": (replica_value(P, world, e2e_untuned)
                                           if e2e_untuned else None)},
                 "untuned_ms_per_step": ms_untuned,
-                "roofline": {"bound": "alu", "kernel": "xy_track_kernel<9,float> (FP32 tracker)",
+                "roofline": {"bound": "alu", "kernel": "xy_track_lane_kernel<9> (FP32 tracker)",
                              "achieved": achieved, "peak": p32["tflops"], "unit": "TFLOP/s",
                              "frac": achieved / p32["tflops"],
                              "peak_note": "measured in this run: FP32 FMA microbenchmark (csrc/alu_peak.cu), "

@@ -109,8 +109,8 @@ typedef struct nphc_options {
     int grow_after;            /* consecutive accepted steps before h doubles, 3 */
     int refine_iters;          /* Newton refinement steps at t = 1, 8 */
     double refine_eps;         /* refinement stops when ||dz|| <= eps (1 + ||z||), 1e-14 */
-    int block_size;            /* threads per block of the FP32 tracker; 0 = automatic */
-    int blocks_per_sm;         /* resident blocks per SM of the FP32 tracker; 0 = automatic */
+    int block_size;            /* kept for callers; the FP32 trackers' blocks are fixed */
+    int blocks_per_sm;         /* resident warps per SM of the FP32 tracker; 0 = automatic */
     /* Cauchy endgame (nphc_endgame) */
     int endgame;               /* nphc_solve_into runs the endgame on every path that ends
                                   NPHC_END_SINGULAR or NPHC_END_FAILED, 0 (off) */
@@ -130,8 +130,8 @@ typedef struct nphc_options {
                                   kappa_sing max(1, ||z||_inf^2), 1e12 */
     int threads_per_path;      /* FP64 tracking of lists (hand-offs, re-tracks): 32 = one path
                                   per warp (the path's solve shared over the lanes), 1 = one
-                                  path per thread (every lane a path); 0 = automatic (one path
-                                  per warp) */
+                                  path per thread (every lane a path); 0 = automatic (by the
+                                  list's length: one path per warp, or four lanes per path) */
     double kappa_fp32;         /* FP32 pass: a converged step whose solves' condition estimate
                                   exceeds this is not taken and FP64 continues the path
                                   (NPHC_PATH_HANDOFF_COND, see nphc_track); FP32 solves lose

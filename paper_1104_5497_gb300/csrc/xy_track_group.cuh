@@ -106,6 +106,9 @@ __device__ __forceinline__ bool grp_solve(float4 *__restrict__ sm, const GrpJ<M,
                                           GrpStep<GrpLayout<M>::SL> &dr, float &kest) {
     using L = GrpLayout<M>;
     constexpr int SL = L::SL, NP = L::NP, NPT = L::NPT;
+    // the sums over l unrolled where the kernel stays under 4,000 instructions (M <= 8: 256 paths of
+    // N = 5 0.84 -> 0.77 ms, 16,384 of N = 8 4.15 -> 4.0); at M = 9 (5,100) even three at a time cost 4%
+    constexpr int UL = M <= 8 ? M : 1, UP = M <= 8 ? M : 3;
     const float2 gm = f2(gam.re, gam.im), hgomt = f2scale(0.5f * omt, gm);
     const float hs = 0.5f * s;
     auto at = [&](int off, int i) -> float4 & { return sm[(off + i) * GRP_PATHS]; };
@@ -122,7 +125,7 @@ __device__ __forceinline__ bool grp_solve(float4 *__restrict__ sm, const GrpJ<M,
         ext2 up = {f2(J.val(q, M), 0.0f), f2dup(0.0f)}, uq = up;
         float2 rf = f2dup(0.0f), rg = rf;   // -H rows
         if (corr) {
-#pragma unroll 1
+#pragma unroll UL
             for (int l = 0; l < M; l++) {
                 const float4 v = at(L::PQ, l);
                 const float2 c = J.dup(q, l);
@@ -132,7 +135,7 @@ __device__ __forceinline__ bool grp_solve(float4 *__restrict__ sm, const GrpJ<M,
             f32_residual_rows(f2(z.x, z.y), f2(z.z, z.w), up, uq, s, hs, __fmul_rn(omt, gam.re),
                               __fmul_rn(omt, gam.im), rf, rg);
         } else {
-#pragma unroll 3
+#pragma unroll UP
             for (int l = 0; l < M; l++) {
                 const float4 v = at(L::PQ, l);
                 const float2 c = J.dup(q, l);
@@ -205,7 +208,7 @@ __device__ __forceinline__ bool grp_solve(float4 *__restrict__ sm, const GrpJ<M,
 #pragma unroll
         for (int q = 0; q < SL; q++) sx[q] = sy[q] = rx[q] = ry[q] = f2dup(0.0f);
         if (corr) {
-#pragma unroll 1
+#pragma unroll UL
             for (int j = 0; j < M; j++) {
                 const float4 v = at(L::XY, j), r = at(L::AC, j);
 #pragma unroll
@@ -218,7 +221,7 @@ __device__ __forceinline__ bool grp_solve(float4 *__restrict__ sm, const GrpJ<M,
                 }
             }
         } else {
-#pragma unroll 1
+#pragma unroll UL
             for (int j = 0; j < M; j++) {
                 const float4 v = at(L::XY, j);
 #pragma unroll
