@@ -47,20 +47,22 @@ cudaError_t NPHC_CAT(launch_xy_cauchy_m, NPHC_INST_M)(const XYSys &sys, const EG
 // (xy_track_group.cuh).  The first takes fewer instructions per path but one wave of it (19,000 to
 // 90,000 paths) takes its paths' latency however few they are; four lanes shorten every solve
 // and sixteen warps per SM hide each other's latency where four to ten cannot, at the price of
-// the rows that pad M to a multiple of four.  Measured (GB300, FP32 pass alone, group / lane, ms):
-//   no padding    N = 13 80,000 paths (4.1 waves of lanes) 58.1 / 65.6, 262,144 (13.5) 183.7 / 185.6;
-//                 N = 9 65,536 (1.5) 13.8 / 16.8, batches of 262,144 (6) 74 / 74, 524,288 (12) 225 / 188
-//   one row       N = 12 32,768 (1.3) 24.3 / 27.8, 65,536 (2.7) 43.0 / 41.1, 262,144 (11) 154 / 133;
-//                 N = 8 batches of 65,536 (1.2) 19.5 / 20.1, 262,144 (4.9) 86 / 80
-//   two rows      N = 11 32,768 (1.1) 18.7 / 20.6, 49,152 (1.7) 25.7 / 26.4, 65,536 (2.2) 33.2 / 30.0,
-//                 262,144 (9) 118 / 93
-//   three rows    N = 10 16,384 (0.5) 9.0 / 13.5, 24,576 (0.7) 14.0 / 13.6, 32,768 (1.0) 16.4 / 13.8,
-//                 262,144 (7.7) 106 / 73
-// So lanes from that many quarter waves on, by the number of padding rows:
+// the rows that pad M to a multiple of four.  Measured (GB300, FP32 pass alone or the whole batch,
+// group / lane, ms; in brackets the waves of lanes):
+//   no padding    N = 9 65,536 (1.5) 12.5 / 16.9, batches of 262,144 (6) 62 / 67, 524,288 (12) 184 / 168;
+//                 N = 13 262,144 (13.5) 126 / 186
+//   one row       N = 8 batches of 65,536 (1.2) 17.4 / 18.8, 196,608 (3.7) 61.4 / 59.6, 393,216 (7.3)
+//                 123 / 119; N = 12 262,144 (11) 114 / 133
+//   two rows      N = 7 batch of 163,840 (2.4) 46.1 / 47.5; N = 11 65,536 (2.2) 26.7 / 29.9, 131,072 (4.5)
+//                 49.6 / 50.6, 262,144 (9) 95.3 / 93.3
+//   three rows    N = 10 20,000 (0.6) 10.5 / 13.7, 32,768 (1.0) 14.2 / 14.0, 65,536 (1.9) 25.1 / 22.8,
+//                 262,144 (7.7) 96 / 73; N = 6 batch of 131,072 (1.9) 76.5 / 74.4
+// So lanes from that many waves on, by the number of padding rows, and never at M >= 11 (five
+// and four warps per SM).
 template <int M>
 static bool use_group(int64_t items, int64_t wave) {
-    constexpr int quarters[4] = {32, 11, 8, 3};
-    return 4 * items < quarters[GrpLayout<M>::ROWS - M] * wave;
+    constexpr int waves[4] = {8, 4, 6, 1};
+    return M >= 11 || items < waves[GrpLayout<M>::ROWS - M] * wave;
 }
 
 static cudaError_t device_sms(int &sms) {

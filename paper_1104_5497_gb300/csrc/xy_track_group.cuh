@@ -18,8 +18,8 @@
 //     (T on even lanes, R on odd ones).  No rows are swapped.
 //   * Arithmetic in pairs (fma.rn.f32x2): (re, im) where the coefficient is real or a
 //     compensated sum runs, two neighbouring columns where both factors are complex.
-//   * Each path is in its own phase (an RK4 stage or a corrector iteration); a warp runs, for
-//     all paths that wait for one, whichever of a predictor and a corrector solve has more
+//   * Each path is in its own phase (an RK4 stage or a corrector iteration); a warp, or with
+//     full warps the block, runs, for all paths that wait for one, whichever of a predictor and a corrector solve has more
 //     takers (a corrector solve costs about twice as much, so it needs half as many).  In
 //     lockstep a warp runs the correctors its slowest path needs (1.7 per step on average,
 //     three at worst).  A path's own sequence of operations does not depend on its company.
@@ -424,6 +424,13 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
         const int64_t want = (total + warps - 1) / warps;
         if (want < per) per = want < 1 ? 1 : (int)want;
     }
+    // With full warps the block decides which solve runs, so that its four warps go through the same
+    // code at the same time: sixteen warps in sixteen places of a kernel of 60 to 90 KB waited for
+    // instructions two cycles per issue.  The pool of 32 paths fills the phases as well as
+    // eight do (85% in a simulation of the mix).  N = 13 80,000 paths 58 -> 41 ms, N = 12 32,768
+    // 24.4 -> 18.6, N = 11 19.1 -> 15.8, N = 9 65,536 13.7 -> 12.7.  With fewer paths no path waits for
+    // the others of its block.
+    const bool together = per == GRP_PATHS;
     const F32Ctl K(C);
     int64_t e = pth < per ? -1 : -2;   // entry of this path slot; -1 idle, -2 drained
     int inst = 0;                      // instance of the entry (batches)
@@ -517,7 +524,8 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
                 }
             }
         }
-        if (__all_sync(0xffffffffu, e < 0)) break;
+        const bool any = __any_sync(0xffffffffu, e >= 0);
+        if (!together && !any) break;
 
         // ---- a new attempt: its first stage's point z0 + h/2 k1
         const bool act = e >= 0;
@@ -540,10 +548,18 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
 
         // ---- which solve runs now, and for whom
         const bool wants_c = act && (ph == 0 || ph >= 4);
-        const int nc = __popc(__ballot_sync(0xffffffffu, wants_c));
-        const int np = __popc(__ballot_sync(0xffffffffu, act && !wants_c));
+        int nc, np;
+        if (together) {
+            nc = __syncthreads_count(wants_c);
+            np = __syncthreads_count(act && !wants_c);
+            if (nc + np == 0) break;
+        } else {
+            nc = __popc(__ballot_sync(0xffffffffu, wants_c));
+            np = __popc(__ballot_sync(0xffffffffu, act && !wants_c));
+        }
         const bool corr = nc > 0 && 2 * nc >= np;
         const bool w = act && wants_c == corr;
+        if (together && !__any_sync(0xffffffffu, w)) continue;
         const f32_time te = ph == 0 ? P.t : ph < 3 ? P.t + hh / 2 : t1;
         int verdict = STEP_GO_ON, status = NPHC_PATH_RUNNING;
         float zi = 0.0f;

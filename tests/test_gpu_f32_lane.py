@@ -28,8 +28,9 @@ def endpoints(N_, system, gamma, paths):
     return (ep.tensors["z_re"] + 1j * ep.tensors["z_im"]).cpu().numpy().T, ep.tensors["cls"].cpu().numpy()
 
 
-# odd and even M, with and without a column of its own for the second right-hand side
-@pytest.mark.parametrize("N,count", [(10, 40001), (11, 70001), (12, 80001), (13, 180001)])
+# odd and even M, with and without a column of its own for the second right-hand side; the larger
+# rings: blocks of the four-lane kernel that decide together against warps that decide alone
+@pytest.mark.parametrize("N,count", [(10, 40001), (11, 70001), (11, 190001), (12, 80001), (13, 180001)])
 def test_many_paths_match_few(N, count):
     N_ = nphc()
     g = I.draw_pair_normals(np.random.default_rng(60 + N), N)
