@@ -58,11 +58,12 @@ cudaError_t NPHC_CAT(launch_xy_cauchy_m, NPHC_INST_M)(const XYSys &sys, const EG
 //   three rows    N = 10 20,000 (0.6) 10.5 / 13.7, 32,768 (1.0) 14.2 / 14.0, 65,536 (1.9) 25.1 / 22.8,
 //                 262,144 (7.7) 96 / 73; N = 6 batch of 131,072 (1.9) 76.5 / 74.4
 // So lanes from that many waves on, by the number of padding rows, and never at M >= 11 (five
-// and four warps per SM).
+// and four warps per SM): LANE_MAX_M.
+constexpr int LANE_MAX_M = 10;
 template <int M>
 static bool use_group(int64_t items, int64_t wave) {
     constexpr int waves[4] = {8, 4, 6, 1};
-    return M >= 11 || items < waves[GrpLayout<M>::ROWS - M] * wave;
+    return M > LANE_MAX_M || items < waves[GrpLayout<M>::ROWS - M] * wave;
 }
 
 static cudaError_t device_sms(int &sms) {
@@ -86,6 +87,31 @@ static cudaError_t kernel_blocks(K k, int threads, size_t smem, bool &attr, int 
     return e;
 }
 
+// The per-thread kernel where it exists: resident blocks per SM, and the launches.
+template <int M, bool BATCH>
+static cudaError_t lane_blocks(int &per) {
+    per = 0;
+    if constexpr (M <= LANE_MAX_M) {
+        static bool attr = false;
+        const size_t smem = lane_smem_per_block<M>(BATCH);
+        if constexpr (BATCH) return kernel_blocks(xy_track_lane_batch_kernel<M>, NPHC_TRACK_BLOCK, smem, attr, per);
+        else return kernel_blocks(xy_track_lane_kernel<M>, NPHC_TRACK_BLOCK, smem, attr, per);
+    }
+    return cudaSuccess;
+}
+template <int M>
+static void launch_lanes(int grid, const XYSys &sys, const XYCtl &ctl, const EPView &ep, const WorkList &wl,
+                         cudaStream_t st) {
+    if constexpr (M <= LANE_MAX_M)
+        xy_track_lane_kernel<M><<<grid, NPHC_TRACK_BLOCK, lane_smem_per_block<M>(false), st>>>(sys, ctl, ep, wl);
+}
+template <int M>
+static void launch_lanes_batch(int grid, const BatchGroup &bg, const XYCtl &ctl, const WorkList &wl, cudaStream_t st) {
+    if constexpr (M <= LANE_MAX_M)
+        xy_track_lane_batch_kernel<M><<<grid, NPHC_TRACK_BLOCK, lane_smem_per_block<M>(true), st>>>(
+            bg.sys, bg.ep, bg.off, bg.n, ctl, wl);
+}
+
 // Grid of a group launch over `items` paths: every SM filled (or with `warps` warps in all, if
 // given), but no more blocks than the paths need at one warp per scheduler first and eight
 // paths per warp then.
@@ -103,13 +129,12 @@ cudaError_t NPHC_CAT(launch_xy_track_f32_m, NPHC_INST_M)(const XYSys &sys, const
                                                          const EPView &ep, const WorkList &wl,
                                                          int grid, cudaStream_t st) {
     constexpr int M = NPHC_INST_M, BLK = NPHC_TRACK_BLOCK;
-    static bool attr_t = false, attr_g = false;
-    const size_t smem_t = lane_smem_per_block<M>(false), smem_g = grp_smem_per_block<M>(false);
-    auto kt = xy_track_lane_kernel<M>;
+    static bool attr_g = false;
+    const size_t smem_g = grp_smem_per_block<M>(false);
     auto kg = xy_track_group_kernel<M>;
     int sms = 0, per_t = 0, per_g = 0;
     cudaError_t e = device_sms(sms);
-    if (e == cudaSuccess) e = kernel_blocks(kt, BLK, smem_t, attr_t, per_t);
+    if (e == cudaSuccess) e = lane_blocks<M, false>(per_t);
     if (e == cudaSuccess) e = kernel_blocks(kg, 32 * GRP_WARPS, smem_g, attr_g, per_g);
     if (e != cudaSuccess) return e;
     if (use_group<M>(ep.count, (int64_t)sms * per_t * BLK)) {
@@ -121,7 +146,7 @@ cudaError_t NPHC_CAT(launch_xy_track_f32_m, NPHC_INST_M)(const XYSys &sys, const
         if (grid <= 0 || grid > full) grid = full;
         grid = std::min(grid, (int)(wl.state_threads / BLK));   // the scratch holds state for this many
         if (grid <= 0) return cudaErrorInvalidValue;
-        kt<<<grid, BLK, smem_t, st>>>(sys, ctl, ep, wl);
+        launch_lanes<M>(grid, sys, ctl, ep, wl, st);
     }
     nphc_launch_counter(1);
     return cudaGetLastError();
@@ -135,13 +160,12 @@ cudaError_t NPHC_CAT(launch_xy_track_f32_batch_m, NPHC_INST_M)(const BatchGroup 
                                                                cudaStream_t st) {
     constexpr int M = NPHC_INST_M, BLK = NPHC_TRACK_BLOCK;
     if (bg.total <= 0) return cudaSuccess;
-    static bool attr_t = false, attr_g = false;
-    const size_t smem_t = lane_smem_per_block<M>(true), smem_g = grp_smem_per_block<M>(true);
-    auto kt = xy_track_lane_batch_kernel<M>;
+    static bool attr_g = false;
+    const size_t smem_g = grp_smem_per_block<M>(true);
     auto kg = xy_track_group_batch_kernel<M>;
     int sms = 0, per_t = 0, per_g = 0;
     cudaError_t e = device_sms(sms);
-    if (e == cudaSuccess) e = kernel_blocks(kt, BLK, smem_t, attr_t, per_t);
+    if (e == cudaSuccess) e = lane_blocks<M, true>(per_t);
     if (e == cudaSuccess) e = kernel_blocks(kg, 32 * GRP_WARPS, smem_g, attr_g, per_g);
     if (e != cudaSuccess) return e;
     if (use_group<M>(bg.total, (int64_t)sms * per_t * BLK)) {
@@ -155,7 +179,7 @@ cudaError_t NPHC_CAT(launch_xy_track_f32_batch_m, NPHC_INST_M)(const BatchGroup 
         if (grid > need) grid = (int)need;
         grid = std::min(grid, (int)(wl.state_threads / BLK));
         if (grid <= 0) return cudaErrorInvalidValue;
-        kt<<<grid, BLK, smem_t, st>>>(bg.sys, bg.ep, bg.off, bg.n, ctl, wl);
+        launch_lanes_batch<M>(grid, bg, ctl, wl, st);
     }
     nphc_launch_counter(1);
     return cudaGetLastError();

@@ -20,7 +20,7 @@
 // another 1,000 (everything unrolled) it waited a quarter of the time for instructions, 73 -> 90 ms.
 // Measured (GB300, 262,144 paths of N = 10): 109 ms for a lockstep kernel with a path per thread
 // and scalar arithmetic, 73 ms here (issue slots 32% used, the rest waits on shared memory and on
-// results); N = 11 154 -> 93, N = 12 209 -> 133.
+// results); N = 11 154 -> 93.  Up to M = 10 (xy_inst.cu).
 #pragma once
 
 #include "f32_step.cuh"
