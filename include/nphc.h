@@ -238,7 +238,11 @@ nphc_status nphc_workspace_size(const nphc_system *sys, int64_t count, size_t *b
  *          NPHC_PATH_HANDOFF, or NPHC_PATH_HANDOFF_COND when a converged step's condition
  *          estimate (max |U_kk| / min |U_kk| of the pivoted LU factor of the step's Schur
  *          system) exceeded opt->kappa_fp32, and its (z, t, h) for an FP64 call with
- *          resume = 1.
+ *          resume = 1.  Which FP32 kernel runs is chosen by the number of paths, and the
+ *          kernels round differently.  A path that reaches a far endpoint, whose class
+ *          would depend on that, is tracked again by one kernel for all (its steps and
+ *          solves count both passes).  Far: some |Re z_i| or |Im z_i| of at least
+ *          2^floor(log2(0.01 / sqrt(opt->refine_eps))), 65,536 by default.
  * list (device int32, may be NULL) selects entries list[0 .. *list_count - 1]
  * (list_count: device int32); NULL tracks every entry.  resume = 0 starts each selected
  * path at its start point; resume = 1 continues from ep's (z, t, h).  Writes z, t, h,
@@ -256,7 +260,9 @@ nphc_status nphc_track(const nphc_system *sys, const nphc_options *opt, nphc_pre
  * same test passes at Re z, otherwise non-real when ||Im z|| > 2 beta, else undecided.
  * The certificate is taken at the iterate whose Newton correction met the refinement
  * tolerance, from that iteration's own factorisation (beta = the correction's norm); z is
- * its Newton iterate, closer still to the same zero.  Writes z
+ * its Newton iterate, closer still to the same zero.  (At a far endpoint, see nphc_track, the
+ * tolerance is no longer small against the certificate's bound: whether such a solution
+ * certifies depends on the bits of z.)  Writes z
  * (refined), cls, alpha, beta, gamma, resid.  Other statuses get NPHC_END_NONE
  * (diverged) or NPHC_END_FAILED.  list / list_count as in nphc_track. */
 nphc_status nphc_refine_certify(const nphc_system *sys, const nphc_options *opt,

@@ -61,10 +61,11 @@ int64_t table_size_for(int64_t count) {
 }
 
 // Device scratch: [queue counters | tracker path state | dedup cell keys | cell list
-// heads | list links | flags].  The tracker state holds four vectors of n complex
-// doubles for each of NPHC_TRACK_MAX_THREADS threads (enough for either precision).
+// heads | list links | flags | far endpoints' count and list].  The tracker state holds four
+// vectors of n complex doubles for each of NPHC_TRACK_MAX_THREADS threads (enough for either
+// precision).
 struct WsLayout {
-    size_t queue, state, keys, head, next, inlist, total;
+    size_t queue, state, keys, head, next, inlist, far, total;
     int64_t tsize;
 };
 
@@ -78,6 +79,7 @@ WsLayout ws_layout(int n, int64_t count) {
     L.head = o;   o += align256(sizeof(int32_t) * L.tsize * DD_LEVELS);
     L.next = o;   o += align256(sizeof(int32_t) * count * DD_LEVELS);
     L.inlist = o; o += align256(sizeof(int32_t) * count);
+    L.far = o;    o += align256(sizeof(int32_t) * (count + 1));
     L.total = o;
     return L;
 }
@@ -91,6 +93,19 @@ DedupScratch dedup_scratch(void *ws, const WsLayout &L) {
     w.next = reinterpret_cast<int32_t *>(b + L.next);
     w.inlist = reinterpret_cast<int32_t *>(b + L.inlist);
     return w;
+}
+
+constexpr int kFarQueue = 5;   // queue slot of the far endpoints' pass
+
+// What an FP32 pass counts with: its own queue, the far endpoints' queue and their number.
+FillSet fp32_counters(void *ws, int n, int64_t count, int queue_slot) {
+    char *b = static_cast<char *>(ws);
+    const WsLayout L = ws_layout(n, count);
+    FillSet f;
+    f.add(b + L.queue + sizeof(unsigned long long) * queue_slot, sizeof(unsigned long long), 0);
+    f.add(b + L.queue + sizeof(unsigned long long) * kFarQueue, sizeof(unsigned long long), 0);
+    f.add(b + L.far, sizeof(int32_t), 0);
+    return f;
 }
 
 // k with s < 2^k for a rounded sum s >= 0 of non-negative numbers
@@ -515,6 +530,32 @@ EPView view(const nphc_endpoints *e) {
 // 20 ms by warps and 29 by groups (13.5 by warps now).
 constexpr int64_t kFewPerScheduler = 10, kFewListedPerScheduler = 32;
 
+// The far endpoints of an FP32 pass, tracked again by the per-thread kernel (a path's result then
+// never depends on the kernel that the launch's size chose).  The pass cleared queue slot 5 and
+// the count.
+nphc_status far_pass(const nphc_system *S, const nphc_options *o, const EPView &v, const int32_t *list,
+                     const int32_t *list_count, void *ws, cudaStream_t st) {
+    const WsLayout L = ws_layout(S->n, v.count);
+    int32_t *const far = reinterpret_cast<int32_t *>(static_cast<char *>(ws) + L.far);
+    const WorkList from = {list, list_count, nullptr, nullptr, 0};
+    NPHC_CK(launch_far_list(v, S->n, from, far_exponent(o->refine_eps), far + 1, far, st));
+    XYCtl ctl = make_ctl(o, true, false, true);   // the pass's steps and solves count too
+    ctl.sparse = 1;
+    WorkList wl;
+    wl.list = far + 1;
+    wl.list_count = far;
+    wl.queue = ws_queue(ws, kFarQueue);
+    wl.state = static_cast<char *>(ws) + L.state;
+    wl.state_threads = NPHC_TRACK_MAX_THREADS;
+    // one warp per scheduler: a hundred paths, each a chain of dependent solves
+    int dev = 0, sms = 0;
+    NPHC_CK(cudaGetDevice(&dev));
+    NPHC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    NPHC_CK(launch_xy_track_f32_thread(S->M, sys_with_gamma(S, o), ctl, v, wl,
+                                       (int)std::min<int64_t>(4 * sms, v.count), st));
+    return NPHC_OK;
+}
+
 nphc_status track_impl(const nphc_system *S, const nphc_options *o, nphc_precision prec,
                        const nphc_endpoints *ep, const int32_t *list, const int32_t *list_count,
                        bool resume, bool accumulate, void *ws, int queue_slot, cudaStream_t st,
@@ -532,15 +573,21 @@ nphc_status track_impl(const nphc_system *S, const nphc_options *o, nphc_precisi
     wl.queue = ws_queue(ws, queue_slot);
     wl.state = static_cast<char *>(ws) + ws_layout(S->n, 0).state;
     wl.state_threads = NPHC_TRACK_MAX_THREADS;
-    NPHC_CK(cudaMemsetAsync(wl.queue, 0, sizeof(unsigned long long), st));
     int dev = 0, sms = 0;
     NPHC_CK(cudaGetDevice(&dev));
     NPHC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const EPView v = view(ep);
+    if (f32 && !resume && ep->count > 0) {
+        NPHC_CK(launch_fill(fp32_counters(ws, S->n, ep->count, queue_slot), st));
+        NPHC_CK(launch_xy_track_f32(S->M, xs, ctl, v, wl, 0, sms * o->blocks_per_sm, st));
+        return far_pass(S, o, v, list, list_count, ws, st);
+    }
+    NPHC_CK(cudaMemsetAsync(wl.queue, 0, sizeof(unsigned long long), st));
     if (S->quad) {
         NPHC_CK(launch_quad_track(S->n, quad_with_gamma(S, o), ctl, v, wl, st));
     } else if (f32) {
-        NPHC_CK(launch_xy_track_f32(S->M, xs, ctl, v, wl, 0, sms * o->blocks_per_sm, st));
+        // a resumed pass cannot be run again from its points: the per-thread kernel tracks all of it
+        NPHC_CK(launch_xy_track_f32_thread(S->M, xs, ctl, v, wl, sms * o->blocks_per_sm, st));
     } else if (list != nullptr && o->threads_per_path == 1) {   // one path per thread, full warps
         NPHC_CK(launch_xy_track_f64(S->M, xs, ctl, v, wl, 0, 0, st));
     } else if (list != nullptr && o->threads_per_path == 32) {
@@ -898,6 +945,10 @@ nphc_status solve_into_impl(const nphc_system *S, const nphc_options *o, nphc_re
             const Range r("fp32 pass");
             if ((s = track_impl(S, o, NPHC_PREC_MIXED, ep, nullptr, nullptr, false, false, R->ws, 0, st)))
                 return s;
+        } else {
+            const Range r("far endpoints of the group's fp32 pass");
+            NPHC_CK(launch_fill(fp32_counters(R->ws, R->n, R->P, kFarQueue), st));
+            if ((s = far_pass(S, o, v, nullptr, nullptr, R->ws, st))) return s;
         }
         Range r_tail("fp64 hand-offs, refinement, certification");
         // hand-offs: refinement at t = 1 straight from the hand-off point (certified ones

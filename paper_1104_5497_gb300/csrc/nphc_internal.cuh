@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+
 #include "nphc.h"
 
 #define NPHC_MAXN NPHC_MAX_N          // couplings are stored in NPHC_MAXN rows of
@@ -153,6 +155,16 @@ __device__ __forceinline__ ext<double> grid_sub(ext<double> a, ext<double> b) {
     return ext<double>{__dsub_rn(a.hi, b.hi), __dsub_rn(a.lo, b.lo)};
 }
 
+// A far endpoint: some |Re z_i| or |Im z_i| >= 2^far_exponent.  alpha at the refinement's tolerance is
+// gamma refine_eps ||z||, and gamma is 5 to 20 ||z|| on the rings looked at, so within this line
+// (65,536 at the default refine_eps of 1e-14) an endpoint's alpha stays a hundred times below the
+// certificate's bound whichever way the last correction is rounded.  Beyond it the class depends on
+// the rounding of the FP32 pass and of the refinement (xy_track.cuh, xy_refine_far.cuh); the nearest
+// endpoint seen to change its class was at 5e5.
+inline int far_exponent(double refine_eps) {
+    return refine_eps > 0.0 ? std::ilogb(0.01 / std::sqrt(refine_eps)) : 2000;   // 2000: never
+}
+
 // ------------------------------------------------------ launch arguments --
 // Couplings and homotopy constants of one XY ring, passed by value so that the
 // unrolled kernels read them as constant-bank operands.
@@ -284,6 +296,9 @@ cudaError_t launch_xy_track_f32(int M, const XYSys &sys, const XYCtl &ctl, const
                                 const WorkList &wl, int block, int grid, cudaStream_t st);
 cudaError_t launch_xy_track_f64(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
                                 const WorkList &wl, int block, int grid, cudaStream_t st);
+// FP32 tracking by the per-thread kernel (xy_track.cuh): far endpoints, resumed passes.
+cudaError_t launch_xy_track_f32_thread(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
+                                       const WorkList &wl, int grid, cudaStream_t st);
 // The FP32 pass over every path of a batch group (ring size M), one persistent launch.
 cudaError_t launch_xy_track_f32_batch(int M, const BatchGroup &bg, const XYCtl &ctl,
                                       const WorkList &wl, int grid, cudaStream_t st);

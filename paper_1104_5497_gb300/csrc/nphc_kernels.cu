@@ -64,6 +64,20 @@ __global__ void compact_kernel(const EPView ep, int pred, int32_t *flags, int32_
     }
 }
 
+__global__ void far_list_kernel(const EPView ep, int n, const WorkList wl, int far_exp, int32_t *list,
+                                int32_t *count) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= worklist_size(wl, ep.count)) return;
+    const int64_t e = worklist_entry(wl, i, ep.count);
+    if (e < 0 || ep.status[e] != NPHC_PATH_REACHED) return;
+    int ez = -2000;
+    for (int k = 0; k < n; k++) ez = max(ez, max(gexp(ep.z_re[k * ep.count + e]), gexp(ep.z_im[k * ep.count + e])));
+    if (ez < far_exp) return;
+    const int32_t k = atomicAdd(count, 1);
+    if (k < ep.count) list[k] = (int32_t)e;
+    else atomicSub(count, 1);   // a caller's list that names entries twice can overrun the room
+}
+
 // Marks the entries of a list re-tracked (used for the duplicate re-track).
 __global__ void flag_list_kernel(const int32_t *list, const int32_t *count, int32_t *flags,
                                  int32_t bit, int64_t cap) {
@@ -460,6 +474,14 @@ cudaError_t launch_compact(const EPView &ep, int pred, int32_t *flags, int32_t *
                            int32_t *count, cudaStream_t st) {
     if (ep.count == 0) return cudaSuccess;
     compact_kernel<<<blocks_for(ep.count, 256), 256, 0, st>>>(ep, pred, flags, list, count);
+    nphc_launch_counter(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_far_list(const EPView &ep, int n, const WorkList &wl, int far_exp, int32_t *list,
+                            int32_t *count, cudaStream_t st) {
+    if (ep.count == 0) return cudaSuccess;
+    far_list_kernel<<<blocks_for(ep.count, 128), 128, 0, st>>>(ep, n, wl, far_exp, list, count);
     nphc_launch_counter(1);
     return cudaGetLastError();
 }

@@ -50,6 +50,9 @@ cudaError_t nphc_debug_read(int *code);
 
 cudaError_t launch_compact(const EPView &ep, int pred, int32_t *flags, int32_t *list,
                            int32_t *count, cudaStream_t st);
+// The entries (of wl's list, or all) of n unknowns that reached t = 1 at a far endpoint.
+cudaError_t launch_far_list(const EPView &ep, int n, const WorkList &wl, int far_exp, int32_t *list,
+                            int32_t *count, cudaStream_t st);
 cudaError_t launch_flag_list(const int32_t *list, const int32_t *count, int64_t cap,
                              int32_t *flags, int32_t bit, cudaStream_t st);
 // Marks duplicates among the certified entries of ep.  mlist / mcount (device, may be

@@ -16,6 +16,13 @@ cudaError_t launch_xy_track_f32_batch(int M, const BatchGroup &bg, const XYCtl &
 #undef C
 }
 
+cudaError_t launch_xy_track_f32_thread(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
+                                       const WorkList &wl, int grid, cudaStream_t st) {
+#define C(MM) case MM: return launch_xy_track_f32t_m##MM(sys, ctl, ep, wl, grid, st);
+    switch (M) { NPHC_FOR_EACH_M(C) default: return cudaErrorInvalidValue; }
+#undef C
+}
+
 cudaError_t launch_xy_track_f64(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
                                 const WorkList &wl, int block, int grid, cudaStream_t st) {
     (void)block;

@@ -39,9 +39,47 @@ cudaError_t NPHC_CAT(launch_xy_cauchy_m, NPHC_INST_M)(const XYSys &sys, const EG
 }
 #endif
 
+#if NPHC_INST_KIND == 0 || NPHC_INST_KIND == 1
+#include "xy_track.cuh"
+
+// The per-thread tracker (xy_track.cuh) over the list or every entry of the launch.
+template <int M, class R>
+static cudaError_t launch_per_thread(const XYSys &sys, const XYCtl &ctl, const EPView &ep,
+                                     const WorkList &wl, int grid, cudaStream_t st) {
+    constexpr int BLK = NPHC_TRACK_BLOCK;
+    const size_t smem = xy_smem_per_thread<M, R>() * BLK;
+    auto k = xy_track_kernel<M, R, BLK>;
+    static bool attr_set = false;   // once per process for this instantiation
+    if (!attr_set) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
+    int dev = 0, sms = 0, per = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, BLK, smem);
+    if (e != cudaSuccess) return e;
+    const int full = sms * (per > 0 ? per : 1);   // persistent grid: every SM filled
+    if (grid <= 0 || grid > full) grid = full;
+    const int cap = (int)(wl.state_threads / BLK);  // the scratch holds state for this many
+    if (grid > cap) grid = cap;
+    if (grid <= 0) return cudaErrorInvalidValue;
+    k<<<grid, BLK, smem, st>>>(sys, ctl, ep, wl);
+    nphc_launch_counter(1);
+    return cudaGetLastError();
+}
+#endif
+
 #if NPHC_INST_KIND == 0
 #include "xy_track_group.cuh"
 #include "xy_track_lane.cuh"
+
+cudaError_t NPHC_CAT(launch_xy_track_f32t_m, NPHC_INST_M)(const XYSys &sys, const XYCtl &ctl,
+                                                          const EPView &ep, const WorkList &wl,
+                                                          int grid, cudaStream_t st) {
+    return launch_per_thread<NPHC_INST_M, float>(sys, ctl, ep, wl, grid, st);
+}
 
 // The FP32 pass has two kernels: one path per thread (xy_track_lane.cuh) and four lanes per path
 // (xy_track_group.cuh).  The first takes fewer instructions per path but one wave of it (19,000 to
@@ -253,28 +291,7 @@ cudaError_t NPHC_CAT(launch_xy_track_f64g_m, NPHC_INST_M)(const XYSys &sys, cons
 cudaError_t NPHC_CAT(launch_xy_track_f64_m, NPHC_INST_M)(const XYSys &sys, const XYCtl &ctl,
                                                          const EPView &ep, const WorkList &wl,
                                                          int grid, cudaStream_t st) {
-    constexpr int M = NPHC_INST_M, BLK = NPHC_TRACK_BLOCK;
-    const size_t smem = xy_smem_per_thread<M, double>() * BLK;
-    auto k = xy_track_kernel<M, BLK>;
-    static bool attr_set = false;   // once per process for this instantiation
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
-    int dev = 0, sms = 0, per = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, BLK, smem);
-    if (e != cudaSuccess) return e;
-    const int full = sms * (per > 0 ? per : 1);   // persistent grid: every SM filled
-    if (grid <= 0 || grid > full) grid = full;
-    const int cap = (int)(wl.state_threads / BLK);  // the scratch holds state for this many
-    if (grid > cap) grid = cap;
-    if (grid <= 0) return cudaErrorInvalidValue;
-    k<<<grid, BLK, smem, st>>>(sys, ctl, ep, wl);
-    nphc_launch_counter(1);
-    return cudaGetLastError();
+    return launch_per_thread<NPHC_INST_M, double>(sys, ctl, ep, wl, grid, st);
 }
 #endif
 
@@ -305,7 +322,8 @@ cudaError_t NPHC_CAT(launch_xy_refine_certify_m, NPHC_INST_M)(const XYSys &sys, 
     // and the entries are dealt out evenly), at most one entry per warp
     const int64_t full = (int64_t)sms * (per >= 8 ? 8 : per >= 4 ? 4 : per > 0 ? per : 1);
     const int grid = (int)(cap < full ? cap : full);
-    k<<<grid, 32, smem, st>>>(sys, tol_sol, refine_eps, refine_iters, ep, wl, shortcut);
+    k<<<grid, 32, smem, st>>>(sys, tol_sol, refine_eps, refine_iters, ep, wl, shortcut,
+                              far_exponent(refine_eps));
     nphc_launch_counter(1);
     return cudaGetLastError();
 }

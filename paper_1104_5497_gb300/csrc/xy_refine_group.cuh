@@ -21,10 +21,11 @@
 // An endpoint is in one of two states: it waits for an evaluation (P, the factorisation of DP
 // and the Newton correction at its point) or for a certificate from the factorisation just
 // made.  A warp runs evaluations while any of its endpoints waits for one, then the
-// certificates together; a finished slot takes the next entry.
+// certificates together; a finished slot takes the next entry.  Far endpoints are the whole warp's
+// (xy_refine_far.cuh), one at a time, as the slots come upon them.
 #pragma once
 
-#include "xy_endgame.cuh"
+#include "xy_refine_far.cuh"
 
 constexpr int RG_PATHS = 8;   // endpoints per warp (one warp per block)
 
@@ -40,13 +41,15 @@ struct RGLayout {
     static constexpr int U = QB + M;         // u_j
     static constexpr int W = U + M;          // w_j
     static constexpr int IV = W + M;         // (1 / |(a_j, b_j)|, -)
-    static constexpr int V = IV + M;         // a column per lane, 4 M
-    static constexpr int TOTAL = V + 4 * M;
+    static constexpr int V = IV + M;         // a column per lane, 4 M; of all endpoints together,
+    static constexpr int TOTAL = V + 4 * M;  // between certificates, the working set of a far one,
+    static constexpr int FAR = FarLayout<M>::TOTAL > RG_PATHS * 4 * M   // which takes so many more at M = 12
+                                   ? FarLayout<M>::TOTAL - RG_PATHS * 4 * M : 0;
 };
 
 template <int M>
 constexpr size_t rg_smem_per_block() {
-    return sizeof(cx<double>) * (size_t)(RG_PATHS * RGLayout<M>::TOTAL) +
+    return sizeof(cx<double>) * (size_t)(RG_PATHS * RGLayout<M>::TOTAL + RGLayout<M>::FAR) +
            sizeof(double) * (size_t)(M * (M + 2));   // J rows (the pinned column too), sums of squares
 }
 
@@ -313,11 +316,12 @@ __device__ void rg_norms(const RGPath<M> &G, unsigned long long perm, double &in
 template <int M>
 __global__ void __launch_bounds__(32)
     xy_refine_group_kernel(const __grid_constant__ XYSys S, double tol_sol, double refine_eps,
-                           int refine_iters, const EPView ep, const WorkList wl, int shortcut) {
+                           int refine_iters, const __grid_constant__ EPView ep, const WorkList wl,
+                           int shortcut, int far_exp) {
     using L = RGLayout<M>;
     extern __shared__ __align__(16) unsigned char rgraw[];
     cx<double> *const base = reinterpret_cast<cx<double> *>(rgraw);
-    double *const J = reinterpret_cast<double *>(base + RG_PATHS * L::TOTAL);
+    double *const J = reinterpret_cast<double *>(base + RG_PATHS * L::TOTAL + L::FAR);
     double *const jj = J + M * (M + 1);
     const int lane = threadIdx.x, g = lane >> 3, pth = lane & 7;
     for (int i = lane; i < M * (M + 1); i += 32) J[i] = S.Jd[(i / (M + 1)) * NPHC_JSTRIDE + i % (M + 1)];
@@ -338,7 +342,7 @@ __global__ void __launch_bounds__(32)
     if ((int)blockIdx.x >= warps) return;
     int64_t next = (int64_t)pth * warps + blockIdx.x;
     const int64_t stride = (int64_t)RG_PATHS * warps;
-    enum { IDLE, EVALUATE, CERTIFY, DONE };
+    enum { IDLE, EVALUATE, CERTIFY, FAR, DONE };
     enum { NEWTON, LAST, FINAL, REAL };   // what the evaluation is for: a Newton step, the one
                                           // whose correction met the tolerance, a certificate
                                           // without a step, the real test at Re z
@@ -366,6 +370,17 @@ __global__ void __launch_bounds__(32)
                 for (int k = g; k < 2 * M; k += 4)
                     G.at(L::Z, k) = cx<double>{ep.z_re[k * cnt + e], ep.z_im[k * cnt + e]};
                 state = EVALUATE;
+                if (!sc) {
+                    int ez = -2000;
+#pragma unroll 1
+                    for (int k = g; k < 2 * M; k += 4) {
+                        const cx<double> z = G.at(L::Z, k);
+                        ez = max(ez, max(gexp(z.re), gexp(z.im)));
+                    }
+                    ez = max(ez, __shfl_xor_sync(mine, ez, 8));
+                    ez = max(ez, __shfl_xor_sync(mine, ez, 16));
+                    if (ez >= far_exp) state = FAR;
+                }
                 it = 0;
                 mode = refine_iters > 0 ? NEWTON : FINAL;
             } else if (g == 0) {
@@ -374,6 +389,14 @@ __global__ void __launch_bounds__(32)
             }
         }
         __syncwarp();
+        unsigned fa = __ballot_sync(0xffffffffu, state == FAR) & 0xffu;   // slots with a far endpoint
+        if (fa) {
+            for (; fa; fa &= fa - 1)
+                far_refine<M>(base + RG_PATHS * L::V, J, S, tol_sol, refine_eps, refine_iters, ep,
+                              __shfl_sync(0xffffffffu, e, __ffs(fa) - 1));
+            if (state == FAR) state = IDLE;
+            continue;
+        }
         const unsigned ev = __ballot_sync(0xffffffffu, state == EVALUATE);
         const unsigned ce = __ballot_sync(0xffffffffu, state == CERTIFY);
         if (!ev && !ce) break;   // every slot is done

@@ -219,10 +219,14 @@ __device__ __forceinline__ bool aug_qr_solve(const SMat<M, R, BLOCK> &A, bool tw
 // conflict-free in the interleaved layout) and the rows below take a rank-one update,
 // a load, four FMAs and a store per complex entry, against Householder's extra dot
 // product per entry.  The pivot's reciprocal replaces U_kk for the back substitution.
+// kest (may be NULL) receives max_k |U_kk| / min_k |U_kk|, the usual cheap estimate of the
+// condition number from a pivoted factorisation.
 template <int M, class R, int BLOCK>
-__device__ __forceinline__ bool aug_lu_solve(const SMat<M, R, BLOCK> &A, bool two_rhs) {
+__device__ __forceinline__ bool aug_lu_solve(const SMat<M, R, BLOCK> &A, bool two_rhs,
+                                             R *kest = nullptr) {
     const int ncol = two_rhs ? M + 2 : M + 1;
     bool ok = true;
+    R umax = R(0), umin = R(0);
 #pragma unroll 1
     for (int k = 0; k < M; k++) {
         const int n = M - k;   // active rows k .. M-1, relative index i = 0 .. n-1
@@ -244,6 +248,9 @@ __device__ __forceinline__ bool aug_lu_solve(const SMat<M, R, BLOCK> &A, bool tw
             }
         }
         ok = ok && (best > R(0));
+        const R um = sqrt_r(best);
+        umax = fmax(umax, um);
+        umin = k == 0 ? um : fmin(umin, um);
         const cx<R> ip = crecip(piv);
         // multipliers of rows 1 .. n-1 after the swap (row p holds the old row k)
 #pragma unroll
@@ -295,6 +302,7 @@ __device__ __forceinline__ bool aug_lu_solve(const SMat<M, R, BLOCK> &A, bool tw
         }
     }
 
+    if (kest) *kest = umin > R(0) ? umax / umin : R(INFINITY);
     return ok;
 }
 
@@ -372,7 +380,8 @@ template <int M, class R, int BLOCK, class Out2>
 __device__ __forceinline__ bool xy_solve(const R *__restrict__ J, const SMat<M, R, BLOCK> &A,
                                          const SVec<R, BLOCK> &pt, R s, R omt, cx<R> gam,
                                          bool two_rhs, const SVec<R, BLOCK> &res,
-                                         const SVec<R, BLOCK> &out1, const Out2 &out2, bool wr) {
+                                         const SVec<R, BLOCK> &out1, const Out2 &out2, bool wr,
+                                         R *kest = nullptr) {
     const cx<R> gomt = cscale(omt, gam);
 
     cx<R> p[M], q[M];
@@ -441,7 +450,7 @@ __device__ __forceinline__ bool xy_solve(const R *__restrict__ J, const SMat<M, 
             A.set(k, M + 1, csub(A.get(k, M + 1), cmul_i(cscale(hs, csub(cmul(q[k], sx1[k]), cmul(p[k], sy1[k]))))));
     }
 
-    bool ok = aug_lu_solve<M, R, BLOCK>(A, two_rhs);
+    bool ok = aug_lu_solve<M, R, BLOCK>(A, two_rhs, kest);
 
     // ---- back to (dp, dq) = (sp dwp, sq dwq),
     // (dwp, dwq) = conj(a^, b^) q_j + (b^, -a^) s_j

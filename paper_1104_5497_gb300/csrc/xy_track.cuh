@@ -3,10 +3,19 @@
 // Q_i = z_i^2 - 1, start points z_i = +-1, tracked from t = 0 to t = 1 with a
 // predictor and Newton's corrector).
 //
-// This file: the method, what every tracker shares, and the FP64 tracker with one path per
-// thread, which lists take when asked to (options.threads_per_path = 1).  The others: one path
-// per thread or four lanes per path in FP32 (xy_track_lane.cuh, xy_track_group.cuh), four lanes
-// or a warp per path in FP64 (xy_track_group64.cuh, xy_track_warp.cuh).
+// This file: the method, what every tracker shares, and the tracker with one path per thread.
+// The others: one path per thread or four lanes per path in FP32, written for throughput
+// (xy_track_lane.cuh, xy_track_group.cuh), four lanes or a warp per path in FP64
+// (xy_track_group64.cuh, xy_track_warp.cuh).  This one runs
+//   * in FP64, on lists that ask for it (options.threads_per_path = 1);
+//   * in FP32, over the paths that a pass of the throughput kernels brought to a far endpoint
+//     (launch_far_list), and over resumed passes.  The certificate of a far endpoint is taken
+//     from the first Newton correction within refine_eps (1 + ||z||), which at ||z|| ~ 1e6 certifies
+//     or not depending on the last bits of the FP32 endpoint: one of two kernels of different
+//     rounding, chosen by the launch's size, would make the class of such a solution depend on
+//     the paths it is tracked with.  Measured over 48 samples of 20,011 paths of rings with
+//     N = 8 .. 13: 0.1% of the paths end beyond the line, and 18 of 169,326 certified
+//     endpoints had another class by the throughput kernels, all of them among these.
 //
 // Layout here: a persistent grid pulls paths from a device work counter (warp-aggregated
 // atomics) until the list is drained.  The warp runs its 32 paths in lockstep through the same
@@ -22,7 +31,7 @@
 // side, same factorisation), and at t = 0 it is known in closed form
 // (H_z = 2 gamma diag(z), H_t = P(z)), so each step costs 3 stage solves.
 // Corrector: Newton at t + h, its residual evaluated with compensated sums
-// (float-float in FP32, double-double in FP64).  A step is accepted when ||dz|| <= eps (1 + ||z||)
+// (xy_residual_comp: float-float in FP32, double-double in FP64).  A step is accepted when ||dz|| <= eps (1 + ||z||)
 // within max_newton iterations, and rejected when the first correction exceeds
 // trust (1 + ||z||).  Step size doubles after grow_after consecutive accepts and halves
 // on a reject; the final step lands exactly on t = t_end (1, or 1 - r0 before the Cauchy
@@ -47,6 +56,17 @@
 #pragma once
 
 #include "xy_solve.cuh"
+
+template <class R>
+struct JSel;
+template <>
+struct JSel<float> {
+    static __device__ __forceinline__ const float *get(const XYSys &S) { return S.Jf; }
+};
+template <>
+struct JSel<double> {
+    static __device__ __forceinline__ const double *get(const XYSys &S) { return S.Jd; }
+};
 
 #define CRAWL_ZONE 1e-3   // the crawl test applies once 1 - t < CRAWL_ZONE
 // A path in the end zone whose ||z||_inf exceeds FAR_NORM and grew by more than FAR_GROWTH
@@ -77,6 +97,14 @@ __device__ __forceinline__ R vnorm2(const V &v) {
     return sqrt_r(s);
 }
 
+template <int NV, class R, class V>
+__device__ __forceinline__ R vnorminf(const V &v) {
+    R s = R(0);
+#pragma unroll 1
+    for (int i = 0; i < NV; i++) s = fmax(s, sqrt_r(cabs2(v.get(i))));
+    return s;
+}
+
 // The problem a tracker runs on, as a policy for track_body: the unknowns (NV), the
 // per-thread shared matrix (MD x (MD + 2)), the start point with its dz/dt, the
 // corrector residual -H, the linear solve, and the tracker state's relation to the
@@ -84,9 +112,9 @@ __device__ __forceinline__ R vnorm2(const V &v) {
 // z's inf-norm).  XYProblem: the XY ring (structured Schur solve, M = N - 1 free sites,
 // NV = 2M), its state in light-cone coordinates p_k = x_k + i y_k, q_k = x_k - i y_k
 // (xy_solve.cuh): a unitary map times sqrt(2), so 2-norms are the state's over sqrt(2).
-template <int M, int BLK>
+template <int M, class RT, int BLK>
 struct XYProblem {
-    using R = double;
+    using R = RT;
     using Sys = XYSys;
     static constexpr int BLOCK = BLK;
     static constexpr int NV = 2 * M;
@@ -135,7 +163,7 @@ struct XYProblem {
     // H_t = P(z), so dz_i/dt = -P_i(z) / (2 gamma z_i); both in light-cone coordinates
     static __device__ __forceinline__ void start(const Sys &S, int64_t p, const GVec<R> &Z0,
                                                  const GVec<R> &K1) {
-        const R *J = S.Jd;
+        const R *J = JSel<R>::get(S);
         const cx<R> gam = cx<R>{(R)S.gre, (R)S.gim};
         cx<R> x[M], y[M];
 #pragma unroll
@@ -162,7 +190,7 @@ struct XYProblem {
 
     static __device__ __forceinline__ void residual(const Sys &S, const SVec<R, BLOCK> &pt, R s,
                                                     R omt, const SVec<R, BLOCK> &out, bool wr) {
-        xy_residual_comp<M, R, BLOCK>(S.Jd, pt, s, omt, cx<R>{S.gre, S.gim}, out, wr);
+        xy_residual_comp<M, R, BLOCK>(JSel<R>::get(S), pt, s, omt, cx<R>{(R)S.gre, (R)S.gim}, out, wr);
     }
 
     template <class Out2>
@@ -170,9 +198,9 @@ struct XYProblem {
                                                  const SVec<R, BLOCK> &pt, R s, R omt,
                                                  bool two_rhs, const SVec<R, BLOCK> &res,
                                                  const SVec<R, BLOCK> &out1, const Out2 &out2,
-                                                 bool wr) {
-        return xy_solve<M, R, BLOCK>(S.Jd, A, pt, s, omt, cx<R>{S.gre, S.gim}, two_rhs, res, out1,
-                                     out2, wr);
+                                                 bool wr, R *kest = nullptr) {
+        return xy_solve<M, R, BLOCK>(JSel<R>::get(S), A, pt, s, omt, cx<R>{(R)S.gre, (R)S.gim}, two_rhs,
+                                     res, out1, out2, wr, kest);
     }
 };
 
@@ -244,6 +272,7 @@ __device__ __forceinline__ void track_body(const typename P::Sys &S, const XYCtl
     const GVec<R> Z0{st + (0 * NV) * nth + gtid, nth};       // accepted point
     const GVec<R> K1{st + (1 * NV) * nth + gtid, nth};       // dz/dt at Z0
     const GVec<R> AC{st + (2 * NV) * nth + gtid, nth};       // RK4 sum; next K1 in correction
+    const GVec<R> CK{st + (3 * NV) * nth + gtid, nth};       // FP32 pass: hand-off checkpoint
     const int64_t total = worklist_size(wl, ep.count);
 
     // short lists: at most `lanes` paths per warp, so that the list spreads over every SM
@@ -256,8 +285,13 @@ __device__ __forceinline__ void track_body(const typename P::Sys &S, const XYCtl
         lanes = per < 1 ? 1 : (per > 32 ? 32 : (int)per);
     }
     int64_t e = (lane >= lanes) ? -2 : -1;   // entry index; -1 idle, -2 drained
-    double t = 0.0, h = 0.0;
-    int status = 0, run = 0, attempts = 0, steps = 0, solves = 0, newton = 0;
+    double t = 0.0, h = 0.0, hacc = 0.0;
+    double tck = 0.0, hck = 0.0;   // checkpoint: the last clean accepted point with 1 - t < CRAWL_ZONE
+    bool have_ck = false;
+    int clean = 0;                 // accepted steps in a row without a reject between them
+    double tmark = 0.0;   // 1 - t recorded every CRAWL_STEPS accepted steps near t = 1
+    int since = 0;
+    int status = 0, run = 0, rejects = 0, attempts = 0, steps = 0, solves = 0, newton = 0;
     bool need_k1 = false;
     bool far = false;      // heading out: steps capped at KAPPA_FAR (1 - t)
     double zlast = 0.0;    // ||z||_inf at the last accepted point
@@ -279,7 +313,10 @@ __device__ __forceinline__ void track_body(const typename P::Sys &S, const XYCtl
                 } else if (e >= 0) {
                     status = NPHC_PATH_RUNNING;
                     run = 0;
+                    rejects = 0;
                     attempts = 0;
+                    have_ck = false;
+                    clean = 0;
                     if (C.resume) {
                         P::load(ep, e, Z0);
                         t = ep.t[e];
@@ -300,6 +337,9 @@ __device__ __forceinline__ void track_body(const typename P::Sys &S, const XYCtl
                         newton = C.accumulate ? ep.newton[e] : 0;
                         need_k1 = false;
                     }
+                    hacc = h;
+                    tmark = 1.0 - t;
+                    since = 0;
                     far = false;
                     zlast = 0.0;
                 }
@@ -322,6 +362,7 @@ __device__ __forceinline__ void track_body(const typename P::Sys &S, const XYCtl
         bool go = act && !need_k1;
         bool conv = false, bad = false;
         R zpn = R(0);
+        R kstep = R(0);   // the largest condition estimate of this attempt's solves
         const int ph0 = __any_sync(0xffffffffu, act && need_k1) ? 0 : 1;
         const int nph = 4 + C.max_newton;
 #pragma unroll 1
@@ -356,9 +397,11 @@ __device__ __forceinline__ void track_body(const typename P::Sys &S, const XYCtl
             }
             const R tr = (R)te, omt = (R)(1.0 - te);
             if (corr) P::residual(S, ZC, tr, omt, W1, w);
-            const bool oks = P::solve(S, A, ZC, tr, omt, corr, W1, W1, AC, w);
+            R kest = R(0);
+            const bool oks = P::solve(S, A, ZC, tr, omt, corr, W1, W1, AC, w, &kest);
             if (!w) continue;
             solves++;
+            kstep = fmax(kstep, kest);
             if (ph == 0) {
                 // z0 += Newton correction at t; dz/dt from the second right-hand side
 #pragma unroll 6
@@ -368,7 +411,7 @@ __device__ __forceinline__ void track_body(const typename P::Sys &S, const XYCtl
                 }
                 newton++;
                 need_k1 = false;
-                if (!oks) status = NPHC_PATH_NONFINITE;
+                if (!oks) status = C.handoff ? NPHC_PATH_HANDOFF : NPHC_PATH_NONFINITE;
             } else if (!corr) {
                 bad = bad || !oks;
                 if (ph == 1) {
@@ -409,6 +452,19 @@ __device__ __forceinline__ void track_body(const typename P::Sys &S, const XYCtl
         }
         go = go && status == NPHC_PATH_RUNNING;
 
+        // ---- FP32 pass: a converged step whose Schur systems' condition estimate exceeds
+        // kappa (kappa = 0 outside the FP32 pass) is not taken; FP64 continues the path from
+        // its last accepted point (or the end zone's clean checkpoint), where the estimate
+        // was below kappa: the FP32 solve's relative error grows like the condition number
+        // times 6e-8, and a step across an ill-conditioned stretch (two paths passing
+        // close) can land on the neighbouring path.  A step that did not converge lands
+        // nowhere: it is rejected and halved as usual, whatever its estimate (a poor
+        // prediction far off the path can see a large one)
+        if (go && conv && C.kappa > 0.0 && !((double)kstep <= C.kappa)) {
+            status = NPHC_PATH_HANDOFF_COND;
+            go = false;
+        }
+
         // ---- accept or reject
         if (go) {
             attempts++;
@@ -419,27 +475,78 @@ __device__ __forceinline__ void track_body(const typename P::Sys &S, const XYCtl
                     K1.set(k, AC.get(k));
                 }
                 const R zi = P::norminf(ZC);
+                clean = rejects == 0 ? clean + 1 : 1;
                 t = t1;
                 far = 1.0 - t < CRAWL_ZONE && (double)zi > FAR_NORM && (double)zi > FAR_GROWTH * zlast;
                 zlast = (double)zi;
                 steps++;
+                rejects = 0;
+                hacc = h;
                 if (++run >= C.grow_after) {
                     run = 0;
                     h = fmin(2.0 * h, C.hmax);
                 }
-                if ((double)zi > C.rdiv) status = NPHC_PATH_DIVERGED;
-                else if (t >= C.t_end) status = NPHC_PATH_REACHED;
+                if ((double)zi > C.rdiv)
+                    // An FP32 point is accurate to ~eps relative, so a crossing by more
+                    // than RDIV_BAND is one in FP64 too; FP32 leaves only the marginal
+                    // crossings close to t = 1 to FP64
+                    status = (C.handoff && 1.0 - t < NEAR_END &&
+                              (double)zi <= C.rdiv * (1.0 + RDIV_BAND))
+                                 ? NPHC_PATH_HANDOFF
+                                 : NPHC_PATH_DIVERGED;
+                else if (t >= C.t_end)
+                    status = NPHC_PATH_REACHED;
+                // FP32 pass: in the end zone keep the last clean point (accepted, with the
+                // step before it accepted too); a path that the pass later hands off
+                // resumes in FP64 from there, not from the point where FP32 precision ran
+                // out, which can sit off the path.  A converged FP32 point in light-cone
+                // coordinates is on its path to the corrector's tolerance; in (x, y) the
+                // small light-cone coordinate of a far point was lost to cancellation, so
+                // such points could look converged while off the path, and the checkpoint
+                // then had to stay at the end zone's entry.
+                if (C.handoff && (clean >= 2 || !have_ck) && status == NPHC_PATH_RUNNING &&
+                    1.0 - t < CRAWL_ZONE) {
+#pragma unroll 6
+                    for (int k = 0; k < NV; k++) CK.set(k, Z0.get(k));
+                    tck = t;
+                    hck = hacc;
+                    have_ck = true;
+                }
+                // crawl test near t = 1: 1 - t must at least halve every CRAWL_STEPS
+                // accepted steps (paths to nonsingular endpoints finish in a few steps;
+                // a crawl means a singular endpoint, infinity, or precision exhausted)
+                if (status == NPHC_PATH_RUNNING && C.crawl_steps > 0 && 1.0 - t < CRAWL_ZONE) {
+                    if (++since >= C.crawl_steps) {
+                        if (1.0 - t > 0.5 * tmark)
+                            status = C.handoff ? NPHC_PATH_HANDOFF : NPHC_PATH_MIN_STEP;
+                        tmark = 1.0 - t;
+                        since = 0;
+                    }
+                } else {
+                    tmark = 1.0 - t;
+                    since = 0;
+                }
             } else {
                 run = 0;
+                rejects++;
                 h *= 0.5;
-                if (h < C.hmin) status = NPHC_PATH_MIN_STEP;
+                if (h < C.hmin)
+                    status = C.handoff ? NPHC_PATH_HANDOFF : NPHC_PATH_MIN_STEP;
+                else if (C.handoff && rejects >= 10)
+                    status = NPHC_PATH_HANDOFF;
             }
-            if (status == NPHC_PATH_RUNNING && attempts >= C.max_steps) status = NPHC_PATH_STEP_BUDGET;
+            if (status == NPHC_PATH_RUNNING && attempts >= C.max_steps)
+                status = C.handoff ? NPHC_PATH_HANDOFF : NPHC_PATH_STEP_BUDGET;
         }
         if (act && status != NPHC_PATH_RUNNING) {
-            P::store(ep, e, Z0);
-            ep.t[e] = t;
-            ep.h[e] = h;
+            const bool handed = status == NPHC_PATH_HANDOFF || status == NPHC_PATH_HANDOFF_COND;
+            const bool from_ck = handed && have_ck;
+            if (from_ck)
+                P::store(ep, e, CK);
+            else
+                P::store(ep, e, Z0);
+            ep.t[e] = from_ck ? tck : t;
+            ep.h[e] = from_ck ? hck : (handed ? hacc : h);
             ep.status[e] = status;
             ep.steps[e] = steps;
             ep.solves[e] = solves;
@@ -449,9 +556,9 @@ __device__ __forceinline__ void track_body(const typename P::Sys &S, const XYCtl
     }
 }
 
-template <int M, int BLOCK>
+template <int M, class R, int BLOCK>
 __global__ void __launch_bounds__(BLOCK)
     xy_track_kernel(const __grid_constant__ XYSys S, const __grid_constant__ XYCtl C,
                     const EPView ep, const WorkList wl) {
-    track_body<XYProblem<M, BLOCK>>(S, C, ep, wl);
+    track_body<XYProblem<M, R, BLOCK>>(S, C, ep, wl);
 }
