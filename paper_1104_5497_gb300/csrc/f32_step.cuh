@@ -32,8 +32,10 @@ __device__ __forceinline__ float2 f2cfms(float2 a, float2 b, float2 c) {
 
 // Square root and reciprocal square root for the light-cone scales and frames (any scale solves
 // the same system, and the frame's error of two ulp is the row's own rounding), and a pivot's
-// reciprocal with one Newton step: one to three instructions where the IEEE forms take
-// thirteen to fifteen.
+// reciprocal with one Newton step: a few instructions where the IEEE forms take thirteen to
+// fifteen.  Without flushing: |pivot|^2 beyond 2^126 has a subnormal reciprocal, and a reciprocal
+// flushed to 0 stays 0 in the Newton step, sets its unknown to 0 and passes every test of the
+// solve.  (A square root flushed to 0 is below the scales' bound of 1.)
 __device__ __forceinline__ float f32_sqrt(float x) {
     float r;
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -41,12 +43,12 @@ __device__ __forceinline__ float f32_sqrt(float x) {
 }
 __device__ __forceinline__ float f32_rsqrt(float x) {
     float r;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    asm("rsqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
 __device__ __forceinline__ float f32_recip(float x) {
     float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
     return fmaf(fmaf(-x, r, 1.0f), r, r);
 }
 
