@@ -362,13 +362,9 @@ nphc_status nphc_system_create_quadratic(int n, int nterms, const int32_t *eq, c
             }
         }
     }
-    double d2 = 0.0, most = 0.0;
-    for (int i = 0; i < n; i++) {
+    double d2 = 0.0;
+    for (int i = 0; i < n; i++)
         for (double v : m2[i]) d2 += v * v;
-        double sum = 0.0;
-        for (int t = row[i]; t < row[i + 1]; t++) sum += std::fabs(terms[t].cre) + std::fabs(terms[t].cim);
-        most = std::max(most, sum);
-    }
     // the Jacobian's entries: per (variable, equation) cell the list of c w(other)
     std::vector<std::vector<QTerm>> cell((size_t)n * n);
     for (int i = 0; i < n; i++)
@@ -420,7 +416,6 @@ nphc_status nphc_system_create_quadratic(int n, int nterms, const int32_t *eq, c
         return fail(NPHC_ECUDA, std::string("term list upload: ") + cudaGetErrorString(e));
     }
     S->qs.n = n;
-    S->qs.cexp = sum_exponent(most);
     S->qs.row = reinterpret_cast<const int32_t *>(d);
     S->qs.terms = reinterpret_cast<const QTerm *>(d + rbytes);
     S->qs.jrow = reinterpret_cast<const int32_t *>(d + rbytes + tbytes);

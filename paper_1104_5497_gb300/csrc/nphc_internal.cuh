@@ -268,7 +268,6 @@ struct QTerm {
 
 struct QSys {
     int n;
-    int cexp;              // sum over an equation's terms of |Re c| + |Im c| < 2^cexp (gsum)
     const int32_t *row;    // [n + 1] term offsets per equation (device)
     const QTerm *terms;    // [row[n]] (device)
     // dP_i/dz_v = sum of c w(a) over the entries jrow[v n + i] .. jrow[v n + i + 1] - 1 of jac (a

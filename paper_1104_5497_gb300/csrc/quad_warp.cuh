@@ -66,20 +66,38 @@ struct QuadSum {
         }
         return p;
     }
-    // With exact products and compensated sums, on grids (gsum); |P's parts| < 2^(kp - 1).
+    static __device__ __forceinline__ int wexp(const cx<double> *z, int a) {
+        return a < 0 ? 0 : max(gexp(z[a].re), gexp(z[a].im));
+    }
+    // With exact products and compensated sums, on grids (gsum) of each equation's own size: the
+    // variables and equations of a system may differ by many orders.  |P_i's parts| < 2^(kp - 1).
     static __device__ __forceinline__ void compensated(const QSys &S, const cx<double> *z, int lane,
                                                        ext<double> &pr, ext<double> &pi, int &kp) {
-        const cx<double> zl = z[lane < N ? lane : 0];
-        const int ez = __reduce_max_sync(0xffffffffu, max(max(gexp(zl.re), gexp(zl.im)), 0));
-        kp = S.cexp + 2 * ez + 4;
-        const double am = gsum_anchor(2 * ez + 4), ap = gsum_anchor(kp);
-        gsum sr = {ap, 0.0}, si = sr;
         const int i = lane / LE;
+        int kt = -4000;   // exponent of the equation's largest |c| |w(a)| |w(b)|, in integers
+        if (i < N) {
+#pragma unroll 1
+            for (int t = S.row[i] + lane % LE; t < S.row[i + 1]; t += LE) {
+                const QTerm T = S.terms[t];
+                kt = max(kt, max(gexp(T.cre), gexp(T.cim)) + wexp(z, T.a) + wexp(z, T.b));
+            }
+        }
+#pragma unroll
+        for (int o = 1; o < LE; o++) {   // over the equation's lanes
+            const int ko = __shfl_down_sync(0xffffffffu, kt, o);
+            if (lane % LE == 0) kt = max(kt, ko);
+        }
+        kt = __shfl_sync(0xffffffffu, kt, i * LE < 32 ? i * LE : 0);
+        // a term's parts are below 2^(kt + 5), the sum of all below their number times that
+        kp = kt + 6 + (i < N ? 32 - __clz(S.row[i + 1] - S.row[i]) : 0);
+        const double ap = gsum_anchor(kp);
+        gsum sr = {ap, 0.0}, si = sr;
         if (i < N) {
 #pragma unroll 1
             for (int t = S.row[i] + lane % LE; t < S.row[i + 1]; t += LE) {
                 const QTerm T = S.terms[t];
                 const cx<double> wa = quad_w(z, T.a), wb = quad_w(z, T.b);
+                const double am = gsum_anchor(wexp(z, T.a) + wexp(z, T.b) + 4);
                 gsum smr = {am, 0.0}, smi = smr;   // wa wb
                 gsum_acc(smr, wa.re, wb.re);
                 gsum_acc(smr, -wa.im, wb.im);
