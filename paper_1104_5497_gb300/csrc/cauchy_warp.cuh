@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(32 * WARPS)
                 const EffPoint pe = eff_point(eg_ew(lr, radial, j, K, C.lnratio, v), gam, ag);
                 if (vl) P.at(L::ZC, i) = P.at(L::Z0, i);
                 __syncwarp();
-                warp_residual<M>(P, J, S.jexp, pe.s, pe.omt, pe.g);
+                warp_residual<M>(P, J, pe.s, pe.omt, pe.g);
                 const bool ok = warp_solve<M>(P, J, pe.s, pe.omt, pe.g, true, L::AC);
                 solves++;
                 if (vl) {
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(32 * WARPS)
                 // Newton's corrector at v1
 #pragma unroll 1
                 for (int it = 0; it < C.max_newton && !bad; it++) {
-                    warp_residual<M>(P, J, S.jexp, p1.s, p1.omt, p1.g);
+                    warp_residual<M>(P, J, p1.s, p1.omt, p1.g);
                     const bool oks = warp_solve<M>(P, J, p1.s, p1.omt, p1.g, true, L::AC);
                     solves++;
                     const double dn = sqrt(warp_sum(vl ? cabs2(P.at(L::W1, i)) : 0.0));
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(32 * WARPS)
                                     // a solution of P is the endpoint; otherwise a pole
                                     // (growing distance) or an enclosed branch point of
                                     // two other sheets (on to smaller radii)
-                                    warp_residual<M>(P, J, S.jexp, 1.0, 0.0, gam);   // W1 = -P(est)
+                                    warp_residual<M>(P, J, 1.0, 0.0, gam);   // W1 = -P(est)
                                     const double res = warp_max(vl ? sqrt(cabs2(P.at(L::W1, i))) : 0.0);
                                     const double zi2 = warp_max(vl ? sqrt(cabs2(P.at(L::ZC, i))) : 0.0);
                                     if (res <= C.tol_res * (zi2 > 1.0 ? zi2 * zi2 : 1.0))

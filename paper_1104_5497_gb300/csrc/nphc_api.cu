@@ -108,12 +108,6 @@ FillSet fp32_counters(void *ws, int n, int64_t count, int queue_slot) {
     return f;
 }
 
-// k with s < 2^k for a rounded sum s >= 0 of non-negative numbers
-int sum_exponent(double s) {
-    if (!(s > 0.0)) return -1023;
-    return std::isfinite(s) ? std::ilogb(s * (1.0 + 1e-12)) + 1 : 1024;
-}
-
 unsigned long long *ws_queue(void *ws, int slot) {
     return reinterpret_cast<unsigned long long *>(static_cast<char *>(ws)) + slot;
 }
@@ -280,21 +274,15 @@ nphc_status nphc_system_create_xy(int N, double sigma, const double *J, nphc_sys
     S->J = Jv;
     std::memset(&S->xs, 0, sizeof(S->xs));
     S->xs.N = N;
-    double row = 0.0;         // the largest sum_j |J_ij|
     double d2 = 2.0 * S->M;   // each constraint c^2 + s^2 - 1 contributes ||M_g||_F^2 = 2
-    for (int i = 0; i < N; i++) {
-        double sum = 0.0;
+    for (int i = 0; i < N; i++)
         for (int j = 0; j < N; j++) {
-            sum += std::fabs(Jv[i * N + j]);
             S->xs.Jf[i * NPHC_JSTRIDE + j] = (float)Jv[i * N + j];
             S->xs.Jd[i * NPHC_JSTRIDE + j] = Jv[i * N + j];
             // gradient row i: J_ij (s_i c_j - s_j c_i) puts J_ij / 2 on four symmetric
             // entries when j is free, so ||M_fi||_F^2 gains J_ij^2
             if (i < S->M && j < S->M && i != j) d2 += Jv[i * N + j] * Jv[i * N + j];
         }
-        row = std::max(row, sum);
-    }
-    S->xs.jexp = sum_exponent(row);
     S->xs.d2norm = std::sqrt(d2);
     S->xs.kappa_sing = 1e12;
     *out = S;

@@ -144,6 +144,15 @@ __device__ __forceinline__ void gsum_acc_ext(gsum &s, double a, ext<double> b) {
     gsum_acc(s, a, b.hi);
     s.lo = __fma_rn(a, b.lo, s.lo);
 }
+__device__ __forceinline__ void gsum_add(gsum &s, ext<double> b) {   // b of any grid
+    const double n = __dadd_rn(s.h, b.hi);
+    s.lo = __dadd_rn(s.lo, __dadd_rn(__dsub_rn(b.hi, __dsub_rn(n, s.h)), b.lo));
+    s.h = n;
+}
+// k for the sum of a coupling row's at most 13 products, e the largest of their factors'
+// exponents' sums: every term is below 2^(e + 2).  A row's own e, not the ring's: couplings and
+// coordinates of different sites may differ by many orders.
+__device__ __forceinline__ int gsum_row(int e) { return e + 7; }
 // hi on the grid (sums and differences of such hi are exact), lo not small against it
 __device__ __forceinline__ ext<double> gsum_ext(gsum s, double anchor) {
     return ext<double>{__dsub_rn(s.h, anchor), s.lo};
@@ -170,7 +179,6 @@ inline int far_exponent(double refine_eps) {
 // unrolled kernels read them as constant-bank operands.
 struct XYSys {
     int N;                                  // ring size; M = N - 1 free sites
-    int jexp;                               // sum_j |J_kj| < 2^jexp for every k (gsum)
     alignas(16) float Jf[NPHC_MAXN * NPHC_JSTRIDE];   // J in FP32 (row k, column j at
                                                       // k * NPHC_JSTRIDE + j; zeros beyond)
     double Jd[NPHC_MAXN * NPHC_JSTRIDE];    // J in FP64

@@ -79,7 +79,6 @@ struct RGPath {
     cx<double> *sm;      // this endpoint's column of the shared memory
     const double *J;     // J[k * (M + 1) + l], l = M the pinned site
     const double *jj;    // sum over free l of J_kl^2
-    int jexp;            // XYSys::jexp
     int g;               // lane of the endpoint
     unsigned m;          // the lanes that run this code together (whole endpoints)
     __device__ __forceinline__ cx<double> &at(int off, int i) const { return sm[(off + i) * RG_PATHS]; }
@@ -95,6 +94,52 @@ __device__ __forceinline__ int fill_warps(int64_t total, int slots) {
     return total <= (int64_t)half * slots ? half : (int)gridDim.x;
 }
 
+// P's rows of site j, as sums on grids: f = y u - x w and g = x^2 + y^2 - 1, and u, w.
+template <int M>
+__device__ __forceinline__ void rg_row(const RGPath<M> &G, int j, cx<double> &f, cx<double> &gg, cx<double> &u,
+                                       cx<double> &w) {
+    using L = RGLayout<M>;
+    const double *Jj = G.J + j * (M + 1);
+    int er = gexp(Jj[M]);
+#pragma unroll 1
+    for (int l = 0; l < M; l++) er = max(er, gexp(Jj[l]) + gexp_max(G.at(L::Z, l), G.at(L::Z, M + l)));
+    const int ku = gsum_row(er);   // |u|, |w| < 2^(ku - 1)
+    const double au = gsum_anchor(ku);
+    gsum sur = gsum_start(au, Jj[M]), sui = {au, 0.0}, swr = sui, swi = sui;
+#pragma unroll 1
+    for (int l = 0; l < M; l++) {   // J_jj = 0 adds exact zeros
+        const cx<double> xl = G.at(L::Z, l), yl = G.at(L::Z, M + l);
+        const double c = Jj[l];
+        gsum_acc(sur, c, xl.re);
+        gsum_acc(sui, c, xl.im);
+        gsum_acc(swr, c, yl.re);
+        gsum_acc(swi, c, yl.im);
+    }
+    const ext<double> ur = gsum_ext(sur, au), ui = gsum_ext(sui, au), wr = gsum_ext(swr, au), wi = gsum_ext(swi, au);
+    const cx<double> x = G.at(L::Z, j), y = G.at(L::Z, M + j);
+    const int ek = gexp_max(x, y);
+    const double af = gsum_anchor(ek + ku + 3), ag = gsum_anchor(max(0, 2 * ek + 4) + 2);
+    gsum fr = {af, 0.0}, fi = fr, gr = gsum_start(ag, -1.0), gi = {ag, 0.0};
+    gsum_acc_ext(fr, y.re, ur);
+    gsum_acc_ext(fr, -y.im, ui);
+    gsum_acc_ext(fr, -x.re, wr);
+    gsum_acc_ext(fr, x.im, wi);
+    gsum_acc_ext(fi, y.re, ui);
+    gsum_acc_ext(fi, y.im, ur);
+    gsum_acc_ext(fi, -x.re, wi);
+    gsum_acc_ext(fi, -x.im, wr);
+    gsum_acc(gr, x.re, x.re);
+    gsum_acc(gr, -x.im, x.im);
+    gsum_acc(gr, y.re, y.re);
+    gsum_acc(gr, -y.im, y.im);
+    gsum_acc(gi, 2.0 * x.re, x.im);
+    gsum_acc(gi, 2.0 * y.re, y.im);
+    f = cx<double>{ext_val(gsum_ext(fr, af)), ext_val(gsum_ext(fi, af))};
+    gg = cx<double>{ext_val(gsum_ext(gr, ag)), ext_val(gsum_ext(gi, ag))};
+    u = cx<double>{ext_val(ur), ext_val(ui)};
+    w = cx<double>{ext_val(wr), ext_val(wi)};
+}
+
 // P, the factorisation of DP and the Newton correction D = -DP^-1 P (into QA, QB) at Z.  res = ||P||_inf,
 // dn2 = ||D||_2^2, z2 = ||z||_2^2; perm: the row of S behind each row of the factor, four bits
 // each.  False when the Schur matrix is singular.
@@ -103,49 +148,12 @@ __device__ bool rg_evaluate(const RGPath<M> &G, double &res, double &dn2, double
     using L = RGLayout<M>;
     const int g = G.g;
     double pmax = 0.0;
-    int ez = 0;   // exponent of max(1, ||z||_inf)
-#pragma unroll 1
-    for (int j = g; j < M; j += 4) ez = max(ez, gexp_max(G.at(L::Z, j), G.at(L::Z, M + j)));
-    ez = max(ez, __shfl_xor_sync(G.m, ez, 8));
-    ez = max(ez, __shfl_xor_sync(G.m, ez, 16));
-    const int ku = G.jexp + ez + 2;   // |u_j|, |w_j| < 2^(ku - 1)
-    const double au = gsum_anchor(ku);
 #pragma unroll 1
     for (int j = g; j < M; j += 4) {
-        const double *Jj = G.J + j * (M + 1);
-        gsum sur = gsum_start(au, Jj[M]), sui = {au, 0.0}, swr = sui, swi = sui;
-#pragma unroll 1
-        for (int l = 0; l < M; l++) {   // J_jj = 0 adds exact zeros
-            const cx<double> xl = G.at(L::Z, l), yl = G.at(L::Z, M + l);
-            const double c = Jj[l];
-            gsum_acc(sur, c, xl.re);
-            gsum_acc(sui, c, xl.im);
-            gsum_acc(swr, c, yl.re);
-            gsum_acc(swi, c, yl.im);
-        }
-        const ext<double> ur = gsum_ext(sur, au), ui = gsum_ext(sui, au), wr = gsum_ext(swr, au), wi = gsum_ext(swi, au);
         const cx<double> x = G.at(L::Z, j), y = G.at(L::Z, M + j);
-        const int ek = gexp_max(x, y);
-        const double af = gsum_anchor(ek + ku + 3), ag = gsum_anchor(max(0, 2 * ek + 4) + 2);
-        gsum fr = {af, 0.0}, fi = fr, gr = gsum_start(ag, -1.0), gi = {ag, 0.0};
-        gsum_acc_ext(fr, y.re, ur);   // f = y u - x w
-        gsum_acc_ext(fr, -y.im, ui);
-        gsum_acc_ext(fr, -x.re, wr);
-        gsum_acc_ext(fr, x.im, wi);
-        gsum_acc_ext(fi, y.re, ui);
-        gsum_acc_ext(fi, y.im, ur);
-        gsum_acc_ext(fi, -x.re, wi);
-        gsum_acc_ext(fi, -x.im, wr);
-        gsum_acc(gr, x.re, x.re);     // g = x^2 + y^2 - 1
-        gsum_acc(gr, -x.im, x.im);
-        gsum_acc(gr, y.re, y.re);
-        gsum_acc(gr, -y.im, y.im);
-        gsum_acc(gi, 2.0 * x.re, x.im);
-        gsum_acc(gi, 2.0 * y.re, y.im);
-        const cx<double> f = {ext_val(gsum_ext(fr, af)), ext_val(gsum_ext(fi, af))};
-        const cx<double> gg = {ext_val(gsum_ext(gr, ag)), ext_val(gsum_ext(gi, ag))};
+        cx<double> f, gg, u, w;
+        rg_row<M>(G, j, f, gg, u, w);
         pmax = fmax(pmax, fmax(cabs2(f), cabs2(gg)));
-        const cx<double> u = {ext_val(ur), ext_val(ui)}, w = {ext_val(wr), ext_val(wi)};
         const cx<double> a = cscale(2.0, x), b = cscale(2.0, y);
         const double iv = rsqrt(cabs2(a) + cabs2(b));
         const cx<double> ah = cscale(iv, a), bh = cscale(iv, b);
@@ -332,7 +340,7 @@ __global__ void __launch_bounds__(32)
         jj[lane] = s;
     }
     __syncwarp();
-    RGPath<M> G{base + pth, J, jj, S.jexp, g, 0xffffffffu};
+    RGPath<M> G{base + pth, J, jj, g, 0xffffffffu};
     const unsigned mine = 0x01010101u << pth;   // this endpoint's four lanes
     const double alpha0 = NPHC_ALPHA_CERT;
     const int64_t cnt = ep.count, total = worklist_size(wl, cnt);

@@ -45,7 +45,6 @@ struct G64Path {
     using L = G64Layout<M>;
     cx<double> *sm;
     const double *J;     // J[k * (M + 1) + l], l = M the pinned site
-    int jexp;            // XYSys::jexp
     int g;
     unsigned m;          // the lanes that run this code together (whole paths)
     __device__ __forceinline__ cx<double> &at(int off, int i) const { return sm[(off + i) * G64_PATHS]; }
@@ -67,9 +66,11 @@ __device__ __forceinline__ void f64_residual_rows(cx<double> p, cx<double> q, co
                                                   const ext<double> &upi, const ext<double> &uqr,
                                                   const ext<double> &uqi, int ku, double s, double hs,
                                                   double gr, double gi, cx<double> &rf, cx<double> &rg) {
-    const int ek = max(max(gexp(p.re), gexp(p.im)), max(gexp(q.re), gexp(q.im)));
-    const int eg = max(gexp(gr), gexp(gi)), kd = ek + ku + 3, kh = max(0, 2 * ek + 2) + 2;
-    const double ad = gsum_anchor(kd), ah = gsum_anchor(kh);
+    const int ep = max(gexp(p.re), gexp(p.im)), eq = max(gexp(q.re), gexp(q.im)), ek = max(ep, eq);
+    const int eg = max(gexp(gr), gexp(gi)), kd = ek + ku + 3;
+    // h has a grid of its own: near infinity p q stays near 1 where p^2 or q^2 is huge
+    const int kh = max(0, ep + eq + 2) + 2, kx = max(2 * ek + 3, kh) + 1;
+    const double ad = gsum_anchor(kd), ah = gsum_anchor(kh), ax = gsum_anchor(kx);
     gsum sdr = {ad, 0.0}, sdi = sdr;   // D = q U_p - p U_q, f = i D / 2
     gsum_acc_ext(sdr, q.re, upr);
     gsum_acc_ext(sdr, -q.im, upi);
@@ -82,7 +83,7 @@ __device__ __forceinline__ void f64_residual_rows(cx<double> p, cx<double> q, co
     const ext<double> dr = gsum_ext(sdr, ad), di = gsum_ext(sdi, ad);
     // h = (p q - 2) / 2, B = (p^2 + q^2) / 4: x^2 - 1 = h + B, y^2 - 1 = h - B, p q - 1 = 2 h + 1
     const cx<double> ph = cscale(0.5, p), qh = cscale(0.5, q);
-    gsum shr = gsum_start(ah, -1.0), shi = {ah, 0.0}, sbr = shi, sbi = shi;
+    gsum shr = gsum_start(ah, -1.0), shi = {ah, 0.0}, sbr = {ax, 0.0}, sbi = sbr;
     gsum_acc(shr, ph.re, q.re);
     gsum_acc(shr, -ph.im, q.im);
     gsum_acc(shi, ph.re, q.im);
@@ -93,12 +94,17 @@ __device__ __forceinline__ void f64_residual_rows(cx<double> p, cx<double> q, co
     gsum_acc(sbr, -qh.im, qh.im);
     gsum_acc(sbi, ph.re, p.im);
     gsum_acc(sbi, qh.re, q.im);
-    const ext<double> hr = gsum_ext(shr, ah), hi = gsum_ext(shi, ah), br = gsum_ext(sbr, ah), bi = gsum_ext(sbi, ah);
-    const ext<double> xr = grid_add(hr, br), xi = grid_add(hi, bi), yr = grid_sub(hr, br), yi = grid_sub(hi, bi);
+    const ext<double> hr = gsum_ext(shr, ah), hi = gsum_ext(shi, ah), br = gsum_ext(sbr, ax), bi = gsum_ext(sbi, ax);
+    gsum tr = {__dsub_rn(ax, br.hi), -br.lo}, ti = {__dsub_rn(ax, bi.hi), -bi.lo};   // -B
+    gsum_add(sbr, hr);
+    gsum_add(sbi, hi);
+    gsum_add(tr, hr);
+    gsum_add(ti, hi);
+    const ext<double> xr = gsum_ext(sbr, ax), xi = gsum_ext(sbi, ax), yr = gsum_ext(tr, ax), yi = gsum_ext(ti, ax);
     // H_f = gomt X + t f ;  H_g = gomt Y + t (2 h + 1)
     const double s2 = 2.0 * s;
-    const double af = gsum_anchor(max(eg + kh + 2, gexp(hs) + kd) + 2);
-    const double ag = gsum_anchor(max(eg + kh + 2, gexp(s2) + kh + 1) + 2);
+    const double af = gsum_anchor(max(eg + kx + 2, gexp(hs) + kd) + 2);
+    const double ag = gsum_anchor(max(eg + kx + 2, gexp(s2) + kh + 1) + 2);
     gsum fr = {af, 0.0}, fi = fr, kr = gsum_start(ag, s), ki = {ag, 0.0};
     gsum_acc_ext(fr, gr, xr);
     gsum_acc_ext(fr, -gi, xi);
@@ -116,6 +122,36 @@ __device__ __forceinline__ void f64_residual_rows(cx<double> p, cx<double> q, co
     rg = cx<double>{-ext_val(gsum_ext(kr, ag)), -ext_val(gsum_ext(ki, ag))};
 }
 
+// -H's rows of site j at PQ, and U_p, U_q.
+template <int M>
+__device__ __forceinline__ void g64_residual(const G64Path<M> &G, int j, double s, double gr, double gi, cx<double> &Up,
+                                             cx<double> &Uq, cx<double> &rf, cx<double> &rg) {
+    using L = G64Layout<M>;
+    const double *Jj = G.J + j * (M + 1);
+    int er = gexp(Jj[M]);
+#pragma unroll 1
+    for (int l = 0; l < M; l++) {
+        const cx<double> pl = G.at(L::PQ, l), ql = G.at(L::PQ, M + l);
+        er = max(er, gexp(Jj[l]) + max(max(gexp(pl.re), gexp(pl.im)), max(gexp(ql.re), gexp(ql.im))));
+    }
+    const int ku = gsum_row(er);
+    const double au = gsum_anchor(ku);
+    gsum spr = gsum_start(au, Jj[M]), spi = {au, 0.0}, sqr = spr, sqi = spi;
+#pragma unroll 1
+    for (int l = 0; l < M; l++) {   // J_jj = 0 adds exact zeros
+        const cx<double> pl = G.at(L::PQ, l), ql = G.at(L::PQ, M + l);
+        const double c = Jj[l];
+        gsum_acc(spr, c, pl.re);
+        gsum_acc(spi, c, pl.im);
+        gsum_acc(sqr, c, ql.re);
+        gsum_acc(sqi, c, ql.im);
+    }
+    const ext<double> upr = gsum_ext(spr, au), upi = gsum_ext(spi, au), uqr = gsum_ext(sqr, au), uqi = gsum_ext(sqi, au);
+    f64_residual_rows(G.at(L::PQ, j), G.at(L::PQ, M + j), upr, upi, uqr, uqi, ku, s, 0.5 * s, gr, gi, rf, rg);
+    Up = cx<double>{ext_val(upr), ext_val(upi)};
+    Uq = cx<double>{ext_val(uqr), ext_val(uqi)};
+}
+
 // One solve of H_z(z, t) d = r at PQ: r = -H_t, d into W (corr false); r = -H (compensated), d into
 // W, and r = -H_t, d into AC (corr true; uniform over G.m).  False when the system is singular or
 // the result is not finite.
@@ -125,18 +161,6 @@ __device__ bool g64_solve(const G64Path<M> &G, double s, double omt, cx<double> 
     const int g = G.g;
     const cx<double> gomt = cscale(omt, gam);
     const double hs = 0.5 * s;
-    int ku = 0;
-    if (corr) {   // the grid of the U sums, from the exponent of max(1, max |p|, |q|)
-#pragma unroll 1
-        for (int k = g; k < M; k += 4)
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const cx<double> v = G.at(L::PQ, k + h * M);
-                ku = max(ku, max(gexp(v.re), gexp(v.im)));
-            }
-        ku = max(ku, __shfl_xor_sync(G.m, ku, 8));
-        ku = max(ku, __shfl_xor_sync(G.m, ku, 16)) + G.jexp + 2;
-    }
     // ---- site by site: U sums, residual rows, frames, the diagonal's terms
 #pragma unroll 1
     for (int j = g; j < M; j += 4) {
@@ -144,22 +168,7 @@ __device__ bool g64_solve(const G64Path<M> &G, double s, double omt, cx<double> 
         const cx<double> p = G.at(L::PQ, j), q = G.at(L::PQ, M + j);
         cx<double> Up = {Jj[M], 0.0}, Uq = Up, rf, rg;
         if (corr) {
-            const double au = gsum_anchor(ku);
-            gsum spr = gsum_start(au, Jj[M]), spi = {au, 0.0}, sqr = spr, sqi = spi;
-#pragma unroll 1
-            for (int l = 0; l < M; l++) {   // J_jj = 0 adds exact zeros
-                const cx<double> pl = G.at(L::PQ, l), ql = G.at(L::PQ, M + l);
-                const double c = Jj[l];
-                gsum_acc(spr, c, pl.re);
-                gsum_acc(spi, c, pl.im);
-                gsum_acc(sqr, c, ql.re);
-                gsum_acc(sqi, c, ql.im);
-            }
-            const ext<double> upr = gsum_ext(spr, au), upi = gsum_ext(spi, au), uqr = gsum_ext(sqr, au), uqi = gsum_ext(sqi, au);
-            f64_residual_rows(p, q, upr, upi, uqr, uqi, ku, s, hs, EFT<double>::mul(omt, gam.re),
-                              EFT<double>::mul(omt, gam.im), rf, rg);
-            Up = cx<double>{ext_val(upr), ext_val(upi)};
-            Uq = cx<double>{ext_val(uqr), ext_val(uqi)};
+            g64_residual<M>(G, j, s, EFT<double>::mul(omt, gam.re), EFT<double>::mul(omt, gam.im), Up, Uq, rf, rg);
         } else {
 #pragma unroll 1
             for (int l = 0; l < M; l++) {
@@ -324,7 +333,7 @@ __global__ void __launch_bounds__(32)
     double *const J = reinterpret_cast<double *>(base + G64_PATHS * L::TOTAL);
     const int lane = threadIdx.x, g = lane >> 3, pth = lane & 7;
     for (int i = lane; i < M * (M + 1); i += 32) J[i] = S.Jd[(i / (M + 1)) * NPHC_JSTRIDE + i % (M + 1)];
-    G64Path<M> G{base + pth, J, S.jexp, g, 0xffffffffu};
+    G64Path<M> G{base + pth, J, g, 0xffffffffu};
     const cx<double> gam = {S.gre, S.gim};
     // few paths: fewer per warp, so that every scheduler has some
     const int64_t want = (total + gridDim.x - 1) / gridDim.x;

@@ -114,9 +114,9 @@ struct WarpPath {
 // Cauchy endgame), f = y u - x w; LC == true: the light-cone coordinates (p, q), f = i D / 2 with
 // D = q U_p - p U_q (xy_residual_comp in xy_solve.cuh).  Row pair k: lane k sums u_k (U_p,k) and forms
 // the f row, lane 16 + k sums w_k (U_q,k), hands its share of f (D) to lane k and forms the g row;
-// both halves run the same instructions.  |J row| < 2^jexp.
+// both halves run the same instructions.
 template <int M, bool LC = false>
-__device__ void warp_residual(const WarpPath<M> &P, const double *__restrict__ J, int jexp, double s,
+__device__ void warp_residual(const WarpPath<M> &P, const double *__restrict__ J, double s,
                               double omt, cx<double> gam) {
     static_assert(M <= 16, "one row pair per lane pair");
     using L = WarpLayout<M>;
@@ -128,10 +128,13 @@ __device__ void warp_residual(const WarpPath<M> &P, const double *__restrict__ J
         zk = P.at(L::ZC, k);
         wk = P.at(L::ZC, M + k);
     }
-    const int ek = max(max(gexp(zk.re), gexp(zk.im)), max(gexp(wk.re), gexp(wk.im)));
-    const int ku = __reduce_max_sync(0xffffffffu, max(ek, 0)) + jexp + 2, kd = ek + ku + 3;
-    const double au = gsum_anchor(ku), ad = gsum_anchor(kd);
+    const int ez = max(gexp(zk.re), gexp(zk.im)), ew = max(gexp(wk.re), gexp(wk.im)), ek = max(ez, ew);
     const double *Jk = J + (on ? k : 0) * NPHC_JSTRIDE;
+    int er = gexp(Jk[M]);
+#pragma unroll 1
+    for (int l = 0; l < M; l++) er = max(er, gexp(Jk[l]) + __shfl_sync(0xffffffffu, ek, l));
+    const int ku = gsum_row(er), kd = ek + ku + 3;   // the same on both halves
+    const double au = gsum_anchor(ku), ad = gsum_anchor(kd);
     const int off = hi ? L::ZC + M : L::ZC;
     gsum sr = gsum_start(au, (hi && !LC) ? 0.0 : Jk[M]), si = {au, 0.0};
 #pragma unroll 1
@@ -152,13 +155,15 @@ __device__ void warp_residual(const WarpPath<M> &P, const double *__restrict__ J
     fr = grid_add(fr, shfl_down16(fr));
     fi = grid_add(fi, shfl_down16(fi));
     // lane k: X = x^2 - 1, lane 16 + k: Y = y^2 - 1 and G = x^2 + y^2 - 1
-    const int kh = max(0, 2 * ek + 2) + 2;
+    // (h has a grid of its own: near infinity p q stays near 1 where p^2 or q^2 is huge)
+    const int kh = max(0, (LC ? ez + ew : 2 * ek) + 2) + 2, kx = LC ? max(2 * ek + 3, kh) + 1 : kh;
     const double ah = gsum_anchor(kh);
     ext<double> ar, ai, tr, ti;   // X or Y; what t multiplies: f (or D), or G - 1
     double cr, ci;
     if (LC) {   // h = (p q - 2) / 2, B = (p^2 + q^2) / 4: X = h + B, Y = h - B, G = p q - 1 = 2 h + 1
         const cx<double> ph = cscale(0.5, zk), qh = cscale(0.5, wk);
-        gsum shr = gsum_start(ah, -1.0), shi = {ah, 0.0}, sbr = shi, sbi = shi;
+        const double ax = gsum_anchor(kx);
+        gsum shr = gsum_start(ah, -1.0), shi = {ah, 0.0}, sbr = {ax, 0.0}, sbi = sbr;
         gsum_acc(shr, ph.re, wk.re);
         gsum_acc(shr, -ph.im, wk.im);
         gsum_acc(shi, ph.re, wk.im);
@@ -169,14 +174,16 @@ __device__ void warp_residual(const WarpPath<M> &P, const double *__restrict__ J
         gsum_acc(sbr, -qh.im, qh.im);
         gsum_acc(sbi, ph.re, zk.im);
         gsum_acc(sbi, qh.re, wk.im);
-        ext<double> br = gsum_ext(sbr, ah), bi = gsum_ext(sbi, ah);
-        if (hi) {
-            br = ext<double>{-br.hi, -br.lo};
-            bi = ext<double>{-bi.hi, -bi.lo};
+        const ext<double> br = gsum_ext(sbr, ax), bi = gsum_ext(sbi, ax);
+        if (hi) {   // -B
+            sbr = gsum{__dsub_rn(ax, br.hi), -br.lo};
+            sbi = gsum{__dsub_rn(ax, bi.hi), -bi.lo};
         }
         const ext<double> hr = gsum_ext(shr, ah), hm = gsum_ext(shi, ah);
-        ar = grid_add(hr, br);
-        ai = grid_add(hm, bi);
+        gsum_add(sbr, hr);
+        gsum_add(sbi, hm);
+        ar = gsum_ext(sbr, ax);
+        ai = gsum_ext(sbi, ax);
         tr = hi ? hr : fi;
         ti = hi ? hm : fr;
         cr = hi ? 2.0 * s : -0.5 * s;
@@ -197,7 +204,7 @@ __device__ void warp_residual(const WarpPath<M> &P, const double *__restrict__ J
     // H_f = gomt X + t f, H_g = gomt Y + t G
     const double gr = E::mul(omt, gam.re), gi = E::mul(omt, gam.im);
     const int kt = hi ? kh + 1 : kd;
-    const double av = gsum_anchor(max(max(gexp(gr), gexp(gi)) + kh + 2, gexp(cr) + kt + 1) + 2);
+    const double av = gsum_anchor(max(max(gexp(gr), gexp(gi)) + kx + 2, gexp(cr) + kt + 1) + 2);
     gsum vr = gsum_start(av, hi ? s : 0.0), vi = {av, 0.0};
     gsum_acc_ext(vr, gr, ar);
     gsum_acc_ext(vr, -gi, ai);
@@ -479,7 +486,7 @@ struct WarpXY {
         }
     }
     static __device__ __forceinline__ void residual(const Path &P, const Sys &S, double s, double omt) {
-        warp_residual<M, true>(P, S.Jd, S.jexp, s, omt, cx<double>{S.gre, S.gim});
+        warp_residual<M, true>(P, S.Jd, s, omt, cx<double>{S.gre, S.gim});
     }
     static __device__ __forceinline__ bool solve(const Path &P, const Sys &S, double s, double omt,
                                                  bool two_rhs, int out2) {
