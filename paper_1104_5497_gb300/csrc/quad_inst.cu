@@ -1,22 +1,18 @@
 // quad_inst.cu -- the generic quadratic-system kernels for one system size per
 // compilation.  Compiled with -DNPHC_QUAD_NV=<n> (unknowns, 1 .. NPHC_QUAD_MAX_N).
 #include "quad.cuh"
+#include "smem_optin.h"
 #include "xy_dispatch.cuh"
 
 namespace {
 
-template <class K>
-cudaError_t persistent_grid(K k, int block, size_t smem, int &grid) {
-    static bool attr_set = false;   // once per process for this instantiation
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+template <auto Kernel>
+cudaError_t persistent_grid(int block, size_t smem, int &grid) {
     int dev = 0, sms = 0, per = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    cudaError_t e = allow_dynamic_smem<Kernel>(smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, block, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, Kernel, block, smem);
     if (e != cudaSuccess) return e;
     grid = sms * (per > 0 ? per : 1);
     return cudaSuccess;
@@ -31,9 +27,9 @@ cudaError_t NPHC_CAT(launch_quad_track_n, NPHC_QUAD_NV)(const QSys &sys, const X
                                                         cudaStream_t st) {
     if (ep.count <= 0) return cudaSuccess;
     const size_t smem = sizeof(cx<double>) * QuadLayout<NPHC_QUAD_NV>::TOTAL * QUAD_WARPS;
-    auto k = quad_track_warp_kernel<NPHC_QUAD_NV, QUAD_WARPS>;
+    constexpr auto k = quad_track_warp_kernel<NPHC_QUAD_NV, QUAD_WARPS>;
     int full = 0;
-    cudaError_t e = persistent_grid(k, 32 * QUAD_WARPS, smem, full);
+    cudaError_t e = persistent_grid<k>(32 * QUAD_WARPS, smem, full);
     if (e != cudaSuccess) return e;
     const int64_t need = (ep.count + QUAD_WARPS - 1) / QUAD_WARPS;   // a list is at most ep.count long
     k<<<(int)(need < full ? need : full), 32 * QUAD_WARPS, smem, st>>>(sys, ctl, ep, wl);
@@ -49,9 +45,9 @@ cudaError_t NPHC_CAT(launch_quad_refine_certify_n, NPHC_QUAD_NV)(const QSys &sys
                                                                  cudaStream_t st) {
     if (cap <= 0) return cudaSuccess;
     const size_t smem = sizeof(cx<double>) * QuadRefineLayout<NPHC_QUAD_NV>::TOTAL * QUAD_WARPS;
-    auto k = quad_refine_warp_kernel<NPHC_QUAD_NV, QUAD_WARPS>;
+    constexpr auto k = quad_refine_warp_kernel<NPHC_QUAD_NV, QUAD_WARPS>;
     int full = 0;
-    cudaError_t e = persistent_grid(k, 32 * QUAD_WARPS, smem, full);
+    cudaError_t e = persistent_grid<k>(32 * QUAD_WARPS, smem, full);
     if (e != cudaSuccess) return e;
     const int64_t need = (cap + QUAD_WARPS - 1) / QUAD_WARPS;
     k<<<(int)(need < full ? need : full), 32 * QUAD_WARPS, smem, st>>>(sys, tol_sol, refine_eps, refine_iters,
@@ -67,9 +63,9 @@ cudaError_t NPHC_CAT(launch_quad_cauchy_n, NPHC_QUAD_NV)(const QSys &sys, const 
     using P = QuadProblem<NPHC_QUAD_NV>;
     if (ep.count <= 0) return cudaSuccess;
     const size_t smem = track_smem_per_thread<P>() * P::BLOCK;
-    auto k = quad_cauchy_kernel<NPHC_QUAD_NV>;
+    constexpr auto k = quad_cauchy_kernel<NPHC_QUAD_NV>;
     int full = 0;
-    cudaError_t e = persistent_grid(k, P::BLOCK, smem, full);
+    cudaError_t e = persistent_grid<k>(P::BLOCK, smem, full);
     if (e != cudaSuccess) return e;
     const int64_t need = (ep.count + P::BLOCK - 1) / P::BLOCK;   // the list is at most ep.count long
     const int64_t cap = wl.state_threads / P::BLOCK;

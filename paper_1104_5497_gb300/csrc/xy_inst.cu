@@ -5,6 +5,7 @@
 //   certification, classification, adjoint) or 3 (Cauchy endgame)
 #include <algorithm>
 
+#include "smem_optin.h"
 #include "xy_dispatch.cuh"
 
 #if NPHC_INST_KIND == 3
@@ -18,15 +19,10 @@ cudaError_t NPHC_CAT(launch_xy_cauchy_m, NPHC_INST_M)(const XYSys &sys, const EG
     constexpr int M = NPHC_INST_M, WARPS = 4;
     if (ep.count <= 0) return cudaSuccess;
     const size_t smem = cauchy_warp_smem_per_warp<M>() * WARPS;
-    auto k = xy_cauchy_warp_kernel<M, WARPS>;
-    static bool attr_set = false;   // once per process for this instantiation
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    constexpr auto k = xy_cauchy_warp_kernel<M, WARPS>;
     int dev = 0, sms = 0, per = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    cudaError_t e = allow_dynamic_smem<k>(smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 32 * WARPS, smem);
     if (e != cudaSuccess) return e;
@@ -48,15 +44,10 @@ static cudaError_t launch_per_thread(const XYSys &sys, const XYCtl &ctl, const E
                                      const WorkList &wl, int grid, cudaStream_t st) {
     constexpr int BLK = NPHC_TRACK_BLOCK;
     const size_t smem = xy_smem_per_thread<M, R>() * BLK;
-    auto k = xy_track_kernel<M, R, BLK>;
-    static bool attr_set = false;   // once per process for this instantiation
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    constexpr auto k = xy_track_kernel<M, R, BLK>;
     int dev = 0, sms = 0, per = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    cudaError_t e = allow_dynamic_smem<k>(smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, BLK, smem);
     if (e != cudaSuccess) return e;
@@ -111,16 +102,11 @@ static cudaError_t device_sms(int &sms) {
     return e;
 }
 
-// Shared memory limit and resident blocks per SM of a kernel (the limit is set once per process
-// and instantiation: attr).
-template <class K>
-static cudaError_t kernel_blocks(K k, int threads, size_t smem, bool &attr, int &per) {
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, threads, smem);
+// Shared memory opt-in and resident blocks per SM of a kernel.
+template <auto Kernel>
+static cudaError_t kernel_blocks(int threads, size_t smem, int &per) {
+    cudaError_t e = allow_dynamic_smem<Kernel>(smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, Kernel, threads, smem);
     per = std::max(per, 1);
     return e;
 }
@@ -130,10 +116,9 @@ template <int M, bool BATCH>
 static cudaError_t lane_blocks(int &per) {
     per = 0;
     if constexpr (M <= LANE_MAX_M) {
-        static bool attr = false;
         const size_t smem = lane_smem_per_block<M>(BATCH);
-        if constexpr (BATCH) return kernel_blocks(xy_track_lane_batch_kernel<M>, NPHC_TRACK_BLOCK, smem, attr, per);
-        else return kernel_blocks(xy_track_lane_kernel<M>, NPHC_TRACK_BLOCK, smem, attr, per);
+        if constexpr (BATCH) return kernel_blocks<xy_track_lane_batch_kernel<M>>(NPHC_TRACK_BLOCK, smem, per);
+        else return kernel_blocks<xy_track_lane_kernel<M>>(NPHC_TRACK_BLOCK, smem, per);
     }
     return cudaSuccess;
 }
@@ -167,13 +152,12 @@ cudaError_t NPHC_CAT(launch_xy_track_f32_m, NPHC_INST_M)(const XYSys &sys, const
                                                          const EPView &ep, const WorkList &wl,
                                                          int grid, cudaStream_t st) {
     constexpr int M = NPHC_INST_M, BLK = NPHC_TRACK_BLOCK;
-    static bool attr_g = false;
     const size_t smem_g = grp_smem_per_block<M>(false);
-    auto kg = xy_track_group_kernel<M>;
+    constexpr auto kg = xy_track_group_kernel<M>;
     int sms = 0, per_t = 0, per_g = 0;
     cudaError_t e = device_sms(sms);
     if (e == cudaSuccess) e = lane_blocks<M, false>(per_t);
-    if (e == cudaSuccess) e = kernel_blocks(kg, 32 * GRP_WARPS, smem_g, attr_g, per_g);
+    if (e == cudaSuccess) e = kernel_blocks<kg>(32 * GRP_WARPS, smem_g, per_g);
     if (e != cudaSuccess) return e;
     if (use_group<M>(ep.count, (int64_t)sms * per_t * BLK)) {
         const int gg = group_grid(sms, per_g, grid, ep.count, wl.state_threads);
@@ -198,13 +182,12 @@ cudaError_t NPHC_CAT(launch_xy_track_f32_batch_m, NPHC_INST_M)(const BatchGroup 
                                                                cudaStream_t st) {
     constexpr int M = NPHC_INST_M, BLK = NPHC_TRACK_BLOCK;
     if (bg.total <= 0) return cudaSuccess;
-    static bool attr_g = false;
     const size_t smem_g = grp_smem_per_block<M>(true);
-    auto kg = xy_track_group_batch_kernel<M>;
+    constexpr auto kg = xy_track_group_batch_kernel<M>;
     int sms = 0, per_t = 0, per_g = 0;
     cudaError_t e = device_sms(sms);
     if (e == cudaSuccess) e = lane_blocks<M, true>(per_t);
-    if (e == cudaSuccess) e = kernel_blocks(kg, 32 * GRP_WARPS, smem_g, attr_g, per_g);
+    if (e == cudaSuccess) e = kernel_blocks<kg>(32 * GRP_WARPS, smem_g, per_g);
     if (e != cudaSuccess) return e;
     if (use_group<M>(bg.total, (int64_t)sms * per_t * BLK)) {
         const int gg = group_grid(sms, per_g, grid, bg.total, wl.state_threads);
@@ -236,15 +219,10 @@ cudaError_t NPHC_CAT(launch_xy_track_f64w_m, NPHC_INST_M)(const XYSys &sys, cons
     constexpr int M = NPHC_INST_M, WARPS = 4;
     if (ep.count <= 0) return cudaSuccess;
     const size_t smem = warp_track_smem_per_warp<M>() * WARPS;
-    auto k = xy_track_warp64_kernel<M, WARPS>;
-    static bool attr_set = false;   // once per process for this instantiation
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    constexpr auto k = xy_track_warp64_kernel<M, WARPS>;
     int dev = 0, sms = 0, per = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    cudaError_t e = allow_dynamic_smem<k>(smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 32 * WARPS, smem);
     if (e != cudaSuccess) return e;
@@ -270,15 +248,10 @@ cudaError_t NPHC_CAT(launch_xy_track_f64g_m, NPHC_INST_M)(const XYSys &sys, cons
     constexpr int M = NPHC_INST_M;
     if (ep.count <= 0 || ep.count < min_paths) return cudaSuccess;
     const size_t smem = g64_smem_per_block<M>();
-    auto k = xy_track_group64_kernel<M>;
-    static bool attr_set = false;   // once per process for this instantiation
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    constexpr auto k = xy_track_group64_kernel<M>;
     int dev = 0, sms = 0, per = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    cudaError_t e = allow_dynamic_smem<k>(smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 32, smem);
     if (e != cudaSuccess) return e;
@@ -306,15 +279,10 @@ cudaError_t NPHC_CAT(launch_xy_refine_certify_m, NPHC_INST_M)(const XYSys &sys, 
     if (cap <= 0) return cudaSuccess;
     constexpr int M = NPHC_INST_M;
     const size_t smem = rg_smem_per_block<M>();
-    auto k = xy_refine_group_kernel<M>;
-    static bool attr_set = false;   // once per process for this instantiation
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    constexpr auto k = xy_refine_group_kernel<M>;
     int dev = 0, sms = 0, per = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    cudaError_t e = allow_dynamic_smem<k>(smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 32, smem);
     if (e != cudaSuccess) return e;
@@ -335,15 +303,10 @@ cudaError_t NPHC_CAT(launch_xy_adjoint_m, NPHC_INST_M)(const XYSys &sys, int64_t
     if (count <= 0) return cudaSuccess;
     constexpr int M = NPHC_INST_M;
     const size_t smem = adj_smem_per_block<M>();
-    auto k = xy_adjoint_kernel<M>;
-    static bool attr_set = false;   // once per process for this instantiation
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    constexpr auto k = xy_adjoint_kernel<M>;
     int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    cudaError_t e = allow_dynamic_smem<k>(smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     // a warp per scheduler (the FP64 pipe is busy with one), fewer when a warp per point is fewer
@@ -363,15 +326,10 @@ cudaError_t NPHC_CAT(launch_xy_classify_m, NPHC_INST_M)(const XYSys &sys, const 
     if (ep.count <= 0) return cudaSuccess;
     constexpr int M = NPHC_INST_M;
     const size_t smem = cls_smem_per_block<M>();
-    auto k = xy_classify_kernel<M>;
-    static bool attr_set = false;   // once per process for this instantiation
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    constexpr auto k = xy_classify_kernel<M>;
     int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    cudaError_t e = allow_dynamic_smem<k>(smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     // a warp per scheduler, at most one point per warp (a list is at most ep.count long)
