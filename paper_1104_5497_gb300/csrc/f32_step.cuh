@@ -164,7 +164,8 @@ __device__ __forceinline__ F32Site f32_site(float2 p, float2 q, float2 Up, float
 // ------------------------------------------------------------ step control --
 // Time in units of 2^-53, the grid of the doubles in [1/2, 1): 1 - t is exact, and the step
 // logic costs no FP64 instruction (67 cycles of a scheduler each, measured, whatever the
-// number of lanes).
+// number of lanes).  Steps below one unit (an initial or largest step under 1.1e-16) are one unit: a
+// step rounded to 0 would never grow.
 typedef long long f32_time;
 #define F32_ONE (1ll << 53)
 __device__ __forceinline__ f32_time to_f32_time(double t) {   // clamped: beyond 256 no step differs
@@ -177,7 +178,8 @@ struct F32Ctl {   // XYCtl in the trackers' own units
     f32_time h0, hmax, hmin, tend, zone, near_end;
     float rdiv, rband, eps, trust, kappa;
     __device__ __forceinline__ explicit F32Ctl(const XYCtl &C)
-        : h0(to_f32_time(C.h0)), hmax(to_f32_time(C.hmax)), hmin(max(to_f32_time(C.hmin), (f32_time)1)),
+        : h0(max(to_f32_time(C.h0), (f32_time)1)), hmax(max(to_f32_time(C.hmax), (f32_time)1)),
+          hmin(max(to_f32_time(C.hmin), (f32_time)1)),
           tend(to_f32_time(C.t_end)), zone(to_f32_time(CRAWL_ZONE)), near_end(to_f32_time(NEAR_END)),
           rdiv((float)C.rdiv), rband((float)(C.rdiv * (1.0 + RDIV_BAND))), eps((float)C.eps),
           trust((float)C.trust), kappa((float)C.kappa) {}
