@@ -179,7 +179,13 @@ __global__ void __launch_bounds__(32)
                     double cs = 1.0, sn = 0.0;
                     const double apq = q < M ? H(p, q) : 0.0;
                     if (busy && apq != 0.0) {   // tan of the smaller angle: 2 apq / (d +- sqrt(d^2 + 4 apq^2))
-                        const double d = H(q, q) - H(p, p), h = 2.0 * apq;
+                        double d = H(q, q) - H(p, p), h = 2.0 * apq;
+                        const int ex = max(gexp(d), gexp(h));
+                        if (ex < -400 || ex > 400) {   // the squares below must neither vanish nor overflow
+                            const double by = __hiloint2double((1023 - min(max(ex, -1000), 1000)) << 20, 0);
+                            d *= by;
+                            h *= by;
+                        }
                         const double w = sqrt(fma(d, d, h * h));
                         const double tn = h / (d >= 0.0 ? d + w : d - w);
                         cs = rsqrt(fma(tn, tn, 1.0));
