@@ -18,7 +18,8 @@ sample (every path up to N = 10) the gate covers the whole ring.
 
 The list tracker's best shape depends on how long the hand-off list is, so the sample
 must reproduce it: by default it is every path up to N = 10 (262,144).  The result is
-cached in a JSON file under a key made of N, the GPU's name and its SM count.
+cached in a JSON file under a key made of N, the GPU's name, its SM count and the trackers'
+sources: what was measured on other kernels says nothing about these.
 
 Every step runs through the C ABI (nphc_track, nphc_refine_certify on caller-owned device
 buffers); this module only chooses options and times calls with CUDA events.
@@ -26,6 +27,8 @@ buffers); this module only chooses options and times calls with CUDA events.
 from __future__ import annotations
 
 import ctypes
+import functools
+import hashlib
 import json
 import os
 
@@ -33,7 +36,9 @@ import numpy as np
 
 from . import nphc as N_
 
-FP32_CANDIDATES = (0, 7, 6, 5, 4)   # resident warps per SM; 0 = the occupancy maximum
+# resident warps per SM; 0 = the occupancy maximum (7 or 8 with a path per thread, about 16 in blocks
+# of four with four lanes per path)
+FP32_CANDIDATES = (0, 12, 8, 6, 4)
 LIST_CANDIDATES = (2, 1, 3, 4)      # blocks of 4 warps per SM (the default, 2, first)
 # FP32 step control: (max_newton_fp32, eps_fp32); the defaults first
 STEP_CANDIDATES = ((3, 1e-5), (2, 1e-5), (3, 3e-5), (2, 3e-5))
@@ -57,8 +62,20 @@ def pick(timings: dict) -> int:
     return int(best)
 
 
+@functools.lru_cache(maxsize=None)
+def kernels() -> str:
+    """A hash of the trackers' sources (csrc/xy_*, what they include, and their launchers)."""
+    d = os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc")
+    h = hashlib.sha256()
+    for f in sorted(os.listdir(d)):
+        if f.startswith("xy_") or f in ("f32_step.cuh", "nphc_internal.cuh", "nphc_api.cu"):
+            with open(os.path.join(d, f), "rb") as fh:
+                h.update(f.encode() + b"\0" + fh.read())
+    return h.hexdigest()[:16]
+
+
 def cache_key(N: int, device_name: str, sms: int) -> str:
-    return f"N={N}|{device_name}|sms={sms}"
+    return f"N={N}|{device_name}|sms={sms}|kernels={kernels()}"
 
 
 def load_cache(path: str) -> dict:
