@@ -562,7 +562,7 @@ nphc_status track_impl(const nphc_system *S, const nphc_options *o, nphc_precisi
     const EPView v = view(ep);
     if (f32 && !resume && ep->count > 0) {
         NPHC_CK(launch_fill(fp32_counters(ws, S->n, ep->count, queue_slot), st));
-        NPHC_CK(launch_xy_track_f32(S->M, xs, ctl, v, wl, 0, sms * o->blocks_per_sm, st));
+        NPHC_CK(launch_xy_track_f32(S->M, xs, ctl, v, wl, sms * o->blocks_per_sm, st));
         return far_pass(S, o, v, list, list_count, ws, st);
     }
     NPHC_CK(cudaMemsetAsync(wl.queue, 0, sizeof(unsigned long long), st));
@@ -572,13 +572,14 @@ nphc_status track_impl(const nphc_system *S, const nphc_options *o, nphc_precisi
         // a resumed pass cannot be run again from its points: the per-thread kernel tracks all of it
         NPHC_CK(launch_xy_track_f32_thread(S->M, xs, ctl, v, wl, sms * o->blocks_per_sm, st));
     } else if (list != nullptr && o->threads_per_path == 1) {   // one path per thread, full warps
-        NPHC_CK(launch_xy_track_f64(S->M, xs, ctl, v, wl, 0, 0, st));
+        NPHC_CK(launch_xy_track_f64(S->M, xs, ctl, v, wl, 0, st));
     } else if (list != nullptr && o->threads_per_path == 32) {
         NPHC_CK(launch_xy_track_f64_warp(S->M, xs, ctl, v, wl, o->list_blocks_per_sm, INT64_MAX, st));
     } else {
         // One path per warp for few paths, four lanes per path for many; the length of a list
         // is on the device, so both kernels get it and one of them returns at once.
-        const int64_t few = (list != nullptr ? kFewListedPerScheduler : kFewPerScheduler) * 4 * sms;
+        const int64_t few = S->M < NPHC_GROUP64_MIN_M ? INT64_MAX
+                            : (list != nullptr ? kFewListedPerScheduler : kFewPerScheduler) * 4 * sms;
         if (list != nullptr || ep->count < few)
             NPHC_CK(launch_xy_track_f64_warp(S->M, xs, ctl, v, wl, o->list_blocks_per_sm, few, st));
         NPHC_CK(launch_xy_track_f64_group(S->M, xs, ctl, v, wl, few, st));

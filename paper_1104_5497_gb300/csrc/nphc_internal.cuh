@@ -300,9 +300,9 @@ struct BatchGroup {
 // ------------------------------------------------------ kernel launchers --
 // Implemented per precision / ring size in the .cu files; return cudaGetLastError().
 cudaError_t launch_xy_track_f32(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
-                                const WorkList &wl, int block, int grid, cudaStream_t st);
+                                const WorkList &wl, int grid, cudaStream_t st);
 cudaError_t launch_xy_track_f64(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
-                                const WorkList &wl, int block, int grid, cudaStream_t st);
+                                const WorkList &wl, int grid, cudaStream_t st);
 // FP32 tracking by the per-thread kernel (xy_track.cuh): far endpoints, resumed passes.
 cudaError_t launch_xy_track_f32_thread(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
                                        const WorkList &wl, int grid, cudaStream_t st);
@@ -334,5 +334,3 @@ cudaError_t launch_quad_cauchy(int n, const QSys &sys, const EGCtl &ctl, const E
                                const WorkList &wl, int32_t *cyc, int32_t *egst, cudaStream_t st);
 // Host-side count of kernel launches made by this library (for the result counters).
 int64_t nphc_launch_counter(int64_t add);
-int xy_track_f32_block(int M);
-int xy_track_f64_block(int M);

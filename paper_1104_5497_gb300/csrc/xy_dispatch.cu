@@ -2,8 +2,7 @@
 #include "xy_dispatch.cuh"
 
 cudaError_t launch_xy_track_f32(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
-                                const WorkList &wl, int block, int grid, cudaStream_t st) {
-    (void)block;
+                                const WorkList &wl, int grid, cudaStream_t st) {
 #define C(MM) case MM: return launch_xy_track_f32_m##MM(sys, ctl, ep, wl, grid, st);
     switch (M) { NPHC_FOR_EACH_M(C) default: return cudaErrorInvalidValue; }
 #undef C
@@ -24,8 +23,7 @@ cudaError_t launch_xy_track_f32_thread(int M, const XYSys &sys, const XYCtl &ctl
 }
 
 cudaError_t launch_xy_track_f64(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
-                                const WorkList &wl, int block, int grid, cudaStream_t st) {
-    (void)block;
+                                const WorkList &wl, int grid, cudaStream_t st) {
 #define C(MM) case MM: return launch_xy_track_f64_m##MM(sys, ctl, ep, wl, grid, st);
     switch (M) { NPHC_FOR_EACH_M(C) default: return cudaErrorInvalidValue; }
 #undef C
@@ -71,8 +69,6 @@ cudaError_t launch_xy_classify(int M, const XYSys &sys, const EPView &ep, double
 #undef C
 }
 
-int xy_track_f32_block(int M) { (void)M; return NPHC_TRACK_BLOCK; }
-int xy_track_f64_block(int M) { (void)M; return NPHC_TRACK_BLOCK; }
 
 cudaError_t launch_quad_track(int n, const QSys &sys, const XYCtl &ctl, const EPView &ep,
                               const WorkList &wl, cudaStream_t st) {

@@ -7,6 +7,7 @@
 #define NPHC_CAT(a, b) NPHC_CAT2(a, b)
 
 #define NPHC_TRACK_BLOCK 32   // one warp per block: per-thread shared memory, no block sync
+#define NPHC_GROUP64_MIN_M 7  // smaller rings have at most 4,096 paths: FP64 passes by a warp per path
 #define NPHC_M_MIN 2
 #define NPHC_M_MAX 12
 #define NPHC_FOR_EACH_M(X) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12)

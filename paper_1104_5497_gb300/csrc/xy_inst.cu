@@ -87,12 +87,15 @@ cudaError_t NPHC_CAT(launch_xy_track_f32t_m, NPHC_INST_M)(const XYSys &sys, cons
 //   three rows    N = 10 20,000 (0.6) 10.5 / 13.7, 32,768 (1.0) 14.2 / 14.0, 65,536 (1.9) 25.1 / 22.8,
 //                 262,144 (7.7) 96 / 73; N = 6 batch of 131,072 (1.9) 76.5 / 74.4
 // So lanes from that many waves on, by the number of padding rows, and never at M >= 11 (five
-// and four warps per SM): LANE_MAX_M.
-constexpr int LANE_MAX_M = 10;
-template <int M>
+// and four warps per SM): LANE_MAX_M.  One ring has at most 4^M paths, less than the line's waves up
+// to M = 8: only batches run the per-thread kernel there.
+constexpr int LANE_MAX_M = 10, LANE_MIN_M_SINGLE = 9;
+template <int M, bool BATCH>
+constexpr bool has_lanes = M <= LANE_MAX_M && (BATCH || M >= LANE_MIN_M_SINGLE);
+template <int M, bool BATCH>
 static bool use_group(int64_t items, int64_t wave) {
     constexpr int waves[4] = {8, 4, 6, 1};
-    return M > LANE_MAX_M || items < waves[GrpLayout<M>::ROWS - M] * wave;
+    return !has_lanes<M, BATCH> || items < waves[GrpLayout<M>::ROWS - M] * wave;
 }
 
 static cudaError_t device_sms(int &sms) {
@@ -115,7 +118,7 @@ static cudaError_t kernel_blocks(int threads, size_t smem, int &per) {
 template <int M, bool BATCH>
 static cudaError_t lane_blocks(int &per) {
     per = 0;
-    if constexpr (M <= LANE_MAX_M) {
+    if constexpr (has_lanes<M, BATCH>) {
         const size_t smem = lane_smem_per_block<M>(BATCH);
         if constexpr (BATCH) return kernel_blocks<xy_track_lane_batch_kernel<M>>(NPHC_TRACK_BLOCK, smem, per);
         else return kernel_blocks<xy_track_lane_kernel<M>>(NPHC_TRACK_BLOCK, smem, per);
@@ -125,12 +128,12 @@ static cudaError_t lane_blocks(int &per) {
 template <int M>
 static void launch_lanes(int grid, const XYSys &sys, const XYCtl &ctl, const EPView &ep, const WorkList &wl,
                          cudaStream_t st) {
-    if constexpr (M <= LANE_MAX_M)
+    if constexpr (has_lanes<M, false>)
         xy_track_lane_kernel<M><<<grid, NPHC_TRACK_BLOCK, lane_smem_per_block<M>(false), st>>>(sys, ctl, ep, wl);
 }
 template <int M>
 static void launch_lanes_batch(int grid, const BatchGroup &bg, const XYCtl &ctl, const WorkList &wl, cudaStream_t st) {
-    if constexpr (M <= LANE_MAX_M)
+    if constexpr (has_lanes<M, true>)
         xy_track_lane_batch_kernel<M><<<grid, NPHC_TRACK_BLOCK, lane_smem_per_block<M>(true), st>>>(
             bg.sys, bg.ep, bg.off, bg.n, ctl, wl);
 }
@@ -159,7 +162,7 @@ cudaError_t NPHC_CAT(launch_xy_track_f32_m, NPHC_INST_M)(const XYSys &sys, const
     if (e == cudaSuccess) e = lane_blocks<M, false>(per_t);
     if (e == cudaSuccess) e = kernel_blocks<kg>(32 * GRP_WARPS, smem_g, per_g);
     if (e != cudaSuccess) return e;
-    if (use_group<M>(ep.count, (int64_t)sms * per_t * BLK)) {
+    if (use_group<M, false>(ep.count, (int64_t)sms * per_t * BLK)) {
         const int gg = group_grid(sms, per_g, grid, ep.count, wl.state_threads);
         if (gg <= 0) return cudaErrorInvalidValue;
         kg<<<gg, 32 * GRP_WARPS, smem_g, st>>>(sys, ctl, ep, wl);
@@ -189,7 +192,7 @@ cudaError_t NPHC_CAT(launch_xy_track_f32_batch_m, NPHC_INST_M)(const BatchGroup 
     if (e == cudaSuccess) e = lane_blocks<M, true>(per_t);
     if (e == cudaSuccess) e = kernel_blocks<kg>(32 * GRP_WARPS, smem_g, per_g);
     if (e != cudaSuccess) return e;
-    if (use_group<M>(bg.total, (int64_t)sms * per_t * BLK)) {
+    if (use_group<M, true>(bg.total, (int64_t)sms * per_t * BLK)) {
         const int gg = group_grid(sms, per_g, grid, bg.total, wl.state_threads);
         if (gg <= 0) return cudaErrorInvalidValue;
         kg<<<gg, 32 * GRP_WARPS, smem_g, st>>>(bg.sys, bg.ep, bg.off, bg.n, ctl, wl);
@@ -242,6 +245,12 @@ cudaError_t NPHC_CAT(launch_xy_track_f64w_m, NPHC_INST_M)(const XYSys &sys, cons
 }
 
 // four lanes per path, for min_paths paths or more
+#if NPHC_INST_M < NPHC_GROUP64_MIN_M
+cudaError_t NPHC_CAT(launch_xy_track_f64g_m, NPHC_INST_M)(const XYSys &, const XYCtl &, const EPView &ep,
+                                                          const WorkList &, int64_t min_paths, cudaStream_t) {
+    return ep.count < min_paths ? cudaSuccess : cudaErrorInvalidValue;
+}
+#else
 cudaError_t NPHC_CAT(launch_xy_track_f64g_m, NPHC_INST_M)(const XYSys &sys, const XYCtl &ctl,
                                                           const EPView &ep, const WorkList &wl,
                                                           int64_t min_paths, cudaStream_t st) {
@@ -261,6 +270,8 @@ cudaError_t NPHC_CAT(launch_xy_track_f64g_m, NPHC_INST_M)(const XYSys &sys, cons
     nphc_launch_counter(1);
     return cudaGetLastError();
 }
+#endif
+
 cudaError_t NPHC_CAT(launch_xy_track_f64_m, NPHC_INST_M)(const XYSys &sys, const XYCtl &ctl,
                                                          const EPView &ep, const WorkList &wl,
                                                          int grid, cudaStream_t st) {

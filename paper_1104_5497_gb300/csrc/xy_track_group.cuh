@@ -434,7 +434,7 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
     const F32Ctl K(C);
     int64_t e = pth < per ? -1 : -2;   // entry of this path slot; -1 idle, -2 drained
     int inst = 0;                      // instance of the entry (batches)
-    int ph = 0;                        // phase: 0 re-anchor, 1 .. 3 RK4 stages, 4 .. corrector
+    int ph = 1;                        // phase: 1 .. 3 RK4 stages, 4 .. corrector
     F32Step P;
     P.start(0, 0);
     bool bad = false, start = false;   // start: a new step attempt begins
@@ -472,56 +472,33 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
                 const EPView &ep = src.eps(inst);
                 const int64_t cnt = ep.count;
                 P.steps = P.solves = P.newton = 0;
-                if (C.resume || C.accumulate) {
-                    P.steps = ep.steps[e];
-                    P.solves = ep.solves[e];
-                    P.newton = ep.newton[e];
-                }
                 kstep = 0.0f;
                 bad = false;
-                if (C.resume) {
+                const int64_t path = ep.path[e];
+                const cx<float> ig = crecip(gam);
 #pragma unroll 1
-                    for (int q = 0; q < SL; q++) {
-                        const int k = site(q);
-                        const double xr = ep.z_re[k * cnt + e], xi = ep.z_im[k * cnt + e];
-                        const double yr = ep.z_re[(M + k) * cnt + e], yi = ep.z_im[(M + k) * cnt + e];
-                        if (own(q))
-                            at(L::Z0, k) = at(L::PQ, k) = make_float4((float)(xr - yi), (float)(xi + yr),
-                                                                      (float)(xr + yi), (float)(xi - yr));
+                for (int q = 0; q < SL; q++) {
+                    const int k = site(q);
+                    float u = J.val(q, M), v = 0.0f;
+#pragma unroll 1
+                    for (int l = 0; l < M; l++) {
+                        const float jl = J.val(q, l);
+                        u += ((path >> l) & 1) ? -jl : jl;
+                        v += ((path >> (M + l)) & 1) ? -jl : jl;
                     }
-                    // restart with a step on the scale of 1 - t: the FP32 pass may have been
-                    // crawling with a far smaller one
-                    const double t0 = ep.t[e];
-                    P.start(to_f32_time(t0),
-                            to_f32_time(fmax(fmin(fmax(ep.h[e], 0.125 * (1.0 - t0)), C.hmax), C.hmin * 4.0)));
-                    ph = 0;
-                } else {
-                    const int64_t path = ep.path[e];
-                    const cx<float> ig = crecip(gam);
-#pragma unroll 1
-                    for (int q = 0; q < SL; q++) {
-                        const int k = site(q);
-                        float u = J.val(q, M), v = 0.0f;
-#pragma unroll 1
-                        for (int l = 0; l < M; l++) {
-                            const float jl = J.val(q, l);
-                            u += ((path >> l) & 1) ? -jl : jl;
-                            v += ((path >> (M + l)) & 1) ? -jl : jl;
-                        }
-                        const float x = ((path >> k) & 1) ? -1.0f : 1.0f;
-                        const float y = ((path >> (M + k)) & 1) ? -1.0f : 1.0f;
-                        cx<float> rf, rg;
-                        minus_ht_rows<float>(cx<float>{x, 0.0f}, cx<float>{y, 0.0f}, cx<float>{u, 0.0f},
-                                             cx<float>{v, 0.0f}, gam, rf, rg);
-                        const cx<float> dx = cscale(0.5f * x, cmul(ig, rf)), dy = cscale(0.5f * y, cmul(ig, rg));
-                        if (own(q)) {
-                            at(L::Z0, k) = make_float4(x, y, x, -y);   // p = x + i y, q = x - i y
-                            at(L::K1, k) = make_float4(dx.re - dy.im, dx.im + dy.re, dx.re + dy.im, dx.im - dy.re);
-                        }
+                    const float x = ((path >> k) & 1) ? -1.0f : 1.0f;
+                    const float y = ((path >> (M + k)) & 1) ? -1.0f : 1.0f;
+                    cx<float> rf, rg;
+                    minus_ht_rows<float>(cx<float>{x, 0.0f}, cx<float>{y, 0.0f}, cx<float>{u, 0.0f},
+                                         cx<float>{v, 0.0f}, gam, rf, rg);
+                    const cx<float> dx = cscale(0.5f * x, cmul(ig, rf)), dy = cscale(0.5f * y, cmul(ig, rg));
+                    if (own(q)) {
+                        at(L::Z0, k) = make_float4(x, y, x, -y);   // p = x + i y, q = x - i y
+                        at(L::K1, k) = make_float4(dx.re - dy.im, dx.im + dy.re, dx.re + dy.im, dx.im - dy.re);
                     }
-                    P.start(0, K.h0);
-                    start = true;
                 }
+                P.start(0, K.h0);
+                start = true;
             }
         }
         const bool any = __any_sync(0xffffffffu, e >= 0);
@@ -547,7 +524,7 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
         }
 
         // ---- which solve runs now, and for whom
-        const bool wants_c = act && (ph == 0 || ph >= 4);
+        const bool wants_c = act && ph >= 4;
         int nc, np;
         if (together) {
             nc = __syncthreads_count(wants_c);
@@ -560,7 +537,7 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
         const bool corr = nc > 0 && 2 * nc >= np;
         const bool w = act && wants_c == corr;
         if (together && !__any_sync(0xffffffffu, w)) continue;
-        const f32_time te = ph == 0 ? P.t : ph < 3 ? P.t + hh / 2 : t1;
+        const f32_time te = ph < 3 ? P.t + hh / 2 : t1;
         int verdict = STEP_GO_ON, status = NPHC_PATH_RUNNING;
         float zi = 0.0f;
         GrpStep<SL> dt, dr;
@@ -600,8 +577,7 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
                 if (ph == 4 && bad) verdict = STEP_REJECT;
             }
         } else {
-            // ---- corrector iteration (phase 0: a resumed point pulled onto this precision's
-            // path, its dz/dt taken from the same solve)
+            // ---- corrector iteration
             float dd = 0.0f;
 #pragma unroll
             for (int q = 0; q < SL; q++)
@@ -631,10 +607,7 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
                 P.solves++;
                 P.newton++;
                 kstep = fmaxf(kstep, kest);
-                if (ph == 0) {
-                    verdict = STEP_ANCHORED;
-                    if (!oks) status = C.handoff ? NPHC_PATH_HANDOFF : NPHC_PATH_NONFINITE;
-                } else if (move && dn <= K.eps * (1.0f + sqrtf(0.5f * zz))) {
+                if (move && dn <= K.eps * (1.0f + sqrtf(0.5f * zz))) {
                     // a converged step whose systems' condition estimate exceeds kappa (0: no
                     // test) is not taken: FP64 continues the path from its last accepted
                     // point (or the end zone's clean checkpoint)
@@ -645,7 +618,7 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
                 } else {
                     ph++;
                 }
-                if ((verdict == STEP_ACCEPT || verdict == STEP_ANCHORED) && status == NPHC_PATH_RUNNING) {
+                if (verdict == STEP_ACCEPT && status == NPHC_PATH_RUNNING) {
 #pragma unroll
                     for (int q = 0; q < SL; q++)
                         if (own(q)) {
@@ -667,7 +640,7 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
                 for (int q = 0; q < SL; q++)
                     if (own(q)) ck[(g + 4 * q) * slots] = at(L::PQ, g + 4 * q);
             }
-            if (verdict != STEP_ANCHORED) kstep = 0.0f;
+            kstep = 0.0f;
             start = status == NPHC_PATH_RUNNING;
             if (!start) {
                 const EPView &ep = src.eps(inst);

@@ -365,7 +365,7 @@ __device__ __forceinline__ void lane_track_body(const Src &src, const XYCtl &C, 
     const F32Ctl K(C);
     int64_t e = -1;   // entry; -1 idle, -2 drained
     int inst = 0;     // its instance (batches)
-    int ph = 0;       // phase: 0 re-anchor, 1 .. 3 RK4 stages, 4 .. corrector
+    int ph = 1;       // phase: 1 .. 3 RK4 stages, 4 .. corrector
     F32Step P;
     P.start(0, 0);
     bool bad = false, start = false, take = false, save = false;
@@ -393,52 +393,31 @@ __device__ __forceinline__ void lane_track_body(const Src &src, const XYCtl &C, 
                         gam = f2((float)src.sys(inst).gre, (float)src.sys(inst).gim);
                     }
                     P.steps = P.solves = P.newton = 0;
-                    if (C.resume || C.accumulate) {
-                        P.steps = ep.steps[e];
-                        P.solves = ep.solves[e];
-                        P.newton = ep.newton[e];
-                    }
                     kstep = 0.0f;
                     bad = false;
-                    if (C.resume) {
+                    const int64_t path = ep.path[e];
+                    const cx<float> cg = {gam.x, gam.y}, ig = crecip(cg);
 #pragma unroll 1
-                        for (int k = 0; k < M; k++) {
-                            const double xr = ep.z_re[k * cnt + e], xi = ep.z_im[k * cnt + e];
-                            const double yr = ep.z_re[(M + k) * cnt + e], yi = ep.z_im[(M + k) * cnt + e];
-                            Z0.at(k) = mem.pq(k) = make_float4((float)(xr - yi), (float)(xi + yr),
-                                                               (float)(xr + yi), (float)(xi - yr));
+                    for (int k = 0; k < M; k++) {
+                        const float *Jk = J.base + k * J.ROW;
+                        float u = Jk[M], v = 0.0f;
+#pragma unroll 1
+                        for (int l = 0; l < M; l++) {
+                            const float jl = Jk[l];
+                            u += ((path >> l) & 1) ? -jl : jl;
+                            v += ((path >> (M + l)) & 1) ? -jl : jl;
                         }
-                        // restart with a step on the scale of 1 - t: the FP32 pass may have been
-                        // crawling with a far smaller one
-                        const double t0 = ep.t[e];
-                        P.start(to_f32_time(t0),
-                                to_f32_time(fmax(fmin(fmax(ep.h[e], 0.125 * (1.0 - t0)), C.hmax), C.hmin * 4.0)));
-                        ph = 0;
-                    } else {
-                        const int64_t path = ep.path[e];
-                        const cx<float> cg = {gam.x, gam.y}, ig = crecip(cg);
-#pragma unroll 1
-                        for (int k = 0; k < M; k++) {
-                            const float *Jk = J.base + k * J.ROW;
-                            float u = Jk[M], v = 0.0f;
-#pragma unroll 1
-                            for (int l = 0; l < M; l++) {
-                                const float jl = Jk[l];
-                                u += ((path >> l) & 1) ? -jl : jl;
-                                v += ((path >> (M + l)) & 1) ? -jl : jl;
-                            }
-                            const float x = ((path >> k) & 1) ? -1.0f : 1.0f;
-                            const float y = ((path >> (M + k)) & 1) ? -1.0f : 1.0f;
-                            cx<float> rf, rg;
-                            minus_ht_rows<float>(cx<float>{x, 0.0f}, cx<float>{y, 0.0f}, cx<float>{u, 0.0f},
-                                                 cx<float>{v, 0.0f}, cg, rf, rg);
-                            const cx<float> dx = cscale(0.5f * x, cmul(ig, rf)), dy = cscale(0.5f * y, cmul(ig, rg));
-                            Z0.at(k) = make_float4(x, y, x, -y);   // p = x + i y, q = x - i y
-                            K1.at(k) = make_float4(dx.re - dy.im, dx.im + dy.re, dx.re + dy.im, dx.im - dy.re);
-                        }
-                        P.start(0, K.h0);
-                        start = true;
+                        const float x = ((path >> k) & 1) ? -1.0f : 1.0f;
+                        const float y = ((path >> (M + k)) & 1) ? -1.0f : 1.0f;
+                        cx<float> rf, rg;
+                        minus_ht_rows<float>(cx<float>{x, 0.0f}, cx<float>{y, 0.0f}, cx<float>{u, 0.0f},
+                                             cx<float>{v, 0.0f}, cg, rf, rg);
+                        const cx<float> dx = cscale(0.5f * x, cmul(ig, rf)), dy = cscale(0.5f * y, cmul(ig, rg));
+                        Z0.at(k) = make_float4(x, y, x, -y);   // p = x + i y, q = x - i y
+                        K1.at(k) = make_float4(dx.re - dy.im, dx.im + dy.re, dx.re + dy.im, dx.im - dy.re);
                     }
+                    P.start(0, K.h0);
+                    start = true;
                 }
             }
         }
@@ -472,12 +451,12 @@ __device__ __forceinline__ void lane_track_body(const Src &src, const XYCtl &C, 
         }
 
         // ---- which solve runs now, and for whom
-        const bool wants_c = act && (ph == 0 || ph >= 4);
+        const bool wants_c = act && ph >= 4;
         const int nc = __popc(__ballot_sync(0xffffffffu, wants_c));
         const int np = __popc(__ballot_sync(0xffffffffu, act && !wants_c));
         const bool corr = nc > 0 && 2 * nc >= np;
         const bool w = act && wants_c == corr;
-        const f32_time te = ph == 0 ? P.t : ph < 3 ? P.t + hh / 2 : t1;
+        const f32_time te = ph < 3 ? P.t + hh / 2 : t1;
         LanePost<M> post{mem, Z0, K1, AC, w, corr, ph, ph == 1 ? 0.5f * hr : ph == 2 ? hr : hr * (1.0f / 6.0f),
                          0.0f, 0.0f, 0.0f};
         float kest;
@@ -497,10 +476,7 @@ __device__ __forceinline__ void lane_track_body(const Src &src, const XYCtl &C, 
             const float dn = sqrtf(0.5f * post.dd);
             zi = 0.5f * sqrtf(post.zi);    // ||(x, y)||_inf
             const bool fail = !oks || !isfinite(dn) || (ph == 4 && dn > K.trust * (1.0f + zpn));
-            if (ph == 0) {   // a resumed point pulled onto this precision's path
-                verdict = STEP_ANCHORED;
-                if (!oks) status = C.handoff ? NPHC_PATH_HANDOFF : NPHC_PATH_NONFINITE;
-            } else if (!fail && dn <= K.eps * (1.0f + sqrtf(0.5f * post.zz))) {
+            if (!fail && dn <= K.eps * (1.0f + sqrtf(0.5f * post.zz))) {
                 // a converged step whose systems' condition estimate exceeds kappa (0: no test) is
                 // not taken: FP64 continues the path from its last accepted point (or the
                 // end zone's clean checkpoint)
@@ -519,7 +495,7 @@ __device__ __forceinline__ void lane_track_body(const Src &src, const XYCtl &C, 
         if (verdict == STEP_ACCEPT && take) status = P.accept(K, C, t1, zi, save);
         else if (verdict == STEP_REJECT) status = P.reject(K, C);
         status = P.budget(C, status);
-        if (verdict != STEP_ANCHORED) kstep = 0.0f;
+        kstep = 0.0f;
         start = status == NPHC_PATH_RUNNING;
         if (!start) {
             const EPView &ep = src.eps(inst);

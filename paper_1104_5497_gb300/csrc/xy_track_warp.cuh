@@ -532,8 +532,8 @@ __device__ __forceinline__ void warp_track_body(const typename Q::Sys &S, const 
         if ((int64_t)q >= total) break;
         const int64_t e = worklist_entry(wl, (int64_t)q, ep.count);
         if (e < 0) continue;   // rejected by the debug build's check
-        int status = NPHC_PATH_RUNNING, run = 0, rejects = 0, attempts = 0, steps, solves, newton;
-        double t, h, hacc;
+        int status = NPHC_PATH_RUNNING, run = 0, attempts = 0, steps, solves, newton;
+        double t, h;
         bool need_k1;
         if (C.resume) {
             Q::load(P, ep, e);
@@ -553,7 +553,6 @@ __device__ __forceinline__ void warp_track_body(const typename Q::Sys &S, const 
             newton = C.accumulate ? ep.newton[e] : 0;
             need_k1 = false;
         }
-        hacc = h;
         bool far = false;      // heading out: steps capped at KAPPA_FAR (1 - t) (xy_track.cuh)
         double zlast = 0.0;
         __syncwarp();
@@ -646,8 +645,6 @@ __device__ __forceinline__ void warp_track_body(const typename Q::Sys &S, const 
                 far = 1.0 - t < CRAWL_ZONE && zi > FAR_NORM && zi > FAR_GROWTH * zlast;
                 zlast = zi;
                 steps++;
-                rejects = 0;
-                hacc = h;
                 if (++run >= C.grow_after) {
                     run = 0;
                     h = fmin(2.0 * h, C.hmax);
@@ -656,7 +653,6 @@ __device__ __forceinline__ void warp_track_body(const typename Q::Sys &S, const 
                 else if (t >= C.t_end) status = NPHC_PATH_REACHED;
             } else {
                 run = 0;
-                rejects++;
                 h *= 0.5;
                 if (h < C.hmin) status = NPHC_PATH_MIN_STEP;
             }
