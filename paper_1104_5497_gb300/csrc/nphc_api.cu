@@ -513,8 +513,10 @@ EPView view(const nphc_endpoints *e) {
 // 20 ms by warps and 29 by groups (13.5 by warps now).
 constexpr int64_t kFewPerScheduler = 10, kFewListedPerScheduler = 32;
 
-// The far endpoints of an FP32 pass, tracked again by the per-thread kernel (a path's result then
-// never depends on the kernel that the launch's size chose).  The pass cleared queue slot 5 and
+constexpr int64_t kFarPerScheduler = 16;
+
+// The far endpoints of an FP32 pass, tracked again in the per-thread tracker's arithmetic (a path's
+// result then never depends on the kernel that the launch's size chose).  The pass cleared queue slot 5 and
 // the count.
 nphc_status far_pass(const nphc_system *S, const nphc_options *o, const EPView &v, const int32_t *list,
                      const int32_t *list_count, void *ws, cudaStream_t st) {
@@ -530,12 +532,14 @@ nphc_status far_pass(const nphc_system *S, const nphc_options *o, const EPView &
     wl.queue = ws_queue(ws, kFarQueue);
     wl.state = static_cast<char *>(ws) + L.state;
     wl.state_threads = NPHC_TRACK_MAX_THREADS;
-    // one warp per scheduler: a hundred paths, each a chain of dependent solves
     int dev = 0, sms = 0;
     NPHC_CK(cudaGetDevice(&dev));
     NPHC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    NPHC_CK(launch_xy_track_f32_thread(S->M, sys_with_gamma(S, o), ctl, v, wl,
-                                       (int)std::min<int64_t>(4 * sms, v.count), st));
+    // the length of the list is on the device: both kernels get it and one returns at once
+    const XYSys xs = sys_with_gamma(S, o);
+    const int64_t many = kFarPerScheduler * 4 * sms;
+    NPHC_CK(launch_xy_track_f32_warp(S->M, xs, ctl, v, wl, many, st));
+    NPHC_CK(launch_xy_track_f32_thread(S->M, xs, ctl, v, wl, 0, many, st));
     return NPHC_OK;
 }
 
@@ -570,7 +574,7 @@ nphc_status track_impl(const nphc_system *S, const nphc_options *o, nphc_precisi
         NPHC_CK(launch_quad_track(S->n, quad_with_gamma(S, o), ctl, v, wl, st));
     } else if (f32) {
         // a resumed pass cannot be run again from its points: the per-thread kernel tracks all of it
-        NPHC_CK(launch_xy_track_f32_thread(S->M, xs, ctl, v, wl, sms * o->blocks_per_sm, st));
+        NPHC_CK(launch_xy_track_f32_thread(S->M, xs, ctl, v, wl, sms * o->blocks_per_sm, 0, st));
     } else if (list != nullptr && o->threads_per_path == 1) {   // one path per thread, full warps
         NPHC_CK(launch_xy_track_f64(S->M, xs, ctl, v, wl, 0, st));
     } else if (list != nullptr && o->threads_per_path == 32) {

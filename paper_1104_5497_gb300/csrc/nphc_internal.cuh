@@ -303,9 +303,13 @@ cudaError_t launch_xy_track_f32(int M, const XYSys &sys, const XYCtl &ctl, const
                                 const WorkList &wl, int grid, cudaStream_t st);
 cudaError_t launch_xy_track_f64(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
                                 const WorkList &wl, int grid, cudaStream_t st);
-// FP32 tracking by the per-thread kernel (xy_track.cuh): far endpoints, resumed passes.
+// FP32 tracking by the per-thread kernel (xy_track.cuh) of launches and lists of min_paths or more, and
+// with one path per warp (xy_track_warp32.cuh), from t = 0, of those below max_paths; either gives a
+// path the same result bit for bit.  For far endpoints and resumed passes.
 cudaError_t launch_xy_track_f32_thread(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
-                                       const WorkList &wl, int grid, cudaStream_t st);
+                                       const WorkList &wl, int grid, int64_t min_paths, cudaStream_t st);
+cudaError_t launch_xy_track_f32_warp(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
+                                     const WorkList &wl, int64_t max_paths, cudaStream_t st);
 // The FP32 pass over every path of a batch group (ring size M), one persistent launch.
 cudaError_t launch_xy_track_f32_batch(int M, const BatchGroup &bg, const XYCtl &ctl,
                                       const WorkList &wl, int grid, cudaStream_t st);

@@ -16,8 +16,15 @@ cudaError_t launch_xy_track_f32_batch(int M, const BatchGroup &bg, const XYCtl &
 }
 
 cudaError_t launch_xy_track_f32_thread(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
-                                       const WorkList &wl, int grid, cudaStream_t st) {
-#define C(MM) case MM: return launch_xy_track_f32t_m##MM(sys, ctl, ep, wl, grid, st);
+                                       const WorkList &wl, int grid, int64_t min_paths, cudaStream_t st) {
+#define C(MM) case MM: return launch_xy_track_f32t_m##MM(sys, ctl, ep, wl, grid, min_paths, st);
+    switch (M) { NPHC_FOR_EACH_M(C) default: return cudaErrorInvalidValue; }
+#undef C
+}
+
+cudaError_t launch_xy_track_f32_warp(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
+                                     const WorkList &wl, int64_t max_paths, cudaStream_t st) {
+#define C(MM) case MM: return launch_xy_track_f32w_m##MM(sys, ctl, ep, wl, max_paths, st);
     switch (M) { NPHC_FOR_EACH_M(C) default: return cudaErrorInvalidValue; }
 #undef C
 }

@@ -41,7 +41,7 @@ cudaError_t NPHC_CAT(launch_xy_cauchy_m, NPHC_INST_M)(const XYSys &sys, const EG
 // The per-thread tracker (xy_track.cuh) over the list or every entry of the launch.
 template <int M, class R>
 static cudaError_t launch_per_thread(const XYSys &sys, const XYCtl &ctl, const EPView &ep,
-                                     const WorkList &wl, int grid, cudaStream_t st) {
+                                     const WorkList &wl, int grid, int64_t min_paths, cudaStream_t st) {
     constexpr int BLK = NPHC_TRACK_BLOCK;
     const size_t smem = xy_smem_per_thread<M, R>() * BLK;
     constexpr auto k = xy_track_kernel<M, R, BLK>;
@@ -56,7 +56,7 @@ static cudaError_t launch_per_thread(const XYSys &sys, const XYCtl &ctl, const E
     const int cap = (int)(wl.state_threads / BLK);  // the scratch holds state for this many
     if (grid > cap) grid = cap;
     if (grid <= 0) return cudaErrorInvalidValue;
-    k<<<grid, BLK, smem, st>>>(sys, ctl, ep, wl);
+    k<<<grid, BLK, smem, st>>>(sys, ctl, ep, wl, min_paths);
     nphc_launch_counter(1);
     return cudaGetLastError();
 }
@@ -65,11 +65,39 @@ static cudaError_t launch_per_thread(const XYSys &sys, const XYCtl &ctl, const E
 #if NPHC_INST_KIND == 0
 #include "xy_track_group.cuh"
 #include "xy_track_lane.cuh"
+#include "xy_track_warp32.cuh"
+
+static cudaError_t device_sms(int &sms) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return e;
+}
 
 cudaError_t NPHC_CAT(launch_xy_track_f32t_m, NPHC_INST_M)(const XYSys &sys, const XYCtl &ctl,
                                                           const EPView &ep, const WorkList &wl,
-                                                          int grid, cudaStream_t st) {
-    return launch_per_thread<NPHC_INST_M, float>(sys, ctl, ep, wl, grid, st);
+                                                          int grid, int64_t min_paths,
+                                                          cudaStream_t st) {
+    if (ep.count < min_paths) return cudaSuccess;   // a list is at most ep.count long
+    return launch_per_thread<NPHC_INST_M, float>(sys, ctl, ep, wl, grid, min_paths, st);
+}
+
+// one path per warp, 4 warps per block
+cudaError_t NPHC_CAT(launch_xy_track_f32w_m, NPHC_INST_M)(const XYSys &sys, const XYCtl &ctl,
+                                                          const EPView &ep, const WorkList &wl,
+                                                          int64_t max_paths, cudaStream_t st) {
+    constexpr int M = NPHC_INST_M, WARPS = 4;
+    if (ep.count <= 0) return cudaSuccess;
+    constexpr auto k = xy_track_warp32_kernel<M, WARPS>;
+    int sms = 0, per = 0;
+    cudaError_t e = device_sms(sms);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 32 * WARPS, 0);
+    if (e != cudaSuccess) return e;
+    const int64_t full = (int64_t)sms * std::max(per, 1);
+    const int64_t need = (std::min(ep.count, max_paths) + WARPS - 1) / WARPS;
+    k<<<(int)std::min(full, need), 32 * WARPS, 0, st>>>(sys, ctl, ep, wl, max_paths);
+    nphc_launch_counter(1);
+    return cudaGetLastError();
 }
 
 // The FP32 pass has two kernels: one path per thread (xy_track_lane.cuh) and four lanes per path
@@ -96,13 +124,6 @@ template <int M, bool BATCH>
 static bool use_group(int64_t items, int64_t wave) {
     constexpr int waves[4] = {8, 4, 6, 1};
     return !has_lanes<M, BATCH> || items < waves[GrpLayout<M>::ROWS - M] * wave;
-}
-
-static cudaError_t device_sms(int &sms) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return e;
 }
 
 // Shared memory opt-in and resident blocks per SM of a kernel.
@@ -275,7 +296,7 @@ cudaError_t NPHC_CAT(launch_xy_track_f64g_m, NPHC_INST_M)(const XYSys &sys, cons
 cudaError_t NPHC_CAT(launch_xy_track_f64_m, NPHC_INST_M)(const XYSys &sys, const XYCtl &ctl,
                                                          const EPView &ep, const WorkList &wl,
                                                          int grid, cudaStream_t st) {
-    return launch_per_thread<NPHC_INST_M, double>(sys, ctl, ep, wl, grid, st);
+    return launch_per_thread<NPHC_INST_M, double>(sys, ctl, ep, wl, grid, 0, st);
 }
 #endif
 

@@ -256,7 +256,7 @@ struct BatchSrc {
 
 template <class P>
 __device__ __forceinline__ void track_body(const typename P::Sys &S, const XYCtl &C, const EPView &ep,
-                                           const WorkList &wl) {
+                                           const WorkList &wl, int64_t min_paths) {
     using R = typename P::R;
     constexpr int BLOCK = P::BLOCK, NV = P::NV, MD = P::MD;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -274,6 +274,7 @@ __device__ __forceinline__ void track_body(const typename P::Sys &S, const XYCtl
     const GVec<R> AC{st + (2 * NV) * nth + gtid, nth};       // RK4 sum; next K1 in correction
     const GVec<R> CK{st + (3 * NV) * nth + gtid, nth};       // FP32 pass: hand-off checkpoint
     const int64_t total = worklist_size(wl, ep.count);
+    if (total < min_paths) return;   // another kernel's
 
     // short lists: at most `lanes` paths per warp, so that the list spreads over every SM
     // instead of filling the first warps 32 at a time (FP64 continuation of a few
@@ -559,6 +560,6 @@ __device__ __forceinline__ void track_body(const typename P::Sys &S, const XYCtl
 template <int M, class R, int BLOCK>
 __global__ void __launch_bounds__(BLOCK)
     xy_track_kernel(const __grid_constant__ XYSys S, const __grid_constant__ XYCtl C,
-                    const EPView ep, const WorkList wl) {
-    track_body<XYProblem<M, R, BLOCK>>(S, C, ep, wl);
+                    const EPView ep, const WorkList wl, int64_t min_paths) {
+    track_body<XYProblem<M, R, BLOCK>>(S, C, ep, wl, min_paths);
 }

@@ -107,3 +107,31 @@ def test_far_list_follows_the_refinement_tolerance():
     none = track(N_, system, opts, paths).tensors["solves"].cpu().numpy()
     assert base.sum() > none.sum() and more.sum() > base.sum()
     assert (base >= none).all() and (more >= base).all()
+
+
+@pytest.mark.parametrize("N,count", [(8, 65536 // 4), (11, 60001), (12, 80001), (13, 80001)])
+def test_short_and_long_lists_agree_bit_for_bit(N, count):
+    """Far paths are tracked by a warp each, or by a thread each when there are sixteen or more for every
+    scheduler.  With the line at 2^-4 every path that reaches t = 1 is far: the whole launch takes
+    the per-thread kernel (not at N = 8, where both are short lists), a tenth of it the other."""
+    import torch
+    N_ = nphc()
+    system, opts = ring(N_, N, 2000 + N)
+    opts.refine_eps = 0.01
+    paths = (np.arange(count, dtype=np.int64) * 7919) % system.npaths
+    all_ = track(N_, system, opts, paths)
+    reached = int((all_.tensors["status"] == N_.PATH_REACHED).sum())
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert N == 8 or reached >= 16 * 4 * sms
+    some = np.arange(0, count, 10)
+    few = track(N_, system, opts, paths[some])
+    assert (few.tensors["status"] == N_.PATH_REACHED).sum() < 16 * 4 * sms
+    same = all_.tensors["status"].cpu().numpy()[some] == few.tensors["status"].cpu().numpy()
+    assert same.mean() > 0.999   # (two FP32 kernels may run before: another path may be handed off)
+    at = same & (few.tensors["status"].cpu().numpy() == N_.PATH_REACHED)
+    assert at.sum() > 100
+    for k in ("z_re", "z_im", "t", "h", "steps"):
+        a, b = columns(all_, some, [k])[k], few.tensors[k].cpu().numpy()
+        if k == "steps" and N < 12:
+            continue   # counts of the pass before, of either kernel, included
+        assert np.array_equal(a[..., at], b[..., at]), k
