@@ -513,7 +513,11 @@ EPView view(const nphc_endpoints *e) {
 // 20 ms by warps and 29 by groups (13.5 by warps now).
 constexpr int64_t kFewPerScheduler = 10, kFewListedPerScheduler = 32;
 
-constexpr int64_t kFarPerScheduler = 16;
+
+// Far paths per scheduler from which the per-thread kernel beats a warp per path.  Measured (warp / thread,
+// ms): N = 10 193 paths 2.9 / 14.1, 7,294 7.9 / 20.0, 18,438 15.8 / 26.0, 37,032 28.1 / 22.3; N = 13 144
+// paths 3.5 / 16.9, 16,082 15.6 / 31.7, 64,796 56.9 / 60.7.  A default pass has hundreds.
+constexpr int64_t kFarPerScheduler = 64;
 
 // The far endpoints of an FP32 pass, tracked again in the per-thread tracker's arithmetic (a path's
 // result then never depends on the kernel that the launch's size chose).  The pass cleared queue slot 5 and

@@ -9,10 +9,9 @@
 // sums (the tests compare the two kernels' endpoints bit for bit).
 //
 // A pass is followed by one path's chain of dependent solves, so the time is that chain's latency:
-// per thread a solve is ten thousand instructions on one lane (262,144 paths of N = 10: the far ones took
-// 11 ms after a pass of 73; N = 13: 25 ms), here some two thousand.  Longer lists than
-// NPHC_FAR_PER_SCHEDULER for each scheduler are left to the per-thread kernel, which needs fewer
-// instructions per path.
+// per thread a solve is ten thousand instructions on one lane (193 paths of N = 10 14.1 ms, 144 of N = 13
+// 16.9), here some two thousand (2.9 and 3.5 ms).  Very long lists are left to the per-thread kernel, which needs
+// fewer instructions per path (kFarPerScheduler in nphc_api.cu).
 #pragma once
 
 #include "xy_track.cuh"
