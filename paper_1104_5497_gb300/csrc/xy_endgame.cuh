@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(32)
                 if (a <= -M_PI) a = M_PI;
                 theta[k * cnt + e] = a;
                 const double r2 = fma(x, x, y * y);
-                if (r2 > 0.0 && isfinite(r2)) {
+                if (r2 > 1e-280 && isfinite(r2)) {   // a subnormal r2 has lost its digits
                     const double ir = rsqrt(r2);
                     c = x * ir;
                     s = y * ir;
