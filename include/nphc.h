@@ -455,6 +455,9 @@ nphc_status nphc_result_copy_endgame(const nphc_result *res, int64_t cap, int32_
  * solved in mixed precision with the same FP32 step control (gamma and kappa_sing may
  * differ); otherwise, and for generic quadratic systems, each instance runs the whole of
  * nphc_solve_into on its stream.  Deduplication and classification stay per instance.
+ * The number of paths in a launch chooses its FP32 kernel (see nphc_track), so an
+ * instance's endpoints equal its single solve's to rounding, not bit for bit; far endpoints,
+ * whose class depends on rounding, come from one kernel in either.
  * --------------------------------------------------------------------------------- */
 #define NPHC_BATCH_STREAMS 8
 #define NPHC_BATCH_GRAPH 1          /* nphc_batch_solve flag: capture / replay a CUDA graph */

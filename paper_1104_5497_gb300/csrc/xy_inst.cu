@@ -101,19 +101,20 @@ cudaError_t NPHC_CAT(launch_xy_track_f32w_m, NPHC_INST_M)(const XYSys &sys, cons
 }
 
 // The FP32 pass has two kernels: one path per thread (xy_track_lane.cuh) and four lanes per path
-// (xy_track_group.cuh).  The first takes fewer instructions per path but one wave of it (19,000 to
-// 90,000 paths) takes its paths' latency however few they are; four lanes shorten every solve
-// and sixteen warps per SM hide each other's latency where four to ten cannot, at the price of
+// (xy_track_group.cuh).  The first takes fewer instructions per path but one wave of it (38,912 paths
+// up to M = 8, where registers hold it to eight warps per SM, 34,048 at M = 9, 29,184 at M = 10)
+// takes its paths' latency however few they are; four lanes shorten every solve, and eight (M = 12)
+// to fourteen warps per SM hide each other's latency better than six to eight, at the price of
 // the rows that pad M to a multiple of four.  Measured (GB300, FP32 pass alone or the whole batch,
-// group / lane, ms; in brackets the waves of lanes):
-//   no padding    N = 9 65,536 (1.5) 12.5 / 16.9, batches of 262,144 (6) 62 / 67, 524,288 (12) 184 / 168;
+// group / lane, ms; in brackets the waves of lanes; M >= 11 before it lost its lane kernel):
+//   no padding    N = 9 65,536 (1.7) 12.5 / 16.9, batches of 262,144 (6.7) 62 / 67, 524,288 (13.5) 184 / 168;
 //                 N = 13 262,144 (13.5) 126 / 186
-//   one row       N = 8 batches of 65,536 (1.2) 17.4 / 18.8, 196,608 (3.7) 61.4 / 59.6, 393,216 (7.3)
-//                 123 / 119; N = 12 262,144 (11) 114 / 133
-//   two rows      N = 7 batch of 163,840 (2.4) 46.1 / 47.5; N = 11 65,536 (2.2) 26.7 / 29.9, 131,072 (4.5)
-//                 49.6 / 50.6, 262,144 (9) 95.3 / 93.3
+//   one row       N = 8 batches of 65,536 (1.7) 17.4 / 18.8, 196,608 (5.1) 61.4 / 59.6, 393,216 (10.1)
+//                 123 / 119; N = 12 262,144 (10.8) 114 / 133
+//   two rows      N = 7 batch of 163,840 (4.2) 46.1 / 47.5; N = 11 65,536 (2.2) 26.7 / 29.9, 131,072 (4.5)
+//                 49.6 / 50.6, 262,144 (9.0) 95.3 / 93.3
 //   three rows    N = 10 20,000 (0.6) 10.5 / 13.7, 32,768 (1.0) 14.2 / 14.0, 65,536 (1.9) 25.1 / 22.8,
-//                 262,144 (7.7) 96 / 73; N = 6 batch of 131,072 (1.9) 76.5 / 74.4
+//                 262,144 (7.7) 96 / 73; N = 6 batch of 131,072 (3.4) 76.5 / 74.4
 // So lanes from that many waves on, by the number of padding rows, and never at M >= 11 (five
 // and four warps per SM): LANE_MAX_M.  One ring has at most 4^M paths, less than the line's waves up
 // to M = 8: only batches run the per-thread kernel there.

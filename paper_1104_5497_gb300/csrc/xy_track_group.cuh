@@ -19,8 +19,9 @@
 //   * Arithmetic in pairs (fma.rn.f32x2): (re, im) where the coefficient is real or a
 //     compensated sum runs, two neighbouring columns where both factors are complex.
 //   * Each path is in its own phase (an RK4 stage or a corrector iteration); a warp, or with
-//     full warps the block, runs, for all paths that wait for one, whichever of a predictor and a corrector solve has more
-//     takers (a corrector solve costs about twice as much, so it needs half as many).  In
+//     full warps the block, runs, for all paths that wait for one, whichever of a predictor and a
+//     corrector solve has more takers (a corrector solve costs about twice as much, so it needs
+//     half as many).  In
 //     lockstep a warp runs the correctors its slowest path needs (1.7 per step on average,
 //     three at worst).  A path's own sequence of operations does not depend on its company.
 //   * Time is an integer number of 2^-53, the grid of the doubles in [1/2, 1): 1 - t is exact
@@ -425,8 +426,8 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
         if (want < per) per = want < 1 ? 1 : (int)want;
     }
     // With full warps the block decides which solve runs, so that its four warps go through the same
-    // code at the same time: sixteen warps in sixteen places of a kernel of 60 to 90 KB waited for
-    // instructions two cycles per issue.  The pool of 32 paths fills the phases as well as
+    // code at the same time: an SM's warps (eight at M = 12 to fourteen at M <= 9) in as many places of a
+    // kernel of 60 to 90 KB waited for instructions two cycles per issue.  The pool of 32 paths fills the phases as well as
     // eight do (85% in a simulation of the mix).  N = 13 80,000 paths 58 -> 41 ms, N = 12 32,768
     // 24.4 -> 18.6, N = 11 19.1 -> 15.8, N = 9 65,536 13.7 -> 12.7.  With fewer paths no path waits for
     // the others of its block.
@@ -469,12 +470,10 @@ __device__ __forceinline__ void grp_track_body(const Src &src, const XYCtl &C, c
                 __syncwarp();
             }
             if (fresh) {
-                const EPView &ep = src.eps(inst);
-                const int64_t cnt = ep.count;
                 P.steps = P.solves = P.newton = 0;
                 kstep = 0.0f;
                 bad = false;
-                const int64_t path = ep.path[e];
+                const int64_t path = src.eps(inst).path[e];
                 const cx<float> ig = crecip(gam);
 #pragma unroll 1
                 for (int q = 0; q < SL; q++) {

@@ -386,8 +386,6 @@ __device__ __forceinline__ void lane_track_body(const Src &src, const XYCtl &C, 
                 if (i >= total) e = -2;
                 else src.take(i, inst, e);   // -1 (skipped) if the debug build rejects it
                 if (e >= 0) {
-                    const EPView &ep = src.eps(inst);
-                    const int64_t cnt = ep.count;
                     if (BATCH) {
                         J.base = src.sys(inst).Jf;
                         gam = f2((float)src.sys(inst).gre, (float)src.sys(inst).gim);
@@ -395,7 +393,7 @@ __device__ __forceinline__ void lane_track_body(const Src &src, const XYCtl &C, 
                     P.steps = P.solves = P.newton = 0;
                     kstep = 0.0f;
                     bad = false;
-                    const int64_t path = ep.path[e];
+                    const int64_t path = src.eps(inst).path[e];
                     const cx<float> cg = {gam.x, gam.y}, ig = crecip(cg);
 #pragma unroll 1
                     for (int k = 0; k < M; k++) {
