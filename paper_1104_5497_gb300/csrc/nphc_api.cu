@@ -461,6 +461,7 @@ XYSys sys_with_gamma(const nphc_system *S, const nphc_options *o) {
     x.gre = o->gamma_re;
     x.gim = o->gamma_im;
     x.kappa_sing = o->kappa_sing;
+    x.far_exp = far_exponent(o->refine_eps);
     return x;
 }
 
@@ -937,10 +938,6 @@ nphc_status solve_into_impl(const nphc_system *S, const nphc_options *o, nphc_re
             const Range r("fp32 pass");
             if ((s = track_impl(S, o, NPHC_PREC_MIXED, ep, nullptr, nullptr, false, false, R->ws, 0, st)))
                 return s;
-        } else {
-            const Range r("far endpoints of the group's fp32 pass");
-            NPHC_CK(launch_fill(fp32_counters(R->ws, R->n, R->P, kFarQueue), st));
-            if ((s = far_pass(S, o, v, nullptr, nullptr, R->ws, st))) return s;
         }
         Range r_tail("fp64 hand-offs, refinement, certification");
         // hand-offs: refinement at t = 1 straight from the hand-off point (certified ones
@@ -1312,16 +1309,18 @@ struct nphc_batch {
         int M = 0;
         std::vector<int> members;   // instance indices
         int base = 0;               // first row of the group in the device tables
+        int64_t far = 0;            // its first word in d_far
         cudaEvent_t done = nullptr;
     };
     std::vector<const nphc_system *> sys;
     std::vector<nphc_result *> res;
     std::vector<nphc_options> opts;   // options of the captured solve
     std::vector<Group> groups;
-    void *tab = nullptr;              // device: XYSys[count] | EPView[count] | int64_t[count + groups]
+    void *tab = nullptr;              // device: XYSys[count] | EPView[count] | int64_t[count + groups] | d_far
     XYSys *d_sys = nullptr;
     EPView *d_ep = nullptr;
     int64_t *d_off = nullptr;
+    int32_t *d_far = nullptr;         // per group: number and items of its far endpoints
     std::vector<nphc_options> tab_opts;   // options the XYSys rows were written with
     bool tab_valid = false;
     cudaStream_t streams[NPHC_BATCH_STREAMS] = {};
@@ -1412,8 +1411,15 @@ nphc_status batch_enqueue(nphc_batch *B, const nphc_options *opts, int mode, cud
                 grid = sms * o0->blocks_per_sm;
             }
             const Range r("batch group fp32 pass");
-            NPHC_CK(cudaMemsetAsync(wl.queue, 0, sizeof(unsigned long long), gs));
+            bg.far = B->d_far + G.far;
+            bg.far_queue = ws_queue(R0->ws, kFarQueue);
+            FillSet zero;
+            zero.add(wl.queue, sizeof(unsigned long long), 0);
+            zero.add(bg.far_queue, sizeof(unsigned long long), 0);
+            zero.add(bg.far, sizeof(int32_t), 0);
+            NPHC_CK(launch_fill(zero, gs));
             NPHC_CK(launch_xy_track_f32_batch(G.M, bg, ctl, wl, grid, gs));
+            NPHC_CK(launch_xy_track_far_batch(G.M, bg, make_ctl(o0, true, false, true), gs));
             NPHC_CK(cudaEventRecord(G.done, gs));
             for (int i : G.members) group_of[i] = (int)g;
         }
@@ -1512,7 +1518,13 @@ nphc_status nphc_batch_create(int count, const nphc_system *const *systems, nphc
     const size_t nrow = (size_t)(row > 0 ? row : 1), ng = B->groups.size();
     const size_t b_sys = align256(sizeof(XYSys) * nrow), b_ep = align256(sizeof(EPView) * nrow);
     const size_t b_off = align256(sizeof(int64_t) * (nrow + ng + 1));
-    cudaError_t e = cudaMalloc(&B->tab, b_sys + b_ep + b_off);
+    int64_t far = 0;
+    for (auto &G : B->groups) {
+        G.far = far;
+        far++;
+        for (int i : G.members) far += systems[i]->npaths;
+    }
+    cudaError_t e = cudaMalloc(&B->tab, b_sys + b_ep + b_off + sizeof(int32_t) * far);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return bail(fail(e == cudaErrorMemoryAllocation ? NPHC_ENOMEM : NPHC_ECUDA,
@@ -1521,6 +1533,7 @@ nphc_status nphc_batch_create(int count, const nphc_system *const *systems, nphc
     B->d_sys = reinterpret_cast<XYSys *>(B->tab);
     B->d_ep = reinterpret_cast<EPView *>(static_cast<char *>(B->tab) + b_sys);
     B->d_off = reinterpret_cast<int64_t *>(static_cast<char *>(B->tab) + b_sys + b_ep);
+    B->d_far = reinterpret_cast<int32_t *>(static_cast<char *>(B->tab) + b_sys + b_ep + b_off);
     std::vector<EPView> eps(nrow);
     std::vector<int64_t> off;
     for (const auto &G : B->groups) {

@@ -179,6 +179,7 @@ inline int far_exponent(double refine_eps) {
 // unrolled kernels read them as constant-bank operands.
 struct XYSys {
     int N;                                  // ring size; M = N - 1 free sites
+    int far_exp;                            // far_exponent of the call's refine_eps
     alignas(16) float Jf[NPHC_MAXN * NPHC_JSTRIDE];   // J in FP32 (row k, column j at
                                                       // k * NPHC_JSTRIDE + j; zeros beyond)
     double Jd[NPHC_MAXN * NPHC_JSTRIDE];    // J in FP64
@@ -295,6 +296,8 @@ struct BatchGroup {
     const int64_t *off;
     int n;
     int64_t total;   // off[n], on the host
+    int32_t *far;    // [1 + total] the far endpoints' number and items (scratch)
+    unsigned long long *far_queue;
 };
 
 // ------------------------------------------------------ kernel launchers --
@@ -313,6 +316,9 @@ cudaError_t launch_xy_track_f32_warp(int M, const XYSys &sys, const XYCtl &ctl, 
 // The FP32 pass over every path of a batch group (ring size M), one persistent launch.
 cudaError_t launch_xy_track_f32_batch(int M, const BatchGroup &bg, const XYCtl &ctl,
                                       const WorkList &wl, int grid, cudaStream_t st);
+// The group's far endpoints, listed and tracked again (xy_track_warp32.cuh); bg.far[0] and the queue
+// are 0 before.
+cudaError_t launch_xy_track_far_batch(int M, const BatchGroup &bg, const XYCtl &ctl, cudaStream_t st);
 cudaError_t launch_xy_refine_certify(int M, const XYSys &sys, double tol_sol, double refine_eps,
                                      int refine_iters, const EPView &ep, int64_t cap,
                                      const WorkList &wl, int shortcut, cudaStream_t st);

@@ -29,6 +29,12 @@ cudaError_t launch_xy_track_f32_warp(int M, const XYSys &sys, const XYCtl &ctl, 
 #undef C
 }
 
+cudaError_t launch_xy_track_far_batch(int M, const BatchGroup &bg, const XYCtl &ctl, cudaStream_t st) {
+#define C(MM) case MM: return launch_xy_track_far_batch_m##MM(bg, ctl, st);
+    switch (M) { NPHC_FOR_EACH_M(C) default: return cudaErrorInvalidValue; }
+#undef C
+}
+
 cudaError_t launch_xy_track_f64(int M, const XYSys &sys, const XYCtl &ctl, const EPView &ep,
                                 const WorkList &wl, int grid, cudaStream_t st) {
 #define C(MM) case MM: return launch_xy_track_f64_m##MM(sys, ctl, ep, wl, grid, st);

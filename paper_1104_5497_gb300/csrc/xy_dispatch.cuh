@@ -21,6 +21,7 @@
                                            const WorkList &, int, int64_t, cudaStream_t);    \
     cudaError_t launch_xy_track_f32w_m##MM(const XYSys &, const XYCtl &, const EPView &,    \
                                            const WorkList &, int64_t, cudaStream_t);         \
+    cudaError_t launch_xy_track_far_batch_m##MM(const BatchGroup &, const XYCtl &, cudaStream_t); \
     cudaError_t launch_xy_track_f64_m##MM(const XYSys &, const XYCtl &, const EPView &,     \
                                           const WorkList &, int, cudaStream_t);              \
     cudaError_t launch_xy_track_f64w_m##MM(const XYSys &, const XYCtl &, const EPView &,    \

@@ -100,6 +100,26 @@ cudaError_t NPHC_CAT(launch_xy_track_f32w_m, NPHC_INST_M)(const XYSys &sys, cons
     return cudaGetLastError();
 }
 
+cudaError_t NPHC_CAT(launch_xy_track_far_batch_m, NPHC_INST_M)(const BatchGroup &bg, const XYCtl &ctl,
+                                                               cudaStream_t st) {
+    constexpr int M = NPHC_INST_M, WARPS = 4;
+    if (bg.total <= 0) return cudaSuccess;
+    far_list_batch_kernel<M><<<(int)((bg.total + 127) / 128), 128, 0, st>>>(bg.sys, bg.ep, bg.off, bg.n, bg.far + 1,
+                                                                            bg.far);
+    nphc_launch_counter(1);
+    cudaError_t e = cudaGetLastError();
+    constexpr auto k = xy_track_warp32_batch_kernel<M, WARPS>;
+    int sms = 0, per = 0;
+    if (e == cudaSuccess) e = device_sms(sms);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 32 * WARPS, 0);
+    if (e != cudaSuccess) return e;
+    const int64_t full = (int64_t)sms * std::max(per, 1), need = (bg.total + WARPS - 1) / WARPS;
+    k<<<(int)std::min(full, need), 32 * WARPS, 0, st>>>(bg.sys, bg.ep, bg.off, bg.n, ctl, bg.far + 1, bg.far,
+                                                        bg.far_queue);
+    nphc_launch_counter(1);
+    return cudaGetLastError();
+}
+
 // The FP32 pass has two kernels: one path per thread (xy_track_lane.cuh) and four lanes per path
 // (xy_track_group.cuh).  The first takes fewer instructions per path but one wave of it (38,912 paths
 // up to M = 8, where registers hold it to eight warps per SM, 34,048 at M = 9, 29,184 at M = 10)

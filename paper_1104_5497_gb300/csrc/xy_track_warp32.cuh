@@ -291,31 +291,37 @@ struct Warp32 {
     }
 };
 
-// Tracks the listed paths from t = 0; a list of max_paths or more is left to the per-thread kernel.  The
-// control flow (track_body's in FP32) is uniform over the warp.
-template <int M, int WARPS>
-__global__ void __launch_bounds__(32 * WARPS)
-    xy_track_warp32_kernel(const __grid_constant__ XYSys S, const __grid_constant__ XYCtl C,
-                           const __grid_constant__ EPView ep, const WorkList wl, int64_t max_paths) {
+// Tracks the listed paths from t = 0 (the control flow is track_body's in FP32, uniform over the
+// warp).  total: the list's length; src.take(q, inst, e) gives its entry q.
+template <int M, int WARPS, class Src>
+__device__ __forceinline__ void warp32_track_body(const Src &src, const XYCtl &C, int64_t total,
+                                                  unsigned long long *queue) {
     using L = Warp32Layout<M>;
     constexpr int NV = 2 * M;
     __shared__ cx<float> work[WARPS * L::TOTAL];
-    __shared__ float Js[M * NPHC_JSTRIDE];
-    const int64_t total = worklist_size(wl, ep.count);
-    if (total >= max_paths) return;
+    __shared__ float Js[WARPS * M * NPHC_JSTRIDE];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, i = lane;   // i: vector component
-    for (int k = threadIdx.x; k < M * NPHC_JSTRIDE; k += 32 * WARPS) Js[k] = S.Jf[k];
-    __syncthreads();
-    const Warp32<M> P{work + wid * L::TOTAL, Js, lane};
-    const cx<float> gam = {(float)S.gre, (float)S.gim};
+    float *const J = Js + wid * (M * NPHC_JSTRIDE);
+    const Warp32<M> P{work + wid * L::TOTAL, J, lane};
     const float eps = (float)C.eps, trust = (float)C.trust, scale = 0.70710678118654752440f;
+    int inst = 0, have = -1;   // the instance whose couplings are in J
+    cx<float> gam = {1.0f, 0.0f};
     for (;;) {
         unsigned long long take = 0;
-        if (lane == 0) take = atomicAdd(wl.queue, 1ull);
+        if (lane == 0) take = atomicAdd(queue, 1ull);
         take = __shfl_sync(0xffffffffu, take, 0);
         if ((int64_t)take >= total) break;
-        const int64_t e = worklist_entry(wl, (int64_t)take, ep.count);
+        int64_t e;
+        src.take((int64_t)take, inst, e);
         if (e < 0) continue;   // rejected by the debug build's check
+        if (inst != have) {
+            const XYSys &S = src.sys(inst);
+            for (int k = lane; k < M * NPHC_JSTRIDE; k += 32) J[k] = S.Jf[k];
+            gam = cx<float>{(float)S.gre, (float)S.gim};
+            have = inst;
+            __syncwarp();
+        }
+        const EPView &ep = src.eps(inst);
         P.start(ep.path[e], gam);
         double t = 0.0, h = C.h0, hacc = h, tck = 0.0, hck = 0.0, tmark = 1.0, zlast = 0.0;
         bool have_ck = false, far = false;
@@ -438,4 +444,51 @@ __global__ void __launch_bounds__(32 * WARPS)
         }
         __syncwarp();
     }
+}
+
+// One ring's list, when it is shorter than max_paths (longer ones are the per-thread kernel's).
+template <int M, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS)
+    xy_track_warp32_kernel(const __grid_constant__ XYSys S, const __grid_constant__ XYCtl C,
+                           const __grid_constant__ EPView ep, const WorkList wl, int64_t max_paths) {
+    const int64_t total = worklist_size(wl, ep.count);
+    if (total < max_paths) warp32_track_body<M, WARPS>(SingleSrc<XYSys>{S, ep, wl}, C, total, wl.queue);
+}
+
+// A batch group's: list[q] is an item of the group (BatchSrc).
+template <int M, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS)
+    xy_track_warp32_batch_kernel(const XYSys *__restrict__ sys, const EPView *__restrict__ eps,
+                                 const int64_t *__restrict__ off, int n, const __grid_constant__ XYCtl C,
+                                 const int32_t *list, const int32_t *count, unsigned long long *queue) {
+    struct Src : BatchSrc<XYSys> {
+        const int32_t *list;
+        __device__ __forceinline__ void take(int64_t q, int &g, int64_t &e) const {
+            BatchSrc<XYSys>::take(list[q], g, e);
+        }
+    };
+    Src src;
+    src.S = sys;
+    src.ep = eps;
+    src.off = off;
+    src.n = n;
+    src.list = list;
+    warp32_track_body<M, WARPS>(src, C, *count, queue);
+}
+
+// The items of a batch group that reached a far endpoint (launch_far_list for a batch).
+template <int M>
+__global__ void far_list_batch_kernel(const XYSys *__restrict__ sys, const EPView *__restrict__ eps,
+                                      const int64_t *__restrict__ off, int n, int32_t *list, int32_t *count) {
+    const BatchSrc<XYSys> src = {sys, eps, off, n};
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= src.total()) return;
+    int g;
+    int64_t e;
+    src.take(i, g, e);
+    if (e < 0 || eps[g].status[e] != NPHC_PATH_REACHED) return;
+    const EPView &ep = eps[g];
+    int ez = -2000;
+    for (int k = 0; k < 2 * M; k++) ez = max(ez, max(gexp(ep.z_re[k * ep.count + e]), gexp(ep.z_im[k * ep.count + e])));
+    if (ez >= sys[g].far_exp) list[atomicAdd(count, 1)] = (int32_t)i;   // every item once: at most total
 }

@@ -135,3 +135,23 @@ def test_short_and_long_lists_agree_bit_for_bit(N, count):
         if k == "steps" and N < 12:
             continue   # counts of the pass before, of either kernel, included
         assert np.array_equal(a[..., at], b[..., at]), k
+
+
+def test_batches_match_single_solves_at_far_endpoints():
+    """Rings of three sizes, two or more of each: a group's far paths are listed and tracked together."""
+    N_ = nphc()
+    rings = [ring(N_, N, seed) for N, seed in ((9, 1009), (8, 1017), (9, 1340), (8, 1034), (9, 1323), (6, 7))]
+    systems, opts = [r[0] for r in rings], [r[1] for r in rings]
+    opts[2].refine_eps = 2e-14   # a line of its own
+    batch = N_.Batch(systems)
+    far = 0
+    for flags in (0, N_.BATCH_GRAPH, N_.BATCH_GRAPH):   # eager, captured, replayed
+        batch.solve(opts, flags)
+        for k in range(len(rings)):
+            a, b = batch.result(k).endpoints(), N_.solve(systems[k], opts[k]).endpoints()
+            at = (b["status"] == N_.PATH_REACHED) & (np.maximum(abs(b["z"].real), abs(b["z"].imag)).max(axis=1) >= FAR)
+            far += int(at.sum())
+            assert np.array_equal(a["status"][at], b["status"][at])
+            assert np.array_equal(a["cls"][at], b["cls"][at]) and np.array_equal(a["z"][at], b["z"][at])
+            assert [a["cls"].tolist().count(c) for c in range(7)] == [b["cls"].tolist().count(c) for c in range(7)]
+    assert far >= 60
