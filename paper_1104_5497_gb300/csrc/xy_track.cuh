@@ -8,12 +8,13 @@
 // (xy_track_lane.cuh, xy_track_group.cuh), four lanes or a warp per path in FP64
 // (xy_track_group64.cuh, xy_track_warp.cuh).  This one runs
 //   * in FP64, on lists that ask for it (options.threads_per_path = 1);
-//   * in FP32, over the paths that a pass of the throughput kernels brought to a far endpoint
-//     (launch_far_list), and over resumed passes.  The certificate of a far endpoint is taken
+//   * in FP32, over resumed passes, and over the paths that a pass of the throughput kernels
+//     brought to a far endpoint (launch_far_list) when there are very many; fewer take its
+//     arithmetic with a warp per path (xy_track_warp32.cuh).  The certificate of a far endpoint is taken
 //     from the first Newton correction within refine_eps (1 + ||z||), which at ||z|| ~ 1e6 certifies
 //     or not depending on the last bits of the FP32 endpoint: one of two kernels of different
 //     rounding, chosen by the launch's size, would make the class of such a solution depend on
-//     the paths it is tracked with.  Measured over 48 samples of 20,011 paths of rings with
+//     the paths it is tracked with.  Over 48 samples of 20,011 paths of rings with
 //     N = 8 .. 13: 0.1% of the paths end beyond the line, and 18 of 169,326 certified
 //     endpoints had another class by the throughput kernels, all of them among these.
 //
